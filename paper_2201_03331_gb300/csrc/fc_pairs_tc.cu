@@ -157,12 +157,17 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1) k_pairs_tc(const __grid_cons
     const int prod = tc_producer_of(warp, a.producers);
     if (prod >= 0) {
         // ---------------- TMA producers ----------------
-        if (lane == 0) {
+        if (elect_one()) {
             const int P = a.producers;
-            uint32_t fill = 0;
-            // Last fill issued into each owned stage (at most two: stages prod
-            // and prod + P).
+            Ring ring;
+            int owner = 0;   // producer of stage ring.s
+            // Parity of the last fill issued into each owned stage (at most
+            // two: stages prod and prod + P), -1 before the first.
             int last0 = -1, last1 = -1;
+            auto step = [&]() {
+                ring.next(stages);
+                owner = ring.s == 0 || owner + 1 == P ? 0 : owner + 1;
+            };
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 const int slot = it % TC_SCHED;
@@ -176,15 +181,14 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1) k_pairs_tc(const __grid_cons
                 for (int c = 0; c < 2 && ok; ++c) {
                     const int nk = c ? kc1 : kc0;
                     const int xbase = c ? kc0 * TC_BK : 0;
-                    for (int kc = 0; kc < nk; ++kc, ++fill) {
-                        const int s = fill % stages;
-                        if (s % P != prod) continue;
-                        const uint32_t n = fill / stages;
-                        if (!mbar_wait(&bar_empty[s], (n & 1) ^ 1, abort_flag, a.err, a.wait_ticks)) { ok = false; break; }
+                    for (int kc = 0; kc < nk; ++kc, step()) {
+                        const int s = ring.s;
+                        if (owner != prod) continue;
+                        if (!mbar_wait(&bar_empty[s], ring.par ^ 1, abort_flag, a.err, a.wait_ticks)) { ok = false; break; }
                         mbar_expect_tx(&bar_full[s], TC_A_BYTES + TC_B_BYTES);
                         tma_load_2d(&tmap, &bar_full[s], stA + (size_t)s * TC_A_BYTES, xbase + kc * TC_BK, I * TC_BM);
                         tma_load_2d(&tmap, &bar_full[s], stB + (size_t)s * TC_B_BYTES, xbase + kc * TC_BK, J * TC_BN);
-                        if (s == prod) last0 = (int)fill; else last1 = (int)fill;
+                        if (s == prod) last0 = (int)ring.par; else last1 = (int)ring.par;
                     }
                 }
             }
@@ -192,18 +196,18 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1) k_pairs_tc(const __grid_cons
             // before the CTA can exit (earlier ones were consumed).
             for (int q = 0; q < 2; ++q) {
                 const int s = prod + q * P;
-                const int f = q ? last1 : last0;
-                if (s >= stages || f < 0) continue;
-                const uint32_t n = (uint32_t)f / stages;
+                const int par = q ? last1 : last0;
+                if (s >= stages || par < 0) continue;
                 long long t0 = clock64();
-                while (!mbar_try(&bar_full[s], n & 1) && clock64() - t0 < WAIT_BUDGET) {}
+                while (!mbar_try(&bar_full[s], (uint32_t)par) && clock64() - t0 < WAIT_BUDGET) {}
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- MMA issue ----------------
             const uint32_t idesc = idesc_e4m3_f32(TC_BM, TC_BN);
-            uint32_t fill = 0;
+            const uint64_t descA = smem_desc_sw128(smem_u32(stA)), descB = smem_desc_sw128(smem_u32(stB));
+            Ring ring;
             bool ok = true;
             // This thread also schedules the tiles, TC_LOOKAHEAD ahead of the
             // one it consumes (another lane of this warp spinning on the ring
@@ -239,18 +243,15 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1) k_pairs_tc(const __grid_cons
                 for (int c = 0; c < 2 && ok; ++c) {
                     const int nk = c ? kc1 : kc0;
                     const uint32_t d = tmem_base + (uint32_t)(b * 256 + c * 128);
-                    for (int kc = 0; kc < nk; ++kc, ++fill) {
-                        const int s = fill % stages;
-                        const uint32_t n = fill / stages;
-                        if (!mbar_wait(&bar_full[s], n & 1, abort_flag, a.err, a.wait_ticks)) { ok = false; break; }
+                    for (int kc = 0; kc < nk; ++kc, ring.next(stages)) {
+                        const int s = ring.s;
+                        if (!mbar_wait(&bar_full[s], ring.par, abort_flag, a.err, a.wait_ticks)) { ok = false; break; }
                         tc_fence_after();
-                        const uint32_t aaddr = smem_u32(stA + (size_t)s * TC_A_BYTES);
-                        const uint32_t baddr = smem_u32(stB + (size_t)s * TC_B_BYTES);
+                        const uint64_t ad = descA + (uint64_t)s * (TC_A_BYTES >> 4);
+                        const uint64_t bd = descB + (uint64_t)s * (TC_B_BYTES >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < TC_BK / 32; ++kk) {
-                            mma_e4m3(d, smem_desc_sw128(aaddr + kk * 32), smem_desc_sw128(baddr + kk * 32), idesc,
-                                     (kc > 0 || kk > 0) ? 1u : 0u);
-                        }
+                        for (int kk = 0; kk < TC_BK / 32; ++kk)
+                            mma_e4m3(d, ad + kk * 2, bd + kk * 2, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
                         mma_commit(&bar_empty[s]);
                     }
                 }

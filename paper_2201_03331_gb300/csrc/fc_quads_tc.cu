@@ -190,12 +190,17 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
     const int prod = tc_producer_of(warp, a.producers);
     if (prod >= 0) {
         // ---------------- TMA producers ----------------
-        if (lane == 0) {
+        if (elect_one()) {
             const int P = a.producers;
-            uint32_t fill = 0;
-            // Last fill issued into each owned stage (at most two: stages prod
-            // and prod + P).
+            Ring ring;
+            int owner = 0;   // producer of stage ring.s
+            // Parity of the last fill issued into each owned stage (at most
+            // two: stages prod and prod + P), -1 before the first.
             int last0 = -1, last1 = -1;
+            auto step = [&]() {
+                ring.next(stages);
+                owner = ring.s == 0 || owner + 1 == P ? 0 : owner + 1;
+            };
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 const int slot = it % TC_SCHED;
@@ -210,33 +215,32 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
                 // The chunks in the order the MMA thread takes them (the
                 // case chunks, then the control chunks: all of them).
                 const int nk = kc0 + kc1;
-                for (int kc = 0; kc < nk; ++kc, ++fill) {
-                    const int s = fill % stages;
-                    if (s % P != prod) continue;
-                    const uint32_t n = fill / stages;
-                    if (!mbar_wait(&bar_empty[s], (n & 1) ^ 1, abort_flag, a.err)) { ok = false; break; }
+                for (int kc = 0; kc < nk; ++kc, step()) {
+                    const int s = ring.s;
+                    if (owner != prod) continue;
+                    if (!mbar_wait(&bar_empty[s], ring.par ^ 1, abort_flag, a.err)) { ok = false; break; }
                     mbar_expect_tx(&bar_full[s], TC_A_BYTES + B_BYTES);
                     tma_load_2d(&tmapL, &bar_full[s], stA + (size_t)s * TC_A_BYTES, kc * TC_BK, rowL);
                     tma_load_2d(&tmapR, &bar_full[s], stB + (size_t)s * B_BYTES, kc * TC_BK, rowR);
-                    if (s == prod) last0 = (int)fill; else last1 = (int)fill;
+                    if (s == prod) last0 = (int)ring.par; else last1 = (int)ring.par;
                 }
             }
             // Let the last copies into the stages this producer owns land
             // before the CTA can exit (earlier ones were consumed).
             for (int q = 0; q < 2; ++q) {
                 const int s = prod + q * P;
-                const int f = q ? last1 : last0;
-                if (s >= stages || f < 0) continue;
-                const uint32_t n = (uint32_t)f / stages;
+                const int par = q ? last1 : last0;
+                if (s >= stages || par < 0) continue;
                 long long t0 = clock64();
-                while (!mbar_try(&bar_full[s], n & 1) && clock64() - t0 < WAIT_BUDGET) {}
+                while (!mbar_try(&bar_full[s], (uint32_t)par) && clock64() - t0 < WAIT_BUDGET) {}
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- MMA issue ----------------
             const uint32_t idesc = idesc_e4m3_f32(TC_BM, NB);
-            uint32_t fill = 0;
+            const uint64_t descA = smem_desc_sw128(smem_u32(stA)), descB = smem_desc_sw128(smem_u32(stB));
+            Ring ring;
             bool ok = true;
             // This thread also schedules the tiles, TC_LOOKAHEAD ahead of the
             // one it consumes (another lane of this warp spinning on the ring
@@ -310,21 +314,18 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
                 // ENC 0: case chunks into columns [0, 128), control chunks
                 // into [128, 256); ENC 1: every chunk into [0, 256).
                 const int nk = kc0 + kc1;
-                for (int kc = 0; kc < nk && ok; ++kc, ++fill) {
+                for (int kc = 0; kc < nk && ok; ++kc, ring.next(stages)) {
                     const bool ctrl = !ENC && kc >= kc0;
                     const int k0 = ctrl ? kc - kc0 : kc;   // chunk within its accumulator
                     const uint32_t d = tmem_base + (uint32_t)(b * 256 + (ctrl ? 128 : 0));
-                    const int s = fill % stages;
-                    const uint32_t n = fill / stages;
-                    if (!mbar_wait(&bar_full[s], n & 1, abort_flag, a.err)) { ok = false; break; }
+                    const int s = ring.s;
+                    if (!mbar_wait(&bar_full[s], ring.par, abort_flag, a.err)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t aaddr = smem_u32(stA + (size_t)s * TC_A_BYTES);
-                    const uint32_t baddr = smem_u32(stB + (size_t)s * B_BYTES);
+                    const uint64_t ad = descA + (uint64_t)s * (TC_A_BYTES >> 4);
+                    const uint64_t bd = descB + (uint64_t)s * (B_BYTES >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < TC_BK / 32; ++kk) {
-                        mma_e4m3(d, smem_desc_sw128(aaddr + kk * 32), smem_desc_sw128(baddr + kk * 32), idesc,
-                                 (k0 > 0 || kk > 0) ? 1u : 0u);
-                    }
+                    for (int kk = 0; kk < TC_BK / 32; ++kk)
+                        mma_e4m3(d, ad + kk * 2, bd + kk * 2, idesc, (k0 > 0 || kk > 0) ? 1u : 0u);
                     mma_commit(&bar_empty[s]);
                 }
                 if (ok) mma_commit(&bar_tfull[b]);

@@ -156,6 +156,39 @@ __device__ __forceinline__ void mma_e4m3(uint32_t tmem_d, uint64_t adesc, uint64
         : "memory");
 }
 
+// True on one lane of a converged warp.  The MMA and TMA issue loops run
+// under this predicate rather than under lane == 0: the compiler then knows
+// that one thread runs the branch and keeps descriptors and addresses in
+// uniform registers, which the tcgen05 and bulk-copy instructions take
+// directly.  Under lane == 0 every MMA first moved its operands there one by
+// one, and the issue alone took 136 cycles per MMA (128 x 240 x 64 in fp4, 120
+// cycles of tensor work; 172 with the waits and copies of the pipeline)
+// against 120 (both) under elect.sync, measured on GB300 over 6400 chunks.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// Position in a ring of n stages: stage s, and the parity of its current
+// fill (the pipeline's loops step it instead of dividing a fill count).
+struct Ring {
+    int s = 0;
+    uint32_t par = 0;
+    __device__ __forceinline__ void next(int n)
+    {
+        if (++s == n) {
+            s = 0;
+            par ^= 1;
+        }
+    }
+};
+
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(

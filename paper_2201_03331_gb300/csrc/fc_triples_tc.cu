@@ -282,10 +282,12 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             while (!mbar_try(&bar_full[w], last_n & 1) && clock64() - t0 < WAIT_BUDGET) {}
         }
     } else if (warp == 3) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- MMA issue ----------------
             const uint32_t idesc = idesc_f8_f32(TC_BM, Sh::NMMA, BATCH);
-            uint32_t fill = 0;
+            const uint64_t descA = smem_desc_sw128(smem_u32(smem));
+            const uint64_t descB = smem_desc_sw128(smem_u32(smem + TC_A_BYTES));
+            Ring ring;
             bool ok = true;
             int Wt = a.Wt, split = a.W0, cur_job = -1;
             // Scheduler state of a batched launch: the job of the last item
@@ -346,10 +348,9 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 const uint32_t u = (uint32_t)(it >> 1);
                 if (!mbar_wait(&bar_tempty[b], (u & 1) ^ 1, abort_flag, a.err, wt)) break;
                 tc_fence_after();
-                for (int kc = 0; kc < Wt; ++kc, ++fill) {
-                    const int s = (int)(fill % T3_LOADERS);
-                    const uint32_t n = fill / T3_LOADERS;
-                    if (!mbar_wait(&bar_full[s], n & 1, abort_flag, a.err, wt)) {
+                for (int kc = 0; kc < Wt; ++kc, ring.next(T3_LOADERS)) {
+                    const int s = ring.s;
+                    if (!mbar_wait(&bar_full[s], ring.par, abort_flag, a.err, wt)) {
                         ok = false;
                         break;
                     }
@@ -359,12 +360,11 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     const bool acc1 = ENC != 1 && kc >= split;
                     const uint32_t d = tmem_base + (uint32_t)(b * 256 + (acc1 ? 128 : 0));
                     const bool first = ENC == 1 ? kc == 0 : (kc == 0 || kc == split);
-                    const uint32_t aaddr = smem_u32(smem + (size_t)s * Sh::STAGE);
-                    const uint32_t baddr = aaddr + TC_A_BYTES;
+                    const uint64_t ad = descA + (uint64_t)s * (Sh::STAGE >> 4);
+                    const uint64_t bd = descB + (uint64_t)s * (Sh::STAGE >> 4);
 #pragma unroll
                     for (int kk = 0; kk < TC_BK / 32; ++kk)
-                        mma_e4m3(d, smem_desc_sw128(aaddr + kk * 32), smem_desc_sw128(baddr + kk * 32), idesc,
-                                 (!first || kk > 0) ? 1u : 0u);
+                        mma_e4m3(d, ad + kk * 2, bd + kk * 2, idesc, (!first || kk > 0) ? 1u : 0u);
                     mma_commit(&bar_empty[s]);
                 }
                 if (ok) mma_commit(&bar_tfull[b]);
