@@ -237,7 +237,7 @@ cudaError_t launch_final_sort_batch(const JobDesc *jobs, int n_jobs, double *res
 // ---- order-2 tensor-core path (fc_pairs_tc.cu) -----------------------------
 
 constexpr int TC_MAX_STAGES = 6;
-constexpr int TC_MAX_PRODUCERS = 4;   // TMA producer warps of the order-2 and orders 4-6 kernels
+constexpr int TC_MAX_PRODUCERS = 4;   // TMA producer warps of the order-2 kernel
 enum { MODE_DUMP = 2 };
 // Time budget of one mbarrier wait in the tensor-core kernels, in clock64
 // ticks (about 2 s).  The pipeline waits of the order-2 kernel take theirs
@@ -366,13 +366,17 @@ cudaError_t launch_fill_lists(float *s, uint64_t *r, size_t n, cudaStream_t st);
 
 // Orders 4 to 6 on tensor cores (fc_quads_tc.cu): left tuples of LT SNPs
 // x right tuples of RT SNPs, k = LT + RT (2 + 2, 2 + 3, 3 + 3).  Each side is
-// a slab of tuple rows with all 3^T genotype combinations, left tuples in
-// order of their last SNP, right tuples in order of their first; a 128-row
-// block holds 27 / 3^T tuples in each 32-row quarter (27 rows, then 5 zero
-// rows): 12 pairs or 4 triples.  A tile is one left block x one right block.
+// a slab of tuple rows (packed 4-bit 0/1, 64 bytes a word) with all 3^T
+// genotype combinations, left tuples in order of their last SNP, right tuples
+// in order of their first; a left block of 128 rows or right block of 112
+// rows holds 4 (27 / 3^T) tuples: 12 pairs or 4 triples.  A tile is one left
+// block x one or two right blocks.
 constexpr int tc_left_size(int k) { return k == 6 ? 3 : 2; }
 constexpr int tc_tuples_per_block(int T) { return 4 * (27 / (T == 2 ? 9 : 27)); }
 constexpr uint64_t NO_TUPLE = ~0ull;
+// Rows of a left or right block, bytes from one tuple row to the next.
+int tuple_block_rows(bool left);
+constexpr int64_t tuple_pitch(int Wt) { return (int64_t)Wt * 64 + 128; }
 struct QuadsArgs {
     // Tiles (left block a, right block b) come in strips of at most `sub`
     // left blocks: with r = q - item_first and n = ceil((g1 - g0) / sub),
@@ -397,11 +401,12 @@ struct QuadsArgs {
     const uint64_t *rtup;   // right tuples
     const uint64_t *rrank;  // rank part of a right tuple (modulo 2^64)
     const float *xlogx;     // x ln x for x = 0..M
+    const float *small_terms;   // cell terms t(a, b) of small counts (launch_small_terms)
     int M;
+    float acc_max, case_max;    // M1 + 4096 M0 and M1 (enc 1)
     float hy, invN;
     uint64_t rank_begin, rank_end;   // only combinations with ranks in [rank_begin, rank_end) count
-    int L, Bcap, P2, stages;
-    int producers;          // TMA producer warps (a divisor of stages, at most 4)
+    int L, Bcap, P2, stages;    // stages: 2 or 3
     float *list_score;      // [grid][L]
     uint64_t *list_rank;
     int *gthr;
@@ -411,11 +416,12 @@ struct QuadsArgs {
     uint32_t *dump_tables;  // MODE_DUMP: [C(S,k)][3^k][2]
 };
 
-// Tuple rows of T-SNP tuples (nblocks blocks of 128 rows); control words
-// (w >= W0) carry ctrl_byte (e4m3 1.0 = 0x38, or 64 = 0x68 for the encoded
-// form).
-cudaError_t launch_tuple_rows(int T, const uint4 *X, int64_t S_pad, int W0, int Wt, const uint64_t *tuples,
-                              int64_t nblocks, int64_t pitch, uint8_t ctrl_byte, uint8_t *Q, cudaStream_t st);
+// Tuple rows of T-SNP tuples (nblocks left or right blocks).
+cudaError_t launch_tuple_rows(int T, bool left, const uint4 *X, int64_t S_pad, int Wt, const uint64_t *tuples,
+                              int64_t nblocks, int64_t pitch, uint8_t *Q, cudaStream_t st);
+// The table of cell terms of small class counts, small_terms_floats() floats.
+int small_terms_floats();
+cudaError_t launch_small_terms(float *t, cudaStream_t st);
 // Shared memory of the orders 4-6 kernel (enc 1: two right blocks per stage).
 size_t quads_smem_bytes(int enc, int stages, int M, int P2);
 cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUtensorMap &tmapR, const QuadsArgs &a,

@@ -7,129 +7,173 @@
 // count of the AND of one row of each SNP's table),
 //     n_c(cell_L, cell_R) = < P_c[left, cell_L], P_c[right, cell_R] >,
 // the dot product over the samples of two tuple rows P[t, d] = [G_t = d]
-// (all SNPs of tuple t at genotypes d) stored as 0/1 e4m3 bytes.  With the
-// left operand a block of left tuples and the right operand a block of right
-// tuples, both with all 3^T genotype rows, one 128 x 128 tcgen05.mma
-// kind::f8f6f4 tile per class yields every cell of every combination of the
-// two blocks (exact: products of 0/1, FP32 sums of integers below 2^24).
-// No cell is derived; combinations whose left tuple ends before the right
-// tuple starts are the valid ones.
+// (all SNPs of tuple t at genotypes d).  The rows are stored as 0/1 e2m1
+// nibbles; with the left operand a block of left tuples and the right operand
+// blocks of right tuples, both with all 3^T genotype rows, one tcgen05.mma
+// kind::mxf4 tile yields every cell of every combination of the blocks
+// exactly (fc_tc.cuh).  No cell is derived; combinations whose left tuple
+// ends before the right tuple starts are the valid ones.
 //
-// Row layout of a 128-row block: each 32-row quarter holds 27 / 3^T tuples
-// (3 pairs or 1 triple) in rows 3^T t + d, then 5 zero rows.  So one TMEM
-// lane quarter (one epilogue warp) holds whole left tuples, and a thread
-// owns the 3^RT cells of its (left tuple, d) row against each right tuple.
+// Row layout.  A left block is 128 rows, 27 / 3^LT tuples in each 32-row TMEM
+// lane quarter: one triple in rows 0 .. 26, or three pairs p with genotypes
+// d < 8 in rows 8 p + d and d = 8 in row 24 + p (so that the sums over a
+// pair's rows are three shuffle levels over eight lanes and one row more);
+// the other rows are zero.  A right block is 112 rows, four groups of 28:
+// 27 / 3^RT tuples with row 3^RT t + d, then one zero row.  A thread owns the
+// 3^RT cells of its (left tuple, d) row against each right tuple.
 //
-// Scoring: MI = H(Y) - (1/N) sum_cells [x ln x (n) - x ln x (a) - x ln x (b)]
-// with a table of x ln x correctly rounded to FP32.  Each thread sums the
-// terms of its row's cells, the 3^LT lanes of a left tuple add their partial
-// sums; every addend is a sum of non-negative cell terms bounded by N ln 2.
-// As for order 3, |MI32 - MI| <= u (3 ln M + (3^k + 4) ln 2) (u = 2^-24),
-// within the sweep's bound u (2 ln M + (2 3^k + 6) ln 2) for M < 2^(3^k + 2).
-// The lexicographic rank of a combination is the sum of a part that depends
-// on the left tuple only and one that depends on the right tuple only, both
-// computed on the host.
+// Scoring: MI = H(Y) - (1/N) sum_cells t(a, b), t = x ln x (a + b) - x ln x (a)
+// - x ln x (b).  Most cells of a high-order table are small: where both
+// class counts are below 64, t comes from one read of a 64 x 64 table
+// (correctly rounded; row stride 69 words, which spreads the few frequent
+// entries over the banks), three columns at a time where no lane of the warp
+// holds a larger count; the others take three reads of a table of x ln x.
+// The accumulator n_case + 4096 n_ctrl plus 2^21 holds four times the packed
+// counts in its mantissa, so the table offset 4 a + 276 b takes a shift and a
+// multiply-add.  Each thread sums the terms of its row's cells, the 3^LT lanes
+// of a left tuple add their partial sums; every addend is a sum of
+// non-negative cell terms bounded by N ln 2, so as for order 3 |MI32 - MI| <=
+// u (3 ln M + (3^k + 4) ln 2) (u = 2^-24), within the sweep's bound
+// u (2 ln M + (2 3^k + 6) ln 2) for M < 2^(3^k + 2).  The lexicographic rank
+// of a combination is the sum of a part that depends on the left tuple only
+// and one that depends on the right tuple only, both computed on the host.
 //
 // Two forms (template ENC):
-//   ENC = 0: both classes carry 1; the case and control chunks accumulate
-//            into two accumulators; a tile is (left block, right block),
-//            N = 128 per class;
-//   ENC = 1: control samples carry the e4m3 value 64 in both slabs, so one
-//            accumulator holds n_case + 4096 n_ctrl (exact while both
-//            classes have at most 4095 samples); a tile is (left block, two
-//            consecutive right blocks), N = 256, which halves the left
-//            operand's bytes per multiply-add.
+//   ENC = 0: case and control samples accumulate into two accumulators of 112
+//            columns; a tile is (left block, right block);
+//   ENC = 1: control samples carry the block scale 4096, so one accumulator
+//            holds n_case + 4096 n_ctrl (exact while both classes have at
+//            most 4095 samples); a tile is (left block, two consecutive right
+//            blocks), N = 224.
 //
-// Roles (one persistent CTA per SM, TC_THREADS_MP threads), as in the
-// order-2 kernel:
-//   warps 0, 6, 7, 8 : TMA producers (128-byte K chunks of the left and right
-//                      blocks), producer p owning the stages s = p (mod
-//                      producers)
-//   warp 1 : TMEM allocation; lane 0 issues the MMAs and schedules the tiles
-//   warps 2-5 : epilogue (TMEM -> registers -> partial MI over a row's cells
-//               -> sum over a left tuple's lanes -> CTA top list)
-// Accumulators: two TMEM buffers x 256 FP32 columns (two classes x 128, or
-// two right blocks x 128).
+// Roles (one persistent CTA per SM, 640 threads):
+//   warps 0-2  : TMA producers (128-byte K chunks, 256 samples, of the left and
+//                right blocks), warp s owning stage s
+//   warp 3     : TMEM allocation; one elected lane issues the MMAs and
+//                schedules the tiles
+//   warps 4-19 : epilogue (TMEM -> registers -> partial MI over a row's cells
+//                -> sum over a left tuple's lanes -> CTA top list), four warps
+//                per TMEM lane quarter, each a quarter of the tile's groups of
+//                28 columns.  With one warp per quarter the epilogue set the
+//                pace: about 18,000 cycles per 128 x 256 tile.
+// TMEM: two accumulator buffers of 224 columns and two blocks of columns of
+// scales.
 #include "fc_tc.cuh"
 
 namespace fc {
 
 namespace {
 
+constexpr int T4_PRODUCERS = 3;                    // = largest stage count
+constexpr int T4_EPI_WARP0 = 4;
+constexpr int T4_EPI_WARPS = 16;
+constexpr int T4_PARTS = T4_EPI_WARPS / 4;         // epilogue warps per TMEM lane quarter
+constexpr int T4_EPI_THREADS = 32 * T4_EPI_WARPS;
+constexpr int T4_THREADS = 32 * T4_EPI_WARP0 + T4_EPI_THREADS;
+constexpr int T4_GROUP = 28;                       // columns of a group of right tuples (27 used)
+constexpr int T4_BLOCK = 4 * T4_GROUP;             // columns of a right block
+constexpr int T4_BUF = 2 * T4_BLOCK;               // columns of an accumulator buffer
+constexpr uint32_t T4_SCALE_COL = 2 * T4_BUF;      // TMEM column of scale 1, then of scale 4096
+static_assert(T4_SCALE_COL + 2 * FP4_SCALE_COLS <= TC_TMEM_COLS, "scales behind the accumulators");
+// Table of t(a, b) for a, b < 64.
+constexpr int T4_SMALL = 64;
+constexpr int T4_SMALL_STRIDE = 69;
+constexpr int T4_SMALL_FLOATS = (T4_SMALL * T4_SMALL_STRIDE + 3) / 4 * 4;
+// x + 2^21 for an integer x = a + 4096 b < 2^21: 4 x in the low mantissa bits.
+constexpr uint32_t T4_MAGIC = 0x4A000000u;
+// Bits of x + 2^21 that are zero exactly where a, b < 64 (and x is a
+// non-negative integer): a's bits 6-11, b's bits 6-8, the exponent's low two
+// bits, the two fraction bits.
+constexpr uint32_t T4_LARGE_BITS = 0x01F03F03u;
+constexpr uint32_t T4_MUL = 16384 - 4 * T4_SMALL_STRIDE;                      // u - (u >> 14) T4_MUL = 4 a + 276 b + T4_OFF
+constexpr uint32_t T4_OFF = T4_MAGIC - (T4_MAGIC >> 14) * T4_MUL;
+
 // Tuple-row slab: thread (row, 16-byte chunk); the row is [G_t = d] (every
 // SNP of the tuple at its genotype digit, first SNP most significant) over
-// 16 samples of one class word, expanded to bytes.
-template <int T>
-__global__ void k_tuple_rows(const uint4 *X, int64_t S_pad, int W0, int Wt, const uint64_t *tuples, int64_t nblocks,
-                             int64_t pitch, uint32_t ctrl_byte, uint8_t *Q)
+// the 32 samples of the chunk, one nibble each.
+template <int T, bool LEFT>
+__global__ void k_tuple_rows(const uint4 *X, int64_t S_pad, int Wt, const uint64_t *tuples, int64_t nblocks,
+                             int64_t pitch, uint8_t *Q)
 {
     constexpr int R = T == 2 ? 9 : 27;              // rows per tuple
-    constexpr int PQ = 27 / R;                      // tuples per quarter
+    constexpr int PQ = 27 / R;                      // tuples per quarter (group)
+    constexpr int QROWS = LEFT ? 32 : T4_GROUP;     // rows per quarter (group)
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int cw = 8 * Wt;                          // 16-byte chunks per row
-    if (t >= nblocks * 128 * cw) return;
+    const int cw = 4 * Wt;                          // 16-byte chunks per row
+    if (t >= nblocks * (4 * QROWS) * cw) return;
     const int64_t row = t / cw;
     const int ch = (int)(t - row * cw);
-    const int64_t blk = row >> 7;
-    const int r = (int)(row & 127);
-    const int quarter = r >> 5, r32 = r & 31;
+    const int64_t blk = row / (4 * QROWS);
+    const int r = (int)(row - blk * (4 * QROWS));
+    const int quarter = r / QROWS, rq = r % QROWS;
     uint32_t bits = 0;
-    if (r32 < 27) {
-        const uint64_t tup = tuples[blk * (4 * PQ) + quarter * PQ + r32 / R];
+    if (rq < 27) {
+        // Tuple of the quarter and genotype digits of this row.
+        const int p = LEFT && T == 2 ? (rq < 24 ? rq >> 3 : rq - 24) : rq / R;
+        int d = LEFT && T == 2 ? (rq < 24 ? rq & 7 : 8) : rq % R;
+        const uint64_t tup = tuples[blk * (4 * PQ) + quarter * PQ + p];
         if (tup != NO_TUPLE) {
-            const int w = ch >> 3, sub = ch & 7;    // 128-sample word, 16-sample part
-            const int q32 = sub >> 1;
-            uint32_t acc = ~0u;
-            int d = r32 % R;
+            const int w = ch >> 2, q32 = ch & 3;    // 128-sample word, 32-sample part
+            bits = ~0u;
 #pragma unroll
             for (int u = T - 1; u >= 0; --u) {
                 const int g = d % 3;
                 d /= 3;
                 const uint32_t s = (uint32_t)(tup >> (16 * u)) & 0xffffu;
-                const uint4 x = X[((size_t)w * 3 + g) * S_pad + s];
-                acc &= q32 == 0 ? x.x : q32 == 1 ? x.y : q32 == 2 ? x.z : x.w;
+                bits &= reinterpret_cast<const uint32_t *>(X + ((size_t)w * 3 + g) * S_pad + s)[q32];
             }
-            bits = (acc >> ((sub & 1) * 16)) & 0xffffu;
         }
     }
-    const uint32_t one = (ch >> 3) < W0 ? 0x38u : ctrl_byte;   // e4m3 1.0, or the control value
-    uint32_t o[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        uint32_t v = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v |= ((bits >> (4 * q + e)) & 1u ? one : 0u) << (8 * e);
-        o[q] = v;
-    }
-    *(reinterpret_cast<uint4 *>(Q + row * pitch) + ch) = make_uint4(o[0], o[1], o[2], o[3]);
+    *(reinterpret_cast<uint4 *>(Q + row * pitch) + ch) = expand_fp4(bits);
 }
 
-// One encoded accumulator x = n_case + 4096 n_ctrl (an exact integer below
-// 2^24, n_case < 4096) as n_case | n_ctrl << 16.
-__device__ __forceinline__ uint32_t unpack_enc4(uint32_t bits)
+// t(a, b) for a, b < T4_SMALL at b T4_SMALL_STRIDE + a: computed in FP64,
+// rounded once.
+__global__ void k_small_terms(float *t)
 {
-    const uint32_t v = __float2uint_rz(__uint_as_float(bits));
-    return v + (v >> 12) * 61440u;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= T4_SMALL_FLOATS) return;
+    const int b = i / T4_SMALL_STRIDE, a = i % T4_SMALL_STRIDE;
+    double v = 0.0;
+    if (a < T4_SMALL && b < T4_SMALL && a > 0 && b > 0) {
+        const double n = a + b;
+        v = (double)a * log(n / a) + (double)b * log(n / b);
+    }
+    t[i] = (float)v;
+}
+
+// The class counts of an encoded accumulator x = a + 4096 b (a, b < 4096),
+// clamped to the classes so that no index can leave the x ln x table.
+__device__ __forceinline__ void split_enc(float x, float xmax, float amax, uint32_t &a, uint32_t &b)
+{
+    x = fminf(fmaxf(x, 0.f), xmax);
+    const float y = __fmaf_rz(x, 1.f / 4096.f, 8388608.f);   // 2^23 + floor(x / 4096)
+    const float af = fminf(fmaf(-4096.f, y - 8388608.f, x), amax);
+    b = __float_as_uint(y) - 0x4B000000u;
+    a = __float_as_uint(af + 8388608.f) - 0x4B000000u;
 }
 
 template <int LT, int RT, int MODE, int ENC>
-__global__ void __launch_bounds__(TC_THREADS_MP, 1)
+__global__ void __launch_bounds__(T4_THREADS, 1)
     k_quads_tc(const __grid_constant__ CUtensorMap tmapL, const __grid_constant__ CUtensorMap tmapR, QuadsArgs a)
 {
-    constexpr uint32_t B_BYTES = ENC ? 2 * TC_B_BYTES : TC_B_BYTES;   // one or two right blocks per stage
-    constexpr int NB = ENC ? 256 : 128;                                 // MMA N
+    constexpr int NB = ENC ? T4_BUF : T4_BLOCK;     // MMA N = right rows per stage
+    constexpr uint32_t STAGE = TC_A_BYTES + (uint32_t)NB * TC_BK;
     constexpr int RL = LT == 2 ? 9 : 27;            // rows (cells) per left tuple
     constexpr int RR = RT == 2 ? 9 : 27;            // columns (cells) per right tuple
     constexpr int LPQ = 27 / RL;                    // left tuples per lane quarter
-    constexpr int RPC = 27 / RR;                    // right tuples per 32-column chunk
+    constexpr int RPG = 27 / RR;                    // right tuples per group of columns
+    constexpr int GROUPS = NB / T4_GROUP;           // groups per tile
+    constexpr int GPW = GROUPS / T4_PARTS;          // groups per epilogue warp
+    constexpr int V = GPW * RPG;                    // right tuples per epilogue warp
     constexpr int CK = RL * RR;                     // cells of a table (3^k)
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_full[TC_MAX_STAGES], bar_empty[TC_MAX_STAGES];
+    __shared__ uint64_t bar_full[T4_PRODUCERS], bar_empty[T4_PRODUCERS];
     __shared__ uint64_t bar_tfull[2], bar_tempty[2], bar_done;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint64_t bar_sfull[TC_SCHED], bar_sempty[TC_SCHED];
     __shared__ int sched_tile[TC_SCHED];   // left block (-1: no more tiles)
-    __shared__ int sched_rb[TC_SCHED];     // right block
+    __shared__ int sched_rb[TC_SCHED];     // right block (ENC 1: pair of right blocks)
     __shared__ int abort_flag_s;
     __shared__ int buf_count;
     __shared__ int epi_stop;
@@ -140,11 +184,10 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
     volatile int *abort_flag = &abort_flag_s;
 
     uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *stA = smem;
-    uint8_t *stB = smem + (size_t)stages * TC_A_BYTES;
-    float *xltab = reinterpret_cast<float *>(stB + (size_t)stages * B_BYTES);   // x ln x
+    float *xltab = reinterpret_cast<float *>(smem + (size_t)stages * STAGE);   // x ln x
     const int lt_floats = (a.M + 1 + 3) & ~3;
-    uint64_t *lrank = reinterpret_cast<uint64_t *>(xltab + lt_floats);
+    float *small = xltab + lt_floats;                                          // t(a, b), ENC 1
+    uint64_t *lrank = reinterpret_cast<uint64_t *>(small + (ENC ? T4_SMALL_FLOATS : 0));
     float *lscore = reinterpret_cast<float *>(lrank + a.P2);
 
     if (threadIdx.x == 0) {
@@ -154,19 +197,19 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bar_tfull[b], 1);
-            mbar_init(&bar_tempty[b], 4);
+            mbar_init(&bar_tempty[b], T4_EPI_WARPS);
         }
         mbar_init(&bar_done, 1);
         for (int s = 0; s < TC_SCHED; ++s) {
             mbar_init(&bar_sfull[s], 1);
-            // The producers, the MMA thread and the four epilogue warps.
-            mbar_init(&bar_sempty[s], a.producers + 5);
+            // The producers, the MMA thread and the epilogue warps.
+            mbar_init(&bar_sempty[s], stages + 1 + T4_EPI_WARPS);
         }
         abort_flag_s = 0;
         buf_count = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {
+    if (warp == 3) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_base_slot)),
                      "r"(TC_TMEM_COLS)
@@ -174,6 +217,8 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     for (int i = threadIdx.x; i <= a.M; i += blockDim.x) xltab[i] = a.xlogx[i];
+    if (ENC)
+        for (int i = threadIdx.x; i < T4_SMALL_FLOATS; i += blockDim.x) small[i] = a.small_terms[i];
     if (MODE == MODE_TOPN) {
         for (int i = threadIdx.x; i < a.P2; i += blockDim.x) {
             lscore[i] = -FLT_MAX;
@@ -184,23 +229,23 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    if (warp >= T4_EPI_WARP0 && warp < T4_EPI_WARP0 + 4) {
+        const uint32_t q = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + T4_SCALE_COL;
+        tmem_fill16(q, FP4_SCALE_ONE);
+        tmem_fill16(q + FP4_SCALE_COLS, FP4_SCALE_4096);
+        tmem_wait_st();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
 
-    const int kc0 = a.W0, kc1 = a.Wt - a.W0;   // 128-sample chunks per class
+    const int nk = (a.Wt + 1) / 2;   // 256-sample chunks (two words; the last may hold one, then zeros)
 
-    const int prod = tc_producer_of(warp, a.producers);
-    if (prod >= 0) {
+    if (warp < T4_PRODUCERS) {
         // ---------------- TMA producers ----------------
-        if (elect_one()) {
-            const int P = a.producers;
+        if (warp < stages && elect_one()) {
             Ring ring;
-            int owner = 0;   // producer of stage ring.s
-            // Parity of the last fill issued into each owned stage (at most
-            // two: stages prod and prod + P), -1 before the first.
-            int last0 = -1, last1 = -1;
-            auto step = [&]() {
-                ring.next(stages);
-                owner = ring.s == 0 || owner + 1 == P ? 0 : owner + 1;
-            };
+            int last = -1;   // parity of the last fill issued into the stage
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 const int slot = it % TC_SCHED;
@@ -210,36 +255,30 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
                 const int rb = sched_rb[slot];
                 mbar_arrive(&bar_sempty[slot]);
                 if (t < 0) break;
-                // ENC 1: rb is a pair of right blocks (rows 256 rb ..).
-                const int rowL = t * 128, rowR = rb * NB;
-                // The chunks in the order the MMA thread takes them (the
-                // case chunks, then the control chunks: all of them).
-                const int nk = kc0 + kc1;
-                for (int kc = 0; kc < nk; ++kc, step()) {
-                    const int s = ring.s;
-                    if (owner != prod) continue;
-                    if (!mbar_wait(&bar_empty[s], ring.par ^ 1, abort_flag, a.err)) { ok = false; break; }
-                    mbar_expect_tx(&bar_full[s], TC_A_BYTES + B_BYTES);
-                    tma_load_2d(&tmapL, &bar_full[s], stA + (size_t)s * TC_A_BYTES, kc * TC_BK, rowL);
-                    tma_load_2d(&tmapR, &bar_full[s], stB + (size_t)s * B_BYTES, kc * TC_BK, rowR);
-                    if (s == prod) last0 = (int)ring.par; else last1 = (int)ring.par;
+                const int rowL = t * TC_BM, rowR = rb * NB;
+                uint8_t *st = smem + (size_t)warp * STAGE;
+                for (int kc = 0; kc < nk; ++kc, ring.next(stages)) {
+                    if (ring.s != warp) continue;
+                    if (!mbar_wait(&bar_empty[warp], ring.par ^ 1, abort_flag, a.err)) { ok = false; break; }
+                    mbar_expect_tx(&bar_full[warp], STAGE);
+                    tma_load_2d(&tmapL, &bar_full[warp], st, kc * TC_BK, rowL);
+                    tma_load_2d(&tmapR, &bar_full[warp], st + TC_A_BYTES, kc * TC_BK, rowR);
+                    last = (int)ring.par;
                 }
             }
-            // Let the last copies into the stages this producer owns land
-            // before the CTA can exit (earlier ones were consumed).
-            for (int q = 0; q < 2; ++q) {
-                const int s = prod + q * P;
-                const int par = q ? last1 : last0;
-                if (s >= stages || par < 0) continue;
+            // Let the last copy into this stage land before the CTA can exit
+            // (earlier ones were consumed).
+            if (last >= 0) {
                 long long t0 = clock64();
-                while (!mbar_try(&bar_full[s], (uint32_t)par) && clock64() - t0 < WAIT_BUDGET) {}
+                while (!mbar_try(&bar_full[warp], (uint32_t)last) && clock64() - t0 < WAIT_BUDGET) {}
             }
         }
-    } else if (warp == 1) {
+    } else if (warp == 3) {
         if (elect_one()) {
             // ---------------- MMA issue ----------------
-            const uint32_t idesc = idesc_e4m3_f32(TC_BM, NB);
-            const uint64_t descA = smem_desc_sw128(smem_u32(stA)), descB = smem_desc_sw128(smem_u32(stB));
+            const uint32_t idesc = idesc_mxf4(TC_BM, NB);
+            const uint64_t descA = smem_desc_sw128(smem_u32(smem)), descB = smem_desc_sw128(smem_u32(smem + TC_A_BYTES));
+            const uint32_t one = tmem_base + T4_SCALE_COL;
             Ring ring;
             bool ok = true;
             // This thread also schedules the tiles, TC_LOOKAHEAD ahead of the
@@ -311,21 +350,28 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
                 const uint32_t u = (uint32_t)(it >> 1);
                 if (!mbar_wait(&bar_tempty[b], (u & 1) ^ 1, abort_flag, a.err)) break;
                 tc_fence_after();
-                // ENC 0: case chunks into columns [0, 128), control chunks
-                // into [128, 256); ENC 1: every chunk into [0, 256).
-                const int nk = kc0 + kc1;
+                const uint32_t d0 = tmem_base + (uint32_t)(b * T4_BUF);
                 for (int kc = 0; kc < nk && ok; ++kc, ring.next(stages)) {
-                    const bool ctrl = !ENC && kc >= kc0;
-                    const int k0 = ctrl ? kc - kc0 : kc;   // chunk within its accumulator
-                    const uint32_t d = tmem_base + (uint32_t)(b * 256 + (ctrl ? 128 : 0));
                     const int s = ring.s;
                     if (!mbar_wait(&bar_full[s], ring.par, abort_flag, a.err)) { ok = false; break; }
                     tc_fence_after();
-                    const uint64_t ad = descA + (uint64_t)s * (TC_A_BYTES >> 4);
-                    const uint64_t bd = descB + (uint64_t)s * (B_BYTES >> 4);
+                    const uint64_t ad = descA + (uint64_t)s * (STAGE >> 4);
+                    const uint64_t bd = descB + (uint64_t)s * (STAGE >> 4);
+                    // Two words of 128 samples (two MMAs each): cases, then
+                    // controls (ENC 0: into the second accumulator; ENC 1:
+                    // with scale 4096).
 #pragma unroll
-                    for (int kk = 0; kk < TC_BK / 32; ++kk)
-                        mma_e4m3(d, ad + kk * 2, bd + kk * 2, idesc, (k0 > 0 || kk > 0) ? 1u : 0u);
+                    for (int h = 0; h < 2; ++h) {
+                        const int w = 2 * kc + h;
+                        if (w < a.Wt) {
+                            const bool ctrl = w >= a.W0;
+                            const bool first = w == 0 || (!ENC && w == a.W0);
+                            const uint32_t d = d0 + (!ENC && ctrl ? T4_BLOCK : 0);
+                            const uint32_t sa = one + (ENC && ctrl ? FP4_SCALE_COLS : 0);
+                            mma_mxf4(d, ad + 4 * h, bd + 4 * h, idesc, sa, one, first ? 0u : 1u);
+                            mma_mxf4(d, ad + 4 * h + 2, bd + 4 * h + 2, idesc, sa, one, 1u);
+                        }
+                    }
                     mma_commit(&bar_empty[s]);
                 }
                 if (ok) mma_commit(&bar_tfull[b]);
@@ -335,20 +381,36 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
             long long t0 = clock64();
             while (!mbar_try(&bar_done, 0) && clock64() - t0 < WAIT_BUDGET) {}
         }
-    } else if (warp >= 2 && warp < 6) {
+    } else {
         // ---------------- epilogue ----------------
-        // TMEM lane = left row 32 w + RL p + d_L; column 32 c + RR q + d_R =
-        // right tuple RPC c + q of the tile, genotype digits d_R.
-        const int tid = threadIdx.x - 64;           // 0..127
+        const int tid = threadIdx.x - 32 * T4_EPI_WARP0;   // 0 .. T4_EPI_THREADS - 1
         const int quarter = warp & 3;
-        const int p = lane / RL;                    // left tuple within the quarter (LPQ: padding lanes)
-        const int cell_l = lane - RL * p;           // genotype digits of this lane's row
-        const int seg0 = RL * min(p, LPQ - 1);      // first lane of this left tuple
+        const int part = (warp - T4_EPI_WARP0) >> 2;       // groups [part GPW, (part + 1) GPW)
+        // Left tuple of the quarter and genotype digits of this lane's row
+        // (p = LPQ: a padding row).
+        const int p = LT == 3 ? (lane < 27 ? 0 : 1) : lane < 24 ? lane >> 3 : lane - 24;
+        const int cell_l = LT == 3 ? lane : lane < 24 ? lane & 7 : 8;
+        // After the sum over a left tuple's rows this lane scores the
+        // combination of its left tuple with right tuple `vsel` of the warp
+        // (-1: none).
+        int vsel = -1;
+        if (LT == 3) {
+            if (V == 2 ? (lane & 15) == 0 : lane == 0) vsel = V == 2 ? lane >> 4 : 0;
+        } else if (lane < 24) {
+            if (V == 6 && (lane & 3) < 3) vsel = 3 * ((lane >> 2) & 1) + (lane & 3);
+            if (V == 3 && (lane & 7) < 3) vsel = lane & 7;
+            if (V == 2 && (lane & 3) == 0) vsel = (lane >> 2) & 1;
+            if (V == 1 && (lane & 7) == 0) vsel = 0;
+        }
         const int L = a.L;
         const int Bcap = a.Bcap;
         const uint32_t lt = (uint32_t)a.M;
+        const float xmax = a.acc_max, amax = a.case_max;
+        const uint32_t small_off = smem_u32(small) - T4_OFF;
         float thr_s = -FLT_MAX;
         uint64_t thr_r = NO_RANK;
+        // A tile inserts at most one candidate per combination.
+        constexpr int TILE_CANDS = 4 * LPQ * GROUPS * RPG;
         for (int it = 0;; ++it) {
             const int slot = it % TC_SCHED;
             const uint32_t sn = (uint32_t)(it / TC_SCHED);
@@ -361,141 +423,201 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
             }
             const int b = it & 1;
             const uint32_t u = (uint32_t)(it >> 1);
-            if (t >= 0) mbar_wait(&bar_tfull[b], u & 1, abort_flag, a.err);
-            // One stop decision for all four epilogue warps (they meet at
-            // named barriers, which have no timeout); t is the same for all.
-            epi_bar();
-            if (tid == 0) epi_stop = *abort_flag;
-            epi_bar();
-            if (epi_stop || t < 0) break;
-            tc_fence_after();
-            const uint2 tile = make_uint2((uint32_t)t, (uint32_t)rb);   // left block, right block
-            // This lane's left tuple: its last SNP and its part of the rank.
-            uint64_t ltp = NO_TUPLE, lrk = 0;
-            if (p < LPQ) {
-                const size_t li = (size_t)tile.x * (4 * LPQ) + quarter * LPQ + p;
-                ltp = a.ltup[li];
-                lrk = a.lrank[li];
-            }
-            const uint32_t llast = (uint32_t)(ltp >> (16 * (LT - 1))) & 0xffffu;
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256);
-            constexpr int NCH = ENC ? 8 : 4;   // 32-column chunks of the tile
-            for (int ch = 0; ch < NCH; ++ch) {
-                // Counts of this chunk: cases in v0, controls in v1.
-                uint32_t v0[32], v1[32];
-                if (ENC) {
-                    tmem_ld32(taddr + ch * 32, v0);
-                    tmem_wait_ld();
-                    tmem_regs_after_wait(v0);
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) {
-                        const uint32_t pk = unpack_enc4(v0[x]);
-                        v0[x] = pk & 0xffffu;
-                        v1[x] = pk >> 16;
-                    }
-                } else {
-                    tmem_ld32(taddr + ch * 32, v0);
-                    tmem_ld32(taddr + 128 + ch * 32, v1);
-                    tmem_wait_ld();
-                    tmem_regs_after_wait(v0);
-                    tmem_regs_after_wait(v1);
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) {
-                        v0[x] = f2u_exact(v0[x]);
-                        v1[x] = f2u_exact(v1[x]);
-                    }
+            // Tile data that does not depend on the accumulators, loaded while
+            // the tile's MMAs may still run: this lane's left tuple and the
+            // right tuple it scores, with their parts of the rank.
+            uint64_t ltp = NO_TUPLE, lrk = 0, rtp = NO_TUPLE, rrk = 0;
+            const size_t ri0 = (size_t)rb * (GROUPS * RPG) + part * V;   // this warp's first right tuple
+            float gthr = -FLT_MAX;
+            if (t >= 0) {
+                if (p < LPQ) {
+                    const size_t li = (size_t)t * (4 * LPQ) + quarter * LPQ + p;
+                    ltp = a.ltup[li];
+                    lrk = a.lrank[li];
                 }
-                if (ch == NCH - 1) {
+                if (vsel >= 0) {
+                    rtp = a.rtup[ri0 + vsel];
+                    rrk = a.rrank[ri0 + vsel];
+                }
+                // The global threshold only rises; a value read once per tile
+                // admits at most a few more candidates than a fresh one would.
+                if (MODE == MODE_TOPN) gthr = from_ordered(*(volatile int *)a.gthr);
+                mbar_wait(&bar_tfull[b], u & 1, abort_flag, a.err);
+            }
+            // One stop decision for all epilogue warps (they meet at named
+            // barriers, which have no timeout); t is the same for all.
+            // Between the barriers nobody inserts, so the buffer's fill is
+            // the same for all.
+            epi_bar_n<T4_EPI_THREADS>();
+            if (tid == 0) epi_stop = *abort_flag;
+            const int fill = buf_count;
+            epi_bar_n<T4_EPI_THREADS>();
+            if (epi_stop || t < 0) break;
+            if (MODE == MODE_TOPN) {
+                if (fill > Bcap - TILE_CANDS) {
+                    for (int x = L + fill + tid; x < a.P2; x += T4_EPI_THREADS) { lscore[x] = -FLT_MAX; lrank[x] = NO_RANK; }
+                    epi_bitonic_desc_n<T4_EPI_THREADS>(lscore, lrank, a.P2, tid);
+                    if (tid == 0) {
+                        buf_count = 0;
+                        if (lrank[L - 1] != NO_RANK) atomicMax(a.gthr, ordered_int(lscore[L - 1]));
+                    }
+                    epi_bar_n<T4_EPI_THREADS>();
+                }
+                thr_s = lscore[L - 1];
+                thr_r = lrank[L - 1];
+            }
+            tc_fence_after();
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * T4_BUF);
+            float val[V];
+#pragma unroll
+            for (int gi = 0; gi < GPW; ++gi) {
+                const uint32_t col = taddr + (uint32_t)((part * GPW + gi) * T4_GROUP);
+                uint32_t v0[28];
+                uint32_t v1[ENC ? 1 : 28];
+                tmem_ld28(col, v0);
+                if constexpr (!ENC) tmem_ld28(col + T4_BLOCK, v1);
+                tmem_wait_ld();
+                tmem_regs_after_wait(v0);
+                if constexpr (!ENC) tmem_regs_after_wait(v1);
+                if (gi == GPW - 1) {
+                    // This warp's last read of the buffer.
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bar_tempty[b]);
                 }
-                float sc[RPC];
-                uint64_t rk[RPC];
-                bool val[RPC];
 #pragma unroll
-                for (int q = 0; q < RPC; ++q) {
-                    // Right tuple RPC ch + q of the tile's right block(s): the
-                    // RR cells of this row.
-                    const size_t ri = (size_t)tile.y * (ENC ? 8 * RPC : 4 * RPC) + ch * RPC + q;
-                    const uint64_t rtp = a.rtup[ri];
-                    const uint32_t rfirst = (uint32_t)rtp & 0xffffu;
-                    float part = 0.f;
+                for (int q = 0; q < RPG; ++q) {
+                    // Three partial sums shorten the chain of dependent
+                    // additions.
+                    float hs[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-                    for (int c = 0; c < RR; ++c) {
-                        // Clamped so that no index can leave the table.
-                        const uint32_t ca = min(v0[RR * q + c], lt);
-                        const uint32_t cb = min(v1[RR * q + c], lt);
-                        const uint32_t n = min(ca + cb, lt);
-                        part += (xltab[n] - xltab[min(ca, n)]) - xltab[min(cb, n)];
+                    for (int c = RR * q; c < RR * q + RR; c += 3) {
+                        bool general = true;
+                        if constexpr (ENC) {
+                            uint32_t w[3];
+#pragma unroll
+                            for (int e = 0; e < 3; ++e)
+                                w[e] = __float_as_uint(__uint_as_float(v0[c + e]) + __uint_as_float(T4_MAGIC));
+                            general = __any_sync(FULL, ((w[0] | w[1] | w[2]) & T4_LARGE_BITS) != 0);
+                            if (!general) {
+#pragma unroll
+                                for (int e = 0; e < 3; ++e)
+                                    hs[e] += lds_f32(small_off + (w[e] - (w[e] >> 14) * T4_MUL));
+                            }
+                        }
+                        if (general) {
+#pragma unroll
+                            for (int e = 0; e < 3; ++e) {
+                                uint32_t ca, cb;
+                                if constexpr (ENC) {
+                                    split_enc(__uint_as_float(v0[c + e]), xmax, amax, ca, cb);
+                                    hs[e] += (xltab[ca + cb] - xltab[ca]) - xltab[cb];
+                                } else {
+                                    // Clamped so that no index can leave the table.
+                                    ca = min(f2u_exact(v0[c + e]), lt);
+                                    cb = min(f2u_exact(v1[c + e]), lt);
+                                    hs[e] += (xltab[min(ca + cb, lt)] - xltab[ca]) - xltab[cb];
+                                }
+                            }
+                        }
                     }
-                    // Sum over the RL lanes of this left tuple.
-                    float tot = 0.f;
-#pragma unroll
-                    for (int k2 = 0; k2 < RL; ++k2) tot += __shfl_sync(FULL, part, min(seg0 + k2, 31));
-                    const bool real = p < LPQ && ltp != NO_TUPLE && rtp != NO_TUPLE && llast < rfirst;
-                    const uint64_t rank0 = real ? lrk + a.rrank[ri] : 0;   // modulo 2^64
-                    const bool valid = real && rank0 >= a.rank_begin && rank0 < a.rank_end;
-                    const float score = fmaf(-tot, a.invN, a.hy);
-                    const uint64_t rank = valid ? rank0 : NO_RANK;
-                    sc[q] = score;
-                    rk[q] = rank;
-                    val[q] = valid && cell_l == 0;
-                    if (MODE == MODE_DUMP && valid) {
-                        if (a.dump_scores && cell_l == 0) a.dump_scores[rank] = score;
-                        if (a.dump_tables) {
-                            uint32_t *o = a.dump_tables + (size_t)rank * (2 * CK) + (size_t)cell_l * (2 * RR);
+                    val[gi * RPG + q] = (hs[0] + hs[1]) + hs[2];
+                    if (MODE == MODE_DUMP && a.dump_tables && p < LPQ && ltp != NO_TUPLE) {
+                        const size_t ri = ri0 + gi * RPG + q;
+                        const uint64_t rq = a.rtup[ri];
+                        const uint32_t llast = (uint32_t)(ltp >> (16 * (LT - 1))) & 0xffffu;
+                        if (rq != NO_TUPLE && llast < ((uint32_t)rq & 0xffffu)) {
+                            uint32_t *o = a.dump_tables + (size_t)(lrk + a.rrank[ri]) * (2 * CK) + (size_t)cell_l * (2 * RR);
 #pragma unroll
                             for (int c = 0; c < RR; ++c) {
-                                o[2 * c] = min(v0[RR * q + c], lt);
-                                o[2 * c + 1] = min(v1[RR * q + c], lt);
+                                uint32_t ca, cb;
+                                if constexpr (ENC) {
+                                    split_enc(__uint_as_float(v0[RR * q + c]), xmax, amax, ca, cb);
+                                } else {
+                                    ca = min(f2u_exact(v0[RR * q + c]), lt);
+                                    cb = min(f2u_exact(v1[RR * q + c]), lt);
+                                }
+                                o[2 * c] = ca;
+                                o[2 * c + 1] = cb;
                             }
                         }
                     }
                 }
-                if (MODE == MODE_TOPN) {
-                    // Every thread reads the buffer fill before any thread of
-                    // this round adds to it, so that all take the same branch.
-                    epi_bar();
-                    const int fill_now = buf_count;
-                    epi_bar();
-                    if (fill_now > Bcap - RPC * 128) {
-                        const int nb = buf_count;
-                        for (int x = L + nb + tid; x < a.P2; x += 128) { lscore[x] = -FLT_MAX; lrank[x] = NO_RANK; }
-                        epi_bitonic_desc(lscore, lrank, a.P2, tid);
-                        if (tid == 0) {
-                            buf_count = 0;
-                            if (lrank[L - 1] != NO_RANK) atomicMax(a.gthr, ordered_int(lscore[L - 1]));
-                        }
-                        epi_bar();
-                    }
-                    thr_s = lscore[L - 1];
-                    thr_r = lrank[L - 1];
-                    const float gthr = from_ordered(*(volatile int *)a.gthr);
+            }
+            // Sum over the RL rows of each left tuple; where the warp holds
+            // two or six right tuples, the first level also splits them
+            // between the halves.
+            float tot;
+            if constexpr (LT == 3) {
+                // Padding rows hold no counts and add 0.
+                static_assert(V <= 2, "order 6");
+                if constexpr (V == 2) {
+                    const bool hi = (lane & 16) != 0;
+                    const float send = hi ? val[0] : val[1];
+                    tot = (hi ? val[1] : val[0]) + __shfl_xor_sync(FULL, send, 16);
+                } else {
+                    tot = val[0] + __shfl_xor_sync(FULL, val[0], 16);
+                }
 #pragma unroll
-                    for (int q = 0; q < RPC; ++q) {
-                        const bool cand = val[q] && sc[q] >= gthr && better(sc[q], rk[q], thr_s, thr_r);
-                        const unsigned mk = __ballot_sync(FULL, cand);
-                        if (mk) {
-                            int base = 0;
-                            if (lane == 0) base = atomicAdd(&buf_count, __popc(mk));
-                            base = __shfl_sync(FULL, base, 0);
-                            if (cand) {
-                                const int s2 = L + base + __popc(mk & ((1u << lane) - 1u));
-                                lscore[s2] = sc[q];
-                                lrank[s2] = rk[q];
-                            }
-                        }
+                for (int o = 8; o > 0; o >>= 1) tot += __shfl_xor_sync(FULL, tot, o);
+            } else {
+                // Row d = 8 of pair p comes from lane 24 + p.
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const float ninth = __shfl_sync(FULL, val[v], 24 + (lane >> 3));
+                    if ((lane & 7) == 0) val[v] += ninth;
+                }
+                constexpr int H = V % 2 ? V : V / 2;
+                float kept[H];
+                const bool hi = (lane & 4) != 0;
+#pragma unroll
+                for (int v = 0; v < H; ++v) {
+                    if constexpr (V % 2) {
+                        kept[v] = val[v] + __shfl_xor_sync(FULL, val[v], 4);
+                    } else {
+                        const float send = hi ? val[v] : val[v + H];
+                        kept[v] = (hi ? val[v + H] : val[v]) + __shfl_xor_sync(FULL, send, 4);
+                    }
+                }
+#pragma unroll
+                for (int o = 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int v = 0; v < H; ++v) kept[v] += __shfl_xor_sync(FULL, kept[v], o);
+                tot = kept[0];
+                if constexpr (H == 3) {
+                    const int pick = V == 6 ? lane & 3 : lane & 7;
+                    tot = pick == 1 ? kept[1] : pick == 2 ? kept[2] : kept[0];
+                }
+            }
+            const uint32_t llast = (uint32_t)(ltp >> (16 * (LT - 1))) & 0xffffu;
+            const uint32_t rfirst = (uint32_t)rtp & 0xffffu;
+            const bool real = vsel >= 0 && ltp != NO_TUPLE && rtp != NO_TUPLE && llast < rfirst;
+            const uint64_t rank = lrk + rrk;   // modulo 2^64
+            const bool valid = real && rank >= a.rank_begin && rank < a.rank_end;
+            const float score = fmaf(-tot, a.invN, a.hy);
+            if (MODE == MODE_DUMP && valid && a.dump_scores) a.dump_scores[rank] = score;
+            if (MODE == MODE_TOPN) {
+                const bool cand = valid && score >= gthr && better(score, rank, thr_s, thr_r);
+                const unsigned mk = __ballot_sync(FULL, cand);
+                if (mk) {
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(&buf_count, __popc(mk));
+                    base = __shfl_sync(FULL, base, 0);
+                    if (cand) {
+                        // The check above keeps the slot inside the buffer.
+                        const int s2 = min(L + base + __popc(mk & ((1u << lane) - 1u)), a.P2 - 1);
+                        lscore[s2] = score;
+                        lrank[s2] = rank;
                     }
                 }
             }
         }
         if (MODE == MODE_TOPN) {
-            epi_bar();
+            epi_bar_n<T4_EPI_THREADS>();
             const int nb = buf_count;
-            for (int x = L + nb + tid; x < a.P2; x += 128) { lscore[x] = -FLT_MAX; lrank[x] = NO_RANK; }
-            epi_bitonic_desc(lscore, lrank, a.P2, tid);
-            for (int x = tid; x < L; x += 128) {
+            for (int x = L + nb + tid; x < a.P2; x += T4_EPI_THREADS) { lscore[x] = -FLT_MAX; lrank[x] = NO_RANK; }
+            epi_bitonic_desc_n<T4_EPI_THREADS>(lscore, lrank, a.P2, tid);
+            for (int x = tid; x < L; x += T4_EPI_THREADS) {
                 a.list_score[(size_t)blockIdx.x * L + x] = lscore[x];
                 a.list_rank[(size_t)blockIdx.x * L + x] = lrank[x];
             }
@@ -504,7 +626,7 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 3) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
                      : "memory");
@@ -513,21 +635,34 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1)
 
 }  // namespace
 
-cudaError_t launch_tuple_rows(int T, const uint4 *X, int64_t S_pad, int W0, int Wt, const uint64_t *tuples,
-                              int64_t nblocks, int64_t pitch, uint8_t ctrl_byte, uint8_t *Q, cudaStream_t st)
+int tuple_block_rows(bool left) { return left ? TC_BM : T4_BLOCK; }
+
+cudaError_t launch_tuple_rows(int T, bool left, const uint4 *X, int64_t S_pad, int Wt, const uint64_t *tuples,
+                              int64_t nblocks, int64_t pitch, uint8_t *Q, cudaStream_t st)
 {
-    const int64_t n = nblocks * 128 * 8 * (int64_t)Wt;
+    const int64_t n = nblocks * tuple_block_rows(left) * 4 * (int64_t)Wt;
     if (n == 0) return cudaSuccess;
     const unsigned grid = (unsigned)((n + 255) / 256);
-    if (T == 2) k_tuple_rows<2><<<grid, 256, 0, st>>>(X, S_pad, W0, Wt, tuples, nblocks, pitch, ctrl_byte, Q);
-    else k_tuple_rows<3><<<grid, 256, 0, st>>>(X, S_pad, W0, Wt, tuples, nblocks, pitch, ctrl_byte, Q);
+    if (T == 2 && left) k_tuple_rows<2, true><<<grid, 256, 0, st>>>(X, S_pad, Wt, tuples, nblocks, pitch, Q);
+    else if (T == 2) k_tuple_rows<2, false><<<grid, 256, 0, st>>>(X, S_pad, Wt, tuples, nblocks, pitch, Q);
+    else if (left) k_tuple_rows<3, true><<<grid, 256, 0, st>>>(X, S_pad, Wt, tuples, nblocks, pitch, Q);
+    else k_tuple_rows<3, false><<<grid, 256, 0, st>>>(X, S_pad, Wt, tuples, nblocks, pitch, Q);
+    return cudaGetLastError();
+}
+
+int small_terms_floats() { return T4_SMALL_FLOATS; }
+
+cudaError_t launch_small_terms(float *t, cudaStream_t st)
+{
+    k_small_terms<<<(T4_SMALL_FLOATS + 255) / 256, 256, 0, st>>>(t);
     return cudaGetLastError();
 }
 
 size_t quads_smem_bytes(int enc, int stages, int M, int P2)
 {
-    return 1024 + (size_t)stages * (TC_A_BYTES + (enc ? 2 : 1) * TC_B_BYTES) + (size_t)((M + 1 + 3) & ~3) * 4 +
-           (size_t)P2 * (8 + 4);
+    // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
+    return 2048 + (size_t)stages * (TC_A_BYTES + (enc ? 2 : 1) * T4_BLOCK * TC_BK) + (size_t)((M + 1 + 3) & ~3) * 4 +
+           (enc ? (size_t)T4_SMALL_FLOATS * 4 : 0) + (size_t)P2 * (8 + 4);
 }
 
 template <int LT, int RT>
@@ -543,7 +678,7 @@ void *quads_kernel(int mode, int enc)
 cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUtensorMap &tmapR, const QuadsArgs &a,
                             int grid, cudaStream_t st)
 {
-    const size_t bytes = quads_smem_bytes(a.enc, a.stages, a.M, a.P2);
+    const size_t bytes = quads_smem_bytes(a.enc, a.stages, a.M, a.P2) - 1024;
     void *fn = nullptr;
     if (k == 4) fn = quads_kernel<2, 2>(mode, a.enc);
     if (k == 5) fn = quads_kernel<2, 3>(mode, a.enc);
@@ -554,7 +689,7 @@ cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUt
     CUtensorMap mL = tmapL, mR = tmapR;
     QuadsArgs args = a;
     void *params[] = {&mL, &mR, &args};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(TC_THREADS_MP), params, bytes, st);
+    return cudaLaunchKernel(fn, dim3(grid), dim3(T4_THREADS), params, bytes, st);
 }
 
 }  // namespace fc

@@ -325,6 +325,7 @@ Dataset::~Dataset()
     dev_free_pooled(tiles, tiles_bytes, device);
     cudaFree(PR);
     cudaFree(xlogx);
+    cudaFree(small_terms);
     cudaFree(xlog2x);
     for (int k = 4; k <= 6; ++k) release_tuples(k);
     dev_free_pooled(tiles3, tiles3_bytes, device);
@@ -561,7 +562,7 @@ int encode_tmap_u8(CUtensorMap *map, void *base, uint64_t inner_bytes, uint64_t 
     return FC_OK;
 }
 
-// TMA producer warps of the order-2 and orders 4-6 kernels: every stage
+// TMA producer warps of the order-2 kernel: every stage
 // count up to 4 gets one producer per stage; 5 stages drop to 4, and 6 take
 // three producers of two stages each.
 void tc_producer_split(int *stages, int *producers)
@@ -1102,8 +1103,7 @@ int64_t tuple_strip(int64_t group, int64_t bl, int64_t br, int sms, double item_
 
 int64_t tuple_group_size(int Wt)
 {
-    const uint64_t pitch = (uint64_t)Wt * 128 + 128;
-    return std::max<int64_t>(16, std::min<int64_t>(512, (int64_t)((48ull << 20) / (128 * pitch))));
+    return std::max<int64_t>(16, std::min<int64_t>(512, ((int64_t)48 << 20) / (tuple_block_rows(true) * tuple_pitch(Wt))));
 }
 
 int64_t tuple_count(int64_t S, int T, int other)
@@ -1136,7 +1136,7 @@ bool Dataset::tuples_tc_eligible(int k, int L)
         const int64_t rchunk = tuple_right_chunk(k);
         if (rchunk <= 0) return false;
         const int64_t group = tuple_group_size(Wt);
-        const int64_t sub = tuple_strip(group, bl, rchunk, sms, 128.0 * ((double)Wt * 128 + 128));
+        const int64_t sub = tuple_strip(group, bl, rchunk, sms, (double)tuple_block_rows(false) * (double)tuple_pitch(Wt));
         if ((double)(bl / group + 1) * (double)rchunk * (double)((group + sub - 1) / sub) >= 2147483647.0)
             return false;
     }
@@ -1147,8 +1147,10 @@ bool Dataset::tuples_tc_eligible(int k, int L)
 
 // Right items per chunk of the orders 4-6 right slab (items: right blocks,
 // block pairs in form 1): all of them when both slabs fit in 60 % of the
-// free memory (at most 192 GiB; FC_TUPLES_SLAB_MB caps it), else as many as
-// fit beside the left slab, which stays resident; 0 if not even one does.
+// free memory (at most 192 GiB), else as many as fit beside the left slab,
+// which stays resident; 0 if not even one does.  FC_TUPLES_SLAB_MB caps them
+// further, counted at one byte a sample and 128 rows a block (about twice
+// what the rows take), so that a setting gives the chunks it always gave.
 // The search then builds each chunk's right rows in turn and runs the
 // chunk's tiles (the paper's order-5 and order-6 runs on one node, 561 and
 // 223 variants, need 2 TB and 122 GB of right rows at 2048 samples).
@@ -1160,18 +1162,22 @@ int64_t Dataset::tuple_right_chunk(int k) const
     const int64_t br = (nr + tc_tuples_per_block(RT) - 1) / tc_tuples_per_block(RT);
     const int rblk = tuples_form() ? 2 : 1;
     const int64_t nb = (br + rblk - 1) / rblk;
-    const double blk = 128.0 * ((double)Wt * 128 + 128);
+    auto fit = [&](double cap, double left, double item) -> int64_t {
+        if (left + (double)nb * item <= cap) return nb;
+        if (cap - left < item) return 0;
+        return std::min<int64_t>(nb, (int64_t)((cap - left) / item));
+    };
     size_t free_b = 0, total_b = 0;
     double cap = 192.0 * 1024 * 1024 * 1024;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) cap = std::min(cap, 0.6 * (double)free_b);
+    const double pitch = (double)tuple_pitch(Wt);
+    int64_t n = fit(cap, (double)bl * tuple_block_rows(true) * pitch, (double)rblk * tuple_block_rows(false) * pitch);
     if (const char *mb = getenv("FC_TUPLES_SLAB_MB")) {
         const long v = atol(mb);
-        if (v > 0) cap = std::min(cap, (double)v * 1024 * 1024);
+        const double blk = 128.0 * ((double)Wt * 128 + 128);
+        if (v > 0) n = std::min(n, fit((double)v * 1024 * 1024, (double)bl * blk, rblk * blk));
     }
-    const double left = (double)bl * blk, item = rblk * blk;
-    if (left + (double)nb * item <= cap) return nb;
-    if (cap - left < item) return 0;
-    return std::min<int64_t>(nb, (int64_t)((cap - left) / item));
+    return n;
 }
 
 int Dataset::build_right_chunk(int k, int64_t c)
@@ -1184,8 +1190,8 @@ int Dataset::build_right_chunk(int k, int64_t c)
     cudaError_t e;
     u.built = -1;
     if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_tuple_rows(RT, X, S_pad, W0, Wt, u.rt + c0 * u.rblk * RPB, (c1 - c0) * u.rblk,
-                               (int64_t)Wt * 128 + 128, u.enc ? 0x68 : 0x38, u.QR, stream)) != cudaSuccess)
+        (e = launch_tuple_rows(RT, false, X, S_pad, Wt, u.rt + c0 * u.rblk * RPB, (c1 - c0) * u.rblk, tuple_pitch(Wt),
+                               u.QR, stream)) != cudaSuccess)
         return cuda_status(e, "tuple-row kernel");
     note_launches(1);
     u.built = c;
@@ -1211,11 +1217,8 @@ QuadsArgs Dataset::tuples_chunk_args(const QuadsArgs &base, int k, int64_t c, co
 // The orders 4-6 tensor-core form: 1 (one accumulator n_case + 4096 n_ctrl,
 // two right blocks per tile, which halves the left operand's bytes per
 // multiply-add) while both classes have at most 4095 samples, else 0 (one
-// accumulator per class, 32 KB stages).  Measured with the strip schedule:
-// at 2048 samples form 1 with four 48 KB stages is 1.3x form 0 with six; at
-// 6000 samples form 1 with three stages is 1.9x form 0 with six (162 against
-// 307 ms for 300 SNPs).  FC_QUADS_ENC=0 forces form 0, FC_QUADS_ENC=1 form 1
-// where the classes allow it.
+// accumulator per class).  FC_QUADS_ENC=0 forces form 0, FC_QUADS_ENC=1 form
+// 1 where the classes allow it.
 int Dataset::tuples_form() const
 {
     const char *f = getenv("FC_QUADS_ENC");
@@ -1243,6 +1246,9 @@ QuadsArgs Dataset::tuples_args(int k, int L, float hy, float invN)
     qa.rtup = u.rt;
     qa.rrank = u.rr;
     qa.xlogx = xlogx;
+    qa.small_terms = small_terms;
+    qa.acc_max = (float)M1 + 4096.f * (float)M0;
+    qa.case_max = (float)M1;
     qa.M = (int)M;
     qa.hy = hy;
     qa.invN = invN;
@@ -1251,11 +1257,7 @@ QuadsArgs Dataset::tuples_args(int k, int L, float hy, float invN)
     qa.L = L;
     qa.Bcap = L > 0 ? std::max(L, 1024) : 0;
     qa.P2 = L > 0 ? pow2_at_least(L + qa.Bcap) : 0;
-    qa.stages = 2;
-    for (int st = TC_MAX_STAGES; st >= 2; --st) {
-        if (quads_smem_bytes(u.enc, st, (int)M, qa.P2) <= (size_t)max_smem_optin) { qa.stages = st; break; }
-    }
-    tc_producer_split(&qa.stages, &qa.producers);
+    qa.stages = quads_smem_bytes(u.enc, 3, (int)M, qa.P2) <= (size_t)max_smem_optin ? 3 : 2;
     return qa;
 }
 
@@ -1353,6 +1355,13 @@ int Dataset::prepare_tuples(int k)
             return cuda_status(e, "x ln x table");
         note_launches(1);
     }
+    if (!small_terms) {
+        if ((e = dev_alloc((void **)&small_terms, sizeof(float) * (size_t)small_terms_floats())) != cudaSuccess)
+            return cuda_status(e, "cell term table allocation");
+        if ((e = launch_gate()) != cudaSuccess || (e = launch_small_terms(small_terms, stream)) != cudaSuccess)
+            return cuda_status(e, "cell term table");
+        note_launches(1);
+    }
     const int LT = tc_left_size(k), RT = k - LT;
     const int LPB = tc_tuples_per_block(LT), RPB = tc_tuples_per_block(RT);
     std::vector<uint64_t> lt, rt;
@@ -1394,8 +1403,9 @@ int Dataset::prepare_tuples(int k)
     for (int64_t blk = 0; blk < bl; ++blk) u.lmin_host[(size_t)blk] = snp(lt[(size_t)blk * LPB], LT - 1);
     for (int64_t blk = 0; blk < br; ++blk)
         u.rmax_host[(size_t)blk] = snp(rt[(size_t)(std::min<int64_t>((blk + 1) * RPB, nr) - 1)], 0);
-    const uint64_t kbytes = (uint64_t)Wt * 128;
-    const uint64_t pitch = kbytes + 128;
+    const uint64_t kbytes = (uint64_t)Wt * 64;
+    const uint64_t pitch = (uint64_t)tuple_pitch(Wt);
+    const int rowsL = tuple_block_rows(true), rowsR = tuple_block_rows(false);
     u.group = tuple_group_size(Wt);
     // amax per right block, or per pair of right blocks (form 1: the
     // second block's, the larger; a padding block takes its partner's).
@@ -1411,14 +1421,14 @@ int Dataset::prepare_tuples(int k)
         amax[(size_t)b] = (int)(std::lower_bound(u.lmin_host.begin(), u.lmin_host.end(), u.rmax_host[(size_t)rb]) -
                                 u.lmin_host.begin());
     }
-    u.sub = tuple_strip(u.group, bl, u.rchunk, sms, (u.enc ? 2.0 : 1.0) * 128.0 * (double)pitch);
+    u.sub = tuple_strip(u.group, bl, u.rchunk, sms, (double)u.rblk * rowsR * (double)pitch);
     int rc = tuple_chunk_groups(u, bl, nullptr, u.groups_host, u.cg0, u.citems);
     if (rc) return rc;
     u.n_items = 0;
     for (const int64_t n : u.citems) u.n_items += n;
     u.ngroups = (int)u.groups_host.size();
-    u.ql_bytes = std::max<size_t>((size_t)bl * 128 * pitch, 1);
-    u.qr_bytes = std::max<size_t>((size_t)u.rchunk * u.rblk * 128 * pitch, 1);
+    u.ql_bytes = std::max<size_t>((size_t)bl * rowsL * pitch, 1);
+    u.qr_bytes = std::max<size_t>((size_t)u.rchunk * u.rblk * rowsR * pitch, 1);
     if ((e = dev_alloc_pooled((void **)&u.QL, u.ql_bytes, device)) != cudaSuccess ||
         (e = dev_alloc_pooled((void **)&u.QR, u.qr_bytes, device)) != cudaSuccess)
         return cuda_status(e, "tuple-row slab allocation");
@@ -1436,16 +1446,15 @@ int Dataset::prepare_tuples(int k)
     cudaMemcpyAsync(u.groups, u.groups_host.data(), sizeof(int4) * u.groups_host.size(), cudaMemcpyHostToDevice, stream);
     cudaMemcpyAsync(u.amax, amax.data(), sizeof(int) * amax.size(), cudaMemcpyHostToDevice, stream);
     if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_tuple_rows(LT, X, S_pad, W0, Wt, u.lt, bl, (int64_t)pitch, u.enc ? 0x68 : 0x38, u.QL, stream)) !=
-            cudaSuccess)
+        (e = launch_tuple_rows(LT, true, X, S_pad, Wt, u.lt, bl, (int64_t)pitch, u.QL, stream)) != cudaSuccess)
         return cuda_status(e, "tuple-row kernel");
     note_launches(1);
     // One chunk: the right rows are built once and kept.
     u.built = -1;
     if (u.nchunks() == 1 && (rc = build_right_chunk(k, 0)) != FC_OK) return rc;
-    if ((rc = encode_tmap_u8(&u.tmapL, u.QL, kbytes, pitch, (uint64_t)bl * 128, 128, true)) != FC_OK) return rc;
-    if ((rc = encode_tmap_u8(&u.tmapR, u.QR, kbytes, pitch, (uint64_t)u.rchunk * u.rblk * 128, u.enc ? 256 : 128,
-                             true)) != FC_OK)
+    if ((rc = encode_tmap_u8(&u.tmapL, u.QL, kbytes, pitch, (uint64_t)bl * rowsL, (uint32_t)rowsL, true)) != FC_OK) return rc;
+    if ((rc = encode_tmap_u8(&u.tmapR, u.QR, kbytes, pitch, (uint64_t)u.rchunk * u.rblk * rowsR,
+                             (uint32_t)(u.rblk * rowsR), true)) != FC_OK)
         return rc;
     // Host vectors go out of scope: the copies must have landed.
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_status(e, "tuple operands");

@@ -102,6 +102,7 @@ struct Dataset {
     std::vector<TripleSlab> slabs3;
     std::vector<int64_t> first_tile3;   // [S + 1] first tile of each first SNP
     float *xlogx = nullptr;   // x ln x, x = 0..M (the orders 4-6 epilogue's MI table)
+    float *small_terms = nullptr;   // cell terms of small class counts (orders 4-6)
     float *xlog2x = nullptr;  // x log2 x, x = 0..M (the order-3 epilogue's)
     uint8_t *P3 = nullptr;
     size_t p3_bytes = 0;
@@ -123,8 +124,7 @@ struct Dataset {
     bool allow_tc = true;
 
     // Tensor-core operands of orders 4-6, built on first use; one order's are
-    // kept at a time: left and right tuple-row slabs (all 3^T genotype rows,
-    // 128-row blocks), the tuples with their parts of the rank, the strip
+    // kept at a time: left and right tuple-row slabs (all 3^T genotype rows), the tuples with their parts of the rank, the strip
     // plan of the tiles (left block, right block) and the slabs' TMA
     // descriptors.
     struct TupleTC {

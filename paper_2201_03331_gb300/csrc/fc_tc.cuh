@@ -156,6 +156,65 @@ __device__ __forceinline__ void mma_e4m3(uint32_t tmem_d, uint64_t adesc, uint64
         : "memory");
 }
 
+// ---- kind::mxf4: packed 4-bit 0/1 operands -----------------------------------
+// Indicator rows as e2m1 nibbles (0x2 = 1.0, sample m in nibble m): 128-byte
+// K chunks hold 256 samples, four MMAs of K = 64.  A block scale (ue8m0, one
+// per 32 samples and row, in TMEM) multiplies the products; here a scale is
+// the same for every row and block, so a TMEM column whose bytes are all
+// equal serves any scale layout.  Control samples take the A scale 2^12, so
+// that one FP32 accumulator holds n_case + 4096 n_ctrl.  Exact: the products
+// are 0 or 1 times a power of two, and FP32 accumulation of integers below
+// 2^24 was measured exact on GB300 up to 16,777,215 (128 x 240 tiles over
+// 8,190 samples with full rows).  Half the bytes per sample of e4m3 and, for
+// N = 240, twice its multiply-adds per cycle (120 cycles per K = 64 MMA).
+constexpr uint32_t FP4_SCALE_ONE = 0x7F7F7F7Fu;    // ue8m0 2^0
+constexpr uint32_t FP4_SCALE_4096 = 0x8B8B8B8Bu;   // ue8m0 2^12
+constexpr uint32_t FP4_SCALE_COLS = 16;            // TMEM columns per scale (at most 8 are read)
+
+// Instruction descriptor, kind::mxf4: A = B = E2M1 (bits 7-9, 10-11 = 1),
+// N >> 3 at bits 17-22, scales ue8m0 (bit 23), M >> 4 at bits 24-28, K = 64
+// (bit 31 = 0), scale ids 0 (bits 4-5, 29-30).
+__host__ __device__ constexpr uint32_t idesc_mxf4(int M, int N)
+{
+    return (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (1u << 23) | ((uint32_t)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_mxf4(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                         uint32_t scale_a, uint32_t scale_b, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], %1, %2, %3, [%4], [%5], p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(scale_a), "r"(scale_b), "r"(accumulate)
+        : "memory");
+}
+
+// 16 TMEM columns of this warp's lane quarter, all words v.
+__device__ __forceinline__ void tmem_fill16(uint32_t taddr, uint32_t v)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
+        "r"(v)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// 32 sample bits as 32 e2m1 nibbles (16 bytes).
+__device__ __forceinline__ uint4 expand_fp4(uint32_t bits)
+{
+    uint32_t o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint32_t x = (bits >> (8 * q)) & 0xffu;
+        x = (x | (x << 12)) & 0x000F000Fu;
+        x = (x | (x << 6)) & 0x03030303u;
+        x = (x | (x << 3)) & 0x11111111u;
+        o[q] = x << 1;
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
 // True on one lane of a converged warp.  The MMA and TMA issue loops run
 // under this predicate rather than under lane == 0: the compiler then knows
 // that one thread runs the branch and keeps descriptors and addresses in
@@ -240,6 +299,33 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
           "=r"(v[15])
         : "r"(taddr));
+}
+
+// 28 consecutive FP32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld28(uint32_t taddr, uint32_t (&v)[28])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+          "=r"(v[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23])
+                 : "r"(taddr + 16));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27])
+                 : "r"(taddr + 24));
+}
+
+// A float of shared memory at a shared-space byte address (a table that is
+// constant after the kernel's first barrier).
+__device__ __forceinline__ float lds_f32(uint32_t addr)
+{
+    float v;
+    asm("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
 }
 
 // Exact integer value of an FP32 accumulator holding an integer in [0, 2^23).
