@@ -370,16 +370,19 @@ cudaError_t launch_fill_lists(float *s, uint64_t *r, size_t n, cudaStream_t st);
 // genotype combinations, left tuples in order of their last SNP, right tuples
 // in order of their first; a left block of 128 rows or right block of 112
 // rows holds 4 (27 / 3^T) tuples: 12 pairs or 4 triples.  A tile is one left
-// block x one or two right blocks.
+// block x one right block (form 0) or two x two (form 1).
 constexpr int tc_left_size(int k) { return k == 6 ? 3 : 2; }
 constexpr int tc_tuples_per_block(int T) { return 4 * (27 / (T == 2 ? 9 : 27)); }
 constexpr uint64_t NO_TUPLE = ~0ull;
 // Rows of a left or right block, bytes from one tuple row to the next.
 int tuple_block_rows(bool left);
+// Blocks that the tiles of a form take together, on either side.
+constexpr int tuple_tile_blocks(int enc) { return enc ? 2 : 1; }
 constexpr int64_t tuple_pitch(int Wt) { return (int64_t)Wt * 64 + 128; }
 struct QuadsArgs {
-    // Tiles (left block a, right block b) come in strips of at most `sub`
-    // left blocks: with r = q - item_first and n = ceil((g1 - g0) / sub),
+    // Tiles (left block a, right block b; enc 1: pairs of consecutive left and
+    // of right blocks in place of blocks) come in strips of at most `sub` left
+    // blocks: with r = q - item_first and n = ceil((g1 - g0) / sub),
     // item q of the launch is (group g, right block b = lo + r / n, strip
     // r % n) of the group {g0, g1, lo, item_first} with the first
     // item_first <= q, and its tiles are the left blocks a in
@@ -387,10 +390,10 @@ struct QuadsArgs {
     // with include[a] set, if include is not null).  Within a group the right
     // blocks stream while the group's left blocks stay in L2; consecutive
     // items share a right block, so the CTAs in flight hold few of them.
-    const int4 *groups;     // by item_first (enc 1: right block pairs in place of right blocks)
+    const int4 *groups;     // by item_first
     int ngroups;
     int sub;
-    int enc;                // 1: one accumulator n_case + 4096 n_ctrl, two right blocks per tile
+    int enc;                // 1: one accumulator n_case + 4096 n_ctrl, tiles of CTA pairs
     int n_items;
     const int *amax;        // [right blocks]: left blocks whose smallest last SNP is below the block's largest first SNP
     const uint8_t *include;
@@ -406,7 +409,7 @@ struct QuadsArgs {
     float acc_max, case_max;    // M1 + 4096 M0 and M1 (enc 1)
     float hy, invN;
     uint64_t rank_begin, rank_end;   // only combinations with ranks in [rank_begin, rank_end) count
-    int L, Bcap, P2, stages;    // stages: 2 or 3
+    int L, Bcap, P2, stages;    // stages: 2 .. TC_MAX_STAGES
     float *list_score;      // [grid][L]
     uint64_t *list_rank;
     int *gthr;
@@ -422,7 +425,7 @@ cudaError_t launch_tuple_rows(int T, bool left, const uint4 *X, int64_t S_pad, i
 // The table of cell terms of small class counts, small_terms_floats() floats.
 int small_terms_floats();
 cudaError_t launch_small_terms(float *t, cudaStream_t st);
-// Shared memory of the orders 4-6 kernel (enc 1: two right blocks per stage).
+// Shared memory of the orders 4-6 kernel.
 size_t quads_smem_bytes(int enc, int stages, int M, int P2);
 cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUtensorMap &tmapR, const QuadsArgs &a,
                             int grid, cudaStream_t st);

@@ -40,17 +40,25 @@
 //
 // Two forms (template ENC):
 //   ENC = 0: case and control samples accumulate into two accumulators of 112
-//            columns; a tile is (left block, right block);
+//            columns; a tile is (left block, right block), one CTA each;
 //   ENC = 1: control samples carry the block scale 4096, so one accumulator
 //            holds n_case + 4096 n_ctrl (exact while both classes have at
-//            most 4095 samples); a tile is (left block, two consecutive right
-//            blocks), N = 224.
+//            most 4095 samples); a tile is (two left blocks, two right
+//            blocks), worked on by a pair of CTAs (cta_group::2, M = 256, N =
+//            224): each CTA loads one left and one right block and scores
+//            its left block against both right blocks.  With 128-row tiles
+//            per CTA the copies of both right blocks set the pace (44 KB a
+//            chunk and CTA at 65 bytes a cycle, the same with the scoring
+//            left out); the pair loads 30 KB.
 //
 // Roles (one persistent CTA per SM, 640 threads):
-//   warps 0-2  : TMA producers (128-byte K chunks, 256 samples, of the left and
-//                right blocks), warp s owning stage s
-//   warp 3     : TMEM allocation; one elected lane issues the MMAs and
-//                schedules the tiles
+//   warps 0, 1 : TMA producers (128-byte K chunks, 256 samples, of the left and
+//                right blocks), warp w owning the stages s = w (mod 2)
+//   warp 2     : one lane (ENC 1: of the pair's leader) schedules the tiles
+//   warp 3     : TMEM allocation; one elected lane (ENC 1: of the pair's
+//                leader) issues the MMAs.  With the scheduling in the same
+//                thread, the tensor cores idled about 700 cycles between
+//                tiles (3,584 cycles of MMAs at 2,048 samples)
 //   warps 4-19 : epilogue (TMEM -> registers -> partial MI over a row's cells
 //                -> sum over a left tuple's lanes -> CTA top list), four warps
 //                per TMEM lane quarter, each a quarter of the tile's groups of
@@ -64,7 +72,7 @@ namespace fc {
 
 namespace {
 
-constexpr int T4_PRODUCERS = 3;                    // = largest stage count
+constexpr int T4_PRODUCERS = 2;
 constexpr int T4_EPI_WARP0 = 4;
 constexpr int T4_EPI_WARPS = 16;
 constexpr int T4_PARTS = T4_EPI_WARPS / 4;         // epilogue warps per TMEM lane quarter
@@ -157,8 +165,9 @@ template <int LT, int RT, int MODE, int ENC>
 __global__ void __launch_bounds__(T4_THREADS, 1)
     k_quads_tc(const __grid_constant__ CUtensorMap tmapL, const __grid_constant__ CUtensorMap tmapR, QuadsArgs a)
 {
-    constexpr int NB = ENC ? T4_BUF : T4_BLOCK;     // MMA N = right rows per stage
-    constexpr uint32_t STAGE = TC_A_BYTES + (uint32_t)NB * TC_BK;
+    constexpr bool PAIR = ENC == 1;                 // a tile per CTA pair
+    constexpr int NB = ENC ? T4_BUF : T4_BLOCK;     // MMA N
+    constexpr uint32_t STAGE = TC_A_BYTES + (uint32_t)T4_BLOCK * TC_BK;   // one left and one right block
     constexpr int RL = LT == 2 ? 9 : 27;            // rows (cells) per left tuple
     constexpr int RR = RT == 2 ? 9 : 27;            // columns (cells) per right tuple
     constexpr int LPQ = 27 / RL;                    // left tuples per lane quarter
@@ -168,12 +177,13 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
     constexpr int V = GPW * RPG;                    // right tuples per epilogue warp
     constexpr int CK = RL * RR;                     // cells of a table (3^k)
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_full[T4_PRODUCERS], bar_empty[T4_PRODUCERS];
+    __shared__ uint64_t bar_full[TC_MAX_STAGES], bar_empty[TC_MAX_STAGES];
     __shared__ uint64_t bar_tfull[2], bar_tempty[2], bar_done;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint64_t bar_sfull[TC_SCHED], bar_sempty[TC_SCHED];
-    __shared__ int sched_tile[TC_SCHED];   // left block (-1: no more tiles)
-    __shared__ int sched_rb[TC_SCHED];     // right block (ENC 1: pair of right blocks)
+    // Left and right block of each slot of the ring (ENC 1: pairs of blocks;
+    // left block -1: no more tiles).
+    __shared__ __align__(8) int2 sched_tile[TC_SCHED];
     __shared__ int abort_flag_s;
     __shared__ int buf_count;
     __shared__ int epi_stop;
@@ -181,6 +191,7 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int stages = a.stages;
+    const uint32_t crank = PAIR ? cluster_rank() : 0;   // CTA of the pair (0: its leader)
     volatile int *abort_flag = &abort_flag_s;
 
     uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -197,24 +208,33 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bar_tfull[b], 1);
-            mbar_init(&bar_tempty[b], T4_EPI_WARPS);
+            mbar_init(&bar_tempty[b], (PAIR ? 2 : 1) * T4_EPI_WARPS);
         }
         mbar_init(&bar_done, 1);
         for (int s = 0; s < TC_SCHED; ++s) {
             mbar_init(&bar_sfull[s], 1);
-            // The producers, the MMA thread and the epilogue warps.
-            mbar_init(&bar_sempty[s], stages + 1 + T4_EPI_WARPS);
+            // The MMA thread, and the producers and epilogue warps (of both
+            // CTAs of a pair).
+            mbar_init(&bar_sempty[s], 1 + (PAIR ? 2 : 1) * (T4_PRODUCERS + T4_EPI_WARPS));
         }
         abort_flag_s = 0;
         buf_count = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 3) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tmem_base_slot)),
-                     "r"(TC_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_slot)),
+                         "r"(TC_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_slot)),
+                         "r"(TC_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     for (int i = threadIdx.x; i <= a.M; i += blockDim.x) xltab[i] = a.xlogx[i];
     if (ENC)
@@ -236,56 +256,86 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
         tmem_wait_st();
     }
     tc_fence_before();
-    __syncthreads();
+    // Barriers and scales of both CTAs are ready before either uses them.
+    if constexpr (PAIR) cluster_sync(); else __syncthreads();
     tc_fence_after();
+
+    // A consumer's word that it has read a slot of the tile ring.
+    const uint32_t sempty0 = PAIR ? cluster_addr(&bar_sempty[0], 0) : 0;
+    auto slot_read = [&](int slot) {
+        if constexpr (PAIR) mbar_arrive_cluster(sempty0 + 8 * slot);
+        else mbar_arrive(&bar_sempty[slot]);
+    };
 
     const int nk = (a.Wt + 1) / 2;   // 256-sample chunks (two words; the last may hold one, then zeros)
 
     if (warp < T4_PRODUCERS) {
         // ---------------- TMA producers ----------------
-        if (warp < stages && elect_one()) {
+        if (elect_one()) {
             Ring ring;
-            int last = -1;   // parity of the last fill issued into the stage
+            int owner = 0;   // producer of stage ring.s
+            // Parity of the last fill issued into each owned stage (at most
+            // three: stages warp, warp + 2, warp + 4), -1 before the first.
+            int last[3] = {-1, -1, -1};
+            auto step = [&]() {
+                ring.next(stages);
+                owner = ring.s == 0 || owner + 1 == T4_PRODUCERS ? 0 : owner + 1;
+            };
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 const int slot = it % TC_SCHED;
                 const uint32_t sn = (uint32_t)(it / TC_SCHED);
-                if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err)) break;
-                const int t = sched_tile[slot];
-                const int rb = sched_rb[slot];
-                mbar_arrive(&bar_sempty[slot]);
+                if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err)) { ok = false; break; }
+                const int t = sched_tile[slot].x;
+                const int rb = sched_tile[slot].y;
+                slot_read(slot);
                 if (t < 0) break;
-                const int rowL = t * TC_BM, rowR = rb * NB;
-                uint8_t *st = smem + (size_t)warp * STAGE;
-                for (int kc = 0; kc < nk; ++kc, ring.next(stages)) {
-                    if (ring.s != warp) continue;
-                    if (!mbar_wait(&bar_empty[warp], ring.par ^ 1, abort_flag, a.err)) { ok = false; break; }
-                    mbar_expect_tx(&bar_full[warp], STAGE);
-                    tma_load_2d(&tmapL, &bar_full[warp], st, kc * TC_BK, rowL);
-                    tma_load_2d(&tmapR, &bar_full[warp], st + TC_A_BYTES, kc * TC_BK, rowR);
-                    last = (int)ring.par;
+                const int rowL = (PAIR ? 2 * t + (int)crank : t) * TC_BM;
+                const int rowR = (PAIR ? 2 * rb + (int)crank : rb) * T4_BLOCK;
+                for (int kc = 0; kc < nk; ++kc, step()) {
+                    if (owner != warp) continue;
+                    const int s = ring.s;
+                    uint8_t *st = smem + (size_t)s * STAGE;
+                    if (!mbar_wait(&bar_empty[s], ring.par ^ 1, abort_flag, a.err)) { ok = false; break; }
+                    if constexpr (PAIR) {
+                        // The leader's barrier counts the bytes of both CTAs.
+                        if (crank == 0) mbar_expect_tx(&bar_full[s], 2 * STAGE);
+                        tma_load_2d_pair(&tmapL, &bar_full[s], st, kc * TC_BK, rowL);
+                        tma_load_2d_pair(&tmapR, &bar_full[s], st + TC_A_BYTES, kc * TC_BK, rowR);
+                    } else {
+                        mbar_expect_tx(&bar_full[s], STAGE);
+                        tma_load_2d(&tmapL, &bar_full[s], st, kc * TC_BK, rowL);
+                        tma_load_2d(&tmapR, &bar_full[s], st + TC_A_BYTES, kc * TC_BK, rowR);
+                    }
+                    last[0] = s == warp ? (int)ring.par : last[0];
+                    last[1] = s == warp + T4_PRODUCERS ? (int)ring.par : last[1];
+                    last[2] = s == warp + 2 * T4_PRODUCERS ? (int)ring.par : last[2];
                 }
             }
-            // Let the last copy into this stage land before the CTA can exit
-            // (earlier ones were consumed).
-            if (last >= 0) {
-                long long t0 = clock64();
-                while (!mbar_try(&bar_full[warp], (uint32_t)last) && clock64() - t0 < WAIT_BUDGET) {}
+            // Let the last copies into the stages this producer owns land
+            // before the CTA can exit (earlier ones were consumed).  A pair's
+            // copies complete on its leader's barriers, and neither CTA exits
+            // before the other (the cluster barrier below); where a wait ran
+            // out, the second CTA allows its own copies a millisecond.
+            if (crank == 0) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int s = warp + q * T4_PRODUCERS;
+                    const int par = last[q];
+                    if (s >= stages || par < 0) continue;
+                    long long t0 = clock64();
+                    while (!mbar_try(&bar_full[s], (uint32_t)par) && clock64() - t0 < WAIT_BUDGET) {}
+                }
+            } else if (!ok) {
+                const long long t0 = clock64();
+                while (clock64() - t0 < 2000000) {}
             }
         }
-    } else if (warp == 3) {
-        if (elect_one()) {
-            // ---------------- MMA issue ----------------
-            const uint32_t idesc = idesc_mxf4(TC_BM, NB);
-            const uint64_t descA = smem_desc_sw128(smem_u32(smem)), descB = smem_desc_sw128(smem_u32(smem + TC_A_BYTES));
-            const uint32_t one = tmem_base + T4_SCALE_COL;
-            Ring ring;
-            bool ok = true;
-            // This thread also schedules the tiles, TC_LOOKAHEAD ahead of the
-            // one it consumes (another lane of this warp spinning on the ring
-            // delayed the MMA issue).
-            int published = 0;
-            bool sched_done = false;
+    } else if (warp == 2) {
+        if (crank == 0 && lane == 0) {
+            // ---------------- scheduler ----------------
+            const uint32_t peer_tile = PAIR ? cluster_addr(&sched_tile[0], 1) : 0;
+            const uint32_t peer_sfull = PAIR ? cluster_addr(&bar_sfull[0], 1) : 0;
             // The strip being handed out: right block s_b, left blocks
             // [s_a, s_aend); the group of the last item taken.
             int s_b = 0, s_a = 0, s_aend = 0;
@@ -323,27 +373,31 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
                     s_aend = min(min(s_a + a.sub, s_g1), a.amax[s_b]);
                 }
             };
-            auto publish = [&](int k) -> bool {
-                const int pslot = k % TC_SCHED;
-                const uint32_t psn = (uint32_t)(k / TC_SCHED);
-                if (!mbar_wait(&bar_sempty[pslot], (psn & 1) ^ 1, abort_flag, a.err)) return false;
+            for (int it = 0;; ++it) {
+                const int slot = it % TC_SCHED;
+                const uint32_t sn = (uint32_t)(it / TC_SCHED);
+                if (!mbar_wait(&bar_sempty[slot], (sn & 1) ^ 1, abort_flag, a.err)) break;
                 int ta = -1, tb = 0;
-                if (!sched_done && !next_tile(ta, tb)) {
-                    ta = -1;
-                    sched_done = true;
-                }
-                sched_tile[pslot] = ta;
-                sched_rb[pslot] = tb;
-                mbar_arrive(&bar_sfull[pslot]);
-                return true;
-            };
-            for (; published < TC_LOOKAHEAD && ok; ++published) ok = publish(published);
+                if (!next_tile(ta, tb)) ta = -1;
+                sched_tile[slot] = make_int2(ta, tb);
+                mbar_arrive(&bar_sfull[slot]);
+                if constexpr (PAIR) cluster_post2(peer_tile + 8 * slot, peer_sfull + 8 * slot, ta, tb);
+                if (ta < 0) break;
+            }
+        }
+    } else if (warp == 3) {
+        if (crank == 0 && elect_one()) {
+            // ---------------- MMA issue ----------------
+            const uint32_t idesc = idesc_mxf4(PAIR ? 2 * TC_BM : TC_BM, NB);
+            const uint64_t descA = smem_desc_sw128(smem_u32(smem)), descB = smem_desc_sw128(smem_u32(smem + TC_A_BYTES));
+            const uint32_t one = tmem_base + T4_SCALE_COL;
+            Ring ring;
+            bool ok = true;
             for (int it = 0; ok; ++it) {
-                if (!(ok = publish(published++))) break;
                 const int slot = it % TC_SCHED;
                 const uint32_t sn = (uint32_t)(it / TC_SCHED);
                 if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err)) break;
-                const int t = sched_tile[slot];
+                const int t = sched_tile[slot].x;
                 mbar_arrive(&bar_sempty[slot]);
                 if (t < 0) break;
                 const int b = it & 1;
@@ -368,16 +422,23 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
                             const bool first = w == 0 || (!ENC && w == a.W0);
                             const uint32_t d = d0 + (!ENC && ctrl ? T4_BLOCK : 0);
                             const uint32_t sa = one + (ENC && ctrl ? FP4_SCALE_COLS : 0);
-                            mma_mxf4(d, ad + 4 * h, bd + 4 * h, idesc, sa, one, first ? 0u : 1u);
-                            mma_mxf4(d, ad + 4 * h + 2, bd + 4 * h + 2, idesc, sa, one, 1u);
+                            if constexpr (PAIR) {
+                                mma_mxf4_pair(d, ad + 4 * h, bd + 4 * h, idesc, sa, one, first ? 0u : 1u);
+                                mma_mxf4_pair(d, ad + 4 * h + 2, bd + 4 * h + 2, idesc, sa, one, 1u);
+                            } else {
+                                mma_mxf4(d, ad + 4 * h, bd + 4 * h, idesc, sa, one, first ? 0u : 1u);
+                                mma_mxf4(d, ad + 4 * h + 2, bd + 4 * h + 2, idesc, sa, one, 1u);
+                            }
                         }
                     }
-                    mma_commit(&bar_empty[s]);
+                    if constexpr (PAIR) mma_commit_pair(&bar_empty[s]); else mma_commit(&bar_empty[s]);
                 }
-                if (ok) mma_commit(&bar_tfull[b]);
+                if (ok) {
+                    if constexpr (PAIR) mma_commit_pair(&bar_tfull[b]); else mma_commit(&bar_tfull[b]);
+                }
             }
             // All MMAs issued by this thread complete before TMEM is released.
-            mma_commit(&bar_done);
+            if constexpr (PAIR) mma_commit_pair(&bar_done); else mma_commit(&bar_done);
             long long t0 = clock64();
             while (!mbar_try(&bar_done, 0) && clock64() - t0 < WAIT_BUDGET) {}
         }
@@ -405,6 +466,7 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
         const int L = a.L;
         const int Bcap = a.Bcap;
         const uint32_t lt = (uint32_t)a.M;
+        const uint32_t tempty0 = PAIR ? cluster_addr(&bar_tempty[0], 0) : 0;
         const float xmax = a.acc_max, amax = a.case_max;
         const uint32_t small_off = smem_u32(small) - T4_OFF;
         float thr_s = -FLT_MAX;
@@ -415,12 +477,13 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
             const int slot = it % TC_SCHED;
             const uint32_t sn = (uint32_t)(it / TC_SCHED);
             const bool ok = mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err);
-            const int t = ok ? sched_tile[slot] : -1;
-            const int rb = ok ? sched_rb[slot] : 0;
+            int t = ok ? sched_tile[slot].x : -1;
+            const int rb = ok ? sched_tile[slot].y : 0;
             if (ok) {
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bar_sempty[slot]);
+                if (lane == 0) slot_read(slot);
             }
+            if (PAIR && t >= 0) t = 2 * t + (int)crank;   // this CTA's left block
             const int b = it & 1;
             const uint32_t u = (uint32_t)(it >> 1);
             // Tile data that does not depend on the accumulators, loaded while
@@ -483,7 +546,10 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
                     // This warp's last read of the buffer.
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&bar_tempty[b]);
+                    if (lane == 0) {
+                        if constexpr (PAIR) mbar_arrive_cluster(tempty0 + 8 * b);
+                        else mbar_arrive(&bar_tempty[b]);
+                    }
                 }
 #pragma unroll
                 for (int q = 0; q < RPG; ++q) {
@@ -626,10 +692,25 @@ __global__ void __launch_bounds__(T4_THREADS, 1)
 
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) {
+        // Neither CTA of a pair leaves while the other may still signal it or
+        // an MMA may read its shared memory (the leader has waited for its
+        // last commit above).
+        if (crank == 1 && threadIdx.x == 0) {
+            const long long t0 = clock64();
+            while (!mbar_try(&bar_done, 0) && clock64() - t0 < WAIT_BUDGET) {}
+        }
+        __syncwarp();
+        cluster_sync();
+    }
     if (warp == 3) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
-                     : "memory");
+        if constexpr (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
+                         : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
+                         : "memory");
     }
 }
 
@@ -661,7 +742,7 @@ cudaError_t launch_small_terms(float *t, cudaStream_t st)
 size_t quads_smem_bytes(int enc, int stages, int M, int P2)
 {
     // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
-    return 2048 + (size_t)stages * (TC_A_BYTES + (enc ? 2 : 1) * T4_BLOCK * TC_BK) + (size_t)((M + 1 + 3) & ~3) * 4 +
+    return 2048 + (size_t)stages * (TC_A_BYTES + T4_BLOCK * TC_BK) + (size_t)((M + 1 + 3) & ~3) * 4 +
            (enc ? (size_t)T4_SMALL_FLOATS * 4 : 0) + (size_t)P2 * (8 + 4);
 }
 
@@ -689,7 +770,19 @@ cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUt
     CUtensorMap mL = tmapL, mR = tmapR;
     QuadsArgs args = a;
     void *params[] = {&mL, &mR, &args};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(T4_THREADS), params, bytes, st);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(T4_THREADS);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = a.enc ? 1 : 0;   // form 1: CTA pairs (an even grid)
+    return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
 }  // namespace fc

@@ -1077,7 +1077,7 @@ void enum_tuples(int64_t S, int T, bool left, int other, std::vector<uint64_t> &
     }
 }
 
-// Left blocks per group: ~48 MB of them, about a third of L2 (two dies share
+// Left blocks (form 1: pairs of them) per group: ~48 MB of them, about a third of L2 (two dies share
 // the 129 MB), so that a group stays resident while the right blocks stream.
 // A scheduler item is a strip of at most `sub` of them against one right
 // block (form 1: block pair), so that the CTAs in flight share right blocks:
@@ -1101,9 +1101,10 @@ int64_t tuple_strip(int64_t group, int64_t bl, int64_t br, int sms, double item_
     }
 }
 
-int64_t tuple_group_size(int Wt)
+int64_t tuple_group_size(int Wt, int enc)
 {
-    return std::max<int64_t>(16, std::min<int64_t>(512, ((int64_t)48 << 20) / (tuple_block_rows(true) * tuple_pitch(Wt))));
+    const int64_t bytes = tuple_tile_blocks(enc) * tuple_block_rows(true) * tuple_pitch(Wt);
+    return std::max<int64_t>(16, std::min<int64_t>(512, ((int64_t)48 << 20) / bytes));
 }
 
 int64_t tuple_count(int64_t S, int T, int other)
@@ -1126,7 +1127,9 @@ bool Dataset::tuples_tc_eligible(int k, int L)
     if (W0 == 0 || Wt == W0) return false;
     const int LT = tc_left_size(k), RT = k - LT;
     const int64_t nl = tuple_count(S, LT, RT), nr = tuple_count(S, RT, LT);
-    const int64_t bl = (nl + tc_tuples_per_block(LT) - 1) / tc_tuples_per_block(LT);
+    const int enc = tuples_form();
+    const int64_t LPB = tuple_tile_blocks(enc) * tc_tuples_per_block(LT);
+    const int64_t bl = (nl + LPB - 1) / LPB;
     const int64_t br = (nr + tc_tuples_per_block(RT) - 1) / tc_tuples_per_block(RT);
     // Block indices and strips (group, right block) are ints (the group size
     // as in prepare_tuples).
@@ -1135,14 +1138,15 @@ bool Dataset::tuples_tc_eligible(int k, int L)
         // The left slab stays resident; the right one in chunks beside it.
         const int64_t rchunk = tuple_right_chunk(k);
         if (rchunk <= 0) return false;
-        const int64_t group = tuple_group_size(Wt);
-        const int64_t sub = tuple_strip(group, bl, rchunk, sms, (double)tuple_block_rows(false) * (double)tuple_pitch(Wt));
+        const int64_t group = tuple_group_size(Wt, enc);
+        const int64_t sub = tuple_strip(group, bl, rchunk, sms,
+                                        (double)tuple_tile_blocks(enc) * tuple_block_rows(false) * (double)tuple_pitch(Wt));
         if ((double)(bl / group + 1) * (double)rchunk * (double)((group + sub - 1) / sub) >= 2147483647.0)
             return false;
     }
     const int Bcap = std::max(L, 1024);
     const int P2 = pow2_at_least(L + Bcap);
-    return quads_smem_bytes(tuples_form(), 2, (int)M, P2) <= (size_t)max_smem_optin;
+    return quads_smem_bytes(enc, 2, (int)M, P2) <= (size_t)max_smem_optin;
 }
 
 // Right items per chunk of the orders 4-6 right slab (items: right blocks,
@@ -1160,7 +1164,7 @@ int64_t Dataset::tuple_right_chunk(int k) const
     const int64_t nl = tuple_count(S, LT, RT), nr = tuple_count(S, RT, LT);
     const int64_t bl = (nl + tc_tuples_per_block(LT) - 1) / tc_tuples_per_block(LT);
     const int64_t br = (nr + tc_tuples_per_block(RT) - 1) / tc_tuples_per_block(RT);
-    const int rblk = tuples_form() ? 2 : 1;
+    const int rblk = tuple_tile_blocks(tuples_form());
     const int64_t nb = (br + rblk - 1) / rblk;
     auto fit = [&](double cap, double left, double item) -> int64_t {
         if (left + (double)nb * item <= cap) return nb;
@@ -1171,7 +1175,7 @@ int64_t Dataset::tuple_right_chunk(int k) const
     double cap = 192.0 * 1024 * 1024 * 1024;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) cap = std::min(cap, 0.6 * (double)free_b);
     const double pitch = (double)tuple_pitch(Wt);
-    int64_t n = fit(cap, (double)bl * tuple_block_rows(true) * pitch, (double)rblk * tuple_block_rows(false) * pitch);
+    int64_t n = fit(cap, (double)((bl + rblk - 1) / rblk * rblk) * tuple_block_rows(true) * pitch, (double)rblk * tuple_block_rows(false) * pitch);
     if (const char *mb = getenv("FC_TUPLES_SLAB_MB")) {
         const long v = atol(mb);
         const double blk = 128.0 * ((double)Wt * 128 + 128);
@@ -1198,7 +1202,7 @@ int Dataset::build_right_chunk(int k, int64_t c)
     return FC_OK;
 }
 
-QuadsArgs Dataset::tuples_chunk_args(const QuadsArgs &base, int k, int64_t c, const int4 *groups,
+QuadsArgs Dataset::tuples_chunk_args(const QuadsArgs &base, int k, int64_t c, const int4 *groups, const int *amax,
                                      const std::vector<int> &cg0, const std::vector<int64_t> &citems) const
 {
     const TupleTC &u = tup[k - 4];
@@ -1208,7 +1212,7 @@ QuadsArgs Dataset::tuples_chunk_args(const QuadsArgs &base, int k, int64_t c, co
     qa.groups = groups + cg0[(size_t)c];
     qa.ngroups = cg0[(size_t)c + 1] - cg0[(size_t)c];
     qa.n_items = (int)citems[(size_t)c];
-    qa.amax = u.amax + c0;
+    qa.amax = amax + c0;
     qa.rtup = u.rt + c0 * u.rblk * RPB;
     qa.rrank = u.rr + c0 * u.rblk * RPB;
     return qa;
@@ -1255,9 +1259,15 @@ QuadsArgs Dataset::tuples_args(int k, int L, float hy, float invN)
     qa.rank_begin = 0;
     qa.rank_end = ~0ull;
     qa.L = L;
-    qa.Bcap = L > 0 ? std::max(L, 1024) : 0;
-    qa.P2 = L > 0 ? pow2_at_least(L + qa.Bcap) : 0;
-    qa.stages = quads_smem_bytes(u.enc, 3, (int)M, qa.P2) <= (size_t)max_smem_optin ? 3 : 2;
+    // A buffer of at least 512 candidates (a tile adds up to 288), the rest
+    // of shared memory to the load stages: with 30 KB a stage the copies in
+    // flight, not the L2 bandwidth, limit the stream (three stages of 44 KB
+    // gave 65 bytes a cycle and SM, four 98).
+    qa.P2 = L > 0 ? pow2_at_least(L + 512) : 0;
+    qa.Bcap = qa.P2 - L;
+    qa.stages = 2;
+    for (int st = TC_MAX_STAGES; st >= 2; --st)
+        if (quads_smem_bytes(u.enc, st, (int)M, qa.P2) <= (size_t)max_smem_optin) { qa.stages = st; break; }
     return qa;
 }
 
@@ -1268,6 +1278,7 @@ void Dataset::release_tuples(int k)
     if (stream) cudaStreamSynchronize(stream);
     dev_free_pooled(u.QL, u.ql_bytes, device);
     dev_free_pooled(u.QR, u.qr_bytes, device);
+    dev_free_pooled(u.QX, u.qx_bytes, device);
     cudaFree(u.lt);
     cudaFree(u.lr);
     cudaFree(u.rt);
@@ -1318,12 +1329,14 @@ int64_t tuple_groups(int64_t group, int64_t sub, int64_t bl, const std::vector<i
 }
 }  // namespace
 
+namespace {
 // Groups of every right chunk of the plan of order k (those of left blocks
 // with include set, if include is not null), back to back: chunk c's are
 // groups[cg0[c] .. cg0[c + 1]), with citems[c] items.  FC_ERANGE if a
 // chunk's items overflow an int.
-int tuple_chunk_groups(const Dataset::TupleTC &u, int64_t bl, const std::vector<char> *include,
-                       std::vector<int4> &groups, std::vector<int> &cg0, std::vector<int64_t> &citems)
+int tuple_chunk_groups(const Dataset::TupleTC &u, const std::vector<int> &amax, int64_t sub, int64_t bl,
+                       const std::vector<char> *include, std::vector<int4> &groups, std::vector<int> &cg0,
+                       std::vector<int64_t> &citems)
 {
     groups.clear();
     cg0.assign(1, 0);
@@ -1331,8 +1344,8 @@ int tuple_chunk_groups(const Dataset::TupleTC &u, int64_t bl, const std::vector<
     std::vector<int4> gc;
     for (int64_t c = 0; c < u.nchunks(); ++c) {
         const int64_t c0 = c * u.rchunk, c1 = std::min(u.nb, c0 + u.rchunk);
-        const std::vector<int> slice(u.amax_host.begin() + c0, u.amax_host.begin() + c1);
-        const int64_t items = tuple_groups(u.group, u.sub, bl, slice, include, gc);
+        const std::vector<int> slice(amax.begin() + c0, amax.begin() + c1);
+        const int64_t items = tuple_groups(u.group, sub, bl, slice, include, gc);
         if (items >= ((int64_t)1 << 31)) return set_error(FC_ERANGE, "tensor-core strip plan too large");
         groups.insert(groups.end(), gc.begin(), gc.end());
         cg0.push_back((int)groups.size());
@@ -1340,6 +1353,25 @@ int tuple_chunk_groups(const Dataset::TupleTC &u, int64_t bl, const std::vector<
     }
     return FC_OK;
 }
+
+// The last SNP of a left tuple of LT SNPs.
+int64_t tuple_last(uint64_t t, int LT) { return (int64_t)((t >> (16 * (LT - 1))) & 0xffffu); }
+
+// amax of every right item of the plan for left blocks whose smallest last
+// SNPs are lmin (ascending): the number of left blocks that hold a tuple
+// ending before the item's largest first SNP.
+std::vector<int> tuple_amax(const Dataset::TupleTC &u, const std::vector<int64_t> &lmin)
+{
+    std::vector<int> amax((size_t)u.nb);
+    const int64_t br = (int64_t)u.rmax_host.size();
+    for (int64_t b = 0; b < u.nb; ++b) {
+        // The item's last right block (a padding block takes its partner's).
+        const int64_t rb = std::min<int64_t>(u.rblk * b + u.rblk - 1, br - 1);
+        amax[(size_t)b] = (int)(std::lower_bound(lmin.begin(), lmin.end(), u.rmax_host[(size_t)rb]) - lmin.begin());
+    }
+    return amax;
+}
+}  // namespace
 
 int Dataset::prepare_tuples(int k)
 {
@@ -1363,14 +1395,16 @@ int Dataset::prepare_tuples(int k)
         note_launches(1);
     }
     const int LT = tc_left_size(k), RT = k - LT;
-    const int LPB = tc_tuples_per_block(LT), RPB = tc_tuples_per_block(RT);
+    // Form 1 takes blocks in pairs on either side: a "block" of the left
+    // side is then a pair, and the right slab gets an even count.
+    u.enc = tuples_form();
+    u.rblk = tuple_tile_blocks(u.enc);
+    const int LPB = u.rblk * tc_tuples_per_block(LT), RPB = tc_tuples_per_block(RT);
     std::vector<uint64_t> lt, rt;
     enum_tuples(S, LT, true, RT, lt);
     enum_tuples(S, RT, false, LT, rt);
     const int64_t nl = (int64_t)lt.size(), nr = (int64_t)rt.size();
     const int64_t bl = (nl + LPB - 1) / LPB, br = (nr + RPB - 1) / RPB;
-    // Form 1 takes right blocks in pairs: the right slab gets an even count.
-    u.enc = tuples_form();
     const int64_t br2 = u.enc ? (br + 1) / 2 * 2 : br;
     auto snp = [](uint64_t t, int i) { return (int64_t)((t >> (16 * i)) & 0xffffu); };
     std::vector<uint64_t> lr(lt.size()), rr(rt.size());
@@ -1405,24 +1439,16 @@ int Dataset::prepare_tuples(int k)
         u.rmax_host[(size_t)blk] = snp(rt[(size_t)(std::min<int64_t>((blk + 1) * RPB, nr) - 1)], 0);
     const uint64_t kbytes = (uint64_t)Wt * 64;
     const uint64_t pitch = (uint64_t)tuple_pitch(Wt);
-    const int rowsL = tuple_block_rows(true), rowsR = tuple_block_rows(false);
-    u.group = tuple_group_size(Wt);
-    // amax per right block, or per pair of right blocks (form 1: the
-    // second block's, the larger; a padding block takes its partner's).
-    std::vector<int> &amax = u.amax_host;
+    const int rowsL = u.rblk * tuple_block_rows(true), rowsR = tuple_block_rows(false);
+    u.group = tuple_group_size(Wt, u.enc);
     const int64_t nb = u.enc ? br2 / 2 : br;
     u.nb = nb;
-    u.rblk = u.enc ? 2 : 1;
     u.rchunk = tuple_right_chunk(k);
     if (u.rchunk <= 0) return set_error(FC_ENOMEM, "tuple-row slabs do not fit in device memory");
-    amax.resize((size_t)nb);
-    for (int64_t b = 0; b < nb; ++b) {
-        const int64_t rb = u.enc ? std::min<int64_t>(2 * b + 1, br - 1) : b;
-        amax[(size_t)b] = (int)(std::lower_bound(u.lmin_host.begin(), u.lmin_host.end(), u.rmax_host[(size_t)rb]) -
-                                u.lmin_host.begin());
-    }
+    u.amax_host = tuple_amax(u, u.lmin_host);
+    const std::vector<int> &amax = u.amax_host;
     u.sub = tuple_strip(u.group, bl, u.rchunk, sms, (double)u.rblk * rowsR * (double)pitch);
-    int rc = tuple_chunk_groups(u, bl, nullptr, u.groups_host, u.cg0, u.citems);
+    int rc = tuple_chunk_groups(u, amax, u.sub, bl, nullptr, u.groups_host, u.cg0, u.citems);
     if (rc) return rc;
     u.n_items = 0;
     for (const int64_t n : u.citems) u.n_items += n;
@@ -1446,19 +1472,22 @@ int Dataset::prepare_tuples(int k)
     cudaMemcpyAsync(u.groups, u.groups_host.data(), sizeof(int4) * u.groups_host.size(), cudaMemcpyHostToDevice, stream);
     cudaMemcpyAsync(u.amax, amax.data(), sizeof(int) * amax.size(), cudaMemcpyHostToDevice, stream);
     if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_tuple_rows(LT, true, X, S_pad, Wt, u.lt, bl, (int64_t)pitch, u.QL, stream)) != cudaSuccess)
+        (e = launch_tuple_rows(LT, true, X, S_pad, Wt, u.lt, bl * u.rblk, (int64_t)pitch, u.QL, stream)) != cudaSuccess)
         return cuda_status(e, "tuple-row kernel");
     note_launches(1);
     // One chunk: the right rows are built once and kept.
     u.built = -1;
     if (u.nchunks() == 1 && (rc = build_right_chunk(k, 0)) != FC_OK) return rc;
-    if ((rc = encode_tmap_u8(&u.tmapL, u.QL, kbytes, pitch, (uint64_t)bl * rowsL, (uint32_t)rowsL, true)) != FC_OK) return rc;
+    if ((rc = encode_tmap_u8(&u.tmapL, u.QL, kbytes, pitch, (uint64_t)bl * rowsL, (uint32_t)tuple_block_rows(true),
+                             true)) != FC_OK)
+        return rc;
     if ((rc = encode_tmap_u8(&u.tmapR, u.QR, kbytes, pitch, (uint64_t)u.rchunk * u.rblk * rowsR,
-                             (uint32_t)(u.rblk * rowsR), true)) != FC_OK)
+                             (uint32_t)rowsR, true)) != FC_OK)
         return rc;
     // Host vectors go out of scope: the copies must have landed.
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_status(e, "tuple operands");
     u.lt_host = std::move(lt);
+    u.lr_host = std::move(lr);
     u.ready = true;
     return FC_OK;
 }
@@ -1494,8 +1523,8 @@ int Dataset::tuples_dense(int k, float *scores, uint32_t *tables)
     for (int64_t c = 0; c < u.nchunks(); ++c) {
         if (u.citems[(size_t)c] == 0) continue;
         if ((rc = build_right_chunk(k, c)) != FC_OK) return rc;
-        const QuadsArgs qc = tuples_chunk_args(qa, k, c, u.groups, u.cg0, u.citems);
-        const int grid = (int)std::min<int64_t>(sms, u.citems[(size_t)c]);
+        const QuadsArgs qc = tuples_chunk_args(qa, k, c, u.groups, u.amax, u.cg0, u.citems);
+        const int grid = u.rblk * (int)std::min<int64_t>(sms / u.rblk, u.citems[(size_t)c]);
         cudaMemsetAsync(qa.tile_counter, 0, sizeof(int), stream);
         if ((e = launch_gate()) != cudaSuccess ||
             (e = launch_quads_tc(k, MODE_DUMP, u.tmapL, u.tmapR, qc, grid, stream)) != cudaSuccess)
@@ -1560,11 +1589,15 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         // and the left blocks to take.
         std::vector<int4> range_groups4;
         std::vector<char> include4;
+        // Its own left tuples, their parts of the rank and amax (compact).
+        std::vector<uint64_t> lt4, lr4;
+        std::vector<int> amax4;
         std::vector<int> cg0_4;
         std::vector<int64_t> citems4, launches4;
         struct SlabLaunch { int si; int64_t t0, t1; };
         std::vector<SlabLaunch> launches3;
         int grid = 0;
+        int ctas4 = 0;   // orders 4-6: CTAs of a launch (whole pairs in form 1)
         if (tc) {
             int rc = prepare_pairs();
             if (rc) return rc;
@@ -1600,39 +1633,79 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
             int rc = prepare_tuples(k);
             if (rc) return rc;
             qa = tuples_args(k, L, (float)hy, (float)(1.0 / Nd));
-            const TupleTC &u = tup[k - 4];
+            TupleTC &u = tup[k - 4];
             cg0_4 = u.cg0;
             citems4 = u.citems;
             if (!whole) {
-                const int LT = tc_left_size(k), LPB = tc_tuples_per_block(LT);
-                std::vector<char> &include = include4;
-                include.assign(u.lmin_host.size(), 0);
+                const int LT = tc_left_size(k), LPB = u.rblk * tc_tuples_per_block(LT);
+                // The combinations that extend left tuple t form the rank
+                // range [first, first + count): t followed by its smallest
+                // right tuple, and every right tuple after its last SNP.
+                std::vector<uint64_t> count((size_t)S);
+                for (int64_t c = 0; c < S; ++c) count[(size_t)c] = binom(S - c - 1, k - LT);
+                std::vector<size_t> in;
                 for (size_t x = 0; x < u.lt_host.size(); ++x) {
-                    const uint64_t t = u.lt_host[x];
-                    if (t == NO_TUPLE) continue;
-                    // The combinations that extend left tuple t form the rank
-                    // range [first, first + count): t followed by its smallest
-                    // right tuple, and every right tuple after its last SNP.
-                    uint32_t c[FC_KMAX_SEARCH];
-                    for (int q = 0; q < LT; ++q) c[q] = (uint32_t)((t >> (16 * q)) & 0xffffu);
-                    for (int q = LT; q < k; ++q) c[q] = c[q - 1] + 1;
-                    const uint64_t count = binom(S - (int64_t)c[LT - 1] - 1, k - LT);
-                    if (count == 0) continue;
-                    const uint64_t first = rank_of(S, k, c);
-                    if (first < r1 && first + count > r0) include[x / (size_t)LPB] = 1;
+                    if (u.lt_host[x] == NO_TUPLE) continue;
+                    const uint64_t n = count[(size_t)tuple_last(u.lt_host[x], LT)];
+                    const uint64_t first = u.lr_host[x] - n;
+                    if (n > 0 && first < r1 && first + n > r0) in.push_back(x);
                 }
-                if ((rc = tuple_chunk_groups(u, (int64_t)u.lmin_host.size(), &include, range_groups4, cg0_4,
-                                             citems4)) != FC_OK)
-                    return rc;
+                // Left tuples come in order of their last SNP, so a range
+                // of a few first SNPs holds a few tuples of many blocks:
+                // where at most half of the tuples meet the range their rows
+                // are built again, close together.  (The 41st of 64 ranges of
+                // 1,001 SNPs at order 4 touched 30 % of the tuples of the
+                // blocks it took.)
+                bool compact = 2 * in.size() <= u.lt_host.size() && !in.empty();
+                if (compact) {
+                    const int64_t bx = ((int64_t)in.size() + LPB - 1) / LPB;
+                    const size_t bytes = (size_t)(bx * u.rblk) * tuple_block_rows(true) * (size_t)tuple_pitch(Wt);
+                    if (bytes > u.qx_bytes) {
+                        cudaStreamSynchronize(stream);
+                        dev_free_pooled(u.QX, u.qx_bytes, device);
+                        u.QX = nullptr;
+                        u.qx_bytes = 0;
+                        if (dev_alloc_pooled((void **)&u.QX, bytes, device) == cudaSuccess) {
+                            u.qx_bytes = bytes;
+                        } else {
+                            cudaGetLastError();   // the resident left rows serve
+                            compact = false;
+                        }
+                    }
+                    if (compact) {
+                        lt4.assign((size_t)(bx * LPB), NO_TUPLE);
+                        lr4.assign((size_t)(bx * LPB), 0);
+                        std::vector<int64_t> lmin((size_t)bx);
+                        for (size_t x = 0; x < in.size(); ++x) {
+                            lt4[x] = u.lt_host[in[x]];
+                            lr4[x] = u.lr_host[in[x]];
+                            if (x % (size_t)LPB == 0) lmin[x / (size_t)LPB] = tuple_last(lt4[x], LT);
+                        }
+                        amax4 = tuple_amax(u, lmin);
+                        const int64_t sub = tuple_strip(u.group, bx, u.rchunk, sms,
+                                                        (double)u.rblk * tuple_block_rows(false) * (double)tuple_pitch(Wt));
+                        qa.sub = (int)sub;
+                        rc = tuple_chunk_groups(u, amax4, sub, bx, nullptr, range_groups4, cg0_4, citems4);
+                        if (rc) return rc;
+                    }
+                }
+                if (!compact) {
+                    include4.assign(u.lmin_host.size(), 0);
+                    for (const size_t x : in) include4[x / (size_t)LPB] = 1;
+                    if ((rc = tuple_chunk_groups(u, u.amax_host, u.sub, (int64_t)u.lmin_host.size(), &include4, range_groups4,
+                                                 cg0_4, citems4)) != FC_OK)
+                        return rc;
+                }
                 qa.rank_begin = r0;
                 qa.rank_end = r1;
             }
             // One launch per right chunk with tiles (at least one, whose
-            // CTAs write the empty lists); each writes sms lists.
+            // CTAs write the empty lists); each writes a list per CTA.
             for (int64_t c = 0; c < u.nchunks(); ++c)
                 if (citems4[(size_t)c] > 0) launches4.push_back(c);
             if (launches4.empty()) launches4.push_back(0);
-            grid = sms * (int)launches4.size();
+            ctas4 = sms / u.rblk * u.rblk;
+            grid = ctas4 * (int)launches4.size();
         } else {
             cfg = pick_config(k, L, MODE_TOPN, no_alloc);
             if (cfg.var == VAR_IE) {
@@ -1660,7 +1733,7 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
             p[10] = A.take(sizeof(double) * (size_t)N);
             p[11] = A.take(sizeof(int) * 4);
             p[12] = A.take(sizeof(uint32_t) * range_tiles.size() + sizeof(int4) * range_groups4.size() +
-                           include4.size() + 16);
+                           sizeof(uint64_t) * (lt4.size() + lr4.size()) + sizeof(int) * amax4.size() + include4.size() + 16);
         };
         void *p[13];
         plan(ar, p);
@@ -1717,27 +1790,49 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
             qa.tile_counter = (int *)p[11] + 1;
             qa.err = err;
             const int4 *groups = u.groups;
+            const int *amax = u.amax;
+            CUtensorMap tmapL = u.tmapL;
             if (!whole) {
                 int4 *dg = (int4 *)p[12];
-                uint8_t *di = (uint8_t *)(dg + range_groups4.size());
                 if (!range_groups4.empty())
                     cudaMemcpyAsync(dg, range_groups4.data(), sizeof(int4) * range_groups4.size(),
                                     cudaMemcpyHostToDevice, stream);
-                cudaMemcpyAsync(di, include4.data(), include4.size(), cudaMemcpyHostToDevice, stream);
                 groups = dg;
-                qa.include = di;
+                if (!lt4.empty()) {
+                    const int LT = tc_left_size(k);
+                    uint64_t *dl = (uint64_t *)(dg + range_groups4.size()), *dr = dl + lt4.size();
+                    int *da = (int *)(dr + lr4.size());
+                    cudaMemcpyAsync(dl, lt4.data(), sizeof(uint64_t) * lt4.size(), cudaMemcpyHostToDevice, stream);
+                    cudaMemcpyAsync(dr, lr4.data(), sizeof(uint64_t) * lr4.size(), cudaMemcpyHostToDevice, stream);
+                    cudaMemcpyAsync(da, amax4.data(), sizeof(int) * amax4.size(), cudaMemcpyHostToDevice, stream);
+                    const int64_t blocks = (int64_t)lt4.size() / tc_tuples_per_block(LT), pitch = tuple_pitch(Wt);
+                    if ((e = launch_gate()) != cudaSuccess ||
+                        (e = launch_tuple_rows(LT, true, X, S_pad, Wt, dl, blocks, pitch, u.QX, stream)) != cudaSuccess)
+                        return cuda_status(e, "tuple-row kernel");
+                    note_launches(1);
+                    int rc = encode_tmap_u8(&tmapL, u.QX, (uint64_t)Wt * 64, (uint64_t)pitch,
+                                            (uint64_t)blocks * tuple_block_rows(true), (uint32_t)tuple_block_rows(true), true);
+                    if (rc) return rc;
+                    qa.ltup = dl;
+                    qa.lrank = dr;
+                    amax = da;
+                } else {
+                    uint8_t *di = (uint8_t *)(dg + range_groups4.size());
+                    cudaMemcpyAsync(di, include4.data(), include4.size(), cudaMemcpyHostToDevice, stream);
+                    qa.include = di;
+                }
             }
             cudaMemsetAsync(p[11], 0x80, sizeof(int), stream);
             for (size_t x = 0; x < launches4.size(); ++x) {
                 const int64_t c = launches4[x];
                 int rc = build_right_chunk(k, c);
                 if (rc) return rc;
-                QuadsArgs qc = tuples_chunk_args(qa, k, c, groups, cg0_4, citems4);
-                qc.list_score = (float *)p[0] + x * sms * L;
-                qc.list_rank = (uint64_t *)p[1] + x * sms * L;
+                QuadsArgs qc = tuples_chunk_args(qa, k, c, groups, amax, cg0_4, citems4);
+                qc.list_score = (float *)p[0] + x * ctas4 * L;
+                qc.list_rank = (uint64_t *)p[1] + x * ctas4 * L;
                 cudaMemsetAsync(qa.tile_counter, 0, sizeof(int), stream);
                 if ((e = launch_gate()) != cudaSuccess ||
-                    (e = launch_quads_tc(k, MODE_TOPN, u.tmapL, u.tmapR, qc, sms, stream)) != cudaSuccess)
+                    (e = launch_quads_tc(k, MODE_TOPN, tmapL, u.tmapR, qc, ctas4, stream)) != cudaSuccess)
                     return cuda_status(e, "tensor-core tuple kernel");
                 if (x > 0) note_launches(1);
             }

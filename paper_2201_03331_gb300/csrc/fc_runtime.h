@@ -130,6 +130,9 @@ struct Dataset {
     struct TupleTC {
         uint8_t *QL = nullptr, *QR = nullptr;
         size_t ql_bytes = 0, qr_bytes = 0;
+        // Left rows of a rank-range search's own tuples, kept for the next.
+        uint8_t *QX = nullptr;
+        size_t qx_bytes = 0;
         uint64_t *lt = nullptr, *lr = nullptr, *rt = nullptr, *rr = nullptr;
         int enc = 0;               // form (tuples_form)
         int4 *groups = nullptr;    // {g0, g1, lo, item_first} per group of left blocks
@@ -140,16 +143,17 @@ struct Dataset {
         std::vector<int> amax_host;
         CUtensorMap tmapL{}, tmapR{};
         bool ready = false;
-        // Host copies for rank-range searches: the left tuples, each left
+        // Host copies for rank-range searches: the left tuples and their
+        // parts of the rank, each left
         // block's smallest last SNP, each right block's largest first SNP,
         // and the left blocks per tile group.
-        std::vector<uint64_t> lt_host;
+        std::vector<uint64_t> lt_host, lr_host;
         std::vector<int64_t> lmin_host, rmax_host;
         int64_t group = 0;
         int64_t sub = 1;           // left blocks per strip (scheduler item)
         // The right operand in chunks when the whole right slab does not
         // fit beside the left one: nb right items (blocks; block pairs in
-        // form 1) of rblk blocks, rchunk of them per chunk (nb: one chunk,
+        // form 1) of rblk blocks (the left side's items take as many), rchunk of them per chunk (nb: one chunk,
         // built once and kept); chunk c's groups are groups_host[cg0[c] ..
         // cg0[c + 1]) with citems[c] items; QR holds chunk `built`.
         int64_t nb = 0, rchunk = 0;
@@ -191,7 +195,7 @@ struct Dataset {
     // ext_scratch: if non-null, a device work area of ext_cap bytes used instead
     // of the handle's own (grown-on-demand) scratch allocation.
     // [rank_begin, rank_end): search only the combinations of these
-    // lexicographic ranks (a proper sub-range always takes the sweep).
+    // lexicographic ranks.
     int search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, int64_t *out_count,
                void *ext_scratch = nullptr, size_t ext_cap = 0, uint64_t rank_begin = 0,
                uint64_t rank_end = ~0ull);
@@ -217,8 +221,8 @@ struct Dataset {
     int build_right_chunk(int k, int64_t c);
     // Arguments of the launch over right chunk c (groups from `groups` with
     // chunk offsets cg0, citems).
-    QuadsArgs tuples_chunk_args(const QuadsArgs &base, int k, int64_t c, const int4 *groups, const std::vector<int> &cg0,
-                                const std::vector<int64_t> &citems) const;
+    QuadsArgs tuples_chunk_args(const QuadsArgs &base, int k, int64_t c, const int4 *groups, const int *amax,
+                                const std::vector<int> &cg0, const std::vector<int64_t> &citems) const;
     int tuples_form() const;
     int prepare_tuples(int k);
     void release_tuples(int k);

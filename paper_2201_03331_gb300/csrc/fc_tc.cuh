@@ -190,6 +190,79 @@ __device__ __forceinline__ void mma_mxf4(uint32_t tmem_d, uint64_t adesc, uint64
         : "memory");
 }
 
+// ---- CTA pairs (cta_group::2) ---------------------------------------------------
+// Two CTAs of a cluster (one TPC) work on one M = 256 tile: each holds its
+// 128 rows of A, half of the rows of B and its 128 accumulator lanes; the MMAs
+// are issued by the leader (rank 0) alone.  Copies of both CTAs complete on
+// the leader's barriers, commits arrive on both CTAs' barriers.
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Shared-cluster address of `p` in the CTA of rank `rank`.
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+// Arrive on the barrier at a shared-cluster address.  What crosses the pair
+// this way is only "this slot has been read" and "this accumulator has been
+// read" (ordered by tcgen05 fences); arrivals and waits of cluster scope would
+// add a fence and drop the L1 lines of the waiting SM each time (orders 5 and
+// 6 at 2,048 samples: 174 and 168 ms instead of 126 and 130).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// Writes {x, y} to the 8 bytes at a shared-cluster address, completing the
+// current phase of the barrier at `bar` there (one arrival and these bytes):
+// a waiter on that barrier sees the data.
+__device__ __forceinline__ void cluster_post2(uint32_t addr, uint32_t bar, int x, int y)
+{
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], 8;" ::"r"(bar) : "memory");
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(x),
+                 "r"(y), "r"(bar)
+                 : "memory");
+}
+// Copy into this CTA's shared memory that completes on barrier `bar` (the
+// same offset) of the pair's leader: bit 24 of a shared-cluster address
+// selects the CTA of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(const CUtensorMap *map, uint64_t *bar, void *dst, int x, int y)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+        "[%4];" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar) & 0xFEFFFFFFu)
+        : "memory");
+}
+__device__ __forceinline__ void mma_mxf4_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t scale_a, uint32_t scale_b, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.block32 [%0], %1, %2, %3, [%4], [%5], p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(scale_a), "r"(scale_b), "r"(accumulate)
+        : "memory");
+}
+// Arrives on `bar` (the same offset) of both CTAs once the MMAs issued so far
+// are complete.
+__device__ __forceinline__ void mma_commit_pair(uint64_t *bar)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+}
+
 // 16 TMEM columns of this warp's lane quarter, all words v.
 __device__ __forceinline__ void tmem_fill16(uint32_t taddr, uint32_t v)
 {
