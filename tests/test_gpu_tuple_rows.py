@@ -29,11 +29,11 @@ def combos(S, k):
 
 
 @pytest.mark.parametrize("k", [4, 5, 6])
-@pytest.mark.parametrize("cases,controls", [(4095, 4095), (1, 4095), (128, 129), (129, 127), (63, 64), (64, 63)])
+@pytest.mark.parametrize("cases,controls", [(4095, 4095), (1, 4095), (128, 129), (129, 127), (127, 128), (128, 127)])
 def test_one_accumulator_limits(fc, monkeypatch, k, cases, controls):
     """SNPs without variation put whole classes into one cell: the
-    accumulator n_case + 4096 n_ctrl reaches 2^24 - 1, and counts of 63 and
-    64 take either side of the small-count table.  128- and 129-sample
+    accumulator n_case + 4096 n_ctrl reaches 2^24 - 1, and counts of 127 and
+    128 take either side of the small-count table.  128- and 129-sample
     classes end inside, at and just past a chunk."""
     monkeypatch.setenv("FC_QUADS_ENC", "1")
     S = k + 3
