@@ -141,14 +141,23 @@ int pow2_ge(int v)
 
 // ---- batched order-3 tensor-core form -------------------------------------------
 
-// Plans the batched tensor-core form for the order-3 jobs marked in B.tc:
-// every data set all of whose replicates take the tensor cores and fit one
-// of the two batched forms.  Builds its operands once (the genotype rows of
-// each data set and the class-carrying SNP rows of each job, in the sample
-// order of the data set's first replicate), the tile plans, the TMA
-// descriptors and job table, the buffers of the lists and results, and the
-// slab buffer; groups the data sets into launches whose slabs fit it
-// together.  Jobs it leaves out keep the per-job tensor-core search.
+// The pair rows of a slot's job (the first SNPs 0 .. S - 3 have pairs with a
+// third SNP after them).
+cudaError_t launch_slot_slab(const fc_handle *h, const Tc3Batch &T, const Tc3Batch::Slot &ss, cudaStream_t st)
+{
+    const Dataset &d = *h->jobs[(size_t)ss.job];
+    return launch_pair_rows(T.E + ss.e_off, triples_pitch(d.Wt), d.Wt, d.S, 0, d.S - 2, T.rowbase + ss.rowbase_off,
+                            T.slab + ss.slab_off, st);
+}
+
+// Plans the batched tensor-core form for the order-3 jobs marked in B.tc.
+// Builds every job's SNP rows once, the tile plans (one per SNP count), the
+// TMA descriptors and job table, the buffers of the lists and results, and the
+// slab buffer; groups the jobs into launches whose slabs fit it together.
+// Each job has its own slab, in its own order of cases and controls: the
+// 4-bit rows carry no class, so a slab shared by the replicates of a data set
+// would need class-carrying byte rows (e5m2), whose kernel took twice the time
+// per combination; a slab of 1,000 SNPs x 4,000 samples is written in 0.7 ms.
 int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
 {
     out.reset();
@@ -156,8 +165,7 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
     Dataset &lead = h->ds;
     const char *env = getenv("FC_BATCH_TC3");
     if (env && strcmp(env, "0") == 0) return FC_OK;
-    const int R = B.R;
-    const int grid = lead.sms;
+    const int grid = lead.sms & ~1;   // (form 1 launches CTA pairs)
     // The per-job merge of grid lists in one or two levels of k_merge_jobs.
     const int merge_cap = 16384;   // entries one merge block sorts (12 bytes each in shared memory)
     if (L > 1024 || (int64_t)L * grid > (int64_t)merge_cap * 16) return FC_OK;
@@ -165,100 +173,64 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
     T->L = L;
     T->grid = grid;
     T->smem_cap = lead.max_smem_optin;
-    int64_t maxM = 0;
-    for (int d = 0; d < B.n_data; ++d) {
-        bool all = true, one_acc = true;
-        int64_t cls = 0;   // the largest class of any replicate
-        for (int r = 0; r < R; ++r) {
-            const Dataset &x = *h->jobs[(size_t)d * R + r];
-            all = all && B.tc[(size_t)d * R + r];
-            one_acc = one_acc && x.M1 <= 4095 && x.M0 <= 4095;
-            cls = std::max(cls, std::max(x.M1, x.M0));
-        }
-        if (!all) continue;
-        const Dataset &d0 = *h->jobs[(size_t)d * R];
-        Tc3Batch::Set st;
-        st.first_job = d * R;
-        // The kernel holds an x ln x table of the power of two above the
-        // launch's largest class count (the table serves the class counts;
-        // n ln n of a cell's total comes from the hardware logarithm): one
-        // accumulator where both classes of every replicate have at most
-        // 4095 samples and shared memory fits, else two.
-        if (one_acc && triples_list_fit(1, cls, L, lead.max_smem_optin) > 0) {
-            st.enc = 1;
-        } else {
-            // Two accumulators over the chunks [0, split) and [split, Wt) of
-            // the first replicate's layout, each with at most 4095 samples
-            // (so with at most 4095 of either class in any replicate).
-            int64_t pre = 0;
-            int split = 0;
-            for (int c = 0; c < d0.Wt; ++c) {
-                const int64_t real = c < d0.W0 ? std::min<int64_t>(128, d0.M1 - 128 * (int64_t)c)
-                                               : std::min<int64_t>(128, d0.M0 - 128 * (int64_t)(c - d0.W0));
-                if (pre + real > 4095) break;
-                pre += real;
-                split = c + 1;
-            }
-            if (split <= 0 || split >= d0.Wt || d0.M - pre > 4095) continue;
-            if (triples_list_fit(2, cls, L, lead.max_smem_optin) < 0) continue;
-            st.enc = 2;
-            st.split = split;
-        }
-        st.M = cls;   // table extent
-        st.NP = triples_pairs_per_tile(st.enc);
-        st.pitch = (int64_t)d0.Wt * 128 + 128;
-        st.rows = 2 * ((d0.S + 63) / 64 * 64);
-        T->sets.push_back(st);
-        maxM = std::max(maxM, d0.M);
+    int64_t maxM = 0, minM = INT64_MAX;
+    for (int j = 0; j < (int)h->jobs.size(); ++j) {
+        if (!B.tc[j]) continue;
+        const Dataset &x = *h->jobs[j];
+        Tc3Batch::Slot st;
+        st.job = j;
+        st.enc = x.triples_form(L);
+        st.M = x.M;
+        st.stages = triples_stages((int)st.M, L, (size_t)lead.max_smem_optin);
+        if (st.enc < 0 || st.stages == 0) continue;
+        T->slots.push_back(st);
+        maxM = std::max(maxM, st.M);
+        minM = std::min(minM, st.M);
     }
-    if (T->sets.empty()) return FC_OK;
-    // One-accumulator data sets first, then the two-accumulator ones; within
-    // a form by the size of their x ln x table (a launch takes one size).
-    std::stable_sort(T->sets.begin(), T->sets.end(), [](const Tc3Batch::Set &a, const Tc3Batch::Set &b) {
-        return a.enc != b.enc ? a.enc < b.enc : pow2_at_least((int)a.M + 1) < pow2_at_least((int)b.M + 1);
-    });
-    T->M = (int)maxM;
+    if (T->slots.empty()) return FC_OK;
+    T->scale = triples_scale(minM);
+    // A launch takes one form and one stage count (its x log2 x table spans
+    // its most samples): one-accumulator jobs first, then by stages.
+    auto key = [](const Tc3Batch::Slot &x) { return std::make_pair(-x.enc, -x.stages); };
+    std::stable_sort(T->slots.begin(), T->slots.end(),
+                     [&](const Tc3Batch::Slot &a, const Tc3Batch::Slot &b) { return key(a) < key(b); });
 
-    // Tile plans (one slab per data set).
+    // Tile plans (one slab per job, one plan per SNP count).
     std::vector<uint4> tiles;
     std::vector<int64_t> rowbase;
-    for (Tc3Batch::Set &st : T->sets) {
-        const Dataset &d0 = *h->jobs[(size_t)st.first_job];
-        const std::shared_ptr<const TriplePlan> pl = plan_triples(d0.S, st.NP, INT64_MAX / 4);
-        st.tile_off = (int64_t)tiles.size();
-        st.ntiles = (int64_t)pl->tiles.size();
-        st.rowbase_off = (int64_t)rowbase.size();
-        st.slab_rows = pl->max_rows;
-        tiles.insert(tiles.end(), pl->tiles.begin(), pl->tiles.end());
-        rowbase.insert(rowbase.end(), pl->rowbase.begin(), pl->rowbase.end());
+    std::map<std::pair<int64_t, int>, size_t> plan_of;   // (SNP count, form) -> a slot that holds the plan
+    size_t ebytes = 0;
+    for (size_t x = 0; x < T->slots.size(); ++x) {
+        Tc3Batch::Slot &st = T->slots[x];
+        const Dataset &d = *h->jobs[(size_t)st.job];
+        const auto it = plan_of.find({d.S, st.enc});
+        if (it != plan_of.end()) {
+            const Tc3Batch::Slot &o = T->slots[it->second];
+            st.tile_off = o.tile_off;
+            st.ntiles = o.ntiles;
+            st.rowbase_off = o.rowbase_off;
+            st.slab_rows = o.slab_rows;
+        } else {
+            const std::shared_ptr<const TriplePlan> pl = plan_triples(d.S, st.enc, INT64_MAX / 4);
+            st.tile_off = (int64_t)tiles.size();
+            st.ntiles = (int64_t)pl->tiles.size();
+            st.rowbase_off = (int64_t)rowbase.size();
+            st.slab_rows = pl->max_rows;
+            tiles.insert(tiles.end(), pl->tiles.begin(), pl->tiles.end());
+            rowbase.insert(rowbase.end(), pl->rowbase.begin(), pl->rowbase.end());
+            plan_of[{d.S, st.enc}] = x;
+        }
+        st.e_off = ebytes;
+        ebytes += ((size_t)triples_rows(d.S) * (size_t)triples_pitch(d.Wt) + 1023) / 1024 * 1024;
     }
-    const int nsets = (int)T->sets.size();
-    const int n = nsets * R;
+    const int n = (int)T->slots.size();
     T->n = n;
-    // Slots: data set by data set, replicates in order.
-    T->slot_job.resize((size_t)n);
-    for (int si = 0; si < nsets; ++si)
-        for (int r = 0; r < R; ++r) T->slot_job[(size_t)si * R + r] = T->sets[(size_t)si].first_job + r;
+    for (const Tc3Batch::Slot &st : T->slots) T->slot_job.push_back(st.job);
 
     // Per-job tables of the epilogue (inclusion-exclusion) and of the rescoring.
     for (int j : T->slot_job) {
         const int rc = h->jobs[(size_t)j]->prepare_ie(3);
         if (rc) return rc;
-    }
-
-    // Operands: per data set its genotype rows, per job its SNP rows.
-    size_t ebytes = 0;
-    T->e_off.resize((size_t)nsets);
-    std::vector<size_t> a_off((size_t)n);
-    for (int si = 0; si < nsets; ++si) {
-        const Tc3Batch::Set &st = T->sets[(size_t)si];
-        const size_t one = (size_t)st.rows * (size_t)st.pitch;
-        T->e_off[(size_t)si] = ebytes;
-        ebytes += (one + 1023) / 1024 * 1024;
-        for (int r = 0; r < R; ++r) {
-            a_off[(size_t)si * R + r] = ebytes;
-            ebytes += (one + 1023) / 1024 * 1024;
-        }
     }
     cudaError_t e;
     auto alloc = [&](void **ptr, size_t bytes) -> cudaError_t {
@@ -281,24 +253,15 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
     }
 
     // Other buffers (one arena).
-    std::vector<uint32_t> masks;   // per job: Wt uint4 of control bits
-    std::vector<size_t> mask_off((size_t)n);
-    for (int x = 0; x < n; ++x) {
-        const Tc3Batch::Set &st = T->sets[(size_t)(x / R)];
-        const Dataset &d0 = *h->jobs[(size_t)st.first_job];
-        mask_off[(size_t)x] = masks.size();
-        masks.resize(masks.size() + 4 * (size_t)d0.Wt, 0u);
-    }
     Arena ar;
     void *pm[24];
     auto plan = [&](Arena &A) {
-        pm[0] = A.take(sizeof(CUtensorMap) * ((size_t)n + nsets) + 128);
+        pm[0] = A.take(sizeof(CUtensorMap) * 2 * (size_t)n + 128);
         pm[1] = A.take(sizeof(T3Job) * (size_t)n);
         pm[2] = A.take(sizeof(JobDesc) * (size_t)n);
         pm[3] = A.take(sizeof(JobDesc) * (size_t)n * std::max(G1, 1));
         pm[4] = A.take(sizeof(uint4) * std::max<size_t>(tiles.size(), 1));
         pm[5] = A.take(sizeof(int64_t) * std::max<size_t>(rowbase.size(), 1));
-        pm[6] = A.take(sizeof(uint32_t) * std::max<size_t>(masks.size(), 4));
         pm[7] = A.take(sizeof(float) * (size_t)n * grid * L);
         pm[8] = A.take(sizeof(uint64_t) * (size_t)n * grid * L);
         pm[9] = A.take(sizeof(float) * (size_t)n * std::max(G1, 1) * L);
@@ -311,7 +274,7 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
         pm[16] = A.take(sizeof(uint32_t) * (size_t)n + 16);
         pm[17] = A.take(sizeof(uint32_t) * (size_t)n * n_out * 3);
         pm[18] = A.take(sizeof(double) * (size_t)n * n_out);
-        pm[19] = A.take(sizeof(int) * (size_t)n);
+        pm[19] = A.take(sizeof(int) * (size_t)n * grid);
         pm[20] = A.take(sizeof(int) * 4096);   // tile counters of the launches, kernel error word
         pm[21] = A.take(sizeof(float) * ((size_t)maxM + 1));
     };
@@ -327,7 +290,6 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
     T->d_desc1 = (JobDesc *)pm[3];
     uint4 *d_tiles = (uint4 *)pm[4];
     T->rowbase = (int64_t *)pm[5];
-    uint32_t *d_masks = (uint32_t *)pm[6];
     T->list_s = (float *)pm[7];
     T->list_r = (uint64_t *)pm[8];
     T->mid_s = (float *)pm[9];
@@ -340,65 +302,34 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
     T->job_err = (uint32_t *)pm[16];
     T->out_idx = (uint32_t *)pm[17];
     T->out_score = (double *)pm[18];
-    T->d_gthr = (int *)pm[19];
+    T->d_pub = (int *)pm[19];
     T->d_counter = (int *)pm[20];
     T->xlogx = (float *)pm[21];
 
-    // Control bits of every job in its data set's first-replicate layout:
-    // chunk w < W0 holds that replicate's cases in input order, the rest its
-    // controls.
-    for (int si = 0; si < nsets; ++si) {
-        const Tc3Batch::Set &st = T->sets[(size_t)si];
-        const int d = st.first_job / R;
-        const Dataset &d0 = *h->jobs[(size_t)st.first_job];
-        const int64_t M = d0.M;
-        const std::vector<uint8_t> &ph = B.ph[(size_t)d];
-        std::vector<int64_t> cases, ctrls;
-        for (int64_t m = 0; m < M; ++m) (ph[(size_t)m] ? cases : ctrls).push_back(m);
-        for (int r = 0; r < R; ++r) {
-            uint32_t *mk = masks.data() + mask_off[(size_t)si * R + r];
-            const uint8_t *phr = ph.data() + (size_t)r * M;
-            for (size_t x = 0; x < cases.size(); ++x)
-                if (!phr[cases[x]]) mk[x >> 5] |= 1u << (x & 31);
-            const size_t base = (size_t)d0.W0 * 128;
-            for (size_t x = 0; x < ctrls.size(); ++x)
-                if (!phr[ctrls[x]]) mk[(base + x) >> 5] |= 1u << ((base + x) & 31);
-        }
-    }
     cudaStream_t st = lead.stream;
     cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(uint4) * tiles.size(), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(T->rowbase, rowbase.data(), sizeof(int64_t) * rowbase.size(), cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(d_masks, masks.data(), sizeof(uint32_t) * masks.size(), cudaMemcpyHostToDevice, st);
-    if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(T->xlogx, maxM, st, true)) != cudaSuccess)
-        return cuda_status(e, "x ln x table");
-    for (int si = 0; si < nsets; ++si) {
-        const Tc3Batch::Set &ss = T->sets[(size_t)si];
-        const Dataset &d0 = *h->jobs[(size_t)ss.first_job];
+    if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(T->xlogx, maxM, st, true, T->scale)) != cudaSuccess)
+        return cuda_status(e, "x log2 x table");
+    for (const Tc3Batch::Slot &ss : T->slots) {
+        const Dataset &d = *h->jobs[(size_t)ss.job];
         if ((e = launch_gate()) != cudaSuccess ||
-            (e = launch_expand_e5m2(d0.X, d0.S, d0.S_pad, d0.Wt, ss.rows, ss.pitch, nullptr, T->E + T->e_off[(size_t)si],
-                                    st)) != cudaSuccess)
-            return cuda_status(e, "batched genotype rows");
-        for (int r = 0; r < R; ++r) {
-            const int x = si * R + r;
-            if ((e = launch_gate()) != cudaSuccess ||
-                (e = launch_expand_e5m2(d0.X, d0.S, d0.S_pad, d0.Wt, ss.rows, ss.pitch,
-                                        reinterpret_cast<const uint4 *>(d_masks + mask_off[(size_t)x]),
-                                        T->E + a_off[(size_t)x], st)) != cudaSuccess)
-                return cuda_status(e, "batched SNP rows");
-        }
+            (e = launch_expand_fp4(d.X, d.S, d.S_pad, d.Wt, triples_pitch(d.Wt), T->E + ss.e_off, st)) != cudaSuccess)
+            return cuda_status(e, "batched SNP rows");
     }
 
-    // Launch groups: consecutive data sets of one form whose slabs fit the
-    // slab buffer together.  The buffer takes what the data sets need, at
-    // most three quarters of the free memory less 8 GiB (FC_BATCH_SLAB_MB
-    // caps it), and at least the largest slab.
-    std::vector<size_t> slab_bytes((size_t)nsets);
+    // Launch groups: consecutive jobs of one form and stage count whose slabs fit
+    // the slab buffer together.  The buffer takes what the jobs need, at most
+    // three quarters of the free memory less 8 GiB (FC_BATCH_SLAB_MB caps
+    // it), and at least the largest slab.
+    std::vector<size_t> slab_bytes((size_t)n);
     size_t total_slab = 0, max_slab = 0;
-    for (int si = 0; si < nsets; ++si) {
-        const Tc3Batch::Set &ss = T->sets[(size_t)si];
-        slab_bytes[(size_t)si] = ((size_t)ss.slab_rows * (size_t)ss.pitch + 1023) / 1024 * 1024;
-        total_slab += slab_bytes[(size_t)si];
-        max_slab = std::max(max_slab, slab_bytes[(size_t)si]);
+    for (int x = 0; x < n; ++x) {
+        const Tc3Batch::Slot &ss = T->slots[(size_t)x];
+        const int64_t pitch = triples_pitch(h->jobs[(size_t)ss.job]->Wt);
+        slab_bytes[(size_t)x] = ((size_t)ss.slab_rows * (size_t)pitch + 1023) / 1024 * 1024;
+        total_slab += slab_bytes[(size_t)x];
+        max_slab = std::max(max_slab, slab_bytes[(size_t)x]);
     }
     size_t budget = total_slab;
     size_t free_b = 0, total_b = 0;
@@ -416,60 +347,53 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
         Tc3Batch::Launch cur;
         size_t used = 0;
         int64_t items = 0;
-        auto close = [&](int next_set) {
-            if (cur.sets.empty()) return;
-            cur.j1 = next_set * R;
+        auto close = [&](int next) {
+            cur.j1 = next;
             cur.n_items = (int)items;
-            T->launches.push_back(cur);
+            if (cur.j1 > cur.j0) T->launches.push_back(cur);
             cur = Tc3Batch::Launch{};
+            cur.j0 = next;
             used = 0;
             items = 0;
         };
-        for (int si = 0; si < nsets; ++si) {
-            Tc3Batch::Set &ss = T->sets[(size_t)si];
-            const int64_t add = ss.ntiles * R;
-            if (!cur.sets.empty() &&
-                (ss.enc != cur.enc || pow2_at_least((int)ss.M + 1) != pow2_at_least(cur.M + 1) ||
-                 used + slab_bytes[(size_t)si] > budget || items + add > ((int64_t)1 << 30)))
-                close(si);
-            if (cur.sets.empty()) {
-                cur.j0 = si * R;
-                cur.enc = ss.enc;
-            }
+        for (int x = 0; x < n; ++x) {
+            Tc3Batch::Slot &ss = T->slots[(size_t)x];
+            if (x > cur.j0 && (key(ss) != key(T->slots[(size_t)cur.j0]) || used + slab_bytes[(size_t)x] > budget ||
+                               items + ss.ntiles > ((int64_t)1 << 30)))
+                close(x);
+            cur.enc = ss.enc;
+            cur.stages = ss.stages;
             cur.M = std::max(cur.M, (int)ss.M);
             ss.slab_off = used;
-            used += slab_bytes[(size_t)si];
-            items += add;
-            cur.sets.push_back(si);
+            used += slab_bytes[(size_t)x];
+            items += ss.ntiles;
         }
-        close(nsets);
+        close(n);
     }
     if ((int)T->launches.size() > 4096 - 1) return FC_OK;
     T->rebuild = T->launches.size() > 1;
 
     // TMA descriptors, job table and the per-job descriptors of the merge
     // and the rescoring.
-    std::vector<CUtensorMap> maps((size_t)n + nsets);
+    std::vector<CUtensorMap> maps(2 * (size_t)n);
     std::vector<T3Job> jobs((size_t)n);
     std::vector<JobDesc> desc((size_t)n), desc1;
     for (const Tc3Batch::Launch &ln : T->launches) {
         int item = 0;
-        for (const int si : ln.sets) {
-            const Tc3Batch::Set &ss = T->sets[(size_t)si];
-            const Dataset &d0 = *h->jobs[(size_t)ss.first_job];
-            const uint64_t kbytes = (uint64_t)d0.Wt * 128;
-            int rc = encode_tmap_u8(&maps[(size_t)n + si], T->slab + ss.slab_off, kbytes, (uint64_t)ss.pitch,
-                                    (uint64_t)ss.slab_rows, (uint32_t)(4 * ss.NP), true);
+        for (int x = ln.j0; x < ln.j1; ++x) {
+            const Tc3Batch::Slot &ss = T->slots[(size_t)x];
+            const Dataset &dj = *h->jobs[(size_t)ss.job];
+            const uint64_t kbytes = (uint64_t)dj.Wt * 64, pitch = (uint64_t)triples_pitch(dj.Wt);
+            int rc = encode_tmap_u8(&maps[(size_t)n + x], T->slab + ss.slab_off, kbytes, pitch, (uint64_t)ss.slab_rows,
+                                    (uint32_t)triples_block_rows(), true);
             if (rc) return rc;
-            for (int r = 0; r < R; ++r) {
-                const int x = si * R + r;
-                const Dataset &dj = *h->jobs[(size_t)T->slot_job[(size_t)x]];
-                if ((rc = encode_tmap_u8(&maps[(size_t)x], T->E + a_off[(size_t)x], kbytes, (uint64_t)ss.pitch,
-                                         (uint64_t)ss.rows, 128, true)) != FC_OK)
-                    return rc;
+            if ((rc = encode_tmap_u8(&maps[(size_t)x], T->E + ss.e_off, kbytes, pitch, (uint64_t)triples_rows(dj.S), 128,
+                                     true)) != FC_OK)
+                return rc;
+            {
                 T3Job &jb = jobs[(size_t)x];
                 jb.tmapA = T->d_maps + x;
-                jb.tmapP = T->d_maps + n + si;
+                jb.tmapP = T->d_maps + n + x;
                 jb.tiles = d_tiles + ss.tile_off;
                 jb.marg4 = reinterpret_cast<const uint4 *>(dj.marg);
                 jb.PR = dj.PR;
@@ -478,8 +402,8 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
                 jb.total = binom(dj.S, 3);
                 jb.hy = (float)dj.hy64();
                 jb.invN = (float)(1.0 / (double)dj.M);
-                jb.Wt = d0.Wt;
-                jb.split = ss.split;
+                jb.W0 = dj.W0;
+                jb.Wt = dj.Wt;
                 jb.item_first = item;
                 jb.ntiles = (int)ss.ntiles;
                 jb.slot = x;
@@ -522,14 +446,9 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
     T->desc = desc;
     // A single group: its slabs are built once, here.
     if (!T->rebuild) {
-        for (const int si : T->launches[0].sets) {
-            const Tc3Batch::Set &ss = T->sets[(size_t)si];
-            const Dataset &d0 = *h->jobs[(size_t)ss.first_job];
-            if ((e = launch_gate()) != cudaSuccess ||
-                (e = launch_pair_rows(T->E + T->e_off[(size_t)si], ss.pitch, d0.Wt, d0.S, ss.NP, 0, d0.S - 2,
-                                      T->rowbase + ss.rowbase_off, T->slab + ss.slab_off, st)) != cudaSuccess)
+        for (const Tc3Batch::Slot &ss : T->slots)
+            if ((e = launch_gate()) != cudaSuccess || (e = launch_slot_slab(h, *T, ss, st)) != cudaSuccess)
                 return cuda_status(e, "batched pair-row slab");
-        }
     }
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_status(e, "batched order-3 operands");
 
@@ -557,17 +476,15 @@ TriplesArgs tc3_args(const Tc3Batch &T, const Tc3Batch::Launch &ln, int g)
     a.n_jobs = ln.j1 - ln.j0;
     a.n_items = ln.n_items;
     a.xlogx = T.xlogx;
+    a.scale = T.scale;
     a.M = ln.M;
     a.L = T.L;
-    a.P2 = triples_list_fit(ln.enc, ln.M, T.L, T.smem_cap);
-    a.Bcap = a.P2 - a.L;
-    a.check_rounds = 1;
-    for (int r = 3; r >= 1; --r)
-        if (r * triples_round_candidates() <= a.Bcap) { a.check_rounds = r; break; }
+    a.stages = ln.stages;
     a.wait_ticks = TC_WAIT_TICKS;
     a.list_score = T.list_s;
     a.list_rank = T.list_r;
-    a.gthr = T.d_gthr;
+    a.pub = T.d_pub;
+    triples_publish(T.L, T.grid, &a.pub_m, &a.pub_r);
     a.tile_counter = T.d_counter + g;
     a.err = reinterpret_cast<uint32_t *>(T.d_counter + 4095);
     return a;
@@ -781,12 +698,10 @@ int plan_batch(fc_handle *h, int k, int64_t top_n)
         n2_all = std::max(n2_all, pow2_ge((T->level1 ? T->F : T->grid) * L));
         if (T->level1) n2_all = std::max(n2_all, pow2_ge(((T->grid + T->F - 1) / T->F) * L));
         // Each form's kernel takes the shared memory of its largest launch.
-        size_t bytes[3] = {0, 0, 0};
-        for (const Tc3Batch::Launch &ln : T->launches) {
-            const TriplesArgs a = tc3_args(*T, ln, 0);
-            bytes[ln.enc] = std::max(bytes[ln.enc], triples_smem_bytes(ln.enc, a.M, a.P2));
-        }
-        for (int enc = 1; enc <= 2; ++enc)
+        size_t bytes[2] = {0, 0};
+        for (const Tc3Batch::Launch &ln : T->launches)
+            bytes[ln.enc] = std::max(bytes[ln.enc], triples_smem_bytes(ln.stages, ln.M, T->L));
+        for (int enc = 0; enc <= 1; ++enc)
             if (bytes[enc] && (e = prepare_triples_tc_batch(enc, bytes[enc])) != cudaSuccess)
                 return cuda_status(e, "batched order-3 attributes");
     }
@@ -807,7 +722,7 @@ int plan_batch(fc_handle *h, int k, int64_t top_n)
     }
     if (T) {
         // 0x80808080 is below the ordered image of every finite score.
-        chk(cudaMemsetAsync(T->d_gthr, 0x80, sizeof(int) * (size_t)T->n, st));
+        chk(cudaMemsetAsync(T->d_pub, 0x80, sizeof(int) * (size_t)T->n * T->grid, st));
         chk(cudaMemsetAsync(T->d_counter, 0, sizeof(int) * 4096, st));
         chk(cudaMemsetAsync(T->job_err, 0, sizeof(uint32_t) * (size_t)T->n, st));
         // Lists of jobs a CTA never takes stay empty.
@@ -821,13 +736,7 @@ int plan_batch(fc_handle *h, int k, int64_t top_n)
         for (int g = 0; g < (int)T->launches.size(); ++g) {
             const Tc3Batch::Launch &ln = T->launches[(size_t)g];
             if (T->rebuild) {
-                for (const int si : ln.sets) {
-                    const Tc3Batch::Set &ss = T->sets[(size_t)si];
-                    const Dataset &d0 = *h->jobs[(size_t)ss.first_job];
-                    // The first SNPs 0 .. S - 3 have pairs with a third SNP after them.
-                    chk(launch_pair_rows(T->E + T->e_off[(size_t)si], ss.pitch, d0.Wt, d0.S, ss.NP, 0, d0.S - 2,
-                                         T->rowbase + ss.rowbase_off, T->slab + ss.slab_off, st));
-                }
+                for (int x = ln.j0; x < ln.j1; ++x) chk(launch_slot_slab(h, *T, T->slots[(size_t)x], st));
             }
             chk(launch_triples_tc(MODE_TOPN, none, none, tc3_args(*T, ln, g), T->grid, st, false));
         }
@@ -913,8 +822,6 @@ int fc_load_batch(int n_data, const uint8_t *const *genotypes, const int64_t *S,
         BatchState &B = *h->batch;
         B.n_data = n_data;
         B.R = R;
-        B.ph.resize((size_t)n_data);
-        for (int d = 0; d < n_data; ++d) B.ph[(size_t)d].assign(phenotypes[d], phenotypes[d] + (size_t)R * M[d]);
         cudaStream_t st = h->ds.stream;
         int64_t maxS = 0, maxM = 0;
         for (int d = 0; d < n_data; ++d) { maxS = std::max(maxS, S[d]); maxM = std::max(maxM, M[d]); }
@@ -1010,7 +917,7 @@ int fc_search_batch(fc_handle *h, int k, int64_t top_n, uint32_t *out_idx, doubl
                 if (ns > 0) lead.launches += 4;
                 if (T) {
                     lead.launches += 1 + (int)T->launches.size() + (T->level1 ? 2 : 1) + 2;
-                    if (T->rebuild) lead.launches += (int)T->sets.size();
+                    if (T->rebuild) lead.launches += T->n;
                 }
             }
             if (T && (T->h_err[T->n] & ERR_TIMEOUT))
@@ -1048,8 +955,7 @@ int fc_search_batch(fc_handle *h, int k, int64_t top_n, uint32_t *out_idx, doubl
                     rc = d.search(k, top_n, oi, os, &out_count[j]);
                     d.allow_tc = false;
                     d.release_triples();
-                    d.release_pairs();
-                    if (rc) return rc;
+                                if (rc) return rc;
                     B.job_kind[j] = d.last_path_tc3 ? 6 : (d.last_sweep_var == VAR_IE ? 3 : d.last_sweep_var == VAR_JR ? 4 : 1);
                     continue;
                 }
@@ -1081,8 +987,7 @@ int fc_search_batch(fc_handle *h, int k, int64_t top_n, uint32_t *out_idx, doubl
             rc = d.search(k, top_n, out_idx + (size_t)j * top_n * k, out_score + (size_t)j * top_n, &out_count[j]);
             d.allow_tc = false;
             d.release_triples();
-            d.release_pairs();
-            if (rc) return rc;
+                if (rc) return rc;
             B.job_kind[j] = d.last_path_tc3 ? 6 : (d.last_sweep_var == VAR_IE ? 3 : d.last_sweep_var == VAR_JR ? 4 : 1);
             if (lead.timing) {
                 lead.sweep_ms += d.sweep_ms;
@@ -1118,7 +1023,6 @@ int fc_search_job(fc_handle *h, int job, int k, int64_t top_n, uint32_t *out_idx
         const int rc = d.search(k, top_n, out_idx, out_score, out_count);
         d.allow_tc = false;
         d.release_triples();
-        d.release_pairs();
         return rc;
     });
 }

@@ -107,8 +107,12 @@ struct PackArgs {
 cudaError_t launch_class_index(const PackArgs &a, cudaStream_t st);
 cudaError_t launch_pack(const PackArgs &a, int64_t M1, int64_t M0, cudaStream_t st);
 cudaError_t launch_logtab(float *logtab, int64_t M, cudaStream_t st);
-// x ln x (base2: x log2 x) for x = 0..M, each the FP64 product rounded once.
-cudaError_t launch_xlogx(float *t, int64_t M, cudaStream_t st, bool base2 = false);
+// y ln y (base2: y log2 y), y = scale x, for x = 0..M, each the FP64 product
+// rounded once.
+cudaError_t launch_xlogx(float *t, int64_t M, cudaStream_t st, bool base2 = false, double scale = 1.0);
+// t(a, b) = a log(n/a) + b log(n/b), n = a + b (base2: in bits), for a, b < n_max
+// at b stride + a, each rounded once; 0 in the rest of `floats` entries.
+cudaError_t launch_small_terms(float *t, int n_max, int stride, int floats, bool base2, cudaStream_t st);
 
 struct SearchArgs {
     const uint4 *X;
@@ -124,7 +128,7 @@ struct SearchArgs {
     void *dump;             // MODE_SCORES: float [n]; MODE_TABLES: uint32 [n][3^k][2]
     // Inclusion-exclusion inputs (k <= 3 with cfg.ie).
     const uint4 *marg4;     // per-SNP genotype counts (one uint4 per SNP)
-    const uint4 *PR;        // restricted pair counts [S_pad][S_pad] (k = 3)
+    const uint4 *PR;        // restricted pair counts [S_pad][S_pad] (k = 3), both orders of a pair
     uint32_t nn;            // cases | controls << 16
 };
 
@@ -269,98 +273,104 @@ struct PairsArgs {
 };
 
 size_t pairs_smem_bytes(int stages, int M, int P2);
-// ctrl_byte: the e4m3 byte of a control sample's set bit (0x38 = 1.0, or
-// 0x68 = 64.0 for the order-3 kernel's one-accumulator encoding); case
-// samples (words below W0) always carry 0x38.
 cudaError_t launch_expand_e4m3(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, int64_t rows, int64_t pitch,
                                uint8_t *E, uint8_t ctrl_byte, cudaStream_t st);
 cudaError_t launch_marginals(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, uint16_t *marg,
                              cudaStream_t st);
 cudaError_t launch_pairs_tc(int mode, const CUtensorMap &tmap, const PairsArgs &a, int grid, cudaStream_t st);
 
-// Order-3 tensor-core search (fc_triples_tc.cu).  A tile pairs the 64 SNPs
-// l0 .. l0 + 63 (128 e4m3 rows 2 l + g) with the NP pairs (i, j0 + q), q < NP,
-// of slab rows [rowP, rowP + 4 NP) (pair row (a, q, b) at
-// rowP + 2 NP a + 2 q + b); NP = triples_pairs_per_tile(enc).
+// Order-3 tensor-core search (fc_triples_tc.cu).  A tile pairs the SNPs l0 ..
+// l0 + triples_snps_per_tile - 1 (packed 4-bit rows 2 l + g) with the pairs (i,
+// j0 + q), q < triples_pairs_per_tile, of slab rows from rowP (pair row (q, a, b)
+// at rowP + 4 q + 2 a + b).
+int triples_pairs_per_tile(int enc);
+int triples_snps_per_tile(int enc);
+// Slab rows a CTA loads for a tile (28 pairs).
+int triples_block_rows();
+// SNP rows, zero beyond SNP S: a tile starts at any SNP and never leaves them.
+constexpr int64_t triples_rows(int64_t S) { return 2 * ((S + 63) / 64 * 64 + 128); }
+// Bytes from one row of the SNP rows or of the slab to the next.
+constexpr int64_t triples_pitch(int Wt) { return (int64_t)Wt * 64 + 128; }
 // One job of the batched order-3 launch (a data set with one phenotype
-// replicate).  The replicates of a data set share its sample order (that of
-// its first replicate), its pair-row slab (genotypes only, e5m2 1.0) and its
-// tiles; the job's SNP rows carry its classes (e5m2 1.0 for a case, 4096 for
-// a control), so an accumulator holds n_case + 4096 n_ctrl.
+// replicate), with its own operands and lists.
 struct T3Job {
     const CUtensorMap *tmapA;   // the job's SNP rows, 128 x 128-byte boxes
-    const CUtensorMap *tmapP;   // the data set's slab, 4 NP x 128-byte boxes
-    const uint4 *tiles;         // the data set's tiles {rowP, i, j0, l0}
+    const CUtensorMap *tmapP;   // the job's slab, 112 x 128-byte boxes
+    const uint4 *tiles;         // the job's tiles {rowP, i, j0, l0}
     const uint4 *marg4;         // the job's per-SNP genotype counts
     const uint4 *PR;            // the job's restricted pair table [S_pad][S_pad]
     int64_t S, S_pad;
     uint64_t total;             // C(S, 3)
     float hy, invN;
-    int Wt;                     // 128-sample chunks
-    int split;                  // enc 2: first chunk of the second accumulator
+    int W0, Wt;                 // 128-sample words: cases [0, W0), controls [W0, Wt)
     int item_first, ntiles;     // the job's items [item_first, item_first + ntiles) of its launch
-    int slot;                   // lists [slot][grid][L], threshold gthr[slot]
-    int pad;
+    int slot;                   // lists [slot][grid][L], pub[slot][grid]
 };
 
 struct TriplesArgs {
     const uint4 *tiles;     // {rowP, i, j0, l0} per tile of this launch
     int ntiles;
-    // 1: one accumulator n_case + 4096 n_ctrl (operand with controls = 64);
-    // 0: one accumulator per class; 2 (batched launch only): two accumulators
-    // n_case + 4096 n_ctrl over the chunks [0, split) and [split, Wt).
+    // 1: one accumulator n_case + 4096 n_ctrl, 0: one per class.
     int enc;
     // Batched launch (jobs != null): items of all jobs, job-major; the fields
     // above and below that describe one data set come from the job table,
-    // and list_score, list_rank and gthr are indexed by the job's slot.
+    // and list_score, list_rank and pub are indexed by the job's slot.
     const T3Job *jobs;
     int n_jobs, n_items;
     int64_t S, S_pad;
-    int W0, Wt;             // 128-sample chunks: cases [0, W0), controls [W0, Wt)
+    int W0, Wt;             // 128-sample words: cases [0, W0), controls [W0, Wt)
     const uint4 *marg4;     // per-SNP genotype counts (one uint4 per SNP)
     const uint4 *PR;        // restricted pair table [S_pad][S_pad]
-    const float *xlogx;     // x log2 x for x = 0..M (FP64 rounded once to FP32)
-    int M;                  // extent of the kernel's x log2 x table: at least every class count
+    int stages;             // load stages (triples_stages)
+    const float *xlogx;     // y log2 y, y = scale x, for x = 0..M (FP64 rounded once to FP32)
+    float scale;            // the power of two the kernel scores counts in (triples_scale)
+    int M;                  // extent of the kernel's table: the samples
     float hy, invN;
     uint64_t total;         // C(S, 3)
     uint64_t rank_begin, rank_end;   // only combinations with ranks in [rank_begin, rank_end) count
-    int L, Bcap, P2;        // list, candidate buffer (>= 2048), pow2 >= L + Bcap
-    int check_rounds;       // epilogue rounds between buffer checks (Bcap holds that many rounds)
+    int L;
     long long wait_ticks;   // budget of each pipeline wait (clock64 ticks)
     float *list_score;      // [grid][L] (batched: [slots][grid][L])
     uint64_t *list_rank;
-    int *gthr;              // global score threshold (ordered int; batched: one per slot)
+    // Scores of the lists' entries pub_m - 1 as ordered ints, [grid] (batched:
+    // [slots][grid]), set below every score before the first launch; pub_r of
+    // them bound the score of the last of L combinations (triples_publish).
+    int *pub;
+    int pub_m, pub_r;
     int *tile_counter;      // next tile (item) of this launch, zeroed before launch
     uint32_t *err;
     float *dump_scores;     // MODE_DUMP: [C(S,3)] by rank
     uint32_t *dump_tables;  // MODE_DUMP: [C(S,3)][27][2]
 };
 
-int triples_pairs_per_tile(int enc);
 // The base-2 logarithm the tensor-core epilogues take for n ln n, of
 // max(n & (2^23 - 1), 1), for n[0 .. count).
 cudaError_t launch_log2_approx(const uint32_t *n, int64_t count, float *out, cudaStream_t st);
-// Candidates one round of the kernel's epilogue may add to its buffer.
-int triples_round_candidates();
-size_t triples_smem_bytes(int enc, int M, int P2);
-// Slab rows of the first SNPs [i0, i1) from the e4m3 rows E (pitch bytes per
+// The load stages that fit smem_cap bytes of shared memory beside the x log2 x
+// table of M samples and lists of L; 0 if not even two do.
+int triples_stages(int M, int L, size_t smem_cap);
+size_t triples_smem_bytes(int stages, int M, int L);
+// The power of two the kernel scores the counts of M samples in.
+float triples_scale(int64_t M);
+// pub_m and pub_r for lists of L and `grid` CTAs: pub_m pub_r >= L, pub_r at most
+// about half the CTAs.
+void triples_publish(int L, int grid, int *pub_m, int *pub_r);
+// The SNP rows of a bit table X: row 2 s + g, one nibble a sample.
+cudaError_t launch_expand_fp4(const uint4 *X, int64_t S, int64_t S_pad, int Wt, int64_t pitch, uint8_t *E,
+                              cudaStream_t st);
+// Slab rows of the first SNPs [i0, i1) from the SNP rows E (pitch bytes per
 // row); rowbase[i - i0] is the first slab row of SNP i.
-cudaError_t launch_pair_rows(const uint8_t *E, int64_t pitch, int Wt, int64_t S, int NP, int64_t i0, int64_t i1,
+cudaError_t launch_pair_rows(const uint8_t *E, int64_t pitch, int Wt, int64_t S, int64_t i0, int64_t i1,
                              const int64_t *rowbase, uint8_t *P, cudaStream_t st);
-// tmapA: the e4m3 rows in 128 x 128-byte boxes; tmapP: the slab in 4 NP x
+// tmapA: the SNP rows in 128 x 128-byte boxes; tmapP: the slab in 112 x
 // 128-byte boxes (both with the 128-byte swizzle).
 // set_attr = false skips setting the kernel's shared-memory attribute (set
 // by an earlier call; a graph capture may not set it); grid = 0 only sets it.
 cudaError_t launch_triples_tc(int mode, const CUtensorMap &tmapA, const CUtensorMap &tmapP, const TriplesArgs &a,
                               int grid, cudaStream_t st, bool set_attr = true);
-// Shared-memory attribute of the batched kernel of form enc (1 or 2): the
-// largest launch's bytes, set before a graph capture.
+// Shared-memory attribute of the batched kernel of form enc: the largest
+// launch's bytes (triples_smem_bytes), set before a graph capture.
 cudaError_t prepare_triples_tc_batch(int enc, size_t smem_bytes);
-// Operands of the batched form (e5m2; see T3Job): rows 2 s + g of the bit
-// table X, controls of the replicate marked by ctrl (one uint4 of sample
-// bits per chunk; null: no classes).
-cudaError_t launch_expand_e5m2(const uint4 *X, int64_t S, int64_t S_pad, int Wt, int64_t rows, int64_t pitch,
-                               const uint4 *ctrl, uint8_t *E, cudaStream_t st);
 // n list entries (-FLT_MAX, NO_RANK).
 cudaError_t launch_fill_lists(float *s, uint64_t *r, size_t n, cudaStream_t st);
 
@@ -404,7 +414,7 @@ struct QuadsArgs {
     const uint64_t *rtup;   // right tuples
     const uint64_t *rrank;  // rank part of a right tuple (modulo 2^64)
     const float *xlogx;     // x ln x for x = 0..M
-    const float *small_terms;   // cell terms t(a, b) of small counts (launch_small_terms)
+    const float *small_terms;   // cell terms t(a, b) of small counts (launch_quads_small_terms)
     int M;
     float acc_max, case_max;    // M1 + 4096 M0 and M1 (enc 1)
     float hy, invN;
@@ -422,9 +432,9 @@ struct QuadsArgs {
 // Tuple rows of T-SNP tuples (nblocks left or right blocks).
 cudaError_t launch_tuple_rows(int T, bool left, const uint4 *X, int64_t S_pad, int Wt, const uint64_t *tuples,
                               int64_t nblocks, int64_t pitch, uint8_t *Q, cudaStream_t st);
-// The table of cell terms of small class counts, small_terms_floats() floats.
-int small_terms_floats();
-cudaError_t launch_small_terms(float *t, cudaStream_t st);
+// The table of cell terms of small class counts, quads_small_floats() floats.
+int quads_small_floats();
+cudaError_t launch_quads_small_terms(float *t, cudaStream_t st);
 // Shared memory of the orders 4-6 kernel.
 size_t quads_smem_bytes(int enc, int stages, int M, int P2);
 cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUtensorMap &tmapR, const QuadsArgs &a,

@@ -101,19 +101,41 @@ __global__ void k_logtab(float *t, int64_t M)
     if (n <= M) t[n] = n == 0 ? 0.0f : (float)log((double)n);
 }
 
-// x ln x (base2: x log2 x) for x = 0..M (0 ln 0 := 0): the product in FP64
-// rounded once to FP32.
-__global__ void k_xlogx(float *t, int64_t M, bool base2)
+// y ln y (base2: y log2 y), y = scale x, for x = 0..M (0 ln 0 := 0): the product
+// in FP64 rounded once to FP32.
+__global__ void k_xlogx(float *t, int64_t M, bool base2, double scale)
 {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n <= M) t[n] = n == 0 ? 0.0f : (float)((double)n * (base2 ? log2((double)n) : log((double)n)));
+    const double y = scale * (double)n;
+    if (n <= M) t[n] = n == 0 ? 0.0f : (float)(y * (base2 ? log2(y) : log(y)));
+}
+
+// t(a, b) = a log(n/a) + b log(n/b), n = a + b, for a, b < n_max at b stride + a
+// (base2: in bits), in FP64 rounded once; 0 elsewhere.
+__global__ void k_small_terms(float *t, int n_max, int stride, int floats, bool base2)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= floats) return;
+    const int b = i / stride, a = i % stride;
+    double v = 0.0;
+    if (a < n_max && b < n_max && a > 0 && b > 0) {
+        const double n = a + b;
+        v = base2 ? (double)a * log2(n / a) + (double)b * log2(n / b) : (double)a * log(n / a) + (double)b * log(n / b);
+    }
+    t[i] = (float)v;
 }
 
 }  // namespace
 
-cudaError_t launch_xlogx(float *t, int64_t M, cudaStream_t st, bool base2)
+cudaError_t launch_small_terms(float *t, int n_max, int stride, int floats, bool base2, cudaStream_t st)
 {
-    k_xlogx<<<(unsigned)((M + 1 + 255) / 256), 256, 0, st>>>(t, M, base2);
+    k_small_terms<<<(floats + 255) / 256, 256, 0, st>>>(t, n_max, stride, floats, base2);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_xlogx(float *t, int64_t M, cudaStream_t st, bool base2, double scale)
+{
+    k_xlogx<<<(unsigned)((M + 1 + 255) / 256), 256, 0, st>>>(t, M, base2, scale);
     return cudaGetLastError();
 }
 

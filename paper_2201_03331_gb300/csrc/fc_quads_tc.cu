@@ -138,21 +138,6 @@ __global__ void k_tuple_rows(const uint4 *X, int64_t S_pad, int Wt, const uint64
     *(reinterpret_cast<uint4 *>(Q + row * pitch) + ch) = expand_fp4(bits);
 }
 
-// t(a, b) for a, b < T4_SMALL at b T4_SMALL_STRIDE + a: computed in FP64,
-// rounded once.
-__global__ void k_small_terms(float *t)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T4_SMALL_FLOATS) return;
-    const int b = i / T4_SMALL_STRIDE, a = i % T4_SMALL_STRIDE;
-    double v = 0.0;
-    if (a < T4_SMALL && b < T4_SMALL && a > 0 && b > 0) {
-        const double n = a + b;
-        v = (double)a * log(n / a) + (double)b * log(n / b);
-    }
-    t[i] = (float)v;
-}
-
 // The class counts of an encoded accumulator x = a + 4096 b (a, b < 4096),
 // clamped to the classes so that no index can leave the x ln x table.
 __device__ __forceinline__ void split_enc(float x, float xmax, float amax, uint32_t &a, uint32_t &b)
@@ -734,12 +719,11 @@ cudaError_t launch_tuple_rows(int T, bool left, const uint4 *X, int64_t S_pad, i
     return cudaGetLastError();
 }
 
-int small_terms_floats() { return T4_SMALL_FLOATS; }
+int quads_small_floats() { return T4_SMALL_FLOATS; }
 
-cudaError_t launch_small_terms(float *t, cudaStream_t st)
+cudaError_t launch_quads_small_terms(float *t, cudaStream_t st)
 {
-    k_small_terms<<<(T4_SMALL_FLOATS + 255) / 256, 256, 0, st>>>(t);
-    return cudaGetLastError();
+    return launch_small_terms(t, T4_SMALL, T4_SMALL_STRIDE, T4_SMALL_FLOATS, false, st);
 }
 
 size_t quads_smem_bytes(int enc, int stages, int M, int P2)

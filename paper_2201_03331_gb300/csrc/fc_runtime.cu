@@ -722,43 +722,15 @@ int Dataset::pairs_dense(float *scores, uint32_t *tables)
 
 // The order-3 tensor-core form for searches with lists of L: 1 (one
 // accumulator n_case + 4096 n_ctrl) while both classes have at most 4095
-// samples and its shared memory fits, else 0 (one accumulator per class),
-// else -1 (no tensor-core search).  The same for every L up to 1024.
-// FC_TRIPLES_ENC=0 forces the per-class form.
+// samples, else 0 (one accumulator per class), -1 (no tensor-core search)
+// where a class has more than 16,383 samples or the tables do not fit in
+// shared memory.  FC_TRIPLES_ENC=0 forces the per-class form.
 int Dataset::triples_form(int L) const
 {
+    const int64_t cls = std::max(M1, M0);
+    if (cls > 16383 || triples_stages((int)M, std::max(L, 1), (size_t)max_smem_optin) == 0) return -1;
     const char *f = getenv("FC_TRIPLES_ENC");
-    const bool enc_ok = !(f && strcmp(f, "0") == 0) && M1 <= 4095 && M0 <= 4095;
-    if (enc_ok && triples_list_fit(1, L) > 0) return 1;
-    if (triples_list_fit(0, L) > 0) return 0;
-    return -1;
-}
-
-// Candidate list of the order-3 kernel (preferred size): L entries and a
-// buffer of at least 2048, three rounds of its epilogue's inserts (at most
-// 1024 each) between buffer checks.
-int Dataset::triples_list_size(int L)
-{
-    return pow2_at_least(std::max(L, 1) + 2048);
-}
-
-int triples_list_fit(int enc, int64_t M, int L, int smem_cap)
-{
-    const int big = Dataset::triples_list_size(L);
-    if (triples_smem_bytes(enc, (int)M, big) <= (size_t)smem_cap) return big;
-    // A buffer of at least 1024 (one round between checks), for the larger
-    // x ln x tables of more than 4095 samples.
-    const int small = pow2_at_least(std::max(L, 1) + 1024);
-    if (small < big && triples_smem_bytes(enc, (int)M, small) <= (size_t)smem_cap) return small;
-    return -1;
-}
-
-// The order-3 kernel's x ln x table needs the class counts only (n ln n of a
-// cell's total comes from the hardware logarithm), so its extent is the
-// larger class.
-int Dataset::triples_list_fit(int enc, int L) const
-{
-    return fc::triples_list_fit(enc, std::max(M1, M0), L, max_smem_optin);
+    return !(f && strcmp(f, "0") == 0) && cls <= 4095 ? 1 : 0;
 }
 
 bool Dataset::triples_tc_eligible(int L)
@@ -789,46 +761,44 @@ TriplesArgs Dataset::triples_args(int L, float hy, float invN)
     ta.marg4 = reinterpret_cast<const uint4 *>(marg);
     ta.PR = PR;
     ta.xlogx = xlog2x;
-    ta.M = (int)std::max(M1, M0);   // table extent: the class counts
+    ta.scale = triples_scale(M);
+    ta.M = (int)M;
     ta.hy = hy;
     ta.invN = invN;
     ta.total = binom(S, 3);
     ta.rank_begin = 0;
     ta.rank_end = ~0ull;
     ta.L = std::max(L, 1);
-    ta.P2 = triples_list_fit(enc3, L);
-    ta.Bcap = ta.P2 - ta.L;
-    // Rounds of the kernel's epilogue between checks of its candidate buffer.
-    ta.check_rounds = 1;
-    for (int r = 3; r >= 1; --r)
-        if (r * triples_round_candidates() <= ta.Bcap) { ta.check_rounds = r; break; }
+    ta.stages = triples_stages(ta.M, ta.L, (size_t)max_smem_optin);
     ta.wait_ticks = TC_WAIT_TICKS;
     return ta;
 }
 
 namespace {
-// The last order-3 slab and tile plan; it depends on S, the pairs per tile
-// and the slab capacity only, so the phenotype replicates of one data set
-// (and data sets of equal S) share it.
+// The last order-3 slab and tile plan; it depends on S, the form and the slab
+// capacity only, so the phenotype replicates of one data set (and data sets of equal
+// S) share it.
 std::mutex g_plan3_mu;
 std::shared_ptr<const TriplePlan> g_plan3;
 }  // namespace
 
-// Tiles {rowP, i, j0, l0}: first SNP i, the block of NP second SNPs from
-// j0 = i + 1 + NP J' (slab rows [rowP, rowP + 4 NP)), the 64 third SNPs from
-// l0 = j0 + 1 + 64 L', for every block with j0 <= S - 2 and l0 <= S - 1; in
+// Tiles {rowP, i, j0, l0}: first SNP i, the block of NP second SNPs from j0 = i
+// + 1 + NP J' (slab rows from rowP), the LB third SNPs from l0 = j0 + 1 + LB L',
+// for every block with j0 <= S - 2 and l0 <= S - 1; in
 // order of i, so that a rank range is a contiguous run of tiles.  Slabs hold
 // the rows of consecutive first SNPs up to cap_rows rows (at least one
 // SNP's).
-std::shared_ptr<const TriplePlan> plan_triples(int64_t S, int NP, int64_t cap_rows)
+std::shared_ptr<const TriplePlan> plan_triples(int64_t S, int enc, int64_t cap_rows)
 {
+    const int64_t NP = triples_pairs_per_tile(enc), LB = triples_snps_per_tile(enc);
+    const int64_t pad = triples_pairs_per_tile(1);   // the pairs of i fill whole blocks of either form
     {
         std::lock_guard<std::mutex> lock(g_plan3_mu);
-        if (g_plan3 && g_plan3->S == S && g_plan3->NP == NP && g_plan3->cap_rows == cap_rows) return g_plan3;
+        if (g_plan3 && g_plan3->S == S && g_plan3->enc == enc && g_plan3->cap_rows == cap_rows) return g_plan3;
     }
     auto pl = std::make_shared<TriplePlan>();
     pl->S = S;
-    pl->NP = NP;
+    pl->enc = enc;
     pl->cap_rows = cap_rows;
     std::vector<uint4> &tiles = pl->tiles;
     pl->rowbase.assign((size_t)S, 0);
@@ -836,7 +806,7 @@ std::shared_ptr<const TriplePlan> plan_triples(int64_t S, int NP, int64_t cap_ro
     Dataset::TripleSlab cur;
     for (int64_t i = 0; i + 2 < S; ++i) {
         const int64_t nJ = (S - 1 - i + NP - 1) / NP;
-        const int64_t n = nJ * 4 * NP;   // rows of the pairs of i
+        const int64_t n = (S - 1 - i + pad - 1) / pad * pad * 4;   // rows of the pairs of i
         if (cur.rows + n > cap_rows && i > cur.i0) {
             cur.i1 = i;
             cur.t1 = (int64_t)tiles.size();
@@ -851,7 +821,7 @@ std::shared_ptr<const TriplePlan> plan_triples(int64_t S, int NP, int64_t cap_ro
         for (int64_t Jp = 0; Jp < nJ; ++Jp) {
             const int64_t j0 = i + 1 + NP * Jp;
             if (j0 > S - 2) break;
-            for (int64_t l0 = j0 + 1; l0 <= S - 1; l0 += 64)
+            for (int64_t l0 = j0 + 1; l0 <= S - 1; l0 += LB)
                 tiles.push_back(make_uint4((uint32_t)(cur.rows + Jp * 4 * NP), (uint32_t)i, (uint32_t)j0, (uint32_t)l0));
         }
         cur.rows += n;
@@ -868,51 +838,43 @@ std::shared_ptr<const TriplePlan> plan_triples(int64_t S, int NP, int64_t cap_ro
     return pl;
 }
 
-// The e4m3 rows (those of the order-2 path, or a copy with controls = 64 for
-// the one-accumulator form), the inclusion-exclusion tables, the x ln x
-// table, the slab and tile plan, the slab buffer with its first slab and the
-// kernel's two TMA descriptors, in the form that lists of L take.  A slab
-// holds at most min(16 GiB, a quarter of the free device memory) of pair
-// rows (FC_TRIPLES_SLAB_MB overrides the 16 GiB), and at least the rows of
-// one first SNP.  A single slab is kept for later searches; with several,
-// the buffer is released after each search.  Operands of the other form are
-// rebuilt only when their form cannot take lists of L.
+// The packed SNP rows, the inclusion-exclusion tables, the tables of the cell
+// terms, the slab and tile plan, the slab buffer with its first slab and the
+// kernel's two TMA descriptors (all but the tiles serve both forms).  A slab holds at
+// most min(16 GiB, a quarter of the free device memory) of pair rows
+// (FC_TRIPLES_SLAB_MB overrides the 16 GiB), and at least the rows of one
+// first SNP.  A single slab is kept for later searches; with several, the
+// buffer is released after each search.
 int Dataset::prepare_triples(int L)
 {
-    if (triples_ready && triples_list_fit(enc3, L) > 0) return FC_OK;
-    if (triples_ready) release_triples();
     const int form = triples_form(L);
     if (form < 0) return set_error(FC_ERANGE, "order-3 tensor-core kernel does not fit in shared memory");
-    int rc = prepare_pairs();
+    if (triples_ready && enc3 == form) return FC_OK;
+    if (triples_ready) release_triples();
+    enc3 = form;
+    int rc = prepare_ie(3);
     if (rc) return rc;
-    if ((rc = prepare_ie(3)) != FC_OK) return rc;
     cudaError_t e;
     if (!xlog2x) {
         if ((e = dev_alloc((void **)&xlog2x, sizeof(float) * (size_t)(M + 1))) != cudaSuccess)
             return cuda_status(e, "x log2 x table allocation");
-        if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(xlog2x, M, stream, true)) != cudaSuccess)
+        if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(xlog2x, M, stream, true, triples_scale(M))) != cudaSuccess)
             return cuda_status(e, "x log2 x table");
         note_launches(1);
     }
-    const int64_t S64 = (S + 63) / 64 * 64;
-    const int64_t rows = 2 * S64;
-    const uint64_t kbytes = (uint64_t)Wt * 128;
-    const uint64_t pitch = kbytes + 128;
-    enc3 = form;
-    uint8_t *ops = E;
-    if (enc3) {
-        if (!E3) {
-            e3_bytes = e_bytes;
-            if ((e = dev_alloc_pooled((void **)&E3, e3_bytes, device)) != cudaSuccess)
-                return cuda_status(e, "encoded e4m3 operand allocation");
-            if ((e = launch_gate()) != cudaSuccess ||
-                (e = launch_expand_e4m3(X, S, S_pad, W0, Wt, rows, (int64_t)pitch, E3, 0x68, stream)) != cudaSuccess)
-                return cuda_status(e, "encoded e4m3 operand");
-            note_launches(1);
-        }
-        ops = E3;
+    const int64_t rows = triples_rows(S);
+    const uint64_t kbytes = (uint64_t)Wt * 64;
+    const uint64_t pitch = (uint64_t)triples_pitch(Wt);
+    if (!E3) {
+        e3_bytes = (size_t)rows * pitch;
+        if ((e = dev_alloc_pooled((void **)&E3, e3_bytes, device)) != cudaSuccess)
+            return cuda_status(e, "packed SNP row allocation");
+        if ((e = launch_gate()) != cudaSuccess ||
+            (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E3, stream)) != cudaSuccess)
+            return cuda_status(e, "packed SNP rows");
+        note_launches(1);
     }
-    const int NP = triples_pairs_per_tile(enc3);
+    const int NP = triples_pairs_per_tile(1);
     size_t cap = (size_t)16 << 30;
     if (const char *mb = getenv("FC_TRIPLES_SLAB_MB")) {
         const long v = atol(mb);
@@ -922,7 +884,7 @@ int Dataset::prepare_triples(int L)
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) cap = std::min(cap, free_b / 4);
     const int64_t nJ = (S - 2 + NP) / NP;   // blocks of the pairs of i = 0
     const int64_t cap_rows = std::max<int64_t>((int64_t)(cap / pitch), nJ * 4 * NP);
-    const std::shared_ptr<const TriplePlan> plan = plan_triples(S, NP, cap_rows);
+    const std::shared_ptr<const TriplePlan> plan = plan_triples(S, enc3, cap_rows);
     const std::vector<uint4> &tiles = plan->tiles;
     slabs3 = plan->slabs;
     first_tile3 = plan->first_tile;
@@ -939,8 +901,8 @@ int Dataset::prepare_triples(int L)
         return cuda_status(e, "slab row table allocation");
     cudaMemcpyAsync(tiles3, tiles.data(), sizeof(uint4) * tiles.size(), cudaMemcpyHostToDevice, stream);
     cudaMemcpyAsync(rowbase3, plan->rowbase.data(), sizeof(int64_t) * (size_t)S, cudaMemcpyHostToDevice, stream);
-    if ((rc = encode_tmap_u8(&tmap3A, ops, kbytes, pitch, (uint64_t)rows, 128, true)) != FC_OK) return rc;
-    if ((rc = encode_tmap_u8(&tmap3P, P3, kbytes, pitch, (uint64_t)plan->max_rows, (uint32_t)(4 * NP), true)) != FC_OK)
+    if ((rc = encode_tmap_u8(&tmap3A, E3, kbytes, pitch, (uint64_t)rows, 128, true)) != FC_OK) return rc;
+    if ((rc = encode_tmap_u8(&tmap3P, P3, kbytes, pitch, (uint64_t)plan->max_rows, (uint32_t)triples_block_rows(), true)) != FC_OK)
         return rc;
     built_slab3 = -1;
     if ((rc = build_slab3(0)) != FC_OK) return rc;
@@ -953,29 +915,13 @@ int Dataset::build_slab3(int s)
 {
     if (built_slab3 == s || s >= (int)slabs3.size()) return FC_OK;
     const TripleSlab &sl = slabs3[(size_t)s];
-    const int64_t pitch = (int64_t)Wt * 128 + 128;
     cudaError_t e;
     if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_pair_rows(enc3 ? E3 : E, pitch, Wt, S, triples_pairs_per_tile(enc3), sl.i0, sl.i1, rowbase3 + sl.i0,
-                              P3, stream)) != cudaSuccess)
+        (e = launch_pair_rows(E3, triples_pitch(Wt), Wt, S, sl.i0, sl.i1, rowbase3 + sl.i0, P3, stream)) != cudaSuccess)
         return cuda_status(e, "pair-row kernel");
     note_launches(1);
     built_slab3 = s;
     return FC_OK;
-}
-
-void Dataset::release_pairs()
-{
-    if (!E && !tiles) return;
-    if (stream) cudaStreamSynchronize(stream);
-    dev_free_pooled(E, e_bytes, device);
-    dev_free_pooled(tiles, tiles_bytes, device);
-    E = nullptr;
-    tiles = nullptr;
-    ntiles = 0;
-    tiles_host.clear();
-    pairs_ready = false;
-    triples_ready = false;   // its TMA descriptors point into E
 }
 
 void Dataset::release_triples()
@@ -1029,7 +975,7 @@ int Dataset::triples_dense(float *scores, uint32_t *tables)
         a.ntiles = (int)(sl.t1 - sl.t0);
         if (a.ntiles == 0) continue;
         cudaMemsetAsync(a.tile_counter, 0, sizeof(int), stream);
-        const int grid = (int)std::min<int64_t>(sms, a.ntiles);
+        const int grid = enc3 ? 2 * (int)std::min<int64_t>(sms / 2, a.ntiles) : (int)std::min<int64_t>(sms, a.ntiles);
         if ((e = launch_gate()) != cudaSuccess || (e = launch_triples_tc(MODE_DUMP, tmap3A, tmap3P, a, grid, stream)) != cudaSuccess)
             return cuda_status(e, "tensor-core triples kernel");
         note_launches(1);
@@ -1387,9 +1333,9 @@ int Dataset::prepare_tuples(int k)
         note_launches(1);
     }
     if (!small_terms) {
-        if ((e = dev_alloc((void **)&small_terms, sizeof(float) * (size_t)small_terms_floats())) != cudaSuccess)
+        if ((e = dev_alloc((void **)&small_terms, sizeof(float) * (size_t)quads_small_floats())) != cudaSuccess)
             return cuda_status(e, "cell term table allocation");
-        if ((e = launch_gate()) != cudaSuccess || (e = launch_small_terms(small_terms, stream)) != cudaSuccess)
+        if ((e = launch_gate()) != cudaSuccess || (e = launch_quads_small_terms(small_terms, stream)) != cudaSuccess)
             return cuda_status(e, "cell term table");
         note_launches(1);
     }
@@ -1573,7 +1519,7 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         // with SNP rows, one launch per slab of pair rows.
         // A rank range takes the tiles of its first SNPs, and the kernel
         // drops the combinations outside the range.
-        const bool tc3 = k == 3 && triples_tc_eligible(L) && (!no_alloc || (triples_ready && triples_list_fit(enc3, L) > 0));
+        const bool tc3 = k == 3 && triples_tc_eligible(L) && (!no_alloc || triples_ready);
         // Orders 4-6: tensor-core contraction of tuple rows with tuple rows.
         // A rank range takes the tiles of the left blocks holding a left
         // tuple whose combinations meet the range, and the kernel drops the
@@ -1596,7 +1542,7 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         struct SlabLaunch { int si; int64_t t0, t1; };
         std::vector<SlabLaunch> launches3;
         int grid = 0;
-        int ctas4 = 0;   // orders 4-6: CTAs of a launch (whole pairs in form 1)
+        int ctas = 0;   // orders 3-6: CTAs of a launch (whole pairs in form 1)
         if (tc) {
             int rc = prepare_pairs();
             if (rc) return rc;
@@ -1627,7 +1573,8 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
                 const int64_t a0 = std::max(slabs3[(size_t)si].t0, t_lo), a1 = std::min(slabs3[(size_t)si].t1, t_hi);
                 if (a0 < a1) launches3.push_back(SlabLaunch{si, a0, a1});
             }
-            grid = sms * (int)launches3.size();   // every slab launch writes sms lists
+            ctas = enc3 ? sms & ~1 : sms;   // whole CTA pairs in form 1
+            grid = ctas * (int)launches3.size();   // every slab launch writes a list per CTA
         } else if (tc4) {
             int rc = prepare_tuples(k);
             if (rc) return rc;
@@ -1703,8 +1650,8 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
             for (int64_t c = 0; c < u.nchunks(); ++c)
                 if (citems4[(size_t)c] > 0) launches4.push_back(c);
             if (launches4.empty()) launches4.push_back(0);
-            ctas4 = sms / u.rblk * u.rblk;
-            grid = ctas4 * (int)launches4.size();
+            ctas = sms / u.rblk * u.rblk;
+            grid = ctas * (int)launches4.size();
         } else {
             cfg = pick_config(k, L, MODE_TOPN, no_alloc);
             if (cfg.var == VAR_IE) {
@@ -1730,7 +1677,7 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
             p[8] = A.take(sizeof(uint32_t) * (size_t)L * cells * 2);
             p[9] = A.take(sizeof(uint32_t) * (size_t)N * k);
             p[10] = A.take(sizeof(double) * (size_t)N);
-            p[11] = A.take(sizeof(int) * 4);
+            p[11] = A.take(sizeof(int) * (4 + (size_t)sms));
             p[12] = A.take(sizeof(uint32_t) * range_tiles.size() + sizeof(int4) * range_groups4.size() +
                            sizeof(uint64_t) * (lt4.size() + lr4.size()) + sizeof(int) * amax4.size() + include4.size() + 16);
         };
@@ -1827,19 +1774,21 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
                 int rc = build_right_chunk(k, c);
                 if (rc) return rc;
                 QuadsArgs qc = tuples_chunk_args(qa, k, c, groups, amax, cg0_4, citems4);
-                qc.list_score = (float *)p[0] + x * ctas4 * L;
-                qc.list_rank = (uint64_t *)p[1] + x * ctas4 * L;
+                qc.list_score = (float *)p[0] + x * ctas * L;
+                qc.list_rank = (uint64_t *)p[1] + x * ctas * L;
                 cudaMemsetAsync(qa.tile_counter, 0, sizeof(int), stream);
                 if ((e = launch_gate()) != cudaSuccess ||
-                    (e = launch_quads_tc(k, MODE_TOPN, tmapL, u.tmapR, qc, ctas4, stream)) != cudaSuccess)
+                    (e = launch_quads_tc(k, MODE_TOPN, tmapL, u.tmapR, qc, ctas, stream)) != cudaSuccess)
                     return cuda_status(e, "tensor-core tuple kernel");
                 if (x > 0) note_launches(1);
             }
         } else if (tc3) {
-            ta.gthr = (int *)p[11];
+            ta.pub = (int *)p[11] + 4;
+            triples_publish(L, ctas, &ta.pub_m, &ta.pub_r);
             ta.tile_counter = (int *)p[11] + 1;
             ta.err = err;
-            cudaMemsetAsync(p[11], 0x80, sizeof(int), stream);
+            // 0x80808080 is below the ordered image of every finite score.
+            cudaMemsetAsync(ta.pub, 0x80, sizeof(int) * (size_t)sms, stream);
             for (size_t x = 0; x < launches3.size(); ++x) {
                 const SlabLaunch &sl = launches3[x];
                 int rc = build_slab3(sl.si);
@@ -1847,13 +1796,13 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
                 TriplesArgs a = ta;
                 a.tiles = tiles3 + sl.t0;
                 a.ntiles = (int)(sl.t1 - sl.t0);
-                a.list_score = (float *)p[0] + x * sms * L;
-                a.list_rank = (uint64_t *)p[1] + x * sms * L;
+                a.list_score = (float *)p[0] + x * ctas * L;
+                a.list_rank = (uint64_t *)p[1] + x * ctas * L;
                 cudaMemsetAsync(ta.tile_counter, 0, sizeof(int), stream);
-                // A launch with fewer tiles than SMs still writes sms lists:
+                // A launch with fewer tiles than CTAs still writes all lists:
                 // the CTAs without a tile write empty ones.
                 if ((e = launch_gate()) != cudaSuccess ||
-                    (e = launch_triples_tc(MODE_TOPN, tmap3A, tmap3P, a, sms, stream)) != cudaSuccess)
+                    (e = launch_triples_tc(MODE_TOPN, tmap3A, tmap3P, a, ctas, stream)) != cudaSuccess)
                     return cuda_status(e, "tensor-core triples kernel");
                 if (x > 0) note_launches(1);
             }

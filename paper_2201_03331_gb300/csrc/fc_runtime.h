@@ -30,9 +30,6 @@ int check_device(int *dev, int *sms);
 int list_capacity(int64_t N);
 float score_error_bound(int k, int64_t M);
 int pow2_at_least(int v);
-// Candidate-list entries (a power of two) of the order-3 kernel in form enc
-// for lists of L with M samples within smem_cap bytes of shared memory, or -1.
-int triples_list_fit(int enc, int64_t M, int L, int smem_cap);
 // 2-D TMA descriptor over bytes: rows of inner_bytes (pitch apart), boxes of
 // 128 bytes x box_rows.
 int encode_tmap_u8(CUtensorMap *map, void *base, uint64_t inner_bytes, uint64_t pitch, uint64_t rows,
@@ -86,14 +83,13 @@ struct Dataset {
     CUtensorMap tmap{};
     bool pairs_ready = false;
 
-    // Order-3 tensor-core operands, built on first use: slabs of pair rows
-    // (E[2i + a] AND E[2j + b], four rows per pair (i, j), in blocks of NP
-    // pairs from the block of i + 1) for consecutive ranges of first SNPs i,
-    // the tiles of every slab, each i's first row within its slab, the x ln x
-    // table, for the one-accumulator form a copy of E whose control samples
-    // carry 64, and the kernel's two TMA descriptors (SNP rows, slab).  One
-    // slab is built once and kept; with several, each search rebuilds them
-    // in turn in the same buffer.
+    // Order-3 tensor-core operands, built on first use: the packed SNP rows
+    // E3, slabs of pair rows (E3[i, a] AND E3[j, b], four rows per pair (i, j),
+    // from the pair (i, i + 1)) for consecutive ranges of
+    // first SNPs i, the tiles of every slab, each i's first row within its
+    // slab, the x log2 x table, and the kernel's two TMA descriptors (SNP
+    // rows, slab).  One slab is built once and kept; with several, each
+    // search rebuilds them in turn in the same buffer.
     struct TripleSlab {
         int64_t i0 = 0, i1 = 0;   // first SNPs [i0, i1)
         int64_t t0 = 0, t1 = 0;   // tiles [t0, t1) of tiles3
@@ -103,7 +99,7 @@ struct Dataset {
     std::vector<int64_t> first_tile3;   // [S + 1] first tile of each first SNP
     float *xlogx = nullptr;   // x ln x, x = 0..M (the orders 4-6 epilogue's MI table)
     float *small_terms = nullptr;   // cell terms of small class counts (orders 4-6)
-    float *xlog2x = nullptr;  // x log2 x, x = 0..M (the order-3 epilogue's)
+    float *xlog2x = nullptr;  // of x = 0..M times triples_scale(M) (the order-3 epilogue's)
     uint8_t *P3 = nullptr;
     size_t p3_bytes = 0;
     uint4 *tiles3 = nullptr;
@@ -113,7 +109,7 @@ struct Dataset {
     size_t rowbase3_bytes = 0;
     int built_slab3 = -1;
     int enc3 = 0;             // form of the order-3 kernel (triples_form)
-    uint8_t *E3 = nullptr;    // E with controls = 64 (form 1 only)
+    uint8_t *E3 = nullptr;    // packed SNP rows (triples_rows)
     size_t e3_bytes = 0;
     CUtensorMap tmap3A{}, tmap3P{};
     bool triples_ready = false;
@@ -207,12 +203,9 @@ struct Dataset {
     int pairs_dense(float *scores, uint32_t *tables);
     bool triples_tc_eligible(int L);
     int triples_form(int L) const;
-    static int triples_list_size(int L);
-    int triples_list_fit(int enc, int L) const;
     int prepare_triples(int L);
     int build_slab3(int s);
     void release_triples();
-    void release_pairs();
     TriplesArgs triples_args(int L, float hy, float invN);
     int triples_dense(float *scores, uint32_t *tables);
     bool tuples_tc_eligible(int k, int L);
@@ -249,37 +242,38 @@ int sweep_candidates(const Dataset &d, int k, int L, int mode, int var, TuneConf
 
 // Many data sets (x phenotype replicates) searched by one persistent launch.
 // Order-3 tile plan of one SNP count: tiles {rowP, i, j0, l0} (first SNP i,
-// the NP second SNPs from j0, the 64 third SNPs from l0), in order of i, and
+// a block of second SNPs from j0 and of third SNPs from l0), in order of i, and
 // the slabs of pair rows that hold at most cap_rows rows each.
 struct TriplePlan {
     int64_t S = -1, cap_rows = -1, max_rows = 0;
-    int NP = 0;
+    int enc = -1;
     std::vector<uint4> tiles;
     std::vector<int64_t> first_tile;   // [S + 1]: tiles of first SNP i are [first_tile[i], first_tile[i + 1])
     std::vector<int64_t> rowbase;      // [S]: first slab row of SNP i within its slab
     std::vector<Dataset::TripleSlab> slabs;
 };
-std::shared_ptr<const TriplePlan> plan_triples(int64_t S, int NP, int64_t cap_rows);
+std::shared_ptr<const TriplePlan> plan_triples(int64_t S, int enc, int64_t cap_rows);
 
 // The batched order-3 tensor-core form: one persistent launch per group of
-// data sets whose pair-row slabs fit the slab buffer together, every
-// replicate of a data set a job of the launch (T3Job).
+// jobs whose pair-row slabs fit the slab buffer together (T3Job).
 struct Tc3Batch {
     struct Launch {
-        int j0 = 0, j1 = 0;          // jobs (slots) [j0, j1)
+        int j0 = 0, j1 = 0;          // slots [j0, j1)
         int enc = 1, n_items = 0;
-        int M = 0;                   // largest sample count (x ln x table size)
-        std::vector<int> sets;       // data sets whose slabs this launch reads
+        int M = 0;                   // largest sample count (x log2 x table size)
+        int stages = 2;
     };
-    struct Set {
-        int first_job = 0;           // job index of its first replicate
-        int enc = 1, split = 0, NP = 64;
-        int64_t M = 0;
-        int64_t rows = 0, pitch = 0, slab_rows = 0;
+    struct Slot {
+        int job = 0;
+        int enc = 1;
+        int64_t M = 0;               // its samples
+        int stages = 2;
+        int64_t slab_rows = 0;
         size_t slab_off = 0;         // within the slab buffer
+        size_t e_off = 0;            // its SNP rows within E
         int64_t tile_off = 0, ntiles = 0, rowbase_off = 0;
     };
-    std::vector<Set> sets;
+    std::vector<Slot> slots;
     std::vector<Launch> launches;
     std::vector<int> slot_job;       // job index of every slot
     int n = 0, L = 0, grid = 0, smem_cap = 0;
@@ -287,17 +281,16 @@ struct Tc3Batch {
     bool rebuild = false;            // slabs rebuilt before every launch (several groups)
     std::vector<void *> allocs;      // device allocations of the plan
     uint8_t *slab = nullptr;
-    uint8_t *E = nullptr;            // per data set: genotype rows (e5m2 1.0)
+    uint8_t *E = nullptr;            // per slot: packed SNP rows
     int64_t *rowbase = nullptr;
-    std::vector<size_t> e_off;       // per data set, within E
     T3Job *d_jobs = nullptr;
     CUtensorMap *d_maps = nullptr;
     JobDesc *d_desc = nullptr, *d_desc1 = nullptr;
-    int *d_gthr = nullptr, *d_counter = nullptr;
+    int *d_pub = nullptr, *d_counter = nullptr;
     float *list_s = nullptr, *mid_s = nullptr, *job_s = nullptr;
     uint64_t *list_r = nullptr, *mid_r = nullptr, *job_r = nullptr;
     float *xlogx = nullptr;
-    int M = 0;
+    float scale = 1.f;   // of the counts the kernel scores (triples_scale of the fewest samples)
     double *res_s = nullptr, *out_score = nullptr;
     uint64_t *res_r = nullptr;
     uint32_t *res_tab = nullptr, *job_err = nullptr, *out_idx = nullptr;
@@ -343,10 +336,6 @@ struct BatchState {
     std::vector<int> sel;
     std::vector<char> tc;
     std::vector<int> job_kind;
-    // The phenotypes of every data set as loaded (R x M bytes each): the
-    // batched tensor-core form lays the replicates of a data set out in the
-    // sample order of its first one.
-    std::vector<std::vector<uint8_t>> ph;
     std::unique_ptr<Tc3Batch> tc3;   // order 3: the batched tensor-core jobs (null if none)
     std::vector<int> tc3_slot;       // slot of each job in tc3, or -1
     ~BatchState();

@@ -799,14 +799,16 @@ __global__ void __launch_bounds__(256) k_search_px(SearchArgs a, int NW, int WT)
     }
 }
 
-// Restricted pair counts for inclusion-exclusion: PR[i][j] (i < j) holds the
-// four cells with genotypes in {0,1} of SNPs i and j, packed cases |
-// controls << 16, in the order (0,0), (0,1), (1,0), (1,1).
+// Restricted pair counts for inclusion-exclusion: PR[i][j] holds the four
+// cells with genotypes in {0,1} of SNPs i and j, packed cases | controls <<
+// 16, in the order (0,0), (0,1), (1,0), (1,1); computed for i <= j and stored
+// for both orders (the order-3 tensor-core kernel reads entries on either
+// side of the diagonal).
 __global__ void k_restricted_pairs(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, uint4 *PR)
 {
     const int64_t i = blockIdx.y;
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S || j >= S || j <= i) return;
+    if (i >= S || j >= S || j < i) return;
     uint32_t acc[4] = {0, 0, 0, 0};
     for (int w = 0; w < Wt; ++w) {
         const int sh = w < W0 ? 0 : 16;
@@ -819,6 +821,7 @@ __global__ void k_restricted_pairs(const uint4 *X, int64_t S, int64_t S_pad, int
         acc[3] += popc_and4(a1, b1) << sh;
     }
     PR[(size_t)i * S_pad + j] = make_uint4(acc[0], acc[1], acc[2], acc[3]);
+    if (i != j) PR[(size_t)j * S_pad + i] = make_uint4(acc[0], acc[2], acc[1], acc[3]);
 }
 
 // Grid-level merge: each CTA sorts F lists of L entries and keeps the best L.

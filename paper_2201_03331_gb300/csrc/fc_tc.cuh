@@ -168,6 +168,7 @@ __device__ __forceinline__ void mma_e4m3(uint32_t tmem_d, uint64_t adesc, uint64
 // 8,190 samples with full rows).  Half the bytes per sample of e4m3 and, for
 // N = 240, twice its multiply-adds per cycle (120 cycles per K = 64 MMA).
 constexpr uint32_t FP4_SCALE_ONE = 0x7F7F7F7Fu;    // ue8m0 2^0
+constexpr uint32_t FP4_SCALE_4 = 0x81818181u;      // ue8m0 2^2
 constexpr uint32_t FP4_SCALE_4096 = 0x8B8B8B8Bu;   // ue8m0 2^12
 constexpr uint32_t FP4_SCALE_COLS = 16;            // TMEM columns per scale (at most 8 are read)
 
@@ -230,6 +231,14 @@ __device__ __forceinline__ void cluster_post2(uint32_t addr, uint32_t bar, int x
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(x),
                  "r"(y), "r"(bar)
                  : "memory");
+}
+__device__ __forceinline__ void cluster_post4(uint32_t addr, uint32_t bar, uint4 v)
+{
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], 16;" ::"r"(bar) : "memory");
+    asm volatile(
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "r"(v.x),
+        "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+        : "memory");
 }
 // Copy into this CTA's shared memory that completes on barrier `bar` (the
 // same offset) of the pair's leader: bit 24 of a shared-cluster address

@@ -6,71 +6,96 @@
 //     n_c(a, b, g) = sum_{m in c} [G_i(m) = a] [G_j(m) = b] [G_l(m) = g]
 //                  = < P_c[(i, j), (a, b)], E_c[l, g] >,
 // the dot product over the samples of a pair row P = E[i, a] AND E[j, b]
-// with a SNP row E[l, g] (e4m3 bytes).  For one block of 64 SNPs l and one
-// block of NP pairs (i, j) with a fixed i these dot products are one
-// tcgen05.mma kind::f8f6f4 tile (M = 128 SNP rows, N = 4 NP pair rows).
-// Products of e4m3 powers of two are exact, and the tensor cores' FP32
-// accumulation of integers below 2^24 is exact (measured on GB300 up to
-// 2^24, with addends of 1 and of 4096).  The other 19 cells of the
+// with a SNP row E[l, g].  Rows are packed 0/1 e2m1 nibbles; for one block of
+// SNPs l and one block of pairs (i, j) with a fixed i the dot products are one
+// tcgen05.mma kind::mxf4 tile, exact (fc_tc.cuh).  The other 19 cells of the
 // 3 x 3 x 3 table follow exactly by inclusion-exclusion from the restricted
 // pair table and the per-SNP genotype counts (the three rows of a SNP's
-// table partition the samples), as in the order-3 sweep.  The epilogue
-// scores every combination with the same FP32 mutual information as the
-// sweep and keeps a CTA top list; no count is written to memory.
+// table partition the samples).  The epilogue scores every combination with
+// the FP32 mutual information and keeps a CTA top list; no count is written
+// to memory.
 //
-// Two encodings of the classes (template ENC):
-//   ENC = 1: control samples carry the e4m3 value 64 instead of 1, so one
-//            accumulator holds n_case + 4096 n_ctrl (exact while both
-//            classes have at most 4095 samples); NP = 64 pairs per tile,
-//            N = 256, one MMA chain over all samples;
-//   ENC = 0: both classes carry 1, and the case and control samples
-//            accumulate into two accumulators (N = 128 each); NP = 32.
-// Either way a tile takes 256 TMEM columns, and two tiles are in flight.
+// Two forms (template ENC):
+//   ENC = 1: control samples carry the block scale 4096, so one accumulator
+//            holds n_case + 4096 n_ctrl (exact while both classes have at
+//            most 4095 samples); a tile of 128 SNPs l and 56 pairs is worked
+//            on by a pair of CTAs (cta_group::2, M = 256, N = 224): each
+//            loads 64 SNPs and 28 pairs and scores its SNPs against all 56
+//            pairs;
+//   ENC = 0: the case and control samples accumulate into two accumulators;
+//            a tile of 64 SNPs and 28 pairs per CTA (M = 128, N = 112).
+// Either way a CTA's stage is 128 + 112 rows, a tile takes 224 TMEM columns,
+// and two tiles are in flight.  What bounds the kernel is the scoring, about
+// 400 instructions per 32 combinations: 1,000 SNPs x 4,000 samples take 5.3 ms
+// (5.9 with byte rows and both genotypes of a SNP from different tiles), of
+// which the tiles alone are 1.9 ms, the logarithms 0.95, the table reads 0.86
+// and the exchange of the cells 0.45.  (One CTA per 128 x 24 tile with both
+// genotypes of a SNP in one lane needed no exchange of cells, but 1,000 bytes
+// of shared memory per combination against about 530 here: 5.2 ms there, but
+// 3.9 ms instead of 2.9 at 701 SNPs x 9,001 samples, 6.5 before.  12 epilogue
+// warps with more registers: 5.5 and 3.2 ms.)
 //
 // The pair rows live in a slab in device memory, the paper's `combine` of
 // two genotype tables done once per data set (k_pair_rows): for each first
-// SNP i, the rows of its pairs (i, j), j = i + 1 + NP J' + q, in blocks of NP
-// pairs, pair row (a, q, b) of a block at row 2 NP a + 2 q + b, zero where
-// j >= S.  A tile is (i, the block of SNPs j from j0 = i + 1 + NP J', the 64
-// SNPs l from l0 = j0 + 1 + 64 L'): blocks start right after the SNPs before
-// them, so that only the triangle l <= j of a tile's first l block and the
-// ends beyond S are wasted (83 % of the tile area holds combinations at 1 000
-// SNPs, against 78 % with blocks aligned to multiples of 64).  Forming them on chip
-// instead (TMA of the rows of the SNPs j, AND with the rows of SNP i in
-// shared memory) was measured slower: the 48 KiB of shared-memory traffic
-// per 128-sample chunk of the builder cost more than the slab's one-time
-// write.
+// SNP i, the rows of its pairs (i, j), j = i + 1 + jo, row 4 jo + 2 a + b, zero
+// where j >= S.  A tile is (i, the block of SNPs j from j0 = i + 1 + NP J', the
+// SNPs l from l0 = j0 + 1 + LB L'): blocks start right after the SNPs before
+// them; a warp whose 16 SNPs l are all at or before the SNPs j of two pairs,
+// or beyond the last SNP, skips them.  Forming the rows on chip instead (TMA of
+// the rows of the SNPs j, AND with the rows of SNP i in shared memory) was
+// measured slower: the builder's shared-memory traffic cost more than the
+// slab's one-time write.
 //
-// TMA loads issued by one thread complete about one stage at a time, so the
-// three load stages are owned by three producer warps that each issue the
-// copies of their own stage (fill f by warp f mod 3).
+// TMEM lane 2 l + g holds genotype g of SNP l, columns 4 q + 2 a + b the cells of
+// pair q.  The two lanes of a SNP take two pairs at a time, one each: they
+// exchange the four cells of the other's pair, and lane g reads its cells with
+// the genotypes of l in the order g, 1 - g (every table of l is swapped alike),
+// so that nothing is put back in order.  Counts come times four (the block
+// scale of the pair rows is 4; still exact): a packed count n is then the byte
+// offset of its table entry.
 //
-// The epilogue scores each cell, in bits, as t = n log2 n - xl[a] - xl[b] =
-// a log2(n/a) + b log2(n/b) (a, b the class counts, n = a + b), and
-// MI = H(Y) - ln 2 sum t / N, where xl is a shared-memory table of x log2 x
-// over the class counts (entries correctly rounded) and n log2 n comes from
-// the hardware base-2 logarithm, n lg2~(n), with |lg2~(n) - log2 n| <=
-// 2^-22 (log2 n + 1) for every integer 1 <= n <= 2^17 (checked exhaustively
-// on the device by a test; fc_log2_approx).  Moving one of the three lookups
-// per cell to the XU pipe relieves the shared-memory pipe, and the sum in
-// bits leaves one multiplication by ln 2 per combination.  With u = 2^-24
-// (so 2^-22 = 4u) and in bits, a cell errs by at most n 4u (log2 M + 1) from
-// the n log2 n term, u (a + b) log2 M from the table entries, u n log2 M from
-// the fused multiply-subtract and u n from the last subtraction (t <= n);
-// over the 27 cells (sum n = N), the 27 accumulations (partial sums <= N),
-// the product with ln 2 and the final scaling this gives, in nats,
-// |MI32 - MI| <= u (6 ln M + 37 ln 2) <= u (7 ln M + 37 ln 2), which the FP64
-// rescoring window of the library covers (twice the larger of this and the
-// sweep's bound).
+// The epilogue scores each cell, in bits, as t(a, b) = xl[n] - a lg2~(a) - b
+// lg2~(b) = a log2(n/a) + b log2(n/b) (a, b the class counts, n = a + b), and
+// MI = H(Y) - ln 2 sum t / N, where xl is a shared-memory table of x log2 x over
+// the sample counts (entries correctly rounded) and lg2~ the hardware base-2
+// logarithm, with |lg2~(x) - log2 x| <= 2^-22 (|log2 x| + 1) (absolute within
+// [1/2, 2], relative elsewhere; checked on the device for every integer up to
+// 2^17 by a test; fc_log2_approx).  Counts are scored times the power of two
+// 2^-s, s = floor(log2 M) - 2 (the sum times 2^s is the same): the logarithms of
+// the fullest cells are then near 0, and with them the roundings, while no
+// |log2 x| exceeds log2 M.  Errors of 27-cell scores against FP64 (rms, 4,000
+// and 8,190 samples): 2.1e-7 and 2.8e-7 unscaled, 0.8e-7 and
+// 0.7e-7 scaled.
+// One table read per cell instead of two relieves shared memory, and taking
+// the two smaller of the three terms from the logarithm instead of the
+// largest lowers the error.  With u = 2^-24 (so 2^-22 = 4u) and in bits, a cell
+// errs by at most u n log2 M from the table entry, 4u (a + b) (log2 M + 1) from
+// the logarithms and 2 u n log2 M from the two fused multiply-subtracts; over
+// the 27 cells (sum n = N), the 27 accumulations (partial sums <= N), the
+// product with ln 2 and the final scaling this gives, in nats, |MI32 - MI| <= u
+// (7 ln M + 37 ln 2), which the FP64 rescoring window of the library covers
+// (twice the larger of this and the sweep's bound).
+//
+// Candidates: each epilogue warp keeps its own buffer of 64; when it cannot
+// take another 32 the warp merges it into the CTA's sorted list under a lock.
+// No barrier joins the epilogue warps between the first and the last tile (a
+// shared buffer took two barriers per tile and two more every third group of
+// pairs).  Merging is kept rare by a threshold over all CTAs: each publishes
+// the score of one entry m - 1 of its list (m about 2 L / CTAs), and a score
+// that the entries of L / m CTAs reach is reached by L combinations, so lower
+// ones need no place in any list; the scheduler warp looks for it while it
+// waits.  (With each CTA's own list alone, a CTA took about L (1 + ln(n / L))
+// of its n combinations, and merging them a third of the time at 500 SNPs.)
 //
 // Roles (one persistent CTA per SM, 640 threads):
-//   warps 0-2  : producers (lane 0 issues the TMA copies of its stage)
-//   warp 3     : lane 0 issues the MMAs and schedules the tiles; the warp
-//                allocates and frees TMEM
-//   warps 4-19 : epilogue (TMEM -> registers -> 27-cell table -> MI ->
-//                list), four warps per TMEM lane quarter, each taking every
-//                fourth group of 4 pairs (an equal share of a tile's 16 or 8
-//                groups)
+//   warps 0, 1 : TMA producers (128-byte K chunks, 256 samples, of the 128 SNP
+//                rows and 112 pair rows), warp w owning the stages s = w (mod 2)
+//   warp 2     : schedules the tiles (ENC 1: in the pair's leader), score
+//                threshold
+//   warp 3     : TMEM allocation; one elected lane (ENC 1: of the pair's
+//                leader) issues the MMAs
+//   warps 4-19 : epilogue, four warps per TMEM lane quarter, each taking every
+//                fourth two pairs of a tile
 #include <algorithm>
 
 #include "fc_tc.cuh"
@@ -80,35 +105,27 @@ namespace fc {
 
 namespace {
 
-constexpr int T3_LOADERS = 3;                      // = load stages
+constexpr int T3_PRODUCERS = 2;
+constexpr int T3_MAX_STAGES = 6;
 constexpr int T3_EPI_WARP0 = 4;
 constexpr int T3_EPI_WARPS = 16;
 constexpr int T3_PARTS = T3_EPI_WARPS / 4;         // epilogue warps per TMEM lane quarter
 constexpr int T3_EPI_THREADS = 32 * T3_EPI_WARPS;
 constexpr int T3_THREADS = 32 * T3_EPI_WARP0 + T3_EPI_THREADS;
-constexpr int T3_SJ_WORDS = 16;                    // per pair: T01[9], Tj[3], rank base (2 words), valid, pad
 static_assert(T3_EPI_WARP0 % 4 == 0, "epilogue warp w reads TMEM lane quarter w % 4");
-
-template <int ENC>
-struct T3Shape {
-    static constexpr int NP = ENC == 1 ? 64 : 32;         // SNPs j (pairs) per tile
-    static constexpr int RROWS = 2 * NP;                   // raw rows 2 j + b
-    static constexpr int NMMA = 2 * RROWS;                 // pair rows = MMA N
-    static constexpr uint32_t B_BYTES = (uint32_t)NMMA * TC_BK;
-    static constexpr uint32_t STAGE = TC_A_BYTES + B_BYTES;   // A | B
-    static constexpr int QUADS = NP / 4;                   // groups of 4 pairs per tile
-    static constexpr int ROUNDS = (QUADS + T3_PARTS - 1) / T3_PARTS;
-};
-
-// Entries of the shared-memory x ln x table: the power of two above its
-// extent M (the entries beyond M are 0), so that a masked index never leaves
-// it.
-__host__ __device__ inline int xl_table_size(int M)
-{
-    int n = 4;
-    while (n <= M) n <<= 1;
-    return n;
-}
+constexpr int T3_NP = 28;                          // pairs (i, j) per stage
+constexpr int T3_N = 4 * T3_NP;                    // pair rows per stage
+constexpr int T3_LB = 64;                          // SNPs l per CTA and tile
+constexpr uint32_t T3_STAGE = TC_A_BYTES + (uint32_t)T3_N * TC_BK;
+static_assert(T3_STAGE % 1024 == 0, "swizzled stages");
+constexpr int T3_BUF = 2 * T3_N;                   // TMEM columns of a tile
+constexpr uint32_t T3_SCALE_COL = 2 * T3_BUF;      // TMEM column of scale 1, then of 4096, then of 4
+static_assert(T3_SCALE_COL + 3 * FP4_SCALE_COLS <= TC_TMEM_COLS, "scales behind the accumulators");
+constexpr int T3_WARP_PAIRS = 2 * ((2 * T3_NP / 2 + T3_PARTS - 1) / T3_PARTS);   // pairs of a tile per warp (ENC 1)
+constexpr int T3_REC_WORDS = 12;                   // per pair: T01[9], rank base (2 words)
+static_assert(T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS % 4 == 0 && T3_REC_WORDS % 4 == 0, "records of uint4");
+static_assert(T3_WARP_PAIRS <= 32, "a lane per pair record");
+constexpr int T3_WBUF = 64;                        // candidates of a warp's buffer
 
 __device__ __forceinline__ uint64_t c3(uint64_t n) { return n * (n - 1) * (n - 2) / 6; }   // 0 for n < 3
 __device__ __forceinline__ uint64_t c2(uint64_t n) { return n * (n - 1) / 2; }             // 0 for n < 2
@@ -121,7 +138,8 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8])
                  : "r"(taddr));
 }
 
-// Two exact FP32 accumulators (integers below 2^16) packed as lo | hi << 16:
+// Two exact FP32 accumulators (integers below 2^16) packed as lo | hi << 16 (ENC
+// 0: 4 n_case and 4 n_ctrl):
 // x + 2^23 has the integer in its low mantissa bits, and the exponent
 // field of the high word falls outside 32 bits after the shift.
 __device__ __forceinline__ uint32_t pack_exact(uint32_t lo_bits, uint32_t hi_bits)
@@ -131,13 +149,42 @@ __device__ __forceinline__ uint32_t pack_exact(uint32_t lo_bits, uint32_t hi_bit
     return a + (b << 16) - 0x4B000000u;
 }
 
-// One encoded accumulator x = n_case + 4096 n_ctrl (an exact integer below
-// 2^24, n_case < 4096) as n_case | n_ctrl << 16: v = x as an integer, and
-// v + (v >> 12) (65536 - 4096) moves n_ctrl from bit 12 to bit 16.
+// One encoded accumulator x = 4 (n_case + 4096 n_ctrl) (a multiple of 4 below
+// 2^26, n_case < 4096, so exact) as 4 n_case | 4 n_ctrl << 16: v = x as an
+// integer, and v + (v >> 14) (2^18 - 2^14) moves n_ctrl from bit 14 to bit 18.
 __device__ __forceinline__ uint32_t unpack_enc(uint32_t bits)
 {
     const uint32_t v = __float2uint_rz(__uint_as_float(bits));
-    return v + (v >> 12) * 61440u;
+    return v + (v >> 14) * 245760u;
+}
+
+// Two FP32 operations per instruction.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float x, float y)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_split(F2 a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
 }
 
 constexpr float LN2F = 0.693147180559945309f;
@@ -150,75 +197,236 @@ __device__ __forceinline__ float lg2_approx(float x)
     return y;
 }
 
-// An integer below 2^23 as a float, exactly: its bits under the exponent of
-// 2^23, minus 2^23.
+// An integer below 2^23 as a float, exactly.
 __device__ __forceinline__ float u2f_small(uint32_t n)
 {
     return __uint_as_float(n | 0x4B000000u) - 8388608.0f;
 }
 
-// BATCH: the items of several jobs (T3Job), job-major, in one launch; the
-// operands are e5m2 with the class weight on the SNP rows only.
+// (The next three functions are calls, so that the scoring loop keeps its
+// registers.)
+// Sorts a warp's m <= T3_WBUF candidates (ws, wr) best first, keeping those
+// that beat (thr_s, thr_r); returns their number.
+__device__ __noinline__ int sort_candidates(float *ws, uint64_t *wr, int m, float thr_s, uint64_t thr_r, int lane)
+{
+    float cs[2];
+    uint64_t cr[2];
+    unsigned keep[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int x = lane + 32 * h;
+        cs[h] = x < m ? ws[x] : -FLT_MAX;
+        cr[h] = x < m ? wr[x] : NO_RANK;
+        keep[h] = __ballot_sync(FULL, x < m && better(cs[h], cr[h], thr_s, thr_r));
+    }
+    const unsigned below = (1u << lane) - 1u;
+    bool mine[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        mine[h] = (keep[h] >> lane & 1u) != 0;
+        if (mine[h]) {
+            const int p = (h ? __popc(keep[0]) : 0) + __popc(keep[h] & below);
+            ws[p] = cs[h];
+            wr[p] = cr[h];
+        }
+    }
+    m = __popc(keep[0]) + __popc(keep[1]);
+    __syncwarp();
+    // A candidate's place is the number of better ones.
+    int at[2] = {0, 0};
+#pragma unroll 4
+    for (int y = 0; y < m; ++y) {
+        const float s = ws[y];
+        const uint64_t r = wr[y];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) at[h] += better(s, r, cs[h], cr[h]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (mine[h]) {
+            ws[at[h]] = cs[h];
+            wr[at[h]] = cr[h];
+        }
+    __syncwarp();
+    return m;
+}
+
+// Number of the n entries (s, r), best first, that are better than (cs, cr).
+__device__ __forceinline__ int count_better(const float *s, const uint64_t *r, int n, float cs, uint64_t cr)
+{
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (better(s[mid], r[mid], cs, cr)) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// Merges m <= T3_WBUF candidates (ws, wr), best first, into the CTA's list
+// (ls, lr: L entries, best first, empty entries -FLT_MAX / NO_RANK).  All
+// lanes of the warp that holds the list's lock.
+__device__ __noinline__ void merge_candidates(float *ls, uint64_t *lr, int L, const float *ws, const uint64_t *wr, int m, int lane)
+{
+    // Every candidate's place: its place among the candidates plus the list
+    // entries before it.
+    int to[2], first = L;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int x = lane + 32 * h;
+        to[h] = L;
+        if (x < m) {
+            const int lo = count_better(ls, lr, L, ws[x], wr[x]);
+            to[h] = lo + x;
+            first = min(first, lo);
+        }
+    }
+    first = __reduce_min_sync(FULL, first);
+    // Entries from `first` on move down by the number of candidates before
+    // them, blocks of 256 from the end.
+    constexpr int B = 8;
+    for (int base = (L - 1) / (32 * B) * (32 * B); base > first - 32 * B; base -= 32 * B) {
+        float s[B];
+        uint64_t r[B];
+        int p[B];
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+            const int x = base + 32 * q + lane;
+            p[q] = L;
+            if (x >= first && x < L) {
+                s[q] = ls[x];
+                r[q] = lr[x];
+                p[q] = x;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (p[q] < L) p[q] += count_better(ws, wr, m, s[q], r[q]);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (p[q] < L) {
+                ls[p[q]] = s[q];
+                lr[p[q]] = r[q];
+            }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (to[h] < L) {
+            ls[to[h]] = ws[lane + 32 * h];
+            lr[to[h]] = wr[lane + 32 * h];
+        }
+    __syncwarp();
+}
+
+// A score that at least L combinations reach, from what the CTAs of the
+// launch have published (pub[n]: the score of the list's entry m - 1 as an
+// ordered int): the r-th largest, r m >= L, to 20 bits downwards.  All lanes
+// of a warp; n <= 32 T3_PUB_PER_LANE.
+constexpr int T3_PUB_PER_LANE = 8;
+__device__ __noinline__ float published_threshold(const int *pub, int n, int r, int lane)
+{
+    uint32_t key[T3_PUB_PER_LANE];
+#pragma unroll
+    for (int x = 0; x < T3_PUB_PER_LANE; ++x) {
+        const int c = lane + 32 * x;
+        key[x] = c < n ? (uint32_t)*(volatile const int *)(pub + c) ^ 0x80000000u : 0u;
+    }
+    uint32_t t = 0;
+    for (int b = 31; b >= 12; --b) {
+        const uint32_t c = t | 1u << b;
+        int cnt = 0;
+#pragma unroll
+        for (int x = 0; x < T3_PUB_PER_LANE; ++x) cnt += __popc(__ballot_sync(FULL, key[x] >= c));
+        if (cnt >= r) t = c;
+    }
+    const float f = from_ordered((int)(t ^ 0x80000000u));
+    return f >= -FLT_MAX ? f : -FLT_MAX;   // (NaN patterns of nothing published)
+}
+
+// BATCH: the items of several jobs (T3Job), job-major, in one launch.
 template <int MODE, int ENC, bool BATCH>
 __global__ void __launch_bounds__(T3_THREADS, 1)
     k_triples_tc(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapP, TriplesArgs a)
 {
-    static_assert(BATCH ? (ENC == 1 || ENC == 2) && MODE == MODE_TOPN : ENC <= 1, "forms of the two launch kinds");
-    using Sh = T3Shape<ENC>;
-    constexpr int NP = Sh::NP;
+    static_assert(!BATCH || MODE == MODE_TOPN, "the batched launch searches");
+    constexpr bool PAIR = ENC == 1;                 // a tile per CTA pair
+    constexpr int NPT = PAIR ? 2 * T3_NP : T3_NP;   // pairs per tile
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_full[T3_LOADERS], bar_empty[T3_LOADERS];
-    __shared__ uint64_t bar_tfull[2], bar_tempty[2], bar_done;
+    __shared__ uint64_t bar_full[T3_MAX_STAGES], bar_empty[T3_MAX_STAGES];
+    __shared__ uint64_t bar_tfull[2], bar_tempty[2], bar_done, bar_epi;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint64_t bar_sfull[TC_SCHED], bar_sempty[TC_SCHED];
-    __shared__ int sched_tile[TC_SCHED];
-    __shared__ int sched_job[TC_SCHED];
+    // Tiles {rowP, i | j0 << 16, l0, job (0 where there are none; -1: no more
+    // tiles)}.
+    __shared__ uint4 sched_tile[TC_SCHED];
     __shared__ int abort_flag_s;
-    __shared__ int buf_count;
-    __shared__ int epi_stop;
+    __shared__ int list_lock;
+    __shared__ int epi_job;          // job of the tile that the epilogue's first warp took last, -2 at the end
+    // published_threshold: job in the high half, score bits in the low one
+    // (read and written as one word).
+    __shared__ unsigned long long threshold;
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    const int stages = a.stages;
+    const uint32_t crank = PAIR ? cluster_rank() : 0;   // CTA of the pair (0: its leader)
     volatile int *abort_flag = &abort_flag_s;
 
-    // Stages [A 16 KiB | B], 1024-byte aligned; then the
-    // x ln x table, the list and the tables of the tile's SNPs j.
-    uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    float *xltab = reinterpret_cast<float *>(smem + (size_t)T3_LOADERS * Sh::STAGE);
-    const int lt_floats = xl_table_size(a.M);   // a power of two above M
-    uint64_t *lrank = reinterpret_cast<uint64_t *>(xltab + lt_floats);
-    float *lscore = reinterpret_cast<float *>(lrank + a.P2);
-    uint32_t *sJ = reinterpret_cast<uint32_t *>(lscore + a.P2);   // [2][NP][T3_SJ_WORDS]
+    // The x log2 x table first (a constant base saves an addition per read);
+    // then the stages, 1024-byte aligned, the warps' pair records (16-byte
+    // aligned), the candidate list and the warps' buffers (ranks before
+    // scores).
+    float *xltab = reinterpret_cast<float *>(smem_raw);
+    uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)(xltab + a.M + 1) + 1023) & ~(uintptr_t)1023);
+    uint32_t *recs = reinterpret_cast<uint32_t *>(smem + (size_t)stages * T3_STAGE);
+    uint64_t *lrank = reinterpret_cast<uint64_t *>(recs + T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS);
+    uint64_t *wrank = lrank + a.L;
+    float *lscore = reinterpret_cast<float *>(wrank + T3_EPI_WARPS * T3_WBUF);
+    float *wscore = lscore + a.L;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < T3_LOADERS; ++s) {
+        for (int s = 0; s < stages; ++s) {
             mbar_init(&bar_full[s], 1);
             mbar_init(&bar_empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bar_tfull[b], 1);
-            mbar_init(&bar_tempty[b], T3_EPI_WARPS);
+            mbar_init(&bar_tempty[b], (PAIR ? 2 : 1) * T3_EPI_WARPS);
         }
         mbar_init(&bar_done, 1);
+        mbar_init(&bar_epi, T3_EPI_WARPS);
         for (int s = 0; s < TC_SCHED; ++s) {
             mbar_init(&bar_sfull[s], 1);
-            // The producer warps, the MMA thread and the epilogue warps.
-            mbar_init(&bar_sempty[s], T3_LOADERS + 1 + T3_EPI_WARPS);
+            // The MMA thread, and the producer and epilogue warps (of both
+            // CTAs of a pair).
+            mbar_init(&bar_sempty[s], 1 + (PAIR ? 2 : 1) * (T3_PRODUCERS + T3_EPI_WARPS));
         }
         abort_flag_s = 0;
-        buf_count = 0;
+        list_lock = 0;
+        epi_job = -1;
+        threshold = ~0ull << 32;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 3) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tmem_base_slot)),
-                     "r"(TC_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_slot)),
+                         "r"(TC_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_slot)),
+                         "r"(TC_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
-    for (int i = threadIdx.x; i < lt_floats; i += blockDim.x) xltab[i] = i <= a.M ? a.xlogx[i] : 0.f;
+    for (int i = threadIdx.x; i <= a.M; i += blockDim.x) xltab[i] = a.xlogx[i];
     if (MODE == MODE_TOPN) {
-        for (int i = threadIdx.x; i < a.P2; i += blockDim.x) {
+        for (int i = threadIdx.x; i < a.L; i += blockDim.x) {
             lscore[i] = -FLT_MAX;
             lrank[i] = NO_RANK;
         }
@@ -227,500 +435,574 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    if (warp >= T3_EPI_WARP0 && warp < T3_EPI_WARP0 + 4) {
+        const uint32_t q = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + T3_SCALE_COL;
+        tmem_fill16(q, FP4_SCALE_ONE);
+        tmem_fill16(q + FP4_SCALE_COLS, FP4_SCALE_4096);
+        tmem_fill16(q + 2 * FP4_SCALE_COLS, FP4_SCALE_4);
+        tmem_wait_st();
+    }
+    tc_fence_before();
+    // Barriers and scales of both CTAs are ready before either uses them.
+    if constexpr (PAIR) cluster_sync(); else __syncthreads();
+    tc_fence_after();
     const long long wt = a.wait_ticks;
 
-    if (warp < T3_LOADERS) {
-        // ---------------- producers ----------------
-        // Warp w owns stage w and the fills f = w (mod 3); lane 0 issues.
-        const int w = warp;
-        uint8_t *st = smem + (size_t)w * Sh::STAGE;
-        uint32_t fill = 0;
-        uint32_t issued = 0, last_n = 0;
-        bool ok = true;
-        const CUtensorMap *mapA = &tmapA, *mapP = &tmapP;
+    // A consumer's word that it has read a slot of the tile ring.
+    const uint32_t sempty0 = PAIR ? cluster_addr(&bar_sempty[0], 0) : 0;
+    auto slot_read = [&](int slot) {
+        if constexpr (PAIR) mbar_arrive_cluster(sempty0 + 8 * slot);
+        else mbar_arrive(&bar_sempty[slot]);
+    };
+
+    if (warp < T3_PRODUCERS) {
+        // ---------------- TMA producers ----------------
+        if (elect_one()) {
+            Ring ring;
+            int owner = 0;   // producer of stage ring.s
+            // Parity of the last fill issued into each owned stage (at most
+            // three: stages warp, warp + 2, warp + 4), -1 before the first.
+            int last[3] = {-1, -1, -1};
+            auto step = [&]() {
+                ring.next(stages);
+                owner = ring.s == 0 || owner + 1 == T3_PRODUCERS ? 0 : owner + 1;
+            };
+            bool ok = true;
+            const CUtensorMap *mapA = &tmapA, *mapP = &tmapP;
+            int nk = (a.Wt + 1) / 2, cur_job = -1;
+            for (int it = 0; ok; ++it) {
+                const int slot = it % TC_SCHED;
+                const uint32_t sn = (uint32_t)(it / TC_SCHED);
+                if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt)) { ok = false; break; }
+                const uint4 tile = sched_tile[slot];
+                slot_read(slot);
+                const int job = (int)tile.w;
+                if (job < 0) break;
+                if (BATCH && job != cur_job) {
+                    cur_job = job;
+                    const T3Job *jb = a.jobs + job;
+                    mapA = jb->tmapA;
+                    mapP = jb->tmapP;
+                    nk = (jb->Wt + 1) / 2;
+                }
+                const int rowA = 2 * ((int)tile.z + T3_LB * (int)crank), rowP = (int)tile.x + T3_N * (int)crank;
+                for (int kc = 0; kc < nk; ++kc, step()) {
+                    if (owner != warp) continue;
+                    const int s = ring.s;
+                    uint8_t *st = smem + (size_t)s * T3_STAGE;
+                    if (!mbar_wait(&bar_empty[s], ring.par ^ 1, abort_flag, a.err, wt)) { ok = false; break; }
+                    const int x = kc * TC_BK;
+                    if constexpr (PAIR) {
+                        // The leader's barrier counts the bytes of both CTAs.
+                        if (crank == 0) mbar_expect_tx(&bar_full[s], 2 * T3_STAGE);
+                        tma_load_2d_pair(mapA, &bar_full[s], st, x, rowA);
+                        tma_load_2d_pair(mapP, &bar_full[s], st + TC_A_BYTES, x, rowP);
+                    } else {
+                        mbar_expect_tx(&bar_full[s], T3_STAGE);
+                        tma_load_2d(mapA, &bar_full[s], st, x, rowA);
+                        tma_load_2d(mapP, &bar_full[s], st + TC_A_BYTES, x, rowP);
+                    }
+                    last[0] = s == warp ? (int)ring.par : last[0];
+                    last[1] = s == warp + T3_PRODUCERS ? (int)ring.par : last[1];
+                    last[2] = s == warp + 2 * T3_PRODUCERS ? (int)ring.par : last[2];
+                }
+            }
+            // Let the last copies into the owned stages land before the CTA
+            // can exit (earlier ones were consumed).  A pair's copies complete
+            // on its leader's barriers, and neither CTA exits before the other
+            // (the cluster barrier below); where a wait ran out, the second
+            // CTA allows its own copies a millisecond.
+            if (crank == 0) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int s = warp + q * T3_PRODUCERS;
+                    if (s >= stages || last[q] < 0) continue;
+                    const long long t0 = clock64();
+                    while (!mbar_try(&bar_full[s], (uint32_t)last[q]) && clock64() - t0 < WAIT_BUDGET) {}
+                }
+            } else if (!ok) {
+                const long long t0 = clock64();
+                while (clock64() - t0 < 2000000) {}
+            }
+        }
+    } else if (warp == 2) {
+        // ---------------- scheduler, score threshold ----------------
+        // Lane 0 hands out the tiles; while the ring is full the warp renews
+        // the threshold of the job that the epilogue works on.  In a batched
+        // launch: the job of the last item taken and its items [s_first,
+        // s_end); items only grow.
+        int s_job = BATCH ? -1 : 0, s_first = 0, s_end = 0;
         const uint4 *tiles = a.tiles;
-        int Wt = a.Wt, cur_job = -1;
-        for (int it = 0; ok; ++it) {
+        const int n_items = BATCH ? a.n_items : a.ntiles;
+        const uint32_t peer_tile = PAIR ? cluster_addr(&sched_tile[0], 1) : 0;
+        const uint32_t peer_sfull = PAIR ? cluster_addr(&bar_sfull[0], 1) : 0;
+        unsigned pause = 500;
+        long long t0 = clock64();
+        for (int it = 0;;) {
             const int slot = it % TC_SCHED;
             const uint32_t sn = (uint32_t)(it / TC_SCHED);
-            if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt)) break;
-            const int t = sched_tile[slot];
-            const int job = sched_job[slot];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bar_sempty[slot]);
-            if (t < 0) break;
-            if (BATCH && job != cur_job) {
-                cur_job = job;
-                const T3Job *jb = a.jobs + job;
-                mapA = jb->tmapA;
-                mapP = jb->tmapP;
-                tiles = jb->tiles;
-                Wt = jb->Wt;
+            int ready = 0;   // 1: a tile was handed out, 2: no tile is left
+            if (crank == 0 && lane == 0 && mbar_try(&bar_sempty[slot], (sn & 1) ^ 1)) {
+                int t = atomicAdd(a.tile_counter, 1);
+                const bool end = t >= n_items;
+                if (BATCH && !end) {
+                    if (t >= s_end) {
+                        // The last job whose first item is at most t.
+                        int lo = s_job < 0 ? 0 : s_job, hi = a.n_jobs - 1;
+                        while (lo < hi) {
+                            const int mid = (lo + hi + 1) >> 1;
+                            if (a.jobs[mid].item_first <= t) lo = mid; else hi = mid - 1;
+                        }
+                        s_job = lo;
+                        s_first = a.jobs[lo].item_first;
+                        s_end = s_first + a.jobs[lo].ntiles;
+                        tiles = a.jobs[lo].tiles;
+                    }
+                    t -= s_first;
+                }
+                uint4 tile = end ? make_uint4(0, 0, 0, 0) : tiles[t];
+                tile = make_uint4(tile.x, tile.y | tile.z << 16, tile.w, end ? ~0u : (uint32_t)s_job);
+                sched_tile[slot] = tile;
+                mbar_arrive(&bar_sfull[slot]);
+                if constexpr (PAIR) cluster_post4(peer_tile + 16 * slot, peer_sfull + 8 * slot, tile);
+                ready = end ? 2 : 1;
             }
-            if (lane != 0) {
-                fill += (uint32_t)Wt;
+            ready = __shfl_sync(FULL, ready, 0);
+            if (ready == 2) break;
+            if (ready) {
+                ++it;
+                t0 = clock64();
                 continue;
             }
-            const uint4 tile = tiles[t];
-            const int rowP = (int)tile.x, l0 = (int)tile.w;
-            for (int kc = 0; kc < Wt; ++kc, ++fill) {
-                if ((int)(fill % T3_LOADERS) != w) continue;
-                const uint32_t n = fill / T3_LOADERS;
-                if (!mbar_wait(&bar_empty[w], (n & 1) ^ 1, abort_flag, a.err, wt)) { ok = false; break; }
-                const int x = kc * TC_BK;
-                mbar_expect_tx(&bar_full[w], Sh::STAGE);
-                tma_load_2d(mapA, &bar_full[w], st, x, 2 * l0);
-                tma_load_2d(mapP, &bar_full[w], st + TC_A_BYTES, x, rowP);
-                ++issued;
-                last_n = n;
+            // (The second CTA's warp ends with its epilogue.)
+            const int job = __shfl_sync(FULL, *(volatile int *)&epi_job, 0);
+            int stop = 0;
+            if (lane == 0) {
+                if (crank == 0 && clock64() - t0 > wt) {
+                    *abort_flag = 1;
+                    atomicOr(a.err, ERR_TIMEOUT);
+                }
+                stop = *abort_flag || job == -2;
             }
-        }
-        // Let the copies of this stage land before the CTA can exit (one
-        // stage: every earlier fill of it was consumed before this one).
-        if (lane == 0 && issued > 0) {
-            long long t0 = clock64();
-            while (!mbar_try(&bar_full[w], last_n & 1) && clock64() - t0 < WAIT_BUDGET) {}
+            if (__shfl_sync(FULL, stop, 0)) break;
+            if (MODE == MODE_TOPN) {
+                if (job >= 0) {
+                    const int *pub = a.pub + (size_t)(BATCH ? a.jobs[job].slot : 0) * gridDim.x;
+                    const float thr = published_threshold(pub, (int)gridDim.x, a.pub_r, lane);
+                    if (lane == 0)
+                        *(volatile unsigned long long *)&threshold = (unsigned long long)job << 32 | __float_as_uint(thr);
+                }
+            }
+            __nanosleep(pause);
+            pause = min(pause + pause / 2, 4000u);
         }
     } else if (warp == 3) {
-        if (elect_one()) {
+        if (crank == 0 && elect_one()) {
             // ---------------- MMA issue ----------------
-            const uint32_t idesc = idesc_f8_f32(TC_BM, Sh::NMMA, BATCH);
-            const uint64_t descA = smem_desc_sw128(smem_u32(smem));
-            const uint64_t descB = smem_desc_sw128(smem_u32(smem + TC_A_BYTES));
+            const uint32_t idesc = idesc_mxf4(PAIR ? 2 * TC_BM : TC_BM, PAIR ? 2 * T3_N : T3_N);
+            const uint64_t descA = smem_desc_sw128(smem_u32(smem)), descB = smem_desc_sw128(smem_u32(smem + TC_A_BYTES));
+            const uint32_t one = tmem_base + T3_SCALE_COL, four = one + 2 * FP4_SCALE_COLS;
             Ring ring;
             bool ok = true;
-            int Wt = a.Wt, split = a.W0, cur_job = -1;
-            // Scheduler state of a batched launch: the job of the last item
-            // taken and its items [s_first, s_end); items only grow.
-            int s_job = -1, s_first = 0, s_end = 0;
-            const int n_items = BATCH ? a.n_items : a.ntiles;
-            // This thread also schedules the tiles, TC_LOOKAHEAD ahead of the
-            // one it consumes (another lane of this warp spinning on the ring
-            // delayed the MMA issue).
-            int published = 0;
-            bool sched_done = false;
-            auto publish = [&](int k) -> bool {
-                const int pslot = k % TC_SCHED;
-                const uint32_t psn = (uint32_t)(k / TC_SCHED);
-                if (!mbar_wait(&bar_sempty[pslot], (psn & 1) ^ 1, abort_flag, a.err, wt)) return false;
-                int t = -1;
-                if (!sched_done) {
-                    t = atomicAdd(a.tile_counter, 1);
-                    if (t >= n_items) {
-                        t = -1;
-                        sched_done = true;
-                    } else if (BATCH) {
-                        if (t >= s_end) {
-                            // The last job whose first item is at most t.
-                            int lo = s_job < 0 ? 0 : s_job, hi = a.n_jobs - 1;
-                            while (lo < hi) {
-                                const int mid = (lo + hi + 1) >> 1;
-                                if (a.jobs[mid].item_first <= t) lo = mid; else hi = mid - 1;
-                            }
-                            s_job = lo;
-                            s_first = a.jobs[lo].item_first;
-                            s_end = s_first + a.jobs[lo].ntiles;
-                        }
-                        t -= s_first;
-                    }
-                }
-                sched_tile[pslot] = t;
-                sched_job[pslot] = s_job;
-                mbar_arrive(&bar_sfull[pslot]);
-                return true;
-            };
-            for (; published < TC_LOOKAHEAD && ok; ++published) ok = publish(published);
+            int Wt = a.Wt, W0 = a.W0, cur_job = -1;
             for (int it = 0; ok; ++it) {
-                if (!(ok = publish(published++))) break;
                 const int slot = it % TC_SCHED;
                 const uint32_t sn = (uint32_t)(it / TC_SCHED);
                 if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt)) break;
-                const int t = sched_tile[slot];
-                const int job = sched_job[slot];
+                const int job = (int)sched_tile[slot].w;
                 mbar_arrive(&bar_sempty[slot]);
-                if (t < 0) break;
+                if (job < 0) break;
                 if (BATCH && job != cur_job) {
                     cur_job = job;
                     Wt = a.jobs[job].Wt;
-                    split = a.jobs[job].split;
+                    W0 = a.jobs[job].W0;
                 }
                 const int b = it & 1;
                 const uint32_t u = (uint32_t)(it >> 1);
                 if (!mbar_wait(&bar_tempty[b], (u & 1) ^ 1, abort_flag, a.err, wt)) break;
                 tc_fence_after();
-                for (int kc = 0; kc < Wt; ++kc, ring.next(T3_LOADERS)) {
+                const uint32_t d0 = tmem_base + (uint32_t)(b * T3_BUF);
+                for (int kc = 0; 2 * kc < Wt; ++kc, ring.next(stages)) {
                     const int s = ring.s;
                     if (!mbar_wait(&bar_full[s], ring.par, abort_flag, a.err, wt)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    // ENC 0: controls, ENC 2: the chunks from split, into
-                    // the second accumulator.
-                    const bool acc1 = ENC != 1 && kc >= split;
-                    const uint32_t d = tmem_base + (uint32_t)(b * 256 + (acc1 ? 128 : 0));
-                    const bool first = ENC == 1 ? kc == 0 : (kc == 0 || kc == split);
-                    const uint64_t ad = descA + (uint64_t)s * (Sh::STAGE >> 4);
-                    const uint64_t bd = descB + (uint64_t)s * (Sh::STAGE >> 4);
+                    const uint64_t ad = descA + (uint64_t)s * (T3_STAGE >> 4);
+                    const uint64_t bd = descB + (uint64_t)s * (T3_STAGE >> 4);
+                    // Two words of 128 samples (K = 64 twice): cases, then
+                    // controls (ENC 0: into the second accumulator; ENC 1: with
+                    // scale 4096).
 #pragma unroll
-                    for (int kk = 0; kk < TC_BK / 32; ++kk)
-                        mma_e4m3(d, ad + kk * 2, bd + kk * 2, idesc, (!first || kk > 0) ? 1u : 0u);
-                    mma_commit(&bar_empty[s]);
+                    for (int h = 0; h < 2; ++h) {
+                        const int w = 2 * kc + h;
+                        if (w < Wt) {
+                            const bool ctrl = w >= W0;
+                            const bool first = w == 0 || (!PAIR && w == W0);
+                            const uint32_t d = d0 + (!PAIR && ctrl ? T3_N : 0);
+                            const uint32_t sa = one + (PAIR && ctrl ? FP4_SCALE_COLS : 0);
+                            if constexpr (PAIR) {
+                                mma_mxf4_pair(d, ad + 4 * h, bd + 4 * h, idesc, sa, four, first ? 0u : 1u);
+                                mma_mxf4_pair(d, ad + 4 * h + 2, bd + 4 * h + 2, idesc, sa, four, 1u);
+                            } else {
+                                mma_mxf4(d, ad + 4 * h, bd + 4 * h, idesc, sa, four, first ? 0u : 1u);
+                                mma_mxf4(d, ad + 4 * h + 2, bd + 4 * h + 2, idesc, sa, four, 1u);
+                            }
+                        }
+                    }
+                    if constexpr (PAIR) mma_commit_pair(&bar_empty[s]); else mma_commit(&bar_empty[s]);
                 }
-                if (ok) mma_commit(&bar_tfull[b]);
+                if (ok) {
+                    if constexpr (PAIR) mma_commit_pair(&bar_tfull[b]); else mma_commit(&bar_tfull[b]);
+                }
             }
             // All MMAs issued by this thread complete before TMEM is released.
-            mma_commit(&bar_done);
-            long long t0 = clock64();
+            if constexpr (PAIR) mma_commit_pair(&bar_done); else mma_commit(&bar_done);
+            const long long t0 = clock64();
             while (!mbar_try(&bar_done, 0) && clock64() - t0 < WAIT_BUDGET) {}
         }
     } else {
         // ---------------- epilogue ----------------
-        // TMEM lane = A row = 2 l_loc + g; column (within a class for ENC = 0)
-        // 2 NP a + 2 q + b = pair (i, j0 + q) with genotypes (a, b).  Warp w
-        // reads lane quarter w % 4 and the groups of 4 pairs part, part + 3, ..
-        const int tid = threadIdx.x - 32 * T3_EPI_WARP0;   // 0 .. T3_EPI_THREADS - 1
+        const int ew = warp - T3_EPI_WARP0;
         const int quarter = warp & 3;
-        const int part = (warp - T3_EPI_WARP0) >> 2;       // 0 .. T3_PARTS - 1
-        const int row = quarter * 32 + lane;
-        const int l_loc = row >> 1;
-        const int g = row & 1;
+        const int part = ew >> 2;                          // two pairs dp = part, part + 4, .. of a tile
+        const int g = lane & 1;                            // genotype of this lane's row
+        const uint32_t tempty0 = PAIR ? cluster_addr(&bar_tempty[0], 0) : 0;
         const int L = a.L;
-        const uint32_t tmask = (uint32_t)lt_floats - 1;
+        float *ws = wscore + ew * T3_WBUF;
+        uint64_t *wr = wrank + ew * T3_WBUF;
+        uint32_t *rec = recs + ew * (T3_WARP_PAIRS * T3_REC_WORDS);
         // The data set and job of the tile (a batched launch reloads them
         // when the job changes).
-        int64_t S = a.S, Sp = a.S_pad;
+        int S = (int)a.S, Sp = (int)a.S_pad;
         uint64_t total = a.total;
-        float hy = a.hy, invN = a.invN;
+        const float unscale = 1.f / a.scale;   // (exact)
+        float hy = a.hy, invN = a.invN * unscale;
         const uint4 *marg4 = a.marg4, *PR = a.PR;
-        int pjob = -1, pslot = 0;
-        // The job whose candidates the list holds.
-        int ljob = -1, lslot = 0;
+        int cur_job = -1, slot_j = 0;
         const bool whole = BATCH || (a.rank_begin == 0 && a.rank_end >= a.total);
-        // A round inserts at most 2 candidates per thread.  Every
-        // a.check_rounds rounds (and at the start of each tile) the threads
-        // read the buffer's fill between two barriers, where nobody inserts,
-        // and merge it into the list if the next check_rounds rounds might
-        // not fit.
-        const int headroom = a.check_rounds * 2 * T3_EPI_THREADS;
+        // This warp's candidates, and the CTA list's last entry when the
+        // warp last merged: a candidate has to beat it.
+        int cnt = 0;
         float thr_s = -FLT_MAX;
         uint64_t thr_r = NO_RANK;
-        // Merge the buffer into the list (all epilogue threads, uniform).
         auto merge = [&]() {
-            epi_bar_n<T3_EPI_THREADS>();
-            const int nb = min(buf_count, a.Bcap);
-            for (int x = L + nb + tid; x < a.P2; x += T3_EPI_THREADS) {
+            // Sorted outside the lock, against the list's last score then.
+            const float racy = *(volatile float *)(lscore + L - 1);
+            const bool later = racy > thr_s;
+            const int m = sort_candidates(ws, wr, cnt, later ? racy : thr_s, later ? NO_RANK : thr_r, lane);
+            cnt = 0;
+            if (m == 0) return;
+            bool held = true;
+            if (lane == 0) {
+                const long long t0 = clock64();
+                while (atomicCAS(&list_lock, 0, 1) != 0) {
+                    __nanosleep(100);
+                    if (clock64() - t0 > WAIT_BUDGET) {
+                        *abort_flag = 1;
+                        atomicOr(a.err, ERR_TIMEOUT);
+                        held = false;
+                        break;
+                    }
+                }
+                __threadfence_block();
+            }
+            held = __shfl_sync(FULL, held, 0);
+            if (held) {
+                merge_candidates(lscore, lrank, L, ws, wr, m, lane);
+                thr_s = lscore[L - 1];
+                thr_r = lrank[L - 1];
+                __threadfence_block();
+                __syncwarp();
+                if (lane == 0) {
+                    if (lrank[a.pub_m - 1] != NO_RANK)
+                        *(volatile int *)(a.pub + (size_t)slot_j * gridDim.x + blockIdx.x) = ordered_int(lscore[a.pub_m - 1]);
+                    __threadfence_block();
+                    atomicExch(&list_lock, 0);
+                }
+            }
+            __syncwarp();
+        };
+        // All epilogue warps meet, unless a wait ran out in some role.
+        uint32_t epi_par = 0;
+        auto meet = [&]() -> bool {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_epi);
+            const bool met = mbar_wait(&bar_epi, epi_par, abort_flag, a.err, wt);
+            epi_par ^= 1;
+            return __all_sync(FULL, met);
+        };
+        // The CTA's list of the current job, written out as list slot_j of
+        // this CTA (all epilogue warps).
+        auto flush = [&]() -> bool {
+            merge();
+            if (!meet()) return false;
+            const size_t o = ((size_t)slot_j * gridDim.x + blockIdx.x) * L;
+            for (int x = threadIdx.x - 32 * T3_EPI_WARP0; x < L; x += T3_EPI_THREADS) {
+                a.list_score[o + x] = lscore[x];
+                a.list_rank[o + x] = lrank[x];
                 lscore[x] = -FLT_MAX;
                 lrank[x] = NO_RANK;
             }
-            epi_bitonic_desc_n<T3_EPI_THREADS>(lscore, lrank, a.P2, tid);
-            if (tid == 0) {
-                buf_count = 0;
-                if (lrank[L - 1] != NO_RANK) atomicMax(a.gthr + lslot, ordered_int(lscore[L - 1]));
-            }
-            epi_bar_n<T3_EPI_THREADS>();
+            thr_s = -FLT_MAX;
+            thr_r = NO_RANK;
+            return meet();
         };
-        // The list's final order, written out as list lslot of this CTA.
-        auto flush = [&]() {
-            epi_bar_n<T3_EPI_THREADS>();
-            const int nb = min(buf_count, a.Bcap);
-            for (int x = L + nb + tid; x < a.P2; x += T3_EPI_THREADS) { lscore[x] = -FLT_MAX; lrank[x] = NO_RANK; }
-            epi_bitonic_desc_n<T3_EPI_THREADS>(lscore, lrank, a.P2, tid);
-            const size_t o = ((size_t)lslot * gridDim.x + blockIdx.x) * L;
-            for (int x = tid; x < L; x += T3_EPI_THREADS) {
-                a.list_score[o + x] = lscore[x];
-                a.list_rank[o + x] = lrank[x];
-            }
+        // hs + (t(c), t(d)) for two packed cells c, d (4 a | 4 b << 16).
+        auto add_terms = [&](F2 hs, uint32_t c, uint32_t d) -> F2 {
+            // 4 a under the exponent of 2^21 is 2^21 + a; -a q = 2^21 q minus q
+            // times that, exactly (q the scale, a power of two).  The logarithm's
+            // argument is a q + 1e-30, that is a q, or 1e-30 at a = 0, whose
+            // finite logarithm times 0 adds nothing.
+            const F2 minus = f2(-1.f, -1.f), tiny = f2(1e-30f, 1e-30f);
+            const F2 mscale = f2(-a.scale, -a.scale), big = f2(2097152.f * a.scale, 2097152.f * a.scale);
+            const F2 na = f2_fma(f2(__uint_as_float(__byte_perm(c, 0x4A000000u, 0x7610)),
+                                    __uint_as_float(__byte_perm(d, 0x4A000000u, 0x7610))), mscale, big);
+            const F2 nb = f2_fma(f2(__uint_as_float(__byte_perm(c, 0x4A000000u, 0x7632)),
+                                    __uint_as_float(__byte_perm(d, 0x4A000000u, 0x7632))), mscale, big);
+            const float2 aa = f2_split(f2_fma(na, minus, tiny)), bb = f2_split(f2_fma(nb, minus, tiny));
+            // 4 n = 4 a + 4 b is the byte offset of the table entry of n.
+            auto xl = [&](uint32_t x) {
+                return *reinterpret_cast<const float *>(reinterpret_cast<const char *>(xltab) + __dp2a_lo(x, 0x00000101u, 0u));
+            };
+            F2 t = f2_fma(na, f2(lg2_approx(aa.x), lg2_approx(aa.y)), f2(xl(c), xl(d)));
+            t = f2_fma(nb, f2(lg2_approx(bb.x), lg2_approx(bb.y)), t);
+            return f2_add(hs, t);
         };
+        bool ok = true;
         for (int it = 0;; ++it) {
             const int slot = it % TC_SCHED;
             const uint32_t sn = (uint32_t)(it / TC_SCHED);
-            const bool okw = mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt);
-            const int t = okw ? sched_tile[slot] : -1;
-            const int job = okw ? sched_job[slot] : -1;
-            if (okw) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bar_sempty[slot]);
+            ok = mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt);
+            ok = __all_sync(FULL, ok);
+            if (!ok) break;
+            const uint4 tile = sched_tile[slot];
+            const int job = (int)tile.w;
+            __syncwarp();
+            if (lane == 0) slot_read(slot);
+            if (job < 0) break;
+            if (BATCH && job != cur_job) {
+                // A new job: the list of the last one goes out, and the list
+                // starts empty (every epilogue warp sees the same items).
+                if (cur_job >= 0 && !flush()) { ok = false; break; }
+                cur_job = job;
+                const T3Job *jb = a.jobs + job;
+                S = (int)jb->S;
+                Sp = (int)jb->S_pad;
+                total = jb->total;
+                hy = jb->hy;
+                invN = jb->invN * unscale;
+                marg4 = jb->marg4;
+                PR = jb->PR;
+                slot_j = jb->slot;
             }
+            if (MODE == MODE_TOPN && ew == 0 && lane == 0) *(volatile int *)&epi_job = job;
             const int b = it & 1;
             const uint32_t u = (uint32_t)(it >> 1);
-            // Tile data that does not depend on the accumulators, loaded while
-            // the tile's MMAs may still run.
-            int64_t l = 0, j0 = 0;
-            uint32_t Tl[3] = {0, 0, 0}, T02[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-            bool lv = false;
-            uint32_t *sJb = sJ + (size_t)b * NP * T3_SJ_WORDS;
-            const uint4 *tiles = a.tiles;
-            if (BATCH && t >= 0) {
-                const T3Job *jb = a.jobs + job;
-                tiles = jb->tiles;
-                if (job != pjob) {
-                    pjob = job;
-                    S = jb->S;
-                    Sp = jb->S_pad;
-                    total = jb->total;
-                    hy = jb->hy;
-                    invN = jb->invN;
-                    marg4 = jb->marg4;
-                    PR = jb->PR;
-                    pslot = jb->slot;
-                }
+            // Tile data that does not depend on the accumulators, loaded
+            // while the tile's MMAs may still run.
+            const int i = (int)(tile.y & 0xffffu), j0 = (int)(tile.y >> 16);
+            const int lw = (int)tile.z + T3_LB * (int)crank + quarter * 16;   // this warp's first third SNP
+            const int l = lw + (lane >> 1);
+            const bool lv = l < S;
+            // This warp's two pairs dp = part + 4 r, r < nr, that hold some
+            // valid combination: the first pair's j before S and before the
+            // warp's last SNP l.
+            const int jn = lw < S ? min(min(S, lw + 15) - j0, NPT) : 0;    // pairs q < jn
+            const int nr = jn > 2 * part ? ((jn + 1) / 2 - part + T3_PARTS - 1) / T3_PARTS : 0;
+            // Lanes beyond the last SNP count no sample (their rows are
+            // zero): zero tables keep every derived cell a count.  Genotypes
+            // of l in the order g, 1 - g.
+            uint32_t R02[4] = {0, 0, 0, 0}, Tl0 = 0, Tl1 = 0;
+            if (lv) {
+                uint32_t Tl[3];
+                unpack_marg(marg4[l], Tl);
+                Tl0 = (g ? Tl[1] : Tl[0]) << 2;
+                Tl1 = (g ? Tl[0] : Tl[1]) << 2;
+                const uint4 p4 = PR[(size_t)i * Sp + l];
+                R02[0] = (g ? p4.y : p4.x) << 2;
+                R02[1] = (g ? p4.x : p4.y) << 2;
+                R02[2] = (g ? p4.w : p4.z) << 2;
+                R02[3] = (g ? p4.z : p4.w) << 2;
             }
-            if (t >= 0) {
-                const uint4 tile = tiles[t];
-                const int64_t i = tile.y;
-                j0 = tile.z;
-                l = (int64_t)tile.w + l_loc;
-                lv = l < S;
-                const int64_t lc = lv ? l : S - 1;
-                uint32_t Ti[3];
+            __syncwarp();
+            if (lane < 2 * nr) {
+                // The table of pair (i, j), one lane per pair.  Every cell has
+                // to be a count (it is a table offset): where j is no SNP its
+                // rows are zero, those of a SNP of genotype 2 throughout.
+                const int j = j0 + 2 * (part + T3_PARTS * (lane >> 1)) + g;
+                uint32_t Ti[3], T01[9];
                 unpack_marg(marg4[i], Ti);
-                unpack_marg(marg4[lc], Tl);
-                const uint4 p4 = PR[(size_t)i * Sp + lc];
-                const uint32_t R[4] = {p4.x, p4.y, p4.z, p4.w};
-                full2(R, Ti, Tl, T02);
-                // The tables of the tile's SNPs j, one thread per j.
-                if (tid < NP) {
-                    const int64_t j = j0 + tid;
-                    const int64_t jc = j < S ? j : S - 1;
-                    uint32_t Tj[3], T01[9];
-                    unpack_marg(marg4[jc], Tj);
-                    const uint4 q4 = PR[(size_t)i * Sp + jc];
+#pragma unroll
+                for (int x = 0; x < 9; ++x) T01[x] = x % 3 == 2 ? Ti[x / 3] : 0;
+                uint64_t rb = 0;
+                if (j < S) {
+                    uint32_t Tj[3];
+                    unpack_marg(marg4[j], Tj);
+                    const uint4 q4 = PR[(size_t)i * Sp + j];
                     const uint32_t Rq[4] = {q4.x, q4.y, q4.z, q4.w};
                     full2(Rq, Ti, Tj, T01);
                     // rank of (i, j, l) = base_i - C(S - j, 2) + l - j - 1
                     const uint64_t base_i = total - c3((uint64_t)(S - i)) + c2((uint64_t)(S - i - 1));
-                    const uint64_t rb = base_i - c2((uint64_t)(S - jc)) - (uint64_t)jc - 1;
-                    uint4 *rec = reinterpret_cast<uint4 *>(sJb + (size_t)tid * T3_SJ_WORDS);
-                    rec[0] = make_uint4(T01[0], T01[1], T01[2], T01[3]);
-                    rec[1] = make_uint4(T01[4], T01[5], T01[6], T01[7]);
-                    rec[2] = make_uint4(T01[8], Tj[0], Tj[1], Tj[2]);
-                    rec[3] = make_uint4((uint32_t)rb, (uint32_t)(rb >> 32), j < S ? 1u : 0u, 0u);
+                    rb = base_i - c2((uint64_t)(S - j)) - (uint64_t)j - 1;
                 }
-                mbar_wait(&bar_tfull[b], u & 1, abort_flag, a.err, wt);
+#pragma unroll
+                for (int x = 0; x < 9; ++x) T01[x] <<= 2;
+                uint4 *o = reinterpret_cast<uint4 *>(rec + lane * T3_REC_WORDS);
+                o[0] = make_uint4(T01[0], T01[1], T01[2], T01[3]);
+                o[1] = make_uint4(T01[4], T01[5], T01[6], T01[7]);
+                o[2] = make_uint4(T01[8], (uint32_t)rb, (uint32_t)(rb >> 32), 0u);
             }
-            // The global threshold only rises; a value read once per tile
-            // admits at most a few more candidates than a fresh one would.
-            const float gthr = MODE == MODE_TOPN ? from_ordered(*(volatile int *)(a.gthr + (BATCH ? pslot : 0))) : -FLT_MAX;
-            // One stop decision for all epilogue warps (they meet at named
-            // barriers, which have no timeout); t is the same for all.  The
-            // barrier also publishes the tables of the SNPs j, and between
-            // the two barriers the buffer's fill is the same for all.
-            epi_bar_n<T3_EPI_THREADS>();
-            if (tid == 0) epi_stop = *abort_flag;
-            int fill0 = buf_count;
-            epi_bar_n<T3_EPI_THREADS>();
-            if (epi_stop || t < 0) break;
-            if (BATCH && job != ljob) {
-                // A new job: the list of the last one goes out, and the list
-                // starts empty (uniform: every epilogue warp sees the same
-                // items).
-                if (ljob >= 0) {
-                    flush();
-                    for (int x = tid; x < a.P2; x += T3_EPI_THREADS) {
-                        lscore[x] = -FLT_MAX;
-                        lrank[x] = NO_RANK;
-                    }
-                    if (tid == 0) buf_count = 0;
-                    epi_bar_n<T3_EPI_THREADS>();
-                    fill0 = 0;
-                }
-                ljob = job;
-                lslot = pslot;
-            }
-            if (MODE == MODE_TOPN) {
-                if (fill0 > a.Bcap - headroom) merge();
-                thr_s = lscore[L - 1];
-                thr_r = lrank[L - 1];
-            }
+            // PR[j][l] of this lane's next pair.
+            int j = j0 + 2 * part + g;
+            const uint4 *pr = PR + (size_t)j * Sp + l;
+            uint4 pj_next = make_uint4(0, 0, 0, 0);
+            if (nr > 0 && lv && j < S) pj_next = *pr;
+            ok = mbar_wait(&bar_tfull[b], u & 1, abort_flag, a.err, wt);
+            ok = __all_sync(FULL, ok);   // (also orders the records)
+            if (!ok) break;
             tc_fence_after();
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256);
-            const int64_t lc = lv ? l : S - 1;
-            // Pair-table entries PR[j][l] of the first group, then one group ahead.
-            uint4 pjl[2], pjl_next[2];
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * T3_BUF + 8 * part);
+            for (int r = 0; r < nr; ++r, j += 2 * T3_PARTS) {
+                // The cells of two pairs with this lane's genotype of l; those
+                // of the other lane's pair go there.  R[z][2 a + b]: z = 0 this
+                // lane's genotype; packed 4 cases | 4 controls << 16 (all cells
+                // below are).
+                uint32_t R[2][4];
+                {
+                    uint32_t v[8], w[8];
+                    tmem_ld8(taddr + 8 * T3_PARTS * r, v);
+                    if constexpr (!PAIR) tmem_ld8(taddr + T3_N + 8 * T3_PARTS * r, w);
+                    tmem_wait_ld();
+                    tmem_regs_after_wait(v);
+                    if constexpr (!PAIR) tmem_regs_after_wait(w);
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                const int64_t jj = min(j0 + part * 4 + 2 * m + g, S - 1);
-                pjl_next[m] = PR[(size_t)jj * Sp + lc];
-            }
-            // Every warp runs the same number of rounds (a round without a
-            // group scores nothing), because each round meets at a barrier.
-            for (int rnd = 0; rnd < Sh::ROUNDS; ++rnd) {
-                const int qd = part + rnd * T3_PARTS;            // group of pairs 4 qd .. 4 qd + 3
-                const bool has = qd < Sh::QUADS;                 // warp-uniform
-                if (MODE == MODE_TOPN && rnd > 0 && rnd % a.check_rounds == 0) {
-                    epi_bar_n<T3_EPI_THREADS>();
-                    const int fill = buf_count;
-                    epi_bar_n<T3_EPI_THREADS>();
-                    if (fill > a.Bcap - headroom) merge();
-                    thr_s = lscore[L - 1];
-                    thr_r = lrank[L - 1];
-                }
-                pjl[0] = pjl_next[0];
-                pjl[1] = pjl_next[1];
-                if (qd + T3_PARTS < Sh::QUADS) {
+                    for (int x = 0; x < 8; ++x) {
+                        if constexpr (PAIR) v[x] = unpack_enc(v[x]);
+                        else v[x] = pack_exact(v[x], w[x]);
+                    }
 #pragma unroll
-                    for (int m = 0; m < 2; ++m) {
-                        const int64_t jj = min(j0 + (qd + T3_PARTS) * 4 + 2 * m + g, S - 1);
-                        pjl_next[m] = PR[(size_t)jj * Sp + lc];
+                    for (int x = 0; x < 4; ++x) {
+                        R[0][x] = g ? v[4 + x] : v[x];
+                        R[1][x] = __shfl_xor_sync(FULL, g ? v[x] : v[4 + x], 1);
                     }
                 }
-                // This lane's cells (genotype g of SNP l) for the group's 4
-                // pairs q: cell[4 q + 2 a + b], packed cases | controls << 16.
-                uint32_t cell[16];
-#pragma unroll
-                for (int x = 0; x < 16; ++x) cell[x] = 0;
-                if (has) {
-                    const uint32_t c0 = (uint32_t)(8 * qd);            // a = 0: columns 2 q + b
-                    const uint32_t c1 = (uint32_t)(2 * NP + 8 * qd);   // a = 1
-                    if (ENC == 1) {
-                        uint32_t v0[8], v1[8];
-                        tmem_ld8(taddr + c0, v0);
-                        tmem_ld8(taddr + c1, v1);
-                        tmem_wait_ld();
-                        tmem_regs_after_wait(v0);
-                        tmem_regs_after_wait(v1);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-#pragma unroll
-                            for (int bb = 0; bb < 2; ++bb) {
-                                cell[4 * q + bb] = unpack_enc(v0[2 * q + bb]);
-                                cell[4 * q + 2 + bb] = unpack_enc(v1[2 * q + bb]);
-                            }
-                    } else {
-                        uint32_t v0[8], v1[8], w0[8], w1[8];
-                        tmem_ld8(taddr + c0, v0);
-                        tmem_ld8(taddr + 128 + c0, w0);
-                        tmem_ld8(taddr + c1, v1);
-                        tmem_ld8(taddr + 128 + c1, w1);
-                        tmem_wait_ld();
-                        tmem_regs_after_wait(v0);
-                        tmem_regs_after_wait(v1);
-                        tmem_regs_after_wait(w0);
-                        tmem_regs_after_wait(w1);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-#pragma unroll
-                            for (int bb = 0; bb < 2; ++bb) {
-                                if (ENC == 0) {
-                                    cell[4 * q + bb] = pack_exact(v0[2 * q + bb], w0[2 * q + bb]);
-                                    cell[4 * q + 2 + bb] = pack_exact(v1[2 * q + bb], w1[2 * q + bb]);
-                                } else {
-                                    // Two encoded parts; each class sum stays below 2^16.
-                                    cell[4 * q + bb] = unpack_enc(v0[2 * q + bb]) + unpack_enc(w0[2 * q + bb]);
-                                    cell[4 * q + 2 + bb] = unpack_enc(v1[2 * q + bb]) + unpack_enc(w1[2 * q + bb]);
-                                }
-                            }
-                    }
-                    if (qd + T3_PARTS >= Sh::QUADS) {
-                        // This warp's last read of the buffer.
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&bar_tempty[b]);
+                const uint4 pj = pj_next;
+                if (r + 1 < nr) {
+                    pr += (size_t)(2 * T3_PARTS) * Sp;
+                    pj_next = make_uint4(0, 0, 0, 0);
+                    if (lv && j + 2 * T3_PARTS < S) pj_next = *pr;
+                } else {
+                    // This warp's last read of the buffer.
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (PAIR) mbar_arrive_cluster(tempty0 + 8 * b);
+                        else mbar_arrive(&bar_tempty[b]);
                     }
                 }
-                float sc[2];
-                uint64_t rk[2];
-                bool val[2];
+                const uint4 *rq = reinterpret_cast<const uint4 *>(rec + (2 * r + g) * T3_REC_WORDS);
+                const uint4 r0 = rq[0], r1 = rq[1], r2 = rq[2];
+                const uint32_t T01[9] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x};
+                const uint32_t R12[4] = {(g ? pj.y : pj.x) << 2, (g ? pj.x : pj.y) << 2, (g ? pj.w : pj.z) << 2,
+                                         (g ? pj.z : pj.w) << 2};
+                const uint64_t rank = (((uint64_t)r2.z << 32) | r2.y) + (uint64_t)l;
+                // Cells (x, y, 0) and (x, y, 1); (x, y, 2) is the rest of
+                // T01(x, y).
+                F2 hs[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+                uint32_t c2z[2][2];   // cells (x, 2, z), x in {0, 1}
+                uint32_t odd = 0;     // cell (x, y, 2) of the last even (x, y)
 #pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    // This lane scores pair 2m + g of the group; its partner
-                    // lane (genotype 1 - g of the same SNP l) scores 2m + 1 - g.
-                    // Each sends the cells of the other's pair.
-                    uint32_t Rr[8];
+                for (int x = 0; x < 3; ++x)
 #pragma unroll
-                    for (int ab = 0; ab < 4; ++ab) {
-                        const uint32_t own = g ? cell[4 * (2 * m + 1) + ab] : cell[4 * (2 * m) + ab];
-                        const uint32_t other = g ? cell[4 * (2 * m) + ab] : cell[4 * (2 * m + 1) + ab];
-                        const uint32_t recv = __shfl_xor_sync(FULL, other, 1);
-                        Rr[2 * ab] = g ? recv : own;   // Rr[4 a + 2 b + genotype of l]
-                        Rr[2 * ab + 1] = g ? own : recv;
-                    }
-                    const int q = 4 * qd + 2 * m + g;    // pair within the tile
-                    const uint4 *rec = reinterpret_cast<const uint4 *>(sJb + (size_t)(has ? q : 0) * T3_SJ_WORDS);
-                    const uint4 r3 = rec[3];
-                    const int64_t j = j0 + q;
-                    const uint64_t rank0 = (((uint64_t)r3.y << 32) | r3.x) + (uint64_t)l;
-                    const bool valid = has && r3.z != 0 && lv && j < l &&
-                                       (whole || (rank0 >= a.rank_begin && rank0 < a.rank_end));
-                    uint32_t T[27];
-                    float hsum = 0.f;
-                    if (valid) {
-                        const uint4 r0 = rec[0], r1 = rec[1], r2 = rec[2];
-                        const uint32_t T01[9] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x};
-                        const uint32_t Tj[3] = {r2.y, r2.z, r2.w};
-                        uint32_t T12[9];
-                        const uint32_t R12[4] = {pjl[m].x, pjl[m].y, pjl[m].z, pjl[m].w};
-                        full2(R12, Tj, Tl, T12);
-                        full3(Rr, T01, T02, T12, T);
-                        // Three partial sums (nine cells each) shorten the chain
-                        // of dependent additions; every partial sum is still at
-                        // most N ln 2, so the error bound above holds.
-                        float hs[3] = {0.f, 0.f, 0.f};
+                    for (int y = 0; y < 3; ++y) {
+                        uint32_t c[3];
 #pragma unroll
-                        for (int x = 0; x < 27; ++x) {
-                            // Masked so that no index can leave the table
-                            // (exact class counts are below its size).
-                            const uint32_t ca = T[x] & tmask, cb = (T[x] >> 16) & tmask;
-                            const float nf = fmaxf(u2f_small(ca + cb), 1.0f);   // n log2 n = 0 at n = 0, 1
-                            hs[x % 3] += fmaf(nf, lg2_approx(nf), -xltab[ca]) - xltab[cb];
+                        for (int z = 0; z < 2; ++z) {
+                            if (x < 2 && y < 2) c[z] = R[z][2 * x + y];
+                            else if (y < 2) c[z] = R12[2 * y + z] - R[z][y] - R[z][2 + y];
+                            else if (x < 2) c[z] = c2z[x][z] = R02[2 * x + z] - R[z][2 * x] - R[z][2 * x + 1];
+                            else c[z] = ((z ? Tl1 : Tl0) - R12[z] - R12[2 + z]) - c2z[0][z] - c2z[1][z];
                         }
-                        hsum = LN2F * ((hs[0] + hs[1]) + hs[2]);
-                    }
-                    const float score = fmaf(-hsum, invN, hy);
-                    const uint64_t rank = valid ? rank0 : NO_RANK;
-                    sc[m] = score;
-                    rk[m] = rank;
-                    val[m] = valid;
-                    if (MODE == MODE_DUMP && valid) {
-                        if (a.dump_scores) a.dump_scores[rank] = score;
-                        if (a.dump_tables) {
-                            uint32_t *o = a.dump_tables + (size_t)rank * 54;
+                        c[2] = T01[3 * x + y] - c[0] - c[1];
+                        hs[0] = add_terms(hs[0], c[0], c[1]);
+                        if ((3 * x + y) % 2 == 0) odd = c[2];
+                        if ((3 * x + y) % 2 == 1 || 3 * x + y == 8)   // (a cell of no sample adds 0)
+                            hs[1] = add_terms(hs[1], odd, 3 * x + y == 8 ? 0u : c[2]);
+                        if (MODE == MODE_DUMP && a.dump_tables && lv && j < l) {
+                            uint32_t *o = a.dump_tables + (size_t)rank * 54 + 18 * x + 6 * y;
 #pragma unroll
-                            for (int x = 0; x < 27; ++x) { o[2 * x] = T[x] & 0xffffu; o[2 * x + 1] = T[x] >> 16; }
+                            for (int z = 0; z < 3; ++z) {
+                                const int zz = z < 2 ? z ^ g : 2;   // genotype of l
+                                o[2 * zz] = (c[z] & 0xffffu) >> 2;
+                                o[2 * zz + 1] = c[z] >> 18;
+                            }
                         }
                     }
-                }
+                const float2 h2 = f2_split(f2_add(hs[0], hs[1]));
+                const float score = fmaf(-LN2F * (h2.x + h2.y), invN, hy);
+                const bool valid = lv && j < l && (whole || (rank >= a.rank_begin && rank < a.rank_end));
+                if (MODE == MODE_DUMP && valid && a.dump_scores) a.dump_scores[rank] = score;
                 if (MODE == MODE_TOPN) {
-#pragma unroll
-                    for (int m = 0; m < 2; ++m) {
-                        const bool cand = val[m] && sc[m] >= gthr && better(sc[m], rk[m], thr_s, thr_r);
-                        const unsigned mk = __ballot_sync(FULL, cand);
-                        if (mk) {
-                            int base = 0;
-                            if (lane == 0) base = atomicAdd(&buf_count, __popc(mk));
-                            base = __shfl_sync(FULL, base, 0);
-                            if (cand) {
-                                // The headroom keeps the slot inside the buffer.
-                                const int s2 = min(L + base + __popc(mk & ((1u << lane) - 1u)), a.P2 - 1);
-                                lscore[s2] = sc[m];
-                                lrank[s2] = rk[m];
-                            }
+                    // A combination has to reach the list's last score, which
+                    // only rises (a racy read is a score it had at some time),
+                    // and the score that enough combinations of all CTAs are
+                    // known to reach.
+                    const float lthr = *(volatile float *)(lscore + L - 1);
+                    const unsigned long long t2 = *(volatile unsigned long long *)&threshold;
+                    const bool low = (int)(t2 >> 32) == job && score < __uint_as_float((uint32_t)t2);
+                    const bool cand = valid && score >= lthr && !low && better(score, rank, thr_s, thr_r);
+                    const unsigned mk = __ballot_sync(FULL, cand);
+                    if (mk) {
+                        if (cand) {
+                            const int p = cnt + __popc(mk & ((1u << lane) - 1u));
+                            ws[p] = score;
+                            wr[p] = rank;
                         }
+                        cnt += __popc(mk);
+                        __syncwarp();
+                        if (cnt > T3_WBUF - 32) merge();
                     }
+                }
+            }
+            if (nr == 0) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if constexpr (PAIR) mbar_arrive_cluster(tempty0 + 8 * b);
+                    else mbar_arrive(&bar_tempty[b]);
                 }
             }
         }
         // The last list (a batched launch: of the last job this CTA took;
         // its lists of jobs it never took stay as filled before the launch).
-        if (MODE == MODE_TOPN && (!BATCH || ljob >= 0)) flush();
+        if (MODE == MODE_TOPN && ok && (!BATCH || cur_job >= 0)) flush();
+        if (ew == 0 && lane == 0) *(volatile int *)&epi_job = -2;
     }
 
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) {
+        // Neither CTA of a pair leaves while the other may still signal it or
+        // an MMA may read its shared memory (the leader has waited for its
+        // last commit above).
+        if (crank == 1 && threadIdx.x == 0) {
+            const long long t0 = clock64();
+            while (!mbar_try(&bar_done, 0) && clock64() - t0 < WAIT_BUDGET) {}
+        }
+        __syncwarp();
+        cluster_sync();
+    }
     if (warp == 3) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
-                     : "memory");
+        if constexpr (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
+                         : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
+                         : "memory");
     }
-}
-
-template <int ENC>
-size_t smem_bytes_enc(int M, int P2)   // ENC 2 has the shape of ENC 0
-{
-    using Sh = T3Shape<ENC>;
-    return 1024 + (size_t)T3_LOADERS * Sh::STAGE + (size_t)xl_table_size(M) * 4 + (size_t)P2 * (8 + 4) +
-           (size_t)2 * Sh::NP * T3_SJ_WORDS * 4;
 }
 
 template <int MODE, int ENC, bool BATCH>
@@ -730,17 +1012,17 @@ void *kernel_ptr()
 }
 
 // Pair rows of the first SNPs [i0, i1): thread (i - i0, t), t over the
-// pairs (i, j), j = i + 1 + jo, jo < NP ceil((S - 1 - i) / NP), times the
-// 16-byte chunks of a row; the row of pair (a, j, b) is
-// rowbase[i - i0] + (jo / NP) 4 NP + 2 NP a + 2 (jo % NP) + b.
-__global__ void k_pair_rows(const uint8_t *E, int64_t pitch, int Wt, int64_t S, int NP, int64_t i0,
-                            const int64_t *rowbase, uint8_t *P)
+// pairs (i, j), j = i + 1 + jo, jo < 2 NP ceil((S - 1 - i) / (2 NP)), times the
+// 16-byte chunks of a row; the row of pair (j, a, b) is
+// rowbase[i - i0] + 4 jo + 2 a + b.
+__global__ void k_pair_rows(const uint8_t *E, int64_t pitch, int Wt, int64_t S, int64_t i0, const int64_t *rowbase,
+                            uint8_t *P)
 {
     const int64_t ii = blockIdx.y;
     const int64_t i = i0 + ii;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t npairs = (S - 1 - i + NP - 1) / NP * NP;
-    const int cw = 8 * Wt;                         // 16-byte chunks per row
+    const int64_t npairs = (S - 1 - i + 2 * T3_NP - 1) / (2 * T3_NP) * (2 * T3_NP);
+    const int cw = 4 * Wt;                         // 16-byte chunks per row
     if (t >= npairs * cw) return;
     const int64_t jo = t / cw;
     const int ch = (int)(t - jo * cw);
@@ -752,56 +1034,33 @@ __global__ void k_pair_rows(const uint8_t *E, int64_t pitch, int Wt, int64_t S, 
         b0 = *(reinterpret_cast<const uint4 *>(E + (2 * j) * pitch) + ch);
         b1 = *(reinterpret_cast<const uint4 *>(E + (2 * j + 1) * pitch) + ch);
     }
-    const int64_t blk = jo / NP, q = jo % NP;
-    const int64_t row = rowbase[ii] + blk * 4 * NP + 2 * q;
-    auto put = [&](int a, int b, const uint4 &x, const uint4 &y) {
-        *(reinterpret_cast<uint4 *>(P + (row + 2 * NP * a + b) * pitch) + ch) =
+    const int64_t row = rowbase[ii] + 4 * jo;
+    auto put = [&](int r, const uint4 &x, const uint4 &y) {
+        *(reinterpret_cast<uint4 *>(P + (row + r) * pitch) + ch) =
             make_uint4(x.x & y.x, x.y & y.y, x.z & y.z, x.w & y.w);
     };
-    put(0, 0, a0, b0);
-    put(0, 1, a0, b1);
-    put(1, 0, a1, b0);
-    put(1, 1, a1, b1);
+    put(0, a0, b0);
+    put(1, a0, b1);
+    put(2, a1, b0);
+    put(3, a1, b1);
 }
 
-// Rows of the batched form from a bit table X in the sample order of a data
-// set's first replicate: row 2 s + g, byte b of chunk w is e5m2 1.0 (0x3C)
-// where sample 128 w + b carries genotype g of SNP s, or 4096.0 (0x6C) where
-// it is also a control of the job's replicate (bit b of ctrl[w]; ctrl null:
-// the genotype rows without classes), else 0; rows of padding SNPs are zero.
-__global__ void k_expand_e5m2(const uint4 *X, int64_t S, int64_t S_pad, int Wt, int64_t rows, int64_t pitch,
-                              const uint4 *ctrl, uint8_t *E)
+// E[2 s + g]: genotype row g of SNP s as e2m1 nibbles, 64 bytes a word; rows of
+// padding SNPs are zero.  Thread (row, word).
+__global__ void k_expand_fp4(const uint4 *X, int64_t S, int64_t S_pad, int64_t rows, int Wt, int64_t pitch, uint8_t *E)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= rows * Wt) return;
     const int64_t row = t / Wt;
     const int w = (int)(t % Wt);
     const int64_t s = row >> 1;
-    const int g = (int)(row & 1);
     uint4 bits = make_uint4(0, 0, 0, 0);
-    if (s < S) bits = X[((size_t)w * 3 + g) * S_pad + s];
-    const uint4 cm = ctrl ? ctrl[w] : make_uint4(0, 0, 0, 0);
-    const uint32_t b32[4] = {bits.x, bits.y, bits.z, bits.w};
-    const uint32_t c32[4] = {cm.x, cm.y, cm.z, cm.w};
-    uint4 *dst = reinterpret_cast<uint4 *>(E + row * pitch + (int64_t)w * 128);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        uint32_t o[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int bit0 = q * 16 + u * 4;
-            const uint32_t word = b32[bit0 >> 5], cw = c32[bit0 >> 5];
-            const int sh = bit0 & 31;
-            uint32_t v = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const uint32_t byte = ((cw >> (sh + e)) & 1u) ? 0x6Cu : 0x3Cu;
-                v |= (((word >> (sh + e)) & 1u) ? byte : 0u) << (8 * e);
-            }
-            o[u] = v;
-        }
-        dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
+    if (s < S) bits = X[((size_t)w * 3 + (row & 1)) * S_pad + s];
+    uint4 *dst = reinterpret_cast<uint4 *>(E + row * pitch + (int64_t)w * 64);
+    dst[0] = expand_fp4(bits.x);
+    dst[1] = expand_fp4(bits.y);
+    dst[2] = expand_fp4(bits.z);
+    dst[3] = expand_fp4(bits.w);
 }
 
 __global__ void k_fill_lists(float *s, uint64_t *r, size_t n)
@@ -814,11 +1073,11 @@ __global__ void k_fill_lists(float *s, uint64_t *r, size_t n)
 
 }  // namespace
 
-cudaError_t launch_expand_e5m2(const uint4 *X, int64_t S, int64_t S_pad, int Wt, int64_t rows, int64_t pitch,
-                               const uint4 *ctrl, uint8_t *E, cudaStream_t st)
+cudaError_t launch_expand_fp4(const uint4 *X, int64_t S, int64_t S_pad, int Wt, int64_t pitch, uint8_t *E,
+                              cudaStream_t st)
 {
-    const int64_t n = rows * Wt;
-    k_expand_e5m2<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(X, S, S_pad, Wt, rows, pitch, ctrl, E);
+    const int64_t n = triples_rows(S) * Wt;
+    k_expand_fp4<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(X, S, S_pad, triples_rows(S), Wt, pitch, E);
     return cudaGetLastError();
 }
 
@@ -845,42 +1104,66 @@ cudaError_t launch_log2_approx(const uint32_t *n, int64_t count, float *out, cud
     return cudaGetLastError();
 }
 
-int triples_pairs_per_tile(int enc) { return enc == 1 ? T3Shape<1>::NP : T3Shape<0>::NP; }
+int triples_pairs_per_tile(int enc) { return enc ? 2 * T3_NP : T3_NP; }
+int triples_snps_per_tile(int enc) { return enc ? 2 * T3_LB : T3_LB; }
+int triples_block_rows() { return T3_N; }
 
-int triples_round_candidates() { return 2 * T3_EPI_THREADS; }
-
-size_t triples_smem_bytes(int enc, int M, int P2)
+size_t triples_smem_bytes(int stages, int M, int L)
 {
-    return enc == 1 ? smem_bytes_enc<1>(M, P2) : smem_bytes_enc<0>(M, P2);
+    // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
+    return 2048 + (size_t)(M + 1) * 4 + (size_t)stages * T3_STAGE + (size_t)T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS * 4 +
+           (size_t)(L + T3_EPI_WARPS * T3_WBUF) * (8 + 4);
 }
 
-cudaError_t launch_pair_rows(const uint8_t *E, int64_t pitch, int Wt, int64_t S, int NP, int64_t i0, int64_t i1,
+int triples_stages(int M, int L, size_t smem_cap)
+{
+    for (int st = T3_MAX_STAGES; st >= 2; --st)
+        if (triples_smem_bytes(st, M, L) <= smem_cap) return st;
+    return 0;
+}
+
+float triples_scale(int64_t M)
+{
+    float q = 1.f;
+    for (int64_t m = M; m >= 8; m >>= 1) q *= 0.5f;   // 2^-s, s = floor(log2 M) - 2 (8 <= M)
+    return q;
+}
+
+void triples_publish(int L, int grid, int *pub_m, int *pub_r)
+{
+    const int half = std::max(1, std::min(grid, 32 * T3_PUB_PER_LANE) / 2);
+    *pub_m = std::min(L, (L + half - 1) / half);
+    *pub_r = (L + *pub_m - 1) / *pub_m;
+}
+
+cudaError_t launch_pair_rows(const uint8_t *E, int64_t pitch, int Wt, int64_t S, int64_t i0, int64_t i1,
                              const int64_t *rowbase, uint8_t *P, cudaStream_t st)
 {
     if (i1 <= i0) return cudaSuccess;
-    const int64_t maxn = (S - 1 - i0 + NP - 1) / NP * NP * 8 * (int64_t)Wt;   // the pairs of i0, the most
+    const int64_t blk = 2 * T3_NP;
+    const int64_t maxn = (S - 1 - i0 + blk - 1) / blk * blk * 4 * (int64_t)Wt;   // the pairs of i0, the most
     dim3 grid((unsigned)((maxn + 255) / 256), (unsigned)(i1 - i0));
-    k_pair_rows<<<grid, 256, 0, st>>>(E, pitch, Wt, S, NP, i0, rowbase, P);
+    k_pair_rows<<<grid, 256, 0, st>>>(E, pitch, Wt, S, i0, rowbase, P);
     return cudaGetLastError();
 }
 
 cudaError_t prepare_triples_tc_batch(int enc, size_t smem_bytes)
 {
-    if (enc != 1 && enc != 2) return cudaErrorInvalidValue;
-    void *fn = enc == 1 ? kernel_ptr<MODE_TOPN, 1, true>() : kernel_ptr<MODE_TOPN, 2, true>();
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    if (enc != 0 && enc != 1) return cudaErrorInvalidValue;
+    void *fn = enc == 1 ? kernel_ptr<MODE_TOPN, 1, true>() : kernel_ptr<MODE_TOPN, 0, true>();
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes - 1024);
 }
 
 cudaError_t launch_triples_tc(int mode, const CUtensorMap &tmapA, const CUtensorMap &tmapP, const TriplesArgs &a,
                               int grid, cudaStream_t st, bool set_attr)
 {
-    const size_t bytes = triples_smem_bytes(a.enc, a.M, a.P2);
+    const size_t bytes = triples_smem_bytes(a.stages, a.M, a.L) - 1024;
+    if (a.enc != 0 && a.enc != 1) return cudaErrorInvalidValue;
     void *fn = nullptr;
     if (a.jobs) {
-        if (mode != MODE_TOPN || (a.enc != 1 && a.enc != 2)) return cudaErrorInvalidValue;
-        fn = a.enc == 1 ? kernel_ptr<MODE_TOPN, 1, true>() : kernel_ptr<MODE_TOPN, 2, true>();
+        if (mode != MODE_TOPN) return cudaErrorInvalidValue;
+        fn = a.enc ? kernel_ptr<MODE_TOPN, 1, true>() : kernel_ptr<MODE_TOPN, 0, true>();
     } else {
-        if (a.enc != 0 && a.enc != 1) return cudaErrorInvalidValue;
         fn = mode == MODE_TOPN ? (a.enc ? kernel_ptr<MODE_TOPN, 1, false>() : kernel_ptr<MODE_TOPN, 0, false>())
                                : (a.enc ? kernel_ptr<MODE_DUMP, 1, false>() : kernel_ptr<MODE_DUMP, 0, false>());
     }
@@ -892,7 +1175,19 @@ cudaError_t launch_triples_tc(int mode, const CUtensorMap &tmapA, const CUtensor
     CUtensorMap mA = tmapA, mP = tmapP;
     TriplesArgs args = a;
     void *params[] = {&mA, &mP, &args};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(T3_THREADS), params, bytes, st);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(T3_THREADS);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = a.enc ? 1 : 0;   // form 1: CTA pairs (an even grid)
+    return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
 }  // namespace fc
