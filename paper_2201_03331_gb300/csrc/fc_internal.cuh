@@ -30,8 +30,14 @@ __host__ __device__ constexpr int pow3(int k) { return k <= 0 ? 1 : 3 * pow3(k -
 __host__ __device__ inline uint64_t binom(int64_t n, int r)
 {
     if (r < 0 || n < r) return 0;
+    // Unrolled, so that each division is by a constant: a division by a
+    // variable takes some 70 instructions, and a rank is turned into its
+    // combination by up to 30 of these.
     uint64_t c = 1;
-    for (int i = 1; i <= r; ++i) c = c * (uint64_t)(n - r + i) / (uint64_t)i;
+#pragma unroll
+    for (int i = 1; i <= 6; ++i)
+        if (i <= r) c = c * (uint64_t)(n - r + i) / (uint64_t)i;
+    for (int i = 7; i <= r; ++i) c = c * (uint64_t)(n - r + i) / (uint64_t)i;
     return c;
 }
 
@@ -177,12 +183,14 @@ struct RescoreArgs {
     uint64_t total;         // C(S, k)
     double *res_s;          // [L] FP64 scores (-inf where skipped)
     uint64_t *res_r;        // [L]
-    uint32_t *res_tab;      // [L][3^k][2] exact tables (optional)
+    uint32_t *res_c;        // [L][k] combinations
     uint32_t *err;
+    double *out_score;      // [N] the list
+    uint32_t *out_idx;      // [N][k]
+    uint32_t *out_err;      // *err after the rescoring
 };
-cudaError_t launch_rescore(const RescoreArgs &a, cudaStream_t st);
-cudaError_t launch_final_sort(double *res_s, uint64_t *res_r, int L, int N, int k, int64_t S,
-                              uint32_t *out_idx, double *out_score, cudaStream_t st);
+cudaError_t launch_rescore(const RescoreArgs &a, int sms, cudaStream_t st);
+cudaError_t launch_final(const RescoreArgs &a, cudaStream_t st);
 
 // ---- batched persistent search (many data sets / phenotype replicates) -----
 

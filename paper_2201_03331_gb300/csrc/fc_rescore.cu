@@ -1,5 +1,6 @@
 // Exact tables (warp AND/POPC reduction), FP64 rescoring of the FP32
 // candidates and the final ordering by (MI desc, combination asc).
+#include <algorithm>
 #include <cfloat>
 #include "fc_internal.cuh"
 
@@ -74,19 +75,49 @@ __device__ double warp_mi_fp64(const uint32_t *stab, int cells)
     const double n0 = (double)__reduce_add_sync(FULL, c0), n1 = (double)__reduce_add_sync(FULL, c1);
     const double N = n0 + n1;
     if (N <= 0.0) return 0.0;
-    double hx = 0.0, hxy = 0.0;
-    for (int x = lane; x < cells; x += 32) {
-        const double a = stab[2 * x], b = stab[2 * x + 1];
-        const double nx = a + b;
-        if (nx > 0.0) hx -= (nx / N) * log(nx / N);
-        if (a > 0.0) hxy -= (a / N) * log(a / N);
-        if (b > 0.0) hxy -= (b / N) * log(b / N);
+    // log(n / N), 0 for n = 0.
+    auto log_share = [&](double n) { return n > 0.0 ? log(n / N) : 0.0; };
+    double hx = 0.0, hxy = 0.0, l0, l1;
+    if (cells <= 9) {
+        // A logarithm per lane instead of five in a row: those of n, a and b
+        // of cell x on the lanes 3 x, 3 x + 1 and 3 x + 2, those of the classes
+        // on lanes 27 and 28.
+        const int y = lane / 3, kind = lane % 3;
+        double n = lane == 27 ? n0 : lane == 28 ? n1 : 0.0;
+        if (y < cells) {
+            const double a = stab[2 * y], b = stab[2 * y + 1];
+            n = kind == 0 ? a + b : kind == 1 ? a : b;
+        }
+        const double l = log_share(n);
+        l0 = __shfl_sync(FULL, l, 27);
+        l1 = __shfl_sync(FULL, l, 28);
+        const int x = min(lane, 8);
+        const double lx = __shfl_sync(FULL, l, 3 * x), la = __shfl_sync(FULL, l, 3 * x + 1),
+                     lb = __shfl_sync(FULL, l, 3 * x + 2);
+        if (lane < cells) {
+            const double a = stab[2 * lane], b = stab[2 * lane + 1];
+            const double nx = a + b;
+            if (nx > 0.0) hx -= (nx / N) * lx;
+            if (a > 0.0) hxy -= (a / N) * la;
+            if (b > 0.0) hxy -= (b / N) * lb;
+        }
+    } else {
+        for (int x = lane; x < cells; x += 32) {
+            const double a = stab[2 * x], b = stab[2 * x + 1];
+            const double nx = a + b;
+            if (nx > 0.0) hx -= (nx / N) * log(nx / N);
+            if (a > 0.0) hxy -= (a / N) * log(a / N);
+            if (b > 0.0) hxy -= (b / N) * log(b / N);
+        }
+        const double l = log_share(lane == 0 ? n0 : n1);
+        l0 = __shfl_sync(FULL, l, 0);
+        l1 = __shfl_sync(FULL, l, 1);
     }
     hx = warp_sum64(hx);
     hxy = warp_sum64(hxy);
     double hy = 0.0;
-    if (n0 > 0.0) hy -= (n0 / N) * log(n0 / N);
-    if (n1 > 0.0) hy -= (n1 / N) * log(n1 / N);
+    if (n0 > 0.0) hy -= (n0 / N) * l0;
+    if (n1 > 0.0) hy -= (n1 / N) * l1;
     return hx + hy - hxy;
 }
 
@@ -130,45 +161,88 @@ __global__ void k_rescore(RescoreArgs a)
     uint4 *rows;
     uint32_t *stab;
     warp_area(a.k, rows, stab);
-    warp_table(a.X, a.S_pad, a.W0, a.Wt, a.k, c, rows, stab, a.res_tab ? a.res_tab + (size_t)i * cells * 2 : nullptr);
+    warp_table(a.X, a.S_pad, a.W0, a.Wt, a.k, c, rows, stab, nullptr);
     const double mi = warp_mi_fp64(stab, cells);
     if (lane == 0) {
         a.res_s[i] = mi;
         a.res_r[i] = r;
+        for (int t = 0; t < a.k; ++t) a.res_c[(size_t)i * a.k + t] = c[t];
     }
 }
 
-__global__ void k_final_sort(double *res_s, uint64_t *res_r, int L, int N, int k, int64_t S,
-                             uint32_t *out_idx, double *out_score)
+// The rescored candidates in order, their best N and the search's error word to
+// out_score, out_idx and out_err.  In one CTA: the candidates within the
+// window are collected; up to FINAL_COUNT of them take the place that their
+// better ones leave them, several threads counting for one (64-bit integer
+// keys: the chip compares few doubles a cycle), more are sorted.
+constexpr int FINAL_THREADS = 1024;
+constexpr int FINAL_COUNT = 256;
+__global__ void __launch_bounds__(FINAL_THREADS) k_final(RescoreArgs a)
 {
     extern __shared__ uint4 smem4[];
+    __shared__ int taken;
     uint64_t *r = reinterpret_cast<uint64_t *>(smem4);
-    double *s = reinterpret_cast<double *>(r + L);
-    for (int i = threadIdx.x; i < L; i += blockDim.x) { s[i] = res_s[i]; r[i] = res_r[i]; }
-    for (int size = 2; size <= L; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < (L >> 1); i += blockDim.x) {
-                const int lo = 2 * i - (i & (stride - 1));
-                const int hi = lo + stride;
-                const bool desc = (lo & size) == 0;
-                const double s1 = s[lo], s2 = s[hi];
-                const uint64_t r1 = r[lo], r2 = r[hi];
-                const bool sw = desc ? better64(s2, r2, s1, r1) : better64(s1, r1, s2, r2);
-                if (sw) { s[lo] = s2; s[hi] = s1; r[lo] = r2; r[hi] = r1; }
-            }
-        }
+    uint64_t *s = r + a.L;                                 // scores as ordered integers
+    uint32_t *at = reinterpret_cast<uint32_t *>(s + a.L);   // candidate
+    const int tid = threadIdx.x, L = a.L;
+    if (tid == 0) {
+        taken = 0;
+        *a.out_err = *a.err;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        out_score[i] = s[i];
-        uint32_t c[KMAX_TABLES];
-        if (r[i] != NO_RANK) {
-            unrank(S, k, r[i], c);
-        } else {
-            for (int t = 0; t < k; ++t) c[t] = 0xffffffffu;
+    for (int i = tid; i < L; i += FINAL_THREADS) {
+        const uint64_t rk = a.res_r[i];
+        if (rk == NO_RANK) continue;
+        const long long o = __double_as_longlong(a.res_s[i] + 0.0);   // (-0 as +0)
+        const int p = atomicAdd(&taken, 1);
+        r[p] = rk;
+        s[p] = (uint64_t)(o >= 0 ? o : o ^ 0x7fffffffffffffffll) ^ 0x8000000000000000ull;
+        at[p] = (uint32_t)i;
+    }
+    __syncthreads();
+    const int C = taken;
+    auto put = [&](int place, int i) {
+        a.out_score[place] = a.res_s[i];
+        for (int t = 0; t < a.k; ++t) a.out_idx[(size_t)place * a.k + t] = a.res_c[(size_t)i * a.k + t];
+    };
+    if (C <= FINAL_COUNT) {
+        int per = FINAL_THREADS / FINAL_COUNT;
+        while (per < 32 && 2 * per * C <= FINAL_THREADS) per *= 2;
+        const int e = tid / per;
+        int place = 0;
+        if (e < C)
+            for (int x = tid % per; x < C; x += per) place += s[x] > s[e] || (s[x] == s[e] && r[x] < r[e]);
+        for (int o = per / 2; o > 0; o >>= 1) place += __shfl_xor_sync(FULL, place, o);
+        if (e < C && tid % per == 0 && place < a.N) put(place, (int)at[e]);
+    } else {
+        int m = FINAL_COUNT;
+        while (m < C) m *= 2;
+        for (int i = C + tid; i < m; i += FINAL_THREADS) { s[i] = 0; r[i] = NO_RANK; }
+        for (int size = 2; size <= m; size <<= 1) {
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                __syncthreads();
+                for (int i = tid; i < (m >> 1); i += FINAL_THREADS) {
+                    const int lo = 2 * i - (i & (stride - 1));
+                    const int hi = lo + stride;
+                    const bool desc = (lo & size) == 0;
+                    const uint64_t s1 = s[lo], s2 = s[hi], r1 = r[lo], r2 = r[hi];
+                    const bool first2 = s2 > s1 || (s2 == s1 && r2 < r1);
+                    const bool first1 = s1 > s2 || (s1 == s2 && r1 < r2);
+                    if (desc ? first2 : first1) {
+                        s[lo] = s2; s[hi] = s1; r[lo] = r2; r[hi] = r1;
+                        const uint32_t x = at[lo];
+                        at[lo] = at[hi];
+                        at[hi] = x;
+                    }
+                }
+            }
         }
-        for (int t = 0; t < k; ++t) out_idx[(size_t)i * k + t] = c[t];
+        __syncthreads();
+        for (int i = tid; i < min(a.N, C); i += FINAL_THREADS) put(i, (int)at[i]);
+    }
+    for (int i = C + tid; i < a.N; i += FINAL_THREADS) {
+        a.out_score[i] = -DBL_MAX;
+        for (int t = 0; t < a.k; ++t) a.out_idx[(size_t)i * a.k + t] = 0xffffffffu;
     }
 }
 
@@ -272,20 +346,23 @@ static_assert(8 * warp_table_smem(3) <= 48 * 1024 && 4 * warp_table_smem(5) <= 4
 
 }  // namespace
 
-cudaError_t launch_rescore(const RescoreArgs &a, cudaStream_t st)
+cudaError_t launch_rescore(const RescoreArgs &a, int sms, cudaStream_t st)
 {
-    const int wpb = table_warps_per_block(a.k);
+    // As few warps a block as spread the candidates over all SMs: the double
+    // logarithms of one SM go through two lanes a cycle (64 candidates in
+    // blocks of 8 warps took 31 us, one a block 15, with the logarithms spread over the lanes at
+    // orders 1 and 2 and the divisions of the ranks by constants).
+    const int wpb = std::min(table_warps_per_block(a.k), (a.L + sms - 1) / sms);
     k_rescore<<<(a.L + wpb - 1) / wpb, wpb * 32, wpb * warp_table_smem(a.k), st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_final_sort(double *res_s, uint64_t *res_r, int L, int N, int k, int64_t S,
-                              uint32_t *out_idx, double *out_score, cudaStream_t st)
+cudaError_t launch_final(const RescoreArgs &a, cudaStream_t st)
 {
-    const size_t bytes = (size_t)L * 16;
-    cudaError_t e = cudaFuncSetAttribute(k_final_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const size_t bytes = (size_t)a.L * 20;
+    cudaError_t e = cudaFuncSetAttribute(k_final, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    k_final_sort<<<1, 1024, bytes, st>>>(res_s, res_r, L, N, k, S, out_idx, out_score);
+    k_final<<<1, FINAL_THREADS, bytes, st>>>(a);
     return cudaGetLastError();
 }
 

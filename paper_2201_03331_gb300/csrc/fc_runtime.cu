@@ -1503,7 +1503,7 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
     double hy = 0.0;
     if (M1 > 0) hy -= (M1 / Nd) * std::log(M1 / Nd);
     if (M0 > 0) hy -= (M0 / Nd) * std::log(M0 / Nd);
-    const int cells = pow3(k);
+    const size_t result_bytes = (sizeof(double) + sizeof(uint32_t) * k) * (size_t)N + sizeof(uint32_t);
 
     // With caller-provided scratch nothing may be allocated: operands that
     // are built on first use (tensor-core operands, inclusion-exclusion
@@ -1674,14 +1674,13 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
             p[5] = A.take(sizeof(uint64_t) * (size_t)nl1 * L);
             p[6] = A.take(sizeof(double) * L);
             p[7] = A.take(sizeof(uint64_t) * L);
-            p[8] = A.take(sizeof(uint32_t) * (size_t)L * cells * 2);
-            p[9] = A.take(sizeof(uint32_t) * (size_t)N * k);
-            p[10] = A.take(sizeof(double) * (size_t)N);
-            p[11] = A.take(sizeof(int) * (4 + (size_t)sms));
-            p[12] = A.take(sizeof(uint32_t) * range_tiles.size() + sizeof(int4) * range_groups4.size() +
+            p[8] = A.take(sizeof(uint32_t) * (size_t)L * k);
+            p[9] = A.take(result_bytes);   // scores, combinations, error word
+            p[10] = A.take(sizeof(int) * (4 + (size_t)sms));
+            p[11] = A.take(sizeof(uint32_t) * range_tiles.size() + sizeof(int4) * range_groups4.size() +
                            sizeof(uint64_t) * (lt4.size() + lr4.size()) + sizeof(int) * amax4.size() + include4.size() + 16);
         };
-        void *p[13];
+        void *p[12];
         plan(ar, p);
         Arena A2;
         if (ext_scratch) {
@@ -1717,29 +1716,29 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         if (tc) {
             pa.list_score = (float *)p[0];
             pa.list_rank = (uint64_t *)p[1];
-            pa.gthr = (int *)p[11];
-            pa.tile_counter = (int *)p[11] + 1;
+            pa.gthr = (int *)p[10];
+            pa.tile_counter = (int *)p[10] + 1;
             pa.err = err;
             if (!range_tiles.empty()) {
-                cudaMemcpyAsync(p[12], range_tiles.data(), sizeof(uint32_t) * range_tiles.size(),
+                cudaMemcpyAsync(p[11], range_tiles.data(), sizeof(uint32_t) * range_tiles.size(),
                                 cudaMemcpyHostToDevice, stream);
-                pa.tiles = (const uint32_t *)p[12];
+                pa.tiles = (const uint32_t *)p[11];
             }
             // 0x80808080 is below the ordered image of every finite score.
-            cudaMemsetAsync(p[11], 0x80, sizeof(int), stream);
+            cudaMemsetAsync(p[10], 0x80, sizeof(int), stream);
             cudaMemsetAsync(pa.tile_counter, 0, sizeof(int), stream);
             if ((e = launch_gate()) != cudaSuccess || (e = launch_pairs_tc(MODE_TOPN, tmap, pa, grid, stream)) != cudaSuccess)
                 return cuda_status(e, "tensor-core pairs kernel");
         } else if (tc4) {
             const TupleTC &u = tup[k - 4];
-            qa.gthr = (int *)p[11];
-            qa.tile_counter = (int *)p[11] + 1;
+            qa.gthr = (int *)p[10];
+            qa.tile_counter = (int *)p[10] + 1;
             qa.err = err;
             const int4 *groups = u.groups;
             const int *amax = u.amax;
             CUtensorMap tmapL = u.tmapL;
             if (!whole) {
-                int4 *dg = (int4 *)p[12];
+                int4 *dg = (int4 *)p[11];
                 if (!range_groups4.empty())
                     cudaMemcpyAsync(dg, range_groups4.data(), sizeof(int4) * range_groups4.size(),
                                     cudaMemcpyHostToDevice, stream);
@@ -1768,7 +1767,7 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
                     qa.include = di;
                 }
             }
-            cudaMemsetAsync(p[11], 0x80, sizeof(int), stream);
+            cudaMemsetAsync(p[10], 0x80, sizeof(int), stream);
             for (size_t x = 0; x < launches4.size(); ++x) {
                 const int64_t c = launches4[x];
                 int rc = build_right_chunk(k, c);
@@ -1783,9 +1782,9 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
                 if (x > 0) note_launches(1);
             }
         } else if (tc3) {
-            ta.pub = (int *)p[11] + 4;
+            ta.pub = (int *)p[10] + 4;
             triples_publish(L, ctas, &ta.pub_m, &ta.pub_r);
-            ta.tile_counter = (int *)p[11] + 1;
+            ta.tile_counter = (int *)p[10] + 1;
             ta.err = err;
             // 0x80808080 is below the ordered image of every finite score.
             cudaMemsetAsync(ta.pub, 0x80, sizeof(int) * (size_t)sms, stream);
@@ -1834,18 +1833,22 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         ra.X = X; ra.S = S; ra.S_pad = S_pad; ra.W0 = W0; ra.Wt = Wt; ra.k = k;
         ra.N = (int)N; ra.L = L; ra.cand_s = src_s; ra.cand_r = src_r; ra.eps = eps;
         ra.total = r1 - r0;
-        ra.res_s = (double *)p[6]; ra.res_r = (uint64_t *)p[7]; ra.res_tab = (uint32_t *)p[8];
+        ra.res_s = (double *)p[6]; ra.res_r = (uint64_t *)p[7]; ra.res_c = (uint32_t *)p[8];
         ra.err = err;
-        if ((e = launch_rescore(ra, stream)) != cudaSuccess) return cuda_status(e, "rescore kernel");
-        if ((e = launch_final_sort((double *)p[6], (uint64_t *)p[7], L, (int)N, k, S, (uint32_t *)p[9],
-                                   (double *)p[10], stream)) != cudaSuccess)
-            return cuda_status(e, "final sort kernel");
+        ra.out_score = (double *)p[9];
+        ra.out_idx = reinterpret_cast<uint32_t *>(ra.out_score + N);
+        ra.out_err = ra.out_idx + (size_t)N * k;
+        if ((e = launch_rescore(ra, sms, stream)) != cudaSuccess) return cuda_status(e, "rescore kernel");
+        if ((e = launch_final(ra, stream)) != cudaSuccess) return cuda_status(e, "final sort kernel");
         note_launches(2);
-        uint32_t herr = 0;
-        cudaMemcpyAsync(&herr, err, sizeof herr, cudaMemcpyDeviceToHost, stream);
-        cudaMemcpyAsync(out_idx, p[9], sizeof(uint32_t) * (size_t)N * k, cudaMemcpyDeviceToHost, stream);
-        cudaMemcpyAsync(out_score, p[10], sizeof(double) * (size_t)N, cudaMemcpyDeviceToHost, stream);
+        // One copy: each to pageable memory waits for the stream by itself.
+        std::vector<uint8_t> result(result_bytes);
+        cudaMemcpyAsync(result.data(), p[9], result_bytes, cudaMemcpyDeviceToHost, stream);
         if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_status(e, "search");
+        uint32_t herr = 0;
+        memcpy(out_score, result.data(), sizeof(double) * (size_t)N);
+        memcpy(out_idx, result.data() + sizeof(double) * (size_t)N, sizeof(uint32_t) * (size_t)N * k);
+        memcpy(&herr, result.data() + result_bytes - sizeof herr, sizeof herr);
         if (timing) {
             float ms = 0.f;
             if (cudaEventElapsedTime(&ms, ev_sweep0, ev_sweep1) == cudaSuccess) {

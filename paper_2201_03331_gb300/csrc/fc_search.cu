@@ -21,6 +21,7 @@
 //    of restricted pair counts computed once per data set.  The arithmetic
 //    is exact integer subtraction; every intermediate is a count, so the
 //    packed (cases | controls << 16) words never borrow across fields.
+#include <algorithm>
 #include <cfloat>
 #include "fc_internal.cuh"
 #include "fc_ie.cuh"
@@ -824,30 +825,112 @@ __global__ void k_restricted_pairs(const uint4 *X, int64_t S, int64_t S_pad, int
     if (i != j) PR[(size_t)j * S_pad + i] = make_uint4(acc[0], acc[2], acc[1], acc[3]);
 }
 
-// Grid-level merge: each CTA sorts F lists of L entries and keeps the best L.
-__global__ void k_merge(const float *in_s, const uint64_t *in_r, int nlists, int L, int F,
-                        float *out_s, uint64_t *out_r)
+// Grid-level merge: each CTA keeps the best L of up to F lists of L entries (in
+// any order within a list), best first.
+//
+// Only the entries that can be among them are sorted: a bitwise search finds a
+// score that at least L and at most 2 L entries reach (one count per bit over
+// the keys, which stay in shared memory), and those alone are collected and
+// put in order.  Should so many scores tie that there is no such score, a
+// second search takes the smallest ranks among the tied.  Bound by the latency
+// of the counts and of one pass over the lists; 608 lists of 64 take 20 us in
+// two launches, where sorting all entries in blocks of 4096 took 94.
+constexpr int SEL_THREADS = 1024;
+constexpr int SEL_MAX = 32768;   // entries of a block: 128 KiB of keys beside 2 L <= 8192 candidates
+__global__ void __launch_bounds__(SEL_THREADS) k_select(const float *in_s, const uint64_t *in_r, int nlists, int L, int F,
+                                                        float *out_s, uint64_t *out_r)
 {
     extern __shared__ uint4 smem4[];
-    const int n = F * L;
-    uint64_t *r = reinterpret_cast<uint64_t *>(smem4);
-    float *s = reinterpret_cast<float *>(r + n);
-    const int first = blockIdx.x * F;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int lst = first + i / L;
-        if (lst < nlists) {
-            s[i] = in_s[(size_t)first * L + i];
-            r[i] = in_r[(size_t)first * L + i];
-        } else {
-            s[i] = -FLT_MAX;
-            r[i] = NO_RANK;
+    __shared__ int count[1 + 32 + 1 + 64];   // one per count, so that one barrier serves each
+    __shared__ int taken;
+    const int cap = 2 * L;
+    uint64_t *cr = reinterpret_cast<uint64_t *>(smem4);
+    float *cs = reinterpret_cast<float *>(cr + cap);
+    uint32_t *key = reinterpret_cast<uint32_t *>(cs + cap);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const size_t base = (size_t)blockIdx.x * F * L;
+    const int n = min(F, nlists - (int)blockIdx.x * F) * L;
+    for (int i = tid; i < 1 + 32 + 1 + 64; i += SEL_THREADS) count[i] = 0;
+    if (tid == 0) taken = 0;
+    // Keys in the order of the scores (-0 as +0), 0 for an empty entry.
+    for (int i = tid; i < n; i += SEL_THREADS) {
+        const float s = in_s[base + i];
+        const int o = __float_as_int(s + 0.f);
+        key[i] = s == -FLT_MAX ? 0u : (uint32_t)(o >= 0 ? o : o ^ 0x7fffffff) ^ 0x80000000u;
+    }
+    __syncthreads();
+    auto total = [&](int x, int mine) -> int {
+        mine = __reduce_add_sync(0xffffffffu, mine);
+        if (lane == 0 && mine) atomicAdd(&count[x], mine);
+        __syncthreads();
+        return count[x];
+    };
+    auto reaching = [&](int x, uint32_t t) -> int {
+        int c = 0;
+        for (int i = tid; i < n; i += SEL_THREADS) c += key[i] >= t;
+        return total(x, c);
+    };
+    uint32_t t = 1;
+    uint64_t last = NO_RANK;   // of the entries at t itself, the ranks up to this one
+    if (reaching(0, t) > cap) {
+        bool ties = true;
+        t = 0;
+        for (int b = 31; b >= 0; --b) {
+            const int c = reaching(32 - b, t | 1u << b);
+            if (c >= L) t |= 1u << b;
+            if (c >= L && c <= cap) { ties = false; break; }
+        }
+        if (ties) {
+            // Fewer than L entries above t, more than 2 L with it.
+            int c = 0;
+            for (int i = tid; i < n; i += SEL_THREADS) c += key[i] > t;
+            const int above = total(33, c);
+            last = 0;
+            for (int b = 63; b >= 0; --b) {
+                const uint64_t r = last | 1ull << b;
+                c = 0;
+                for (int i = tid; i < n; i += SEL_THREADS)
+                    if (key[i] == t) c += in_r[base + i] < r;
+                if (above + total(97 - b, c) < L) last = r;
+            }
         }
     }
-    block_bitonic_desc(s, r, n);
-    for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        out_s[(size_t)blockIdx.x * L + i] = s[i];
-        out_r[(size_t)blockIdx.x * L + i] = r[i];
+    for (int i = tid; i < n; i += SEL_THREADS) {
+        const uint32_t q = key[i];
+        if (q < t) continue;
+        const uint64_t r = in_r[base + i];
+        if (q == t && r > last) continue;
+        const int p = atomicAdd(&taken, 1);
+        if (p >= cap) continue;   // (not with distinct ranks)
+        cs[p] = in_s[base + i];
+        cr[p] = r;
     }
+    __syncthreads();
+    const int C = min(taken, cap);
+    float *os = out_s + (size_t)blockIdx.x * L;
+    uint64_t *orr = out_r + (size_t)blockIdx.x * L;
+    if (C <= SEL_THREADS / 4) {
+        // An entry's place is the number of better ones: 4 to 32 threads count
+        // for one entry.
+        int per = 4;
+        while (per < 32 && 2 * per * C <= SEL_THREADS) per *= 2;
+        const int e = tid / per;
+        int place = 0;
+        if (e < C)
+            for (int x = tid % per; x < C; x += per) place += better(cs[x], cr[x], cs[e], cr[e]);
+        for (int o = per / 2; o > 0; o >>= 1) place += __shfl_xor_sync(0xffffffffu, place, o);
+        if (e < C && tid % per == 0 && place < L) {
+            os[place] = cs[e];
+            orr[place] = cr[e];
+        }
+        for (int i = C + tid; i < L; i += SEL_THREADS) { os[i] = -FLT_MAX; orr[i] = NO_RANK; }
+        return;
+    }
+    int m = L;   // (a power of two; C <= 2 L)
+    if (C > L) m = cap;
+    for (int i = C + tid; i < m; i += SEL_THREADS) { cs[i] = -FLT_MAX; cr[i] = NO_RANK; }
+    block_bitonic_desc(cs, cr, m);
+    for (int i = tid; i < L; i += SEL_THREADS) { os[i] = cs[i]; orr[i] = cr[i]; }
 }
 
 // Per-job merge of the batched item lists: CTA j merges job j's items.
@@ -1004,13 +1087,14 @@ cudaError_t launch_restricted_pairs(const uint4 *X, int64_t S, int64_t S_pad, in
 cudaError_t launch_merge(const float *in_s, const uint64_t *in_r, int nlists, int L,
                          float *out_s, uint64_t *out_r, int *nout, cudaStream_t st)
 {
-    int F = 4096 / L;
-    if (F < 2) F = 2;
+    // Blocks of 4096 entries (four keys a thread), or of 16 lists where those
+    // are more, which keeps long lists at two or three launches.
+    const int F = std::max(2, std::min(nlists, std::min(SEL_MAX / L, std::max(16, 4096 / L))));
     const int blocks = (nlists + F - 1) / F;
-    const size_t bytes = (size_t)F * L * 12;
-    cudaError_t e = cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const size_t bytes = (size_t)F * L * 4 + (size_t)2 * L * 12;
+    cudaError_t e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    k_merge<<<blocks, 512, bytes, st>>>(in_s, in_r, nlists, L, F, out_s, out_r);
+    k_select<<<blocks, SEL_THREADS, bytes, st>>>(in_s, in_r, nlists, L, F, out_s, out_r);
     *nout = blocks;
     return cudaGetLastError();
 }
