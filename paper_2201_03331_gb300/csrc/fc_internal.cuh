@@ -249,7 +249,6 @@ cudaError_t launch_final_sort_batch(const JobDesc *jobs, int n_jobs, double *res
 // ---- order-2 tensor-core path (fc_pairs_tc.cu) -----------------------------
 
 constexpr int TC_MAX_STAGES = 6;
-constexpr int TC_MAX_PRODUCERS = 4;   // TMA producer warps of the order-2 kernel
 enum { MODE_DUMP = 2 };
 // Time budget of one mbarrier wait in the tensor-core kernels, in clock64
 // ticks (about 2 s).  The pipeline waits of the order-2 kernel take theirs
@@ -258,34 +257,46 @@ enum { MODE_DUMP = 2 };
 constexpr long long TC_WAIT_TICKS = 4000000000ll;
 
 struct PairsArgs {
-    const uint32_t *tiles;  // (I << 16 | J) 64-SNP block pairs, I <= J
+    const uint32_t *tiles;  // (I << 16 | J): SNPs i from pairs_rows_i I, SNPs j from pairs_rows_j J
     int ntiles;
+    int enc;                // 1: one accumulator n_case + 4096 n_ctrl, a tile per CTA pair; 0: one per class
     int64_t S;
-    int W0, Wt;             // 128-sample chunks: cases [0, W0), controls [W0, Wt)
-    const uint16_t *marg;   // [S][8]: cases g0..g2, controls g0..g2, pad
-    const float *logtab;
+    int W0, Wt;             // 128-sample words: cases [0, W0), controls [W0, Wt)
+    const uint4 *marg4;     // per-SNP genotype counts (one uint4 per SNP)
+    int stages;             // load stages (pairs_stages)
+    const float *xlogx;     // y log2 y, y = scale x, for x = 0..M (FP64 rounded once to FP32)
+    float scale;            // the power of two the kernel scores counts in (triples_scale)
     int M;
     float hy, invN;
     uint64_t pair_base;     // C(S, 2)
     uint64_t rank_begin, rank_end;   // only pairs with ranks in [rank_begin, rank_end) count
-    int L, Bcap, P2, stages;
-    int producers;          // TMA producer warps (a divisor of stages, at most 4)
+    int L;
     long long wait_ticks;   // budget of each pipeline wait (clock64 ticks)
     float *list_score;      // [grid][L]
     uint64_t *list_rank;
-    int *gthr;              // global score threshold (ordered int)
+    // Scores of the lists' entries pub_m - 1 as ordered ints, [grid], set below
+    // every score before the launch; pub_r of them bound the score of the last
+    // of L pairs (triples_publish).
+    int *pub;
+    int pub_m, pub_r;
     int *tile_counter;      // next tile of the global order, zeroed before launch
     uint32_t *err;
     float *dump_scores;     // MODE_DUMP: [S][S] (i < j)
     uint32_t *dump_tables;  // MODE_DUMP: [S][S][9][2]
 };
 
-size_t pairs_smem_bytes(int stages, int M, int P2);
-cudaError_t launch_expand_e4m3(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, int64_t rows, int64_t pitch,
-                               uint8_t *E, uint8_t ctrl_byte, cudaStream_t st);
+// SNPs of a tile on either side, and the rows a CTA loads of the SNPs j.
+int pairs_rows_i(int enc);
+int pairs_rows_j(int enc);
+int pairs_block_rows();
+// The load stages that fit smem_cap bytes of shared memory beside the table of
+// M samples and lists of L; 0 if not even two do.
+int pairs_stages(int M, int L, size_t smem_cap);
+size_t pairs_smem_bytes(int stages, int M, int L);
 cudaError_t launch_marginals(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, uint16_t *marg,
                              cudaStream_t st);
-cudaError_t launch_pairs_tc(int mode, const CUtensorMap &tmap, const PairsArgs &a, int grid, cudaStream_t st);
+cudaError_t launch_pairs_tc(int mode, const CUtensorMap &tmapI, const CUtensorMap &tmapJ, const PairsArgs &a, int grid,
+                            cudaStream_t st);
 
 // Order-3 tensor-core search (fc_triples_tc.cu).  A tile pairs the SNPs l0 ..
 // l0 + triples_snps_per_tile - 1 (packed 4-bit rows 2 l + g) with the pairs (i,

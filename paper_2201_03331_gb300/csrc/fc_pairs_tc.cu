@@ -4,67 +4,86 @@
 // contraction (Section "Computing the contingency tables": a cell is the
 // population count of the AND of one row of each SNP's genotype table):
 //     n_c(g, h)[i, j] = sum_{m in class c} [G_i(m) = g] [G_j(m) = h].
-// With the genotype rows g, h in {0, 1} stored as 0/1 e4m3 bytes
-// (E[2s + g][m]), one class's counts for all pairs are E_c E_c^T.  Products
-// of 0/1 are exact and FP32 accumulation of integers below 2^24 is exact,
-// so tcgen05.mma kind::f8f6f4 computes the four {0,1}x{0,1} cells of every
-// pair exactly.  The five cells that involve genotype 2 follow exactly from
-// the per-SNP genotype counts (the rows of each SNP's genotype table
+// With the genotype rows g, h in {0, 1} stored as packed 0/1 e2m1 nibbles
+// (E[2s + g][m]) one class's counts for all pairs are E_c E_c^T, and
+// tcgen05.mma kind::mxf4 computes the four {0,1}x{0,1} cells of every pair
+// exactly (fc_tc.cuh).  The five cells that involve genotype 2 follow exactly
+// from the per-SNP genotype counts (the rows of each SNP's genotype table
 // partition the samples):
 //     n(g,2) = n_i(g) - n(g,0) - n(g,1),   n(2,h) = n_j(h) - n(0,h) - n(1,h),
 //     n(2,2) = n_i(2) - n(2,0) - n(2,1).
-// The epilogue scores each pair with the same FP32 mutual information as the
-// sweep kernel and keeps a CTA top list; the count matrix is never written.
+// The epilogue scores each pair with the FP32 mutual information and keeps a
+// CTA top list; the count matrix is never written.
 //
-// Roles (one persistent CTA per SM, TC_THREADS_MP threads):
-//   warps 0, 6, 7, 8 : TMA producers (128-byte K chunks of the A and B row
-//                      blocks); producer p owns the stages s = p (mod
-//                      producers): copies issued from one thread complete
-//                      about one stage at a time
-//   warp 1 : TMEM allocation; lane 0 issues the MMAs and schedules the tiles
-//   warps 2-5 : epilogue (TMEM -> registers -> table -> MI -> top list)
-// Accumulators: two TMEM buffers x two classes x 128 FP32 columns.
-#include "fc_tc.cuh"
+// Two forms (template ENC), as in the order-3 kernel:
+//   ENC = 1: control samples carry the block scale 4096, so one accumulator
+//            holds n_case + 4096 n_ctrl (exact while both classes have at
+//            most 4095 samples); a tile of 128 SNPs i and 112 SNPs j is worked
+//            on by a pair of CTAs (cta_group::2, M = 256, N = 224): each
+//            loads 64 SNPs i and 56 SNPs j and scores its SNPs i against all
+//            112;
+//   ENC = 0: the case and control samples accumulate into two accumulators;
+//            a tile of 64 SNPs i and 56 SNPs j per CTA (M = 128, N = 112).
+// A tile takes 224 TMEM columns and two tiles are in flight.  The scores are
+// those of the order-3 epilogue over 9 cells (t(a, b) = xl[n] - a lg2~(a) - b
+// lg2~(b), counts times a power of two; the error is derived there): |MI32 - MI|
+// <= u (7 ln M + 19 ln 2).
+//
+// What bounds the kernel: with many samples the operands' way from L2 (60 KB a
+// chunk and tile; 12,000 SNPs x 8,192 samples move 20 GB at 14.5 TB/s, the
+// tensor pipe 33 % active), with few the scoring.  40,000 SNPs x 8,192 samples,
+// lists of 2048: 13.1 ms, x 2,048 samples: 7.5 ms.  (The kernel before, byte rows
+// in 128 x 128 tiles of one CTA and four epilogue warps that met at barriers
+// and sorted a shared buffer of candidates, took 37 ms for the first, and 15 of
+// the 16 ms of a search of 12,001 SNPs x 2,987 samples met once, now 1.5: it
+// sorted after nearly every 16 SNPs while its list filled.)
+//
+// TMEM lane 2 i + g holds genotype g of SNP i, columns 2 j + h genotype h of SNP
+// j.  The two lanes of a SNP i take two SNPs j at a time, one each: they
+// exchange the two cells of the other's SNP, and lane g reads its cells with
+// the genotypes of i in the order g, 1 - g (its table of i is swapped alike).
+//
+// Candidates as in the order-3 kernel: a buffer per epilogue warp, merged into
+// the CTA's sorted list under a lock, and a score threshold over all CTAs.
+//
+// Roles (one persistent CTA per SM, 640 threads):
+//   warps 0, 1 : TMA producers (128-byte K chunks, 256 samples, of 128 rows of
+//                the SNPs i and 112 of the SNPs j), warp w owning the stages
+//                s = w (mod 2)
+//   warp 2     : schedules the tiles (ENC 1: in the pair's leader), score
+//                threshold
+//   warp 3     : TMEM allocation; one elected lane (ENC 1: of the pair's
+//                leader) issues the MMAs
+//   warps 4-19 : epilogue, four warps per TMEM lane quarter, each taking every
+//                fourth four SNPs j of a tile
+#include <algorithm>
+
+#include "fc_candidates.cuh"
+#include "fc_ie.cuh"
 
 namespace fc {
 
 namespace {
 
-// ---- data preparation ------------------------------------------------------
+constexpr int T2_PRODUCERS = 2;
+constexpr int T2_EPI_WARP0 = 4;
+constexpr int T2_EPI_WARPS = 16;
+constexpr int T2_PARTS = T2_EPI_WARPS / 4;         // epilogue warps per TMEM lane quarter
+constexpr int T2_EPI_THREADS = 32 * T2_EPI_WARPS;
+constexpr int T2_THREADS = 32 * T2_EPI_WARP0 + T2_EPI_THREADS;
+static_assert(T2_EPI_WARP0 % 4 == 0, "epilogue warp w reads TMEM lane quarter w % 4");
+constexpr int T2_NJ = 56;                          // SNPs j per stage
+constexpr int T2_N = 2 * T2_NJ;                    // their rows
+constexpr int T2_IB = 64;                          // SNPs i per CTA and tile
+constexpr uint32_t T2_STAGE = TC_A_BYTES + (uint32_t)T2_N * TC_BK;
+static_assert(T2_STAGE % 1024 == 0, "swizzled stages");
+constexpr int T2_BUF = 2 * T2_N;                   // TMEM columns of a tile
+constexpr uint32_t T2_SCALE_COL = 2 * T2_BUF;      // TMEM column of scale 1, then of 4096, then of 4
+static_assert(T2_SCALE_COL + 3 * FP4_SCALE_COLS <= TC_TMEM_COLS, "scales behind the accumulators");
+constexpr int T2_WARP_SNPS = 4 * ((2 * T2_NJ / 4 + T2_PARTS - 1) / T2_PARTS);   // SNPs j of a tile per warp (ENC 1)
+static_assert(T2_WARP_SNPS <= 32, "a lane per SNP record");
 
-// E[2s + g][w*128 + b] = 0x38 (e4m3 1.0), or ctrl_byte for the control words
-// w >= W0, if bit b of word w of genotype row g of SNP s is set, else 0;
-// rows of padding SNPs are zero.
-__global__ void k_expand_e4m3(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, int64_t rows, int64_t pitch,
-                              uint8_t *E, uint32_t ctrl_byte)
-{
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= rows * Wt) return;
-    const int64_t row = t / Wt;
-    const int w = (int)(t % Wt);
-    const int64_t s = row >> 1;
-    const int g = (int)(row & 1);
-    uint4 bits = make_uint4(0, 0, 0, 0);
-    if (s < S) bits = X[((size_t)w * 3 + g) * S_pad + s];
-    const uint32_t b32[4] = {bits.x, bits.y, bits.z, bits.w};
-    uint4 *dst = reinterpret_cast<uint4 *>(E + row * pitch + (int64_t)w * 128);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        uint32_t o[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int bit0 = q * 16 + u * 4;
-            const uint32_t word = b32[bit0 >> 5];
-            const int sh = bit0 & 31;
-            uint32_t v = 0;
-            const uint32_t one = w < W0 ? 0x38u : ctrl_byte;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v |= (((word >> (sh + e)) & 1u) ? one : 0u) << (8 * e);
-            o[u] = v;
-        }
-        dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-}
+// ---- data preparation ------------------------------------------------------
 
 // Per SNP and class, how many samples carry genotype 0, 1, 2:
 // marg[s*8 + c*3 + g], c = 0 cases, 1 controls.
@@ -88,31 +107,40 @@ __global__ void k_marginals(const uint4 *X, int64_t S, int64_t S_pad, int W0, in
 
 // ---- the fused tensor-core kernel ------------------------------------------
 
-template <int MODE>
-__global__ void __launch_bounds__(TC_THREADS_MP, 1) k_pairs_tc(const __grid_constant__ CUtensorMap tmap, PairsArgs a)
+template <int MODE, int ENC>
+__global__ void __launch_bounds__(T2_THREADS, 1) k_pairs_tc(const __grid_constant__ CUtensorMap tmapI,
+                                                            const __grid_constant__ CUtensorMap tmapJ, PairsArgs a)
 {
+    constexpr bool PAIR = ENC == 1;                 // a tile per CTA pair
+    constexpr int NJT = PAIR ? 2 * T2_NJ : T2_NJ;   // SNPs j per tile
+    constexpr int SH = PAIR ? 2 : 0;                // counts come times 2^SH: the block scale of the SNPs j
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[TC_MAX_STAGES], bar_empty[TC_MAX_STAGES];
-    __shared__ uint64_t bar_tfull[2], bar_tempty[2], bar_done;
+    __shared__ uint64_t bar_tfull[2], bar_tempty[2], bar_done, bar_epi;
     __shared__ uint32_t tmem_base_slot;
     __shared__ uint64_t bar_sfull[TC_SCHED], bar_sempty[TC_SCHED];
-    __shared__ int sched_tile[TC_SCHED];
+    __shared__ int2 sched_tile[TC_SCHED];   // {I << 16 | J, 1}, {0, 0}: no more tiles
     __shared__ int abort_flag_s;
-    __shared__ int buf_count;
-    __shared__ int epi_stop;
+    __shared__ int list_lock, list_fill;
+    __shared__ int epi_end;                 // the epilogue has ended
+    __shared__ float threshold;             // published_threshold
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int stages = a.stages;
+    const uint32_t crank = PAIR ? cluster_rank() : 0;   // CTA of the pair (0: its leader)
     volatile int *abort_flag = &abort_flag_s;
 
-    uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *stA = smem;
-    uint8_t *stB = smem + (size_t)stages * TC_A_BYTES;
-    float *logtab = reinterpret_cast<float *>(stB + (size_t)stages * TC_B_BYTES);
-    const int lt_floats = (a.M + 1 + 3) & ~3;
-    uint64_t *lrank = reinterpret_cast<uint64_t *>(logtab + lt_floats);
-    float *lscore = reinterpret_cast<float *>(lrank + a.P2);
+    // The x log2 x table first (a constant base saves an addition per read);
+    // then the stages, 1024-byte aligned, the warps' SNP records, the candidate
+    // list and the warps' buffers (ranks before scores).
+    float *xltab = reinterpret_cast<float *>(smem_raw);
+    uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)(xltab + a.M + 1) + 1023) & ~(uintptr_t)1023);
+    uint2 *recs = reinterpret_cast<uint2 *>(smem + (size_t)stages * T2_STAGE);
+    uint64_t *lrank = reinterpret_cast<uint64_t *>(recs + T2_EPI_WARPS * T2_WARP_SNPS);
+    uint64_t *wrank = lrank + a.L;
+    float *lscore = reinterpret_cast<float *>(wrank + T2_EPI_WARPS * TC_WBUF);
+    float *wscore = lscore + a.L;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -121,28 +149,41 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1) k_pairs_tc(const __grid_cons
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bar_tfull[b], 1);
-            mbar_init(&bar_tempty[b], 4);
+            mbar_init(&bar_tempty[b], (PAIR ? 2 : 1) * T2_EPI_WARPS);
         }
         mbar_init(&bar_done, 1);
+        mbar_init(&bar_epi, T2_EPI_WARPS);
         for (int s = 0; s < TC_SCHED; ++s) {
             mbar_init(&bar_sfull[s], 1);
-            // The producers, the MMA thread and the four epilogue warps.
-            mbar_init(&bar_sempty[s], a.producers + 5);
+            // The MMA thread, and the producer and epilogue warps (of both
+            // CTAs of a pair).
+            mbar_init(&bar_sempty[s], 1 + (PAIR ? 2 : 1) * (T2_PRODUCERS + T2_EPI_WARPS));
         }
         abort_flag_s = 0;
-        buf_count = 0;
+        list_lock = 0;
+        list_fill = 0;
+        epi_end = 0;
+        threshold = -FLT_MAX;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tmem_base_slot)),
-                     "r"(TC_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (warp == 3) {
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_slot)),
+                         "r"(TC_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_slot)),
+                         "r"(TC_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
-    for (int i = threadIdx.x; i <= a.M; i += blockDim.x) logtab[i] = a.logtab[i];
+    for (int i = threadIdx.x; i <= a.M; i += blockDim.x) xltab[i] = a.xlogx[i];
     if (MODE == MODE_TOPN) {
-        for (int i = threadIdx.x; i < a.P2; i += blockDim.x) {
+        for (int i = threadIdx.x; i < a.L; i += blockDim.x) {
             lscore[i] = -FLT_MAX;
             lrank[i] = NO_RANK;
         }
@@ -151,313 +192,504 @@ __global__ void __launch_bounds__(TC_THREADS_MP, 1) k_pairs_tc(const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    if (warp >= T2_EPI_WARP0 && warp < T2_EPI_WARP0 + 4) {
+        const uint32_t q = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + T2_SCALE_COL;
+        tmem_fill16(q, FP4_SCALE_ONE);
+        tmem_fill16(q + FP4_SCALE_COLS, FP4_SCALE_4096);
+        tmem_fill16(q + 2 * FP4_SCALE_COLS, FP4_SCALE_4);
+        tmem_wait_st();
+    }
+    tc_fence_before();
+    // Barriers and scales of both CTAs are ready before either uses them.
+    if constexpr (PAIR) cluster_sync(); else __syncthreads();
+    tc_fence_after();
+    const long long wt = a.wait_ticks;
+    const int nk = (a.Wt + 1) / 2;   // K chunks
 
-    const int kc0 = a.W0, kc1 = a.Wt - a.W0;   // 128-sample chunks per class
+    // A consumer's word that it has read a slot of the tile ring.
+    const uint32_t sempty0 = PAIR ? cluster_addr(&bar_sempty[0], 0) : 0;
+    auto slot_read = [&](int slot) {
+        if constexpr (PAIR) mbar_arrive_cluster(sempty0 + 8 * slot);
+        else mbar_arrive(&bar_sempty[slot]);
+    };
 
-    const int prod = tc_producer_of(warp, a.producers);
-    if (prod >= 0) {
+    if (warp < T2_PRODUCERS) {
         // ---------------- TMA producers ----------------
         if (elect_one()) {
-            const int P = a.producers;
             Ring ring;
             int owner = 0;   // producer of stage ring.s
             // Parity of the last fill issued into each owned stage (at most
-            // two: stages prod and prod + P), -1 before the first.
-            int last0 = -1, last1 = -1;
+            // three: stages warp, warp + 2, warp + 4), -1 before the first.
+            int last[3] = {-1, -1, -1};
             auto step = [&]() {
                 ring.next(stages);
-                owner = ring.s == 0 || owner + 1 == P ? 0 : owner + 1;
+                owner = ring.s == 0 || owner + 1 == T2_PRODUCERS ? 0 : owner + 1;
             };
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 const int slot = it % TC_SCHED;
                 const uint32_t sn = (uint32_t)(it / TC_SCHED);
-                if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, a.wait_ticks)) break;
-                const int t = sched_tile[slot];
-                mbar_arrive(&bar_sempty[slot]);
-                if (t < 0) break;
-                const uint32_t tile = a.tiles[t];
-                const int I = (int)(tile >> 16), J = (int)(tile & 0xffff);
-                for (int c = 0; c < 2 && ok; ++c) {
-                    const int nk = c ? kc1 : kc0;
-                    const int xbase = c ? kc0 * TC_BK : 0;
-                    for (int kc = 0; kc < nk; ++kc, step()) {
-                        const int s = ring.s;
-                        if (owner != prod) continue;
-                        if (!mbar_wait(&bar_empty[s], ring.par ^ 1, abort_flag, a.err, a.wait_ticks)) { ok = false; break; }
-                        mbar_expect_tx(&bar_full[s], TC_A_BYTES + TC_B_BYTES);
-                        tma_load_2d(&tmap, &bar_full[s], stA + (size_t)s * TC_A_BYTES, xbase + kc * TC_BK, I * TC_BM);
-                        tma_load_2d(&tmap, &bar_full[s], stB + (size_t)s * TC_B_BYTES, xbase + kc * TC_BK, J * TC_BN);
-                        if (s == prod) last0 = (int)ring.par; else last1 = (int)ring.par;
+                if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt)) { ok = false; break; }
+                const int2 tile = sched_tile[slot];
+                slot_read(slot);
+                if (!tile.y) break;
+                const int I = (int)((uint32_t)tile.x >> 16), J = tile.x & 0xffff;
+                const int rowI = 2 * T2_IB * ((PAIR ? 2 : 1) * I + (int)crank);
+                const int rowJ = 2 * NJT * J + T2_N * (int)crank;
+                for (int kc = 0; kc < nk; ++kc, step()) {
+                    if (owner != warp) continue;
+                    const int s = ring.s;
+                    uint8_t *st = smem + (size_t)s * T2_STAGE;
+                    if (!mbar_wait(&bar_empty[s], ring.par ^ 1, abort_flag, a.err, wt)) { ok = false; break; }
+                    const int x = kc * TC_BK;
+                    if constexpr (PAIR) {
+                        // The leader's barrier counts the bytes of both CTAs.
+                        if (crank == 0) mbar_expect_tx(&bar_full[s], 2 * T2_STAGE);
+                        tma_load_2d_pair(&tmapI, &bar_full[s], st, x, rowI);
+                        tma_load_2d_pair(&tmapJ, &bar_full[s], st + TC_A_BYTES, x, rowJ);
+                    } else {
+                        mbar_expect_tx(&bar_full[s], T2_STAGE);
+                        tma_load_2d(&tmapI, &bar_full[s], st, x, rowI);
+                        tma_load_2d(&tmapJ, &bar_full[s], st + TC_A_BYTES, x, rowJ);
                     }
+                    last[0] = s == warp ? (int)ring.par : last[0];
+                    last[1] = s == warp + T2_PRODUCERS ? (int)ring.par : last[1];
+                    last[2] = s == warp + 2 * T2_PRODUCERS ? (int)ring.par : last[2];
                 }
             }
-            // Let the last copies into the stages this producer owns land
-            // before the CTA can exit (earlier ones were consumed).
-            for (int q = 0; q < 2; ++q) {
-                const int s = prod + q * P;
-                const int par = q ? last1 : last0;
-                if (s >= stages || par < 0) continue;
-                long long t0 = clock64();
-                while (!mbar_try(&bar_full[s], (uint32_t)par) && clock64() - t0 < WAIT_BUDGET) {}
+            // Let the last copies into the owned stages land before the CTA
+            // can exit (earlier ones were consumed).  A pair's copies complete
+            // on its leader's barriers, and neither CTA exits before the other
+            // (the cluster barrier below); where a wait ran out, the second
+            // CTA allows its own copies a millisecond.
+            if (crank == 0) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int s = warp + q * T2_PRODUCERS;
+                    if (s >= stages || last[q] < 0) continue;
+                    const long long t0 = clock64();
+                    while (!mbar_try(&bar_full[s], (uint32_t)last[q]) && clock64() - t0 < WAIT_BUDGET) {}
+                }
+            } else if (!ok) {
+                const long long t0 = clock64();
+                while (clock64() - t0 < 2000000) {}
             }
         }
-    } else if (warp == 1) {
-        if (elect_one()) {
+    } else if (warp == 2) {
+        // ---------------- scheduler, score threshold ----------------
+        // Lane 0 hands out the tiles; while the ring is full the warp renews
+        // the threshold.
+        const uint32_t peer_tile = PAIR ? cluster_addr(&sched_tile[0], 1) : 0;
+        const uint32_t peer_sfull = PAIR ? cluster_addr(&bar_sfull[0], 1) : 0;
+        unsigned pause = 500;
+        bool done = false;   // all tiles are handed out (the threshold is renewed to the epilogue's end)
+        long long t0 = clock64();
+        for (int it = 0;;) {
+            const int slot = it % TC_SCHED;
+            const uint32_t sn = (uint32_t)(it / TC_SCHED);
+            int ready = 0;   // 1: a tile was handed out, 2: no tile is left
+            if (!done && crank == 0 && lane == 0 && mbar_try(&bar_sempty[slot], (sn & 1) ^ 1)) {
+                const int t = atomicAdd(a.tile_counter, 1);
+                const bool end = t >= a.ntiles;
+                const int2 tile = end ? make_int2(0, 0) : make_int2((int)a.tiles[t], 1);
+                sched_tile[slot] = tile;
+                mbar_arrive(&bar_sfull[slot]);
+                if constexpr (PAIR) cluster_post2(peer_tile + 8 * slot, peer_sfull + 8 * slot, tile.x, tile.y);
+                ready = end ? 2 : 1;
+            }
+            ready = __shfl_sync(FULL, ready, 0);
+            done = done || ready == 2;
+            if (ready == 1) {
+                ++it;
+                t0 = clock64();
+                continue;
+            }
+            int stop = 0;
+            if (lane == 0) {
+                if (!done && crank == 0 && clock64() - t0 > wt) {
+                    *abort_flag = 1;
+                    atomicOr(a.err, ERR_TIMEOUT);
+                }
+                stop = *abort_flag || *(volatile int *)&epi_end;
+            }
+            if (__shfl_sync(FULL, stop, 0)) break;
+            if (MODE == MODE_TOPN) {
+                const float thr = published_threshold(a.pub, (int)gridDim.x, a.pub_r, lane);
+                if (lane == 0) *(volatile float *)&threshold = thr;
+            }
+            __nanosleep(pause);
+            pause = min(pause + pause / 2, 4000u);
+        }
+    } else if (warp == 3) {
+        if (crank == 0 && elect_one()) {
             // ---------------- MMA issue ----------------
-            const uint32_t idesc = idesc_e4m3_f32(TC_BM, TC_BN);
-            const uint64_t descA = smem_desc_sw128(smem_u32(stA)), descB = smem_desc_sw128(smem_u32(stB));
+            const uint32_t idesc = idesc_mxf4(PAIR ? 2 * TC_BM : TC_BM, PAIR ? 2 * T2_N : T2_N);
+            const uint64_t descI = smem_desc_sw128(smem_u32(smem)), descJ = smem_desc_sw128(smem_u32(smem + TC_A_BYTES));
+            const uint32_t one = tmem_base + T2_SCALE_COL, sj = one + (PAIR ? 2 * FP4_SCALE_COLS : 0);
             Ring ring;
             bool ok = true;
-            // This thread also schedules the tiles, TC_LOOKAHEAD ahead of the
-            // one it consumes (another lane of this warp spinning on the ring
-            // delayed the MMA issue).
-            int published = 0;
-            bool sched_done = false;
-            auto publish = [&](int k) -> bool {
-                const int pslot = k % TC_SCHED;
-                const uint32_t psn = (uint32_t)(k / TC_SCHED);
-                if (!mbar_wait(&bar_sempty[pslot], (psn & 1) ^ 1, abort_flag, a.err, a.wait_ticks)) return false;
-                int t = -1;
-                if (!sched_done) {
-                    t = atomicAdd(a.tile_counter, 1);
-                    if (t >= a.ntiles) { t = -1; sched_done = true; }
-                }
-                sched_tile[pslot] = t;
-                mbar_arrive(&bar_sfull[pslot]);
-                return true;
-            };
-            for (; published < TC_LOOKAHEAD && ok; ++published) ok = publish(published);
+            const int Wt = a.Wt, W0 = a.W0;
             for (int it = 0; ok; ++it) {
-                if (!(ok = publish(published++))) break;
                 const int slot = it % TC_SCHED;
                 const uint32_t sn = (uint32_t)(it / TC_SCHED);
-                if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, a.wait_ticks)) break;
-                const int t = sched_tile[slot];
+                if (!mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt)) break;
+                const int more = sched_tile[slot].y;
                 mbar_arrive(&bar_sempty[slot]);
-                if (t < 0) break;
+                if (!more) break;
                 const int b = it & 1;
                 const uint32_t u = (uint32_t)(it >> 1);
-                if (!mbar_wait(&bar_tempty[b], (u & 1) ^ 1, abort_flag, a.err, a.wait_ticks)) break;
+                if (!mbar_wait(&bar_tempty[b], (u & 1) ^ 1, abort_flag, a.err, wt)) break;
                 tc_fence_after();
-                for (int c = 0; c < 2 && ok; ++c) {
-                    const int nk = c ? kc1 : kc0;
-                    const uint32_t d = tmem_base + (uint32_t)(b * 256 + c * 128);
-                    for (int kc = 0; kc < nk; ++kc, ring.next(stages)) {
-                        const int s = ring.s;
-                        if (!mbar_wait(&bar_full[s], ring.par, abort_flag, a.err, a.wait_ticks)) { ok = false; break; }
-                        tc_fence_after();
-                        const uint64_t ad = descA + (uint64_t)s * (TC_A_BYTES >> 4);
-                        const uint64_t bd = descB + (uint64_t)s * (TC_B_BYTES >> 4);
-#pragma unroll
-                        for (int kk = 0; kk < TC_BK / 32; ++kk)
-                            mma_e4m3(d, ad + kk * 2, bd + kk * 2, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-                        mma_commit(&bar_empty[s]);
+                const uint32_t d0 = tmem_base + (uint32_t)(b * T2_BUF);
+                for (int kc = 0; kc < nk; ++kc, ring.next(stages)) {
+                    const int s = ring.s;
+                    if (!mbar_wait(&bar_full[s], ring.par, abort_flag, a.err, wt)) {
+                        ok = false;
+                        break;
                     }
+                    tc_fence_after();
+                    const uint64_t id = descI + (uint64_t)s * (T2_STAGE >> 4);
+                    const uint64_t jd = descJ + (uint64_t)s * (T2_STAGE >> 4);
+                    // Two words of 128 samples (K = 64 twice): cases, then
+                    // controls (ENC 0: into the second accumulator; ENC 1: with
+                    // scale 4096).
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int w = 2 * kc + h;
+                        if (w < Wt) {
+                            const bool ctrl = w >= W0;
+                            const bool first = w == 0 || (!PAIR && w == W0);
+                            const uint32_t d = d0 + (!PAIR && ctrl ? T2_N : 0);
+                            const uint32_t si = one + (PAIR && ctrl ? FP4_SCALE_COLS : 0);
+                            if constexpr (PAIR) {
+                                mma_mxf4_pair(d, id + 4 * h, jd + 4 * h, idesc, si, sj, first ? 0u : 1u);
+                                mma_mxf4_pair(d, id + 4 * h + 2, jd + 4 * h + 2, idesc, si, sj, 1u);
+                            } else {
+                                mma_mxf4(d, id + 4 * h, jd + 4 * h, idesc, si, sj, first ? 0u : 1u);
+                                mma_mxf4(d, id + 4 * h + 2, jd + 4 * h + 2, idesc, si, sj, 1u);
+                            }
+                        }
+                    }
+                    if constexpr (PAIR) mma_commit_pair(&bar_empty[s]); else mma_commit(&bar_empty[s]);
                 }
-                if (ok) mma_commit(&bar_tfull[b]);
+                if (ok) {
+                    if constexpr (PAIR) mma_commit_pair(&bar_tfull[b]); else mma_commit(&bar_tfull[b]);
+                }
             }
             // All MMAs issued by this thread complete before TMEM is released.
-            mma_commit(&bar_done);
-            long long t0 = clock64();
+            if constexpr (PAIR) mma_commit_pair(&bar_done); else mma_commit(&bar_done);
+            const long long t0 = clock64();
             while (!mbar_try(&bar_done, 0) && clock64() - t0 < WAIT_BUDGET) {}
         }
-    } else if (warp >= 2 && warp < 6) {
+    } else {
         // ---------------- epilogue ----------------
-        const int tid = threadIdx.x - 64;           // 0..127
-        const int quarter = warp & 3;               // TMEM lanes 32*quarter ..
-        const int row = quarter * 32 + lane;        // tile row = 2*i_l + g
-        const int i_l = row >> 1;
-        const int g = row & 1;
+        const int ew = warp - T2_EPI_WARP0;
+        const int quarter = warp & 3;
+        const int part = ew >> 2;                          // four SNPs j x = part, part + 4, .. of a tile
+        const int g = lane & 1;                            // genotype of this lane's row
+        const uint32_t tempty0 = PAIR ? cluster_addr(&bar_tempty[0], 0) : 0;
         const int L = a.L;
-        const int Bcap = a.Bcap;
+        float *ws = wscore + ew * TC_WBUF;
+        uint64_t *wr = wrank + ew * TC_WBUF;
+        uint2 *rec = recs + ew * T2_WARP_SNPS;
+        const int S = (int)a.S;
+        const float invN = a.invN * (1.f / a.scale);   // (exact: the scale is a power of two)
+        const bool whole = a.rank_begin == 0 && a.rank_end >= a.pair_base;
+        uint32_t all[3];   // genotype counts of SNP 0, whose sum is the classes
+        unpack_marg(a.marg4[0], all);
+        const uint32_t samples = all[0] + all[1] + all[2];
+        // This warp's candidates, and the CTA list's last entry when the
+        // warp last merged: a candidate has to beat it.
+        int cnt = 0;
         float thr_s = -FLT_MAX;
         uint64_t thr_r = NO_RANK;
+        bool waited = false;
+        // The least score of a candidate by now: that of the list's last entry
+        // (which only rises; a racy read is a score it had at some time), and
+        // the one that enough pairs of all CTAs are known to reach.
+        auto floor_score = [&]() -> float {
+            return fmaxf(*(volatile float *)(lscore + L - 1), *(volatile float *)&threshold);
+        };
+        auto known = [&]() -> bool { return *(volatile float *)&threshold > -FLT_MAX; };
+        auto merge = [&]() {
+            // Sorted outside the lock, against the list's last score then.
+            const float racy = *(volatile float *)(lscore + L - 1);
+            const bool later = racy > thr_s;
+            int m = sort_candidates(ws, wr, cnt, later ? racy : thr_s, later ? NO_RANK : thr_r, lane);
+            cnt = 0;
+            if (m == 0) return;
+            bool held = true;
+            if (lane == 0) {
+                const long long t0 = clock64();
+                while (atomicCAS(&list_lock, 0, 1) != 0) {
+                    __nanosleep(100);
+                    if (clock64() - t0 > WAIT_BUDGET) {
+                        *abort_flag = 1;
+                        atomicOr(a.err, ERR_TIMEOUT);
+                        held = false;
+                        break;
+                    }
+                }
+                __threadfence_block();
+            }
+            held = __shfl_sync(FULL, held, 0);
+            if (held) {
+                // (What the threshold has passed meanwhile is left out.)
+                const float now = floor_score();
+                m = __popc(__ballot_sync(FULL, lane < m && ws[lane] >= now)) +
+                    __popc(__ballot_sync(FULL, lane + 32 < m && ws[lane + 32] >= now));
+                const int fill = merge_candidates(lscore, lrank, L, list_fill, ws, wr, m, lane);
+                if (lane == 0) list_fill = fill;
+                thr_s = lscore[L - 1];
+                thr_r = lrank[L - 1];
+                __threadfence_block();
+                __syncwarp();
+                if (lane == 0) {
+                    if (lrank[a.pub_m - 1] != NO_RANK)
+                        *(volatile int *)(a.pub + blockIdx.x) = ordered_int(lscore[a.pub_m - 1]);
+                    __threadfence_block();
+                    atomicExch(&list_lock, 0);
+                }
+            }
+            __syncwarp();
+            if (waited || L < TC_LONG_LIST) return;
+            // A merge into a long list costs microseconds: after its first
+            // one a warp waits a little for the threshold over all CTAs.
+            waited = true;
+            const long long t0 = clock64();
+            while (clock64() - t0 < TC_FIRST_THRESHOLD_TICKS && !known()) __nanosleep(200);
+            __syncwarp();
+        };
+        // hs + (t(c), t(d)) for two packed cells c, d (a | b << 16, times 2^SH).
+        auto add_terms = [&](F2 hs, uint32_t c, uint32_t d) -> F2 {
+            // a 2^SH under the exponent of 2^(23 - SH) is 2^(23 - SH) + a, and -a q
+            // = 2^(23 - SH) q minus q times that, exactly (q the scale, a power of
+            // two).  The logarithm's argument is a q + 1e-30, that is a q, or
+            // 1e-30 at a = 0, whose finite logarithm times 0 adds nothing.
+            constexpr uint32_t EXP = SH == 2 ? 0x4A000000u : 0x4B000000u;
+            constexpr float BIG = SH == 2 ? 2097152.f : 8388608.f;
+            const F2 minus = f2(-1.f, -1.f), tiny = f2(1e-30f, 1e-30f);
+            const F2 mscale = f2(-a.scale, -a.scale), big = f2(BIG * a.scale, BIG * a.scale);
+            const F2 na = f2_fma(f2(__uint_as_float(__byte_perm(c, EXP, 0x7610)), __uint_as_float(__byte_perm(d, EXP, 0x7610))),
+                                 mscale, big);
+            const F2 nb = f2_fma(f2(__uint_as_float(__byte_perm(c, EXP, 0x7632)), __uint_as_float(__byte_perm(d, EXP, 0x7632))),
+                                 mscale, big);
+            const float2 aa = f2_split(f2_fma(na, minus, tiny)), bb = f2_split(f2_fma(nb, minus, tiny));
+            // The byte offset of the table entry of n = a + b.
+            auto xl = [&](uint32_t x) {
+                return *reinterpret_cast<const float *>(reinterpret_cast<const char *>(xltab) +
+                                                        __dp2a_lo(x, SH == 2 ? 0x00000101u : 0x00000404u, 0u));
+            };
+            F2 t = f2_fma(na, f2(lg2_approx(aa.x), lg2_approx(aa.y)), f2(xl(c), xl(d)));
+            t = f2_fma(nb, f2(lg2_approx(bb.x), lg2_approx(bb.y)), t);
+            return f2_add(hs, t);
+        };
+        bool ok = true;
         for (int it = 0;; ++it) {
             const int slot = it % TC_SCHED;
             const uint32_t sn = (uint32_t)(it / TC_SCHED);
-            const bool ok = mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, a.wait_ticks);
-            const int t = ok ? sched_tile[slot] : -1;
-            if (ok) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bar_sempty[slot]);
-            }
+            ok = mbar_wait(&bar_sfull[slot], sn & 1, abort_flag, a.err, wt);
+            ok = __all_sync(FULL, ok);
+            if (!ok) break;
+            const int2 tile = sched_tile[slot];
+            __syncwarp();
+            if (lane == 0) slot_read(slot);
+            if (!tile.y) break;
             const int b = it & 1;
             const uint32_t u = (uint32_t)(it >> 1);
-            if (t >= 0) mbar_wait(&bar_tfull[b], u & 1, abort_flag, a.err, a.wait_ticks);
-            // One stop decision for all four epilogue warps (they meet at
-            // named barriers, which have no timeout); t is the same for all.
-            epi_bar();
-            if (tid == 0) epi_stop = *abort_flag;
-            epi_bar();
-            if (epi_stop || t < 0) break;
-            tc_fence_after();
-            const uint32_t tile = a.tiles[t];
-            const int I = (int)(tile >> 16), J = (int)(tile & 0xffff);
-            const int64_t i = (int64_t)I * TC_SNPS + i_l;
-            uint32_t mi[2][3] = {{0, 0, 0}, {0, 0, 0}};
-            if (i < a.S) {
-                const uint4 m4 = *reinterpret_cast<const uint4 *>(a.marg + i * 8);
-                mi[0][0] = m4.x & 0xffff; mi[0][1] = m4.x >> 16; mi[0][2] = m4.y & 0xffff;
-                mi[1][0] = m4.y >> 16;    mi[1][1] = m4.z & 0xffff; mi[1][2] = m4.z >> 16;
+            // Tile data that does not depend on the accumulators, loaded
+            // while the tile's MMAs may still run.
+            const int I = (int)((uint32_t)tile.x >> 16), j0 = (tile.x & 0xffff) * NJT;
+            const int iw = T2_IB * ((PAIR ? 2 : 1) * I + (int)crank) + quarter * 16;   // this warp's first SNP i
+            const int i = iw + (lane >> 1);
+            const bool iv = i < S;
+            // This warp's fours of SNPs j, x = part + 4 r, r0 <= r < r1, that
+            // hold some valid pair: their last j after the warp's first i,
+            // their first j before S.
+            const int xlo = j0 + 3 > iw ? 0 : (iw - j0 - 3) / 4 + 1;
+            const int xhi = iw < S ? min(NJT / 4, (S - j0 + 3) / 4) : 0;
+            const int r0 = xlo > part ? (xlo - part + T2_PARTS - 1) / T2_PARTS : 0;
+            const int r1 = xhi > part ? (xhi - part + T2_PARTS - 1) / T2_PARTS : 0;
+            // Every cell has to be a count (it is a table offset): where i is
+            // no SNP its rows are zero, those of a SNP of genotype 2
+            // throughout.  Genotypes of i in the order g, 1 - g.
+            uint32_t Ti[3] = {0, 0, samples << SH};
+            uint64_t rb = 0;   // rank of (i, j) less j
+            if (iv) {
+                uint32_t T[3];
+                unpack_marg(a.marg4[i], T);
+                Ti[0] = (g ? T[1] : T[0]) << SH;
+                Ti[1] = (g ? T[0] : T[1]) << SH;
+                Ti[2] = T[2] << SH;
+                const uint64_t si = (uint64_t)(S - i);
+                rb = a.pair_base - si * (si - 1) / 2 - (uint64_t)i - 1;
             }
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256);
-            for (int ch = 0; ch < TC_BN / 32; ++ch) {
-                uint32_t v0[32], v1[32];
-                tmem_ld32(taddr + ch * 32, v0);
-                tmem_ld32(taddr + 128 + ch * 32, v1);
-                tmem_wait_ld();
-                tmem_regs_after_wait(v0);
-                tmem_regs_after_wait(v1);
-                if (ch == TC_BN / 32 - 1) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&bar_tempty[b]);
+            __syncwarp();
+            if (lane < T2_WARP_SNPS) {
+                // Counts of genotypes 0 and 1 of SNP j, a lane per SNP; no
+                // samples where j is no SNP (its rows are zero).
+                const int j = j0 + 4 * (part + T2_PARTS * (lane >> 2)) + (lane & 3);
+                uint32_t T[3] = {0, 0, 0};
+                if (j < S) unpack_marg(a.marg4[j], T);
+                rec[lane] = make_uint2(T[0] << SH, T[1] << SH);
+            }
+            ok = mbar_wait(&bar_tfull[b], u & 1, abort_flag, a.err, wt);
+            ok = __all_sync(FULL, ok);   // (also orders the records)
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * T2_BUF + 8 * part);
+            auto release = [&]() {
+                // This warp's last read of the buffer.
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if constexpr (PAIR) mbar_arrive_cluster(tempty0 + 8 * b);
+                    else mbar_arrive(&bar_tempty[b]);
                 }
-                float sc[8];
-                uint64_t rk[8];
-                bool val[8];
+            };
+            // Read again whenever a pair passes what was read before.
+            float thr = MODE == MODE_TOPN ? floor_score() : 0.f;
+            const uint32_t after = iv ? (uint32_t)(S - 1 - i) : 0u;   // SNPs j after i
+            if (r0 >= r1) release();
+            for (int r = r0; r < r1; ++r) {
+                uint32_t v[8];
+                {
+                    uint32_t w[8];
+                    tmem_ld8(taddr + 8 * T2_PARTS * r, v);
+                    if constexpr (!PAIR) tmem_ld8(taddr + T2_N + 8 * T2_PARTS * r, w);
+                    tmem_wait_ld();
+                    tmem_regs_after_wait(v);
+                    if constexpr (!PAIR) tmem_regs_after_wait(w);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    // This thread scores j = 2q + g of the chunk; its partner
-                    // lane (the other genotype row of SNP i) scores 2q + 1 - g.
-                    uint32_t own[2][2], oth[2][2];
+                    for (int x = 0; x < 8; ++x) {
+                        if constexpr (PAIR) v[x] = unpack_enc(v[x]);
+                        else v[x] = pack_exact(v[x], w[x]);
+                    }
+                }
+                if (r + 1 == r1) release();
+                // SNPs 2 e and 2 e + 1 of the four: this lane's is 2 e + g.
+                float score[2];
+                const int j = j0 + 4 * (part + T2_PARTS * r) + g;   // (that of e = 0)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const uint2 Tj = rec[4 * r + 2 * e + g];
+                    uint32_t R[2][2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const uint32_t s0 = g ? v0[4 * q + h] : v0[4 * q + 2 + h];
-                        const uint32_t s1 = g ? v1[4 * q + h] : v1[4 * q + 2 + h];
-                        own[0][h] = g ? v0[4 * q + 2 + h] : v0[4 * q + h];
-                        own[1][h] = g ? v1[4 * q + 2 + h] : v1[4 * q + h];
-                        oth[0][h] = __shfl_xor_sync(FULL, s0, 1);
-                        oth[1][h] = __shfl_xor_sync(FULL, s1, 1);
+                        R[0][h] = g ? v[4 * e + 2 + h] : v[4 * e + h];
+                        R[1][h] = __shfl_xor_sync(FULL, g ? v[4 * e + h] : v[4 * e + 2 + h], 1);
                     }
-                    const int jl = ch * 16 + 2 * q + g;
-                    const int64_t j = (int64_t)J * TC_SNPS + jl;
-                    // Lexicographic rank of (i, j): C(S,2) - C(S-i,2) + (j-i-1).
-                    const uint64_t si = (uint64_t)(a.S - i);
-                    const uint64_t rank0 = a.pair_base - si * (si - 1) / 2 + (uint64_t)(j - i - 1);
-                    const bool valid = i < a.S && j < a.S && i < j && rank0 >= a.rank_begin && rank0 < a.rank_end;
-                    uint32_t mj[2][3] = {{0, 0, 0}, {0, 0, 0}};
-                    if (j < a.S) {
-                        const uint4 m4 = *reinterpret_cast<const uint4 *>(a.marg + j * 8);
-                        mj[0][0] = m4.x & 0xffff; mj[0][1] = m4.x >> 16; mj[0][2] = m4.y & 0xffff;
-                        mj[1][0] = m4.y >> 16;    mj[1][1] = m4.z & 0xffff; mj[1][2] = m4.z >> 16;
-                    }
-                    uint32_t cell[2][9];
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const uint32_t n00 = f2u_exact(g ? oth[c][0] : own[c][0]);
-                        const uint32_t n01 = f2u_exact(g ? oth[c][1] : own[c][1]);
-                        const uint32_t n10 = f2u_exact(g ? own[c][0] : oth[c][0]);
-                        const uint32_t n11 = f2u_exact(g ? own[c][1] : oth[c][1]);
-                        const uint32_t n02 = mi[c][0] - n00 - n01;
-                        const uint32_t n12 = mi[c][1] - n10 - n11;
-                        const uint32_t n20 = mj[c][0] - n00 - n10;
-                        const uint32_t n21 = mj[c][1] - n01 - n11;
-                        const uint32_t n22 = mi[c][2] - n20 - n21;
-                        cell[c][0] = n00; cell[c][1] = n01; cell[c][2] = n02;
-                        cell[c][3] = n10; cell[c][4] = n11; cell[c][5] = n12;
-                        cell[c][6] = n20; cell[c][7] = n21; cell[c][8] = n22;
-                    }
-                    float hsum = 0.f;
-                    if (valid) {
-#pragma unroll
-                        for (int x = 0; x < 9; ++x) {
-                            // Clamped so that no index can leave the table.
-                            const uint32_t lt = (uint32_t)a.M;
-                            const uint32_t ca = min(cell[0][x], lt), cb = min(cell[1][x], lt);
-                            const float ln = logtab[min(ca + cb, lt)];
-                            hsum = fmaf((float)ca, ln - logtab[ca], hsum);
-                            hsum = fmaf((float)cb, ln - logtab[cb], hsum);
-                        }
-                    }
-                    const float score = fmaf(-hsum, a.invN, a.hy);
-                    const uint64_t rank = valid ? rank0 : NO_RANK;
-                    sc[q] = score;
-                    rk[q] = rank;
-                    val[q] = valid;
-                    if (MODE == MODE_DUMP && valid) {
-                        if (a.dump_scores) a.dump_scores[i * a.S + j] = score;
+                    const uint32_t c02 = Ti[0] - R[0][0] - R[0][1], c12 = Ti[1] - R[1][0] - R[1][1];
+                    const uint32_t c20 = Tj.x - R[0][0] - R[1][0], c21 = Tj.y - R[0][1] - R[1][1];
+                    const uint32_t c22 = Ti[2] - c20 - c21;
+                    F2 hs[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+                    hs[0] = add_terms(hs[0], R[0][0], R[0][1]);
+                    hs[1] = add_terms(hs[1], R[1][0], R[1][1]);
+                    hs[0] = add_terms(hs[0], c02, c12);
+                    hs[1] = add_terms(hs[1], c20, c21);
+                    hs[0] = add_terms(hs[0], c22, 0u);   // (a cell of no sample adds 0)
+                    const float2 h2 = f2_split(f2_add(hs[0], hs[1]));
+                    score[e] = fmaf(-LN2F * (h2.x + h2.y), invN, a.hy);
+                    if (MODE == MODE_DUMP && (uint32_t)(j + 2 * e - i - 1) < after) {
+                        const size_t at = (size_t)i * (size_t)S + (size_t)(j + 2 * e);
+                        if (a.dump_scores) a.dump_scores[at] = score[e];
                         if (a.dump_tables) {
-                            uint32_t *o = a.dump_tables + (size_t)(i * a.S + j) * 18;
+                            const uint32_t c[9] = {R[g][0], R[g][1], g ? c12 : c02, R[1 - g][0], R[1 - g][1], g ? c02 : c12,
+                                                   c20, c21, c22};
+                            uint32_t *o = a.dump_tables + at * 18;
 #pragma unroll
-                            for (int x = 0; x < 9; ++x) { o[2 * x] = cell[0][x]; o[2 * x + 1] = cell[1][x]; }
+                            for (int x = 0; x < 9; ++x) {
+                                o[2 * x] = (c[x] & 0xffffu) >> SH;
+                                o[2 * x + 1] = c[x] >> (16 + SH);
+                            }
                         }
                     }
                 }
                 if (MODE == MODE_TOPN) {
-                    // Merge the buffer into the list when a full chunk might not fit.
-                    // Every thread reads the buffer fill before any thread of
-                    // this round adds to it, so that all take the same branch.
-                    epi_bar();
-                    const int fill_now = buf_count;
-                    epi_bar();
-                    if (fill_now > Bcap - 1024) {
-                        const int nb = buf_count;
-                        for (int x = L + nb + tid; x < a.P2; x += 128) { lscore[x] = -FLT_MAX; lrank[x] = NO_RANK; }
-                        epi_bitonic_desc(lscore, lrank, a.P2, tid);
-                        if (tid == 0) {
-                            buf_count = 0;
-                            if (lrank[L - 1] != NO_RANK) atomicMax(a.gthr, ordered_int(lscore[L - 1]));
-                        }
-                        epi_bar();
-                    }
-                    thr_s = lscore[L - 1];
-                    thr_r = lrank[L - 1];
-                    const float gthr = from_ordered(*(volatile int *)a.gthr);
+                    // Few pairs reach the threshold: one vote for both scores,
+                    // and ranks only after it.
+                    bool near[2];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const bool cand = val[q] && sc[q] >= gthr && better(sc[q], rk[q], thr_s, thr_r);
-                        const unsigned m = __ballot_sync(FULL, cand);
-                        if (m) {
-                            int base = 0;
-                            if (lane == 0) base = atomicAdd(&buf_count, __popc(m));
-                            base = __shfl_sync(FULL, base, 0);
+                    for (int e = 0; e < 2; ++e) near[e] = (uint32_t)(j + 2 * e - i - 1) < after && score[e] >= thr;
+                    if (__any_sync(FULL, near[0] || near[1])) {
+                        thr = floor_score();
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const uint64_t rank = rb + (uint64_t)(j + 2 * e);
+                            const bool cand = near[e] && score[e] >= thr && (whole || (rank >= a.rank_begin && rank < a.rank_end)) &&
+                                              better(score[e], rank, thr_s, thr_r);
+                            const unsigned mk = __ballot_sync(FULL, cand);
+                            if (mk == 0) continue;
                             if (cand) {
-                                const int slot = L + base + __popc(m & ((1u << lane) - 1u));
-                                lscore[slot] = sc[q];
-                                lrank[slot] = rk[q];
+                                const int p = cnt + __popc(mk & ((1u << lane) - 1u));
+                                ws[p] = score[e];
+                                wr[p] = rank;
                             }
+                            cnt += __popc(mk);
+                            __syncwarp();
+                            if (cnt > TC_WBUF - 32) merge();
                         }
                     }
                 }
             }
         }
         if (MODE == MODE_TOPN) {
-            epi_bar();
-            const int nb = buf_count;
-            for (int x = L + nb + tid; x < a.P2; x += 128) { lscore[x] = -FLT_MAX; lrank[x] = NO_RANK; }
-            epi_bitonic_desc(lscore, lrank, a.P2, tid);
-            for (int x = tid; x < L; x += 128) {
+            // The CTA's list (after a wait that ran out, as far as it got: the
+            // search fails).
+            if (ok) merge();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_epi);
+            mbar_wait(&bar_epi, 0, abort_flag, a.err, wt);
+            for (int x = threadIdx.x - 32 * T2_EPI_WARP0; x < L; x += T2_EPI_THREADS) {
                 a.list_score[(size_t)blockIdx.x * L + x] = lscore[x];
                 a.list_rank[(size_t)blockIdx.x * L + x] = lrank[x];
             }
         }
+        if (ew == 0 && lane == 0) *(volatile int *)&epi_end = 1;
     }
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if constexpr (PAIR) {
+        // Neither CTA of a pair leaves while the other may still signal it or
+        // an MMA may read its shared memory (the leader has waited for its
+        // last commit above).
+        if (crank == 1 && threadIdx.x == 0) {
+            const long long t0 = clock64();
+            while (!mbar_try(&bar_done, 0) && clock64() - t0 < WAIT_BUDGET) {}
+        }
+        __syncwarp();
+        cluster_sync();
+    }
+    if (warp == 3) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
-                     : "memory");
+        if constexpr (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
+                         : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS)
+                         : "memory");
     }
 }
 
 }  // namespace
 
-size_t pairs_smem_bytes(int stages, int M, int P2)
+int pairs_rows_i(int enc) { return (enc ? 2 : 1) * T2_IB; }
+int pairs_rows_j(int enc) { return (enc ? 2 : 1) * T2_NJ; }
+int pairs_block_rows() { return T2_N; }
+
+size_t pairs_smem_bytes(int stages, int M, int L)
 {
-    return 1024 + (size_t)stages * (TC_A_BYTES + TC_B_BYTES) + (size_t)((M + 1 + 3) & ~3) * 4 +
-           (size_t)P2 * (8 + 4);
+    // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
+    return 2048 + (size_t)(M + 1) * 4 + (size_t)stages * T2_STAGE + (size_t)T2_EPI_WARPS * T2_WARP_SNPS * 8 +
+           (size_t)(L + T2_EPI_WARPS * TC_WBUF) * (8 + 4);
 }
 
-cudaError_t launch_expand_e4m3(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, int64_t rows, int64_t pitch,
-                               uint8_t *E, uint8_t ctrl_byte, cudaStream_t st)
+int pairs_stages(int M, int L, size_t smem_cap)
 {
-    const int64_t n = rows * Wt;
-    k_expand_e4m3<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(X, S, S_pad, W0, Wt, rows, pitch, E, ctrl_byte);
-    return cudaGetLastError();
+    for (int st = TC_MAX_STAGES; st >= 2; --st)
+        if (pairs_smem_bytes(st, M, L) <= smem_cap) return st;
+    return 0;
 }
 
 cudaError_t launch_marginals(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, uint16_t *marg,
@@ -467,17 +699,34 @@ cudaError_t launch_marginals(const uint4 *X, int64_t S, int64_t S_pad, int W0, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_pairs_tc(int mode, const CUtensorMap &tmap, const PairsArgs &a, int grid, cudaStream_t st)
+cudaError_t launch_pairs_tc(int mode, const CUtensorMap &tmapI, const CUtensorMap &tmapJ, const PairsArgs &a, int grid,
+                            cudaStream_t st)
 {
-    const size_t bytes = pairs_smem_bytes(a.stages, a.M, a.P2);
-    void *fn = mode == MODE_TOPN ? reinterpret_cast<void *>(&k_pairs_tc<MODE_TOPN>)
-                                 : reinterpret_cast<void *>(&k_pairs_tc<MODE_DUMP>);
+    const size_t bytes = pairs_smem_bytes(a.stages, a.M, a.L) - 1024;
+    void *fn = mode == MODE_TOPN ? (a.enc ? reinterpret_cast<void *>(&k_pairs_tc<MODE_TOPN, 1>)
+                                          : reinterpret_cast<void *>(&k_pairs_tc<MODE_TOPN, 0>))
+                                 : (a.enc ? reinterpret_cast<void *>(&k_pairs_tc<MODE_DUMP, 1>)
+                                          : reinterpret_cast<void *>(&k_pairs_tc<MODE_DUMP, 0>));
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    CUtensorMap map = tmap;
+    CUtensorMap mI = tmapI, mJ = tmapJ;
     PairsArgs args = a;
-    void *params[] = {&map, &args};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(TC_THREADS_MP), params, bytes, st);
+    void *params[] = {&mI, &mJ, &args};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(T2_THREADS);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    if (a.enc) {
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
 }  // namespace fc

@@ -356,15 +356,15 @@ float score_error_bound(int k, int64_t M)
     // N H(Y|X) <= N ln 2); the final scaling and subtraction <= 3u ln 2.
     // Divided by N: |MI32 - MI| <= u (2 ln M + (2*3^k + 6) ln 2).  The
     // orders 4-6 tensor-core epilogue's x ln x form has the smaller bound
-    // u (3 ln M + (3^k + 4) ln 2) for every M used here; the order-3 one,
-    // whose n log2 n terms come from the hardware logarithm (relative error
-    // 2^-22 plus 2^-22 absolute), u (7 ln M + 37 ln 2).  The larger, doubled
-    // for margin.
+    // u (3 ln M + (3^k + 4) ln 2) for every M used here; those of
+    // orders 2 and 3, whose class terms come from the hardware logarithm
+    // (relative error 2^-22 plus 2^-22 absolute), u (7 ln M + 19 ln 2) and u
+    // (7 ln M + 37 ln 2).  The larger, doubled for margin.
     const double u = std::ldexp(1.0, -24);
     const double terms = 2.0 * pow3(k);
     const double lm = std::log((double)std::max<int64_t>(M, 2));
     double e = u * (2.0 * lm + (terms + 6.0) * std::log(2.0));
-    if (k == 3) e = std::max(e, u * (7.0 * lm + 37.0 * std::log(2.0)));
+    if (k == 2 || k == 3) e = std::max(e, u * (7.0 * lm + (k == 2 ? 19.0 : 37.0) * std::log(2.0)));
     return (float)(2.0 * e);
 }
 
@@ -562,20 +562,8 @@ int encode_tmap_u8(CUtensorMap *map, void *base, uint64_t inner_bytes, uint64_t 
     return FC_OK;
 }
 
-// TMA producer warps of the order-2 kernel: every stage
-// count up to 4 gets one producer per stage; 5 stages drop to 4, and 6 take
-// three producers of two stages each.
-void tc_producer_split(int *stages, int *producers)
-{
-    if (*stages == 5) *stages = 4;
-    *producers = *stages <= 4 ? *stages : 3;
-    // FC_TC_PRODUCERS=p (a tuning knob) takes p producers where p divides
-    // the stage count.
-    if (const char *v = getenv("FC_TC_PRODUCERS")) {
-        const int p = atoi(v);
-        if (p >= 1 && p <= TC_MAX_PRODUCERS && *stages % p == 0) *producers = p;
-    }
-}
+// SNPs from which order 2 takes the tensor cores.
+constexpr int64_t PAIRS_TC_MIN_SNPS = 1024;
 
 int pow2_at_least(int v)
 {
@@ -589,13 +577,11 @@ bool Dataset::pairs_tc_eligible(int L)
     const char *mode = getenv("FC_PAIRS_PATH");
     if (mode && strcmp(mode, "popc") == 0) return false;
     const bool forced = mode && strcmp(mode, "tc") == 0;
-    if (!forced && S < 1024) return false;
+    if (!forced && S < PAIRS_TC_MIN_SNPS) return false;
     if (L > 2048) return false;
     // Each class needs at least one K chunk, or its accumulator is never written.
     if (W0 == 0 || Wt == W0) return false;
-    const int Bcap = std::max(L, 1024);
-    const int P2 = pow2_at_least(L + Bcap);
-    return pairs_smem_bytes(2, (int)M, P2) <= (size_t)max_smem_optin;
+    return pairs_stages((int)M, L, (size_t)max_smem_optin) > 0;
 }
 
 PairsArgs Dataset::pairs_args(int L, float hy, float invN)
@@ -603,25 +589,21 @@ PairsArgs Dataset::pairs_args(int L, float hy, float invN)
     PairsArgs pa{};
     pa.tiles = tiles;
     pa.ntiles = ntiles;
+    pa.enc = enc2;
     pa.rank_begin = 0;
     pa.rank_end = ~0ull;
     pa.S = S;
     pa.W0 = W0;
     pa.Wt = Wt;
-    pa.marg = marg;
-    pa.logtab = logtab;
+    pa.marg4 = reinterpret_cast<const uint4 *>(marg);
+    pa.xlogx = xlog2x;
+    pa.scale = triples_scale(M);
     pa.M = (int)M;
     pa.hy = hy;
     pa.invN = invN;
     pa.pair_base = binom(S, 2);
     pa.L = L;
-    pa.Bcap = L > 0 ? std::max(L, 1024) : 0;
-    pa.P2 = L > 0 ? pow2_at_least(L + pa.Bcap) : 0;
-    pa.stages = 2;
-    for (int st = TC_MAX_STAGES; st >= 2; --st) {
-        if (pairs_smem_bytes(st, (int)M, pa.P2) <= (size_t)max_smem_optin) { pa.stages = st; break; }
-    }
-    tc_producer_split(&pa.stages, &pa.producers);
+    pa.stages = pairs_stages(pa.M, L, (size_t)max_smem_optin);
     // FC_TEST_WAIT_TICKS (tests only) shortens the pipeline waits so that
     // they run out and the kernel reports FC_ETIMEOUT.
     pa.wait_ticks = TC_WAIT_TICKS;
@@ -632,44 +614,69 @@ PairsArgs Dataset::pairs_args(int L, float hy, float invN)
     return pa;
 }
 
+int Dataset::pairs_grid(int n) const
+{
+    return enc2 ? std::min(sms & ~1, 2 * n) : std::min(sms, n);
+}
+
+int Dataset::prepare_xlog2x()
+{
+    if (xlog2x) return FC_OK;
+    cudaError_t e;
+    if ((e = dev_alloc((void **)&xlog2x, sizeof(float) * (size_t)(M + 1))) != cudaSuccess)
+        return cuda_status(e, "x log2 x table allocation");
+    if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(xlog2x, M, stream, true, triples_scale(M))) != cudaSuccess)
+        return cuda_status(e, "x log2 x table");
+    note_launches(1);
+    return FC_OK;
+}
+
 int Dataset::prepare_pairs()
 {
     if (pairs_ready) return FC_OK;
-    const int64_t S64 = (S + 63) / 64 * 64;
-    const int64_t rows = 2 * S64;
-    const uint64_t kbytes = (uint64_t)Wt * 128;
-    // Rows are padded by 128 bytes so that the 128 rows of a TMA box do not
-    // fall on a power-of-two stride (which concentrates them in few L2 sets).
-    const uint64_t pitch = kbytes + 128;
+    enc2 = std::max(M1, M0) <= 4095 ? 1 : 0;
+    int rc = prepare_xlog2x();
+    if (rc) return rc;
+    const int64_t rows = triples_rows(S);
+    const uint64_t kbytes = (uint64_t)Wt * 64, pitch = (uint64_t)triples_pitch(Wt);
     cudaError_t e;
-    e_bytes = (size_t)rows * pitch;
-    if ((e = dev_alloc_pooled((void **)&E, e_bytes, device)) != cudaSuccess)
-        return cuda_status(e, "e4m3 operand allocation");
+    if (!E) {
+        e_bytes = (size_t)rows * pitch;
+        if ((e = dev_alloc_pooled((void **)&E, e_bytes, device)) != cudaSuccess)
+            return cuda_status(e, "packed SNP row allocation");
+    }
     const bool need_marg = marg == nullptr;
     if (need_marg && (e = dev_alloc((void **)&marg, sizeof(uint16_t) * 8 * (size_t)S)) != cudaSuccess)
         return cuda_status(e, "marginal allocation");
-    const int nb = (int)(S64 / 64);
+    const int64_t IB = pairs_rows_i(enc2), JB = pairs_rows_j(enc2);
+    const int nI = (int)((S - 1 + IB - 1) / IB), nJ = (int)((S + JB - 1) / JB);
     std::vector<uint32_t> t;
-    t.reserve((size_t)nb * (nb + 1) / 2);
-    // Groups of 16 row blocks sweep all column blocks: a group's A blocks and
-    // the current B block are shared by the CTAs working at the same time.
-    const int Gr = 16;
-    for (int g0 = 0; g0 < nb; g0 += Gr)
-        for (int J = g0; J < nb; ++J)
-            for (int I = g0; I < std::min(g0 + Gr, nb); ++I)
-                if (I <= J) t.push_back(((uint32_t)I << 16) | (uint32_t)J);
+    // Groups of row blocks (2048 SNPs) sweep all column blocks: a group's row
+    // blocks and the current column blocks are shared by the CTAs working at
+    // the same time.
+    const int Gr = (int)(2048 / IB);
+    for (int g0 = 0; g0 < nI; g0 += Gr)
+        for (int J = (int)((g0 * IB + 1) / JB); J < nJ; ++J) {
+            const int64_t j_last = std::min<int64_t>(S, (J + 1) * JB) - 1;
+            for (int I = g0; I < std::min(g0 + Gr, nI); ++I)
+                if (I * IB < j_last) t.push_back(((uint32_t)I << 16) | (uint32_t)J);
+        }
     ntiles = (int)t.size();
     tiles_host = t;
-    tiles_bytes = sizeof(uint32_t) * t.size();
-    if ((e = dev_alloc_pooled((void **)&tiles, tiles_bytes, device)) != cudaSuccess)
-        return cuda_status(e, "tile list allocation");
+    if (!tiles) {
+        tiles_bytes = sizeof(uint32_t) * t.size();
+        if ((e = dev_alloc_pooled((void **)&tiles, tiles_bytes, device)) != cudaSuccess)
+            return cuda_status(e, "tile list allocation");
+    }
     cudaMemcpyAsync(tiles, t.data(), sizeof(uint32_t) * t.size(), cudaMemcpyHostToDevice, stream);
-    if ((e = launch_gate()) != cudaSuccess || (e = launch_expand_e4m3(X, S, S_pad, W0, Wt, rows, (int64_t)pitch, E, 0x38, stream)) != cudaSuccess ||
+    if ((e = launch_gate()) != cudaSuccess ||
+        (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E, stream)) != cudaSuccess ||
         (need_marg && (e = launch_marginals(X, S, S_pad, W0, Wt, marg, stream)) != cudaSuccess))
         return cuda_status(e, "pair operand preparation");
     note_launches(need_marg ? 2 : 1);
-    int rc = encode_tmap_u8(&tmap, E, kbytes, pitch, (uint64_t)rows, 128, true);
-    if (rc) return rc;
+    if ((rc = encode_tmap_u8(&tmapI, E, kbytes, pitch, (uint64_t)rows, 128, true)) != FC_OK ||
+        (rc = encode_tmap_u8(&tmapJ, E, kbytes, pitch, (uint64_t)rows, (uint32_t)pairs_block_rows(), true)) != FC_OK)
+        return rc;
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_status(e, "pair operand preparation");
     pairs_ready = true;
     return FC_OK;
@@ -705,8 +712,8 @@ int Dataset::pairs_dense(float *scores, uint32_t *tables)
     cudaMemsetAsync(pa.tile_counter, 0, sizeof(int), stream);
     if (ns) cudaMemsetAsync(pa.dump_scores, 0, ns, stream);
     if (nt) cudaMemsetAsync(pa.dump_tables, 0, nt, stream);
-    const int grid = std::min(sms, ntiles);
-    if ((e = launch_gate()) != cudaSuccess || (e = launch_pairs_tc(MODE_DUMP, tmap, pa, grid, stream)) != cudaSuccess)
+    if ((e = launch_gate()) != cudaSuccess ||
+        (e = launch_pairs_tc(MODE_DUMP, tmapI, tmapJ, pa, pairs_grid(ntiles), stream)) != cudaSuccess)
         return cuda_status(e, "tensor-core pairs kernel");
     note_launches(1);
     uint32_t herr = 0;
@@ -855,13 +862,7 @@ int Dataset::prepare_triples(int L)
     int rc = prepare_ie(3);
     if (rc) return rc;
     cudaError_t e;
-    if (!xlog2x) {
-        if ((e = dev_alloc((void **)&xlog2x, sizeof(float) * (size_t)(M + 1))) != cudaSuccess)
-            return cuda_status(e, "x log2 x table allocation");
-        if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(xlog2x, M, stream, true, triples_scale(M))) != cudaSuccess)
-            return cuda_status(e, "x log2 x table");
-        note_launches(1);
-    }
+    if ((rc = prepare_xlog2x()) != FC_OK) return rc;
     const int64_t rows = triples_rows(S);
     const uint64_t kbytes = (uint64_t)Wt * 64;
     const uint64_t pitch = (uint64_t)triples_pitch(Wt);
@@ -1551,14 +1552,14 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
                 uint32_t c_lo[2], c_hi[2];
                 unrank(S, 2, r0, c_lo);
                 unrank(S, 2, r1 - 1, c_hi);
-                const uint32_t I_lo = c_lo[0] / 64, I_hi = c_hi[0] / 64;   // 64-SNP row blocks
+                const uint32_t IB = (uint32_t)pairs_rows_i(enc2), I_lo = c_lo[0] / IB, I_hi = c_hi[0] / IB;   // row blocks
                 for (const uint32_t t : tiles_host)
                     if ((t >> 16) >= I_lo && (t >> 16) <= I_hi) range_tiles.push_back(t);
                 pa.ntiles = (int)range_tiles.size();
                 pa.rank_begin = r0;
                 pa.rank_end = r1;
             }
-            grid = std::min(sms, pa.ntiles);
+            grid = pairs_grid(pa.ntiles);
         } else if (tc3) {
             int rc = prepare_triples(L);
             if (rc) return rc;
@@ -1716,7 +1717,8 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         if (tc) {
             pa.list_score = (float *)p[0];
             pa.list_rank = (uint64_t *)p[1];
-            pa.gthr = (int *)p[10];
+            pa.pub = (int *)p[10] + 4;
+            triples_publish(L, grid, &pa.pub_m, &pa.pub_r);
             pa.tile_counter = (int *)p[10] + 1;
             pa.err = err;
             if (!range_tiles.empty()) {
@@ -1725,9 +1727,10 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
                 pa.tiles = (const uint32_t *)p[11];
             }
             // 0x80808080 is below the ordered image of every finite score.
-            cudaMemsetAsync(p[10], 0x80, sizeof(int), stream);
+            cudaMemsetAsync(pa.pub, 0x80, sizeof(int) * (size_t)sms, stream);
             cudaMemsetAsync(pa.tile_counter, 0, sizeof(int), stream);
-            if ((e = launch_gate()) != cudaSuccess || (e = launch_pairs_tc(MODE_TOPN, tmap, pa, grid, stream)) != cudaSuccess)
+            if ((e = launch_gate()) != cudaSuccess ||
+                (e = launch_pairs_tc(MODE_TOPN, tmapI, tmapJ, pa, grid, stream)) != cudaSuccess)
                 return cuda_status(e, "tensor-core pairs kernel");
         } else if (tc4) {
             const TupleTC &u = tup[k - 4];
@@ -2241,6 +2244,13 @@ int fc_timing(fc_handle *h, int enable, double *sweep_ms, int64_t *sweeps, int64
     return FC_OK;
 }
 
+// The samples that the dense outputs take: those whose log table fits beside
+// two 32-KiB load stages in shared memory.
+static bool dense_samples_fit(const Dataset &d)
+{
+    return 1024 + 2 * (size_t)32768 + (size_t)((d.M + 4) & ~3) * 4 <= (size_t)d.max_smem_optin;
+}
+
 int fc_tuples_dense(fc_handle *h, int k, float *scores, uint32_t *tables)
 {
     return guarded([&]() -> int {
@@ -2255,7 +2265,7 @@ int fc_tuples_dense(fc_handle *h, int k, float *scores, uint32_t *tables)
             return set_error(FC_ERANGE, "dense tables need C(S,k) * 3^k <= 2^25");
         if (h->ds.W0 == 0 || h->ds.Wt == h->ds.W0)
             return set_error(FC_EINVAL, "the tensor-core path needs both cases and controls");
-        if ((size_t)pairs_smem_bytes(2, (int)h->ds.M, 0) > (size_t)h->ds.max_smem_optin)
+        if (!dense_samples_fit(h->ds))
             return set_error(FC_ERANGE, "too many samples for the tensor-core path");
         DeviceGuard g(h->ds.device);
         return h->ds.tuples_dense(k, scores, tables);
@@ -2281,7 +2291,7 @@ int fc_triples_dense(fc_handle *h, float *scores, uint32_t *tables)
         if (tables && h->ds.S > 160) return set_error(FC_ERANGE, "dense order-3 tables need S <= 160");
         if (h->ds.W0 == 0 || h->ds.Wt == h->ds.W0)
             return set_error(FC_EINVAL, "the tensor-core path needs both cases and controls");
-        if ((size_t)pairs_smem_bytes(2, (int)h->ds.M, 0) > (size_t)h->ds.max_smem_optin)
+        if (!dense_samples_fit(h->ds))
             return set_error(FC_ERANGE, "too many samples for the tensor-core path");
         DeviceGuard g(h->ds.device);
         return h->ds.triples_dense(scores, tables);
@@ -2298,7 +2308,7 @@ int fc_pairs_dense(fc_handle *h, float *scores, uint32_t *tables)
         if (tables && h->ds.S > 1024) return set_error(FC_ERANGE, "dense tables need S <= 1024");
         if (h->ds.W0 == 0 || h->ds.Wt == h->ds.W0)
             return set_error(FC_EINVAL, "the tensor-core path needs both cases and controls");
-        if ((size_t)pairs_smem_bytes(2, (int)h->ds.M, 0) > (size_t)h->ds.max_smem_optin)
+        if (!dense_samples_fit(h->ds))
             return set_error(FC_ERANGE, "too many samples for the tensor-core path");
         DeviceGuard g(h->ds.device);
         return h->ds.pairs_dense(scores, tables);

@@ -70,9 +70,10 @@ struct Dataset {
     bool last_path_tc = false;
     int max_smem_optin = 0;
 
-    // Order-2 tensor-core operands, built on first use: E = 0/1 e4m3 bytes
-    // [2*S64][Wt*128] (rows 2s+g for genotypes g = 0, 1), per-SNP genotype
-    // counts, the block-pair tile list and E's TMA descriptor.
+    // Order-2 tensor-core operands, built on first use: E = packed SNP rows
+    // (row 2s+g for genotypes g = 0, 1; triples_rows), per-SNP genotype counts,
+    // the block-pair tile list, E's TMA descriptors (boxes of the SNPs i and j)
+    // and the form (PairsArgs::enc).
     uint8_t *E = nullptr;
     size_t e_bytes = 0;
     uint16_t *marg = nullptr;
@@ -80,7 +81,8 @@ struct Dataset {
     size_t tiles_bytes = 0;
     std::vector<uint32_t> tiles_host;   // the same tile list on the host
     int ntiles = 0;
-    CUtensorMap tmap{};
+    CUtensorMap tmapI{}, tmapJ{};
+    int enc2 = 0;
     bool pairs_ready = false;
 
     // Order-3 tensor-core operands, built on first use: the packed SNP rows
@@ -200,6 +202,8 @@ struct Dataset {
     bool pairs_tc_eligible(int L);
     PairsArgs pairs_args(int L, float hy, float invN);
     int prepare_pairs();
+    int prepare_xlog2x();
+    int pairs_grid(int n) const;   // CTAs for n order-2 tiles
     int pairs_dense(float *scores, uint32_t *tables);
     bool triples_tc_eligible(int L);
     int triples_form(int L) const;

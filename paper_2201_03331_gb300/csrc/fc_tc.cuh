@@ -1,4 +1,4 @@
-// Helpers of the tcgen05 kernels (order-2 pairs and order-3 triples):
+// Helpers of the tcgen05 kernels:
 // tile constants, mbarrier waits with a time budget, TMA loads, shared-memory
 // and instruction descriptors, MMA issue and commit, TMEM loads, and the
 // epilogue's named barrier and bitonic sort.  Included by one translation
@@ -11,28 +11,11 @@
 namespace fc {
 namespace {
 
-constexpr int TC_BM = 128;          // tile rows: 64 SNPs x genotype rows {0,1}
-constexpr int TC_BN = 128;          // tile columns
-constexpr int TC_BK = 128;          // K bytes (samples) per pipeline stage
-constexpr int TC_SNPS = 64;         // SNPs per tile side
-constexpr int TC_THREADS = 192;
-// Kernels with several TMA producer warps: warp 0 and warps TC_PROD_WARP1 ..
-// issue the copies (TMA copies issued from one thread complete about one
-// stage at a time); producer p owns the stages s = p (mod producers).
-constexpr int TC_PROD_WARP1 = 6;                              // after warp 1 (MMA) and the four epilogue warps
-constexpr int TC_THREADS_MP = 32 * (TC_PROD_WARP1 + TC_MAX_PRODUCERS - 1);
-
-// Producer index of warp w, or -1 (warp 0 -> 0, warp TC_PROD_WARP1 + q -> q + 1).
-__device__ __forceinline__ int tc_producer_of(int w, int producers)
-{
-    const int p = w == 0 ? 0 : (w >= TC_PROD_WARP1 ? w - TC_PROD_WARP1 + 1 : -1);
-    return p < producers ? p : -1;
-}
+constexpr int TC_BM = 128;          // tile rows of a CTA
+constexpr int TC_BK = 128;          // K bytes per pipeline stage
 constexpr int TC_SCHED = 4;         // depth of the tile-scheduling ring
-constexpr int TC_LOOKAHEAD = 2;     // tiles the MMA thread publishes ahead of the one it consumes
 constexpr uint32_t TC_TMEM_COLS = 512;
 constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK;   // 16 KiB
-constexpr uint32_t TC_B_BYTES = TC_BN * TC_BK;   // 16 KiB
 constexpr unsigned FULL = 0xffffffffu;
 constexpr long long WAIT_BUDGET = TC_WAIT_TICKS;  // clock64 ticks (~2 s) per wait
 
@@ -128,32 +111,6 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
     return d;
-}
-
-// Instruction descriptor, kind::f8f6f4: D = F32 (bits 4-5 = 1), A = B = E4M3
-// (bits 7-9, 10-12 = 0), both K-major (bits 15, 16 = 0), N >> 3 at bits
-// 17-22, M >> 4 at bits 24-28.
-__host__ __device__ constexpr uint32_t idesc_e4m3_f32(int M, int N)
-{
-    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// The same with both operands e4m3 or both e5m2 (A and B type fields,
-// bits 7-9 and 10-12: 0 = E4M3, 1 = E5M2).
-__host__ __device__ constexpr uint32_t idesc_f8_f32(int M, int N, bool e5m2)
-{
-    return idesc_e4m3_f32(M, N) | (e5m2 ? (1u << 7) | (1u << 10) : 0u);
-}
-
-__device__ __forceinline__ void mma_e4m3(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 
 // ---- kind::mxf4: packed 4-bit 0/1 operands -----------------------------------
@@ -340,21 +297,6 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 32 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-          "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
-          "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
-          "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr));
-}
-
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Ties registers written by tcgen05.ld to a point after tcgen05.wait::ld:
@@ -369,19 +311,6 @@ __device__ __forceinline__ void tmem_regs_after_wait(uint32_t (&v)[N])
 // Named barrier 1 over the NT epilogue threads.
 template <int NT>
 __device__ __forceinline__ void epi_bar_n() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
-__device__ __forceinline__ void epi_bar() { epi_bar_n<128>(); }
-
-// 16 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-          "=r"(v[15])
-        : "r"(taddr));
-}
 
 // 28 consecutive FP32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld28(uint32_t taddr, uint32_t (&v)[28])
@@ -444,7 +373,6 @@ __device__ void epi_bitonic_desc_n(float *s, uint64_t *r, int n, int tid)
     }
     epi_bar_n<NT>();
 }
-__device__ void epi_bitonic_desc(float *s, uint64_t *r, int n, int tid) { epi_bitonic_desc_n<128>(s, r, n, tid); }
 
 }  // namespace
 }  // namespace fc

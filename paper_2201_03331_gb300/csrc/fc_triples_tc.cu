@@ -98,7 +98,7 @@
 //                fourth two pairs of a tile
 #include <algorithm>
 
-#include "fc_tc.cuh"
+#include "fc_candidates.cuh"
 #include "fc_ie.cuh"
 
 namespace fc {
@@ -125,225 +125,9 @@ constexpr int T3_WARP_PAIRS = 2 * ((2 * T3_NP / 2 + T3_PARTS - 1) / T3_PARTS);  
 constexpr int T3_REC_WORDS = 12;                   // per pair: T01[9], rank base (2 words)
 static_assert(T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS % 4 == 0 && T3_REC_WORDS % 4 == 0, "records of uint4");
 static_assert(T3_WARP_PAIRS <= 32, "a lane per pair record");
-constexpr int T3_WBUF = 64;                        // candidates of a warp's buffer
 
 __device__ __forceinline__ uint64_t c3(uint64_t n) { return n * (n - 1) * (n - 2) / 6; }   // 0 for n < 3
 __device__ __forceinline__ uint64_t c2(uint64_t n) { return n * (n - 1) / 2; }             // 0 for n < 2
-
-// 8 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "r"(taddr));
-}
-
-// Two exact FP32 accumulators (integers below 2^16) packed as lo | hi << 16 (ENC
-// 0: 4 n_case and 4 n_ctrl):
-// x + 2^23 has the integer in its low mantissa bits, and the exponent
-// field of the high word falls outside 32 bits after the shift.
-__device__ __forceinline__ uint32_t pack_exact(uint32_t lo_bits, uint32_t hi_bits)
-{
-    const uint32_t a = __float_as_uint(__uint_as_float(lo_bits) + 8388608.0f);
-    const uint32_t b = __float_as_uint(__uint_as_float(hi_bits) + 8388608.0f);
-    return a + (b << 16) - 0x4B000000u;
-}
-
-// One encoded accumulator x = 4 (n_case + 4096 n_ctrl) (a multiple of 4 below
-// 2^26, n_case < 4096, so exact) as 4 n_case | 4 n_ctrl << 16: v = x as an
-// integer, and v + (v >> 14) (2^18 - 2^14) moves n_ctrl from bit 14 to bit 18.
-__device__ __forceinline__ uint32_t unpack_enc(uint32_t bits)
-{
-    const uint32_t v = __float2uint_rz(__uint_as_float(bits));
-    return v + (v >> 14) * 245760u;
-}
-
-// Two FP32 operations per instruction.
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 f2(float x, float y)
-{
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float2 f2_split(F2 a)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
-    return r;
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b)
-{
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c)
-{
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-
-constexpr float LN2F = 0.693147180559945309f;
-
-// Hardware base-2 logarithm (MUFU), flush-to-zero; x >= 1 here.
-__device__ __forceinline__ float lg2_approx(float x)
-{
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// An integer below 2^23 as a float, exactly.
-__device__ __forceinline__ float u2f_small(uint32_t n)
-{
-    return __uint_as_float(n | 0x4B000000u) - 8388608.0f;
-}
-
-// (The next three functions are calls, so that the scoring loop keeps its
-// registers.)
-// Sorts a warp's m <= T3_WBUF candidates (ws, wr) best first, keeping those
-// that beat (thr_s, thr_r); returns their number.
-__device__ __noinline__ int sort_candidates(float *ws, uint64_t *wr, int m, float thr_s, uint64_t thr_r, int lane)
-{
-    float cs[2];
-    uint64_t cr[2];
-    unsigned keep[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int x = lane + 32 * h;
-        cs[h] = x < m ? ws[x] : -FLT_MAX;
-        cr[h] = x < m ? wr[x] : NO_RANK;
-        keep[h] = __ballot_sync(FULL, x < m && better(cs[h], cr[h], thr_s, thr_r));
-    }
-    const unsigned below = (1u << lane) - 1u;
-    bool mine[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        mine[h] = (keep[h] >> lane & 1u) != 0;
-        if (mine[h]) {
-            const int p = (h ? __popc(keep[0]) : 0) + __popc(keep[h] & below);
-            ws[p] = cs[h];
-            wr[p] = cr[h];
-        }
-    }
-    m = __popc(keep[0]) + __popc(keep[1]);
-    __syncwarp();
-    // A candidate's place is the number of better ones.
-    int at[2] = {0, 0};
-#pragma unroll 4
-    for (int y = 0; y < m; ++y) {
-        const float s = ws[y];
-        const uint64_t r = wr[y];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) at[h] += better(s, r, cs[h], cr[h]);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (mine[h]) {
-            ws[at[h]] = cs[h];
-            wr[at[h]] = cr[h];
-        }
-    __syncwarp();
-    return m;
-}
-
-// Number of the n entries (s, r), best first, that are better than (cs, cr).
-__device__ __forceinline__ int count_better(const float *s, const uint64_t *r, int n, float cs, uint64_t cr)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (better(s[mid], r[mid], cs, cr)) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
-// Merges m <= T3_WBUF candidates (ws, wr), best first, into the CTA's list
-// (ls, lr: L entries, best first, empty entries -FLT_MAX / NO_RANK).  All
-// lanes of the warp that holds the list's lock.
-__device__ __noinline__ void merge_candidates(float *ls, uint64_t *lr, int L, const float *ws, const uint64_t *wr, int m, int lane)
-{
-    // Every candidate's place: its place among the candidates plus the list
-    // entries before it.
-    int to[2], first = L;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int x = lane + 32 * h;
-        to[h] = L;
-        if (x < m) {
-            const int lo = count_better(ls, lr, L, ws[x], wr[x]);
-            to[h] = lo + x;
-            first = min(first, lo);
-        }
-    }
-    first = __reduce_min_sync(FULL, first);
-    // Entries from `first` on move down by the number of candidates before
-    // them, blocks of 256 from the end.
-    constexpr int B = 8;
-    for (int base = (L - 1) / (32 * B) * (32 * B); base > first - 32 * B; base -= 32 * B) {
-        float s[B];
-        uint64_t r[B];
-        int p[B];
-#pragma unroll
-        for (int q = 0; q < B; ++q) {
-            const int x = base + 32 * q + lane;
-            p[q] = L;
-            if (x >= first && x < L) {
-                s[q] = ls[x];
-                r[q] = lr[x];
-                p[q] = x;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < B; ++q)
-            if (p[q] < L) p[q] += count_better(ws, wr, m, s[q], r[q]);
-        __syncwarp();
-#pragma unroll
-        for (int q = 0; q < B; ++q)
-            if (p[q] < L) {
-                ls[p[q]] = s[q];
-                lr[p[q]] = r[q];
-            }
-        __syncwarp();
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (to[h] < L) {
-            ls[to[h]] = ws[lane + 32 * h];
-            lr[to[h]] = wr[lane + 32 * h];
-        }
-    __syncwarp();
-}
-
-// A score that at least L combinations reach, from what the CTAs of the
-// launch have published (pub[n]: the score of the list's entry m - 1 as an
-// ordered int): the r-th largest, r m >= L, to 20 bits downwards.  All lanes
-// of a warp; n <= 32 T3_PUB_PER_LANE.
-constexpr int T3_PUB_PER_LANE = 8;
-__device__ __noinline__ float published_threshold(const int *pub, int n, int r, int lane)
-{
-    uint32_t key[T3_PUB_PER_LANE];
-#pragma unroll
-    for (int x = 0; x < T3_PUB_PER_LANE; ++x) {
-        const int c = lane + 32 * x;
-        key[x] = c < n ? (uint32_t)*(volatile const int *)(pub + c) ^ 0x80000000u : 0u;
-    }
-    uint32_t t = 0;
-    for (int b = 31; b >= 12; --b) {
-        const uint32_t c = t | 1u << b;
-        int cnt = 0;
-#pragma unroll
-        for (int x = 0; x < T3_PUB_PER_LANE; ++x) cnt += __popc(__ballot_sync(FULL, key[x] >= c));
-        if (cnt >= r) t = c;
-    }
-    const float f = from_ordered((int)(t ^ 0x80000000u));
-    return f >= -FLT_MAX ? f : -FLT_MAX;   // (NaN patterns of nothing published)
-}
 
 // BATCH: the items of several jobs (T3Job), job-major, in one launch.
 template <int MODE, int ENC, bool BATCH>
@@ -362,7 +146,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     // tiles)}.
     __shared__ uint4 sched_tile[TC_SCHED];
     __shared__ int abort_flag_s;
-    __shared__ int list_lock;
+    __shared__ int list_lock, list_fill;
     __shared__ int epi_job;          // job of the tile that the epilogue's first warp took last, -2 at the end
     // published_threshold: job in the high half, score bits in the low one
     // (read and written as one word).
@@ -383,7 +167,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     uint32_t *recs = reinterpret_cast<uint32_t *>(smem + (size_t)stages * T3_STAGE);
     uint64_t *lrank = reinterpret_cast<uint64_t *>(recs + T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS);
     uint64_t *wrank = lrank + a.L;
-    float *lscore = reinterpret_cast<float *>(wrank + T3_EPI_WARPS * T3_WBUF);
+    float *lscore = reinterpret_cast<float *>(wrank + T3_EPI_WARPS * TC_WBUF);
     float *wscore = lscore + a.L;
 
     if (threadIdx.x == 0) {
@@ -405,6 +189,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         }
         abort_flag_s = 0;
         list_lock = 0;
+        list_fill = 0;
         epi_job = -1;
         threshold = ~0ull << 32;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -537,12 +322,13 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         const uint32_t peer_tile = PAIR ? cluster_addr(&sched_tile[0], 1) : 0;
         const uint32_t peer_sfull = PAIR ? cluster_addr(&bar_sfull[0], 1) : 0;
         unsigned pause = 500;
+        bool done = false;   // all tiles are handed out (the threshold is renewed to the epilogue's end)
         long long t0 = clock64();
         for (int it = 0;;) {
             const int slot = it % TC_SCHED;
             const uint32_t sn = (uint32_t)(it / TC_SCHED);
             int ready = 0;   // 1: a tile was handed out, 2: no tile is left
-            if (crank == 0 && lane == 0 && mbar_try(&bar_sempty[slot], (sn & 1) ^ 1)) {
+            if (!done && crank == 0 && lane == 0 && mbar_try(&bar_sempty[slot], (sn & 1) ^ 1)) {
                 int t = atomicAdd(a.tile_counter, 1);
                 const bool end = t >= n_items;
                 if (BATCH && !end) {
@@ -568,17 +354,16 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 ready = end ? 2 : 1;
             }
             ready = __shfl_sync(FULL, ready, 0);
-            if (ready == 2) break;
-            if (ready) {
+            done = done || ready == 2;
+            if (ready == 1) {
                 ++it;
                 t0 = clock64();
                 continue;
             }
-            // (The second CTA's warp ends with its epilogue.)
             const int job = __shfl_sync(FULL, *(volatile int *)&epi_job, 0);
             int stop = 0;
             if (lane == 0) {
-                if (crank == 0 && clock64() - t0 > wt) {
+                if (!done && crank == 0 && clock64() - t0 > wt) {
                     *abort_flag = 1;
                     atomicOr(a.err, ERR_TIMEOUT);
                 }
@@ -670,28 +455,34 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         const int g = lane & 1;                            // genotype of this lane's row
         const uint32_t tempty0 = PAIR ? cluster_addr(&bar_tempty[0], 0) : 0;
         const int L = a.L;
-        float *ws = wscore + ew * T3_WBUF;
-        uint64_t *wr = wrank + ew * T3_WBUF;
+        float *ws = wscore + ew * TC_WBUF;
+        uint64_t *wr = wrank + ew * TC_WBUF;
         uint32_t *rec = recs + ew * (T3_WARP_PAIRS * T3_REC_WORDS);
-        // The data set and job of the tile (a batched launch reloads them
-        // when the job changes).
-        int S = (int)a.S, Sp = (int)a.S_pad;
-        uint64_t total = a.total;
+        // The job of the tile (a batched launch reads the job's data again with
+        // each tile: kept, they cost the scoring loop its registers).
+        int cur_job = BATCH ? -1 : 0;
         const float unscale = 1.f / a.scale;   // (exact)
-        float hy = a.hy, invN = a.invN * unscale;
-        const uint4 *marg4 = a.marg4, *PR = a.PR;
-        int cur_job = -1, slot_j = 0;
         const bool whole = BATCH || (a.rank_begin == 0 && a.rank_end >= a.total);
         // This warp's candidates, and the CTA list's last entry when the
         // warp last merged: a candidate has to beat it.
         int cnt = 0;
         float thr_s = -FLT_MAX;
         uint64_t thr_r = NO_RANK;
+        bool waited = false;
+        // The least score of a candidate by now: that of the list's last entry
+        // (which only rises; a racy read is a score it had at some time), and
+        // the one that enough combinations of all CTAs are known to reach.
+        auto published = [&]() -> float {
+            const unsigned long long t2 = *(volatile unsigned long long *)&threshold;
+            return (int)(t2 >> 32) == cur_job ? __uint_as_float((uint32_t)t2) : -FLT_MAX;
+        };
+        auto floor_score = [&]() -> float { return fmaxf(*(volatile float *)(lscore + L - 1), published()); };
+        auto known = [&]() -> bool { return published() > -FLT_MAX; };
         auto merge = [&]() {
             // Sorted outside the lock, against the list's last score then.
             const float racy = *(volatile float *)(lscore + L - 1);
             const bool later = racy > thr_s;
-            const int m = sort_candidates(ws, wr, cnt, later ? racy : thr_s, later ? NO_RANK : thr_r, lane);
+            int m = sort_candidates(ws, wr, cnt, later ? racy : thr_s, later ? NO_RANK : thr_r, lane);
             cnt = 0;
             if (m == 0) return;
             bool held = true;
@@ -710,18 +501,30 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             }
             held = __shfl_sync(FULL, held, 0);
             if (held) {
-                merge_candidates(lscore, lrank, L, ws, wr, m, lane);
+                // (What the threshold has passed meanwhile is left out.)
+                const float now = floor_score();
+                m = __popc(__ballot_sync(FULL, lane < m && ws[lane] >= now)) +
+                    __popc(__ballot_sync(FULL, lane + 32 < m && ws[lane + 32] >= now));
+                const int fill = merge_candidates(lscore, lrank, L, list_fill, ws, wr, m, lane);
+                if (lane == 0) list_fill = fill;
                 thr_s = lscore[L - 1];
                 thr_r = lrank[L - 1];
                 __threadfence_block();
                 __syncwarp();
                 if (lane == 0) {
                     if (lrank[a.pub_m - 1] != NO_RANK)
-                        *(volatile int *)(a.pub + (size_t)slot_j * gridDim.x + blockIdx.x) = ordered_int(lscore[a.pub_m - 1]);
+                        *(volatile int *)(a.pub + (size_t)(BATCH ? a.jobs[cur_job].slot : 0) * gridDim.x + blockIdx.x) = ordered_int(lscore[a.pub_m - 1]);
                     __threadfence_block();
                     atomicExch(&list_lock, 0);
                 }
             }
+            __syncwarp();
+            if (BATCH || waited || L < TC_LONG_LIST) return;
+            // A merge into a long list costs microseconds: after its first
+            // one a warp waits a little for the threshold over all CTAs.
+            waited = true;
+            const long long t0 = clock64();
+            while (clock64() - t0 < TC_FIRST_THRESHOLD_TICKS && !known()) __nanosleep(200);
             __syncwarp();
         };
         // All epilogue warps meet, unless a wait ran out in some role.
@@ -733,18 +536,20 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             epi_par ^= 1;
             return __all_sync(FULL, met);
         };
-        // The CTA's list of the current job, written out as list slot_j of
+        // The CTA's list of the current job, written out as the list of its
+        // slot of
         // this CTA (all epilogue warps).
         auto flush = [&]() -> bool {
             merge();
             if (!meet()) return false;
-            const size_t o = ((size_t)slot_j * gridDim.x + blockIdx.x) * L;
+            const size_t o = ((size_t)(BATCH ? a.jobs[cur_job].slot : 0) * gridDim.x + blockIdx.x) * L;
             for (int x = threadIdx.x - 32 * T3_EPI_WARP0; x < L; x += T3_EPI_THREADS) {
                 a.list_score[o + x] = lscore[x];
                 a.list_rank[o + x] = lrank[x];
                 lscore[x] = -FLT_MAX;
                 lrank[x] = NO_RANK;
             }
+            if (ew == 0 && lane == 0) list_fill = 0;
             thr_s = -FLT_MAX;
             thr_r = NO_RANK;
             return meet();
@@ -787,16 +592,10 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 // starts empty (every epilogue warp sees the same items).
                 if (cur_job >= 0 && !flush()) { ok = false; break; }
                 cur_job = job;
-                const T3Job *jb = a.jobs + job;
-                S = (int)jb->S;
-                Sp = (int)jb->S_pad;
-                total = jb->total;
-                hy = jb->hy;
-                invN = jb->invN * unscale;
-                marg4 = jb->marg4;
-                PR = jb->PR;
-                slot_j = jb->slot;
             }
+            const T3Job *jb = BATCH ? a.jobs + job : nullptr;
+            const int S = (int)(BATCH ? jb->S : a.S), Sp = (int)(BATCH ? jb->S_pad : a.S_pad);
+            const uint4 *marg4 = BATCH ? jb->marg4 : a.marg4, *PR = BATCH ? jb->PR : a.PR;
             if (MODE == MODE_TOPN && ew == 0 && lane == 0) *(volatile int *)&epi_job = job;
             const int b = it & 1;
             const uint32_t u = (uint32_t)(it >> 1);
@@ -844,7 +643,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     const uint32_t Rq[4] = {q4.x, q4.y, q4.z, q4.w};
                     full2(Rq, Ti, Tj, T01);
                     // rank of (i, j, l) = base_i - C(S - j, 2) + l - j - 1
-                    const uint64_t base_i = total - c3((uint64_t)(S - i)) + c2((uint64_t)(S - i - 1));
+                    const uint64_t base_i = (BATCH ? jb->total : a.total) - c3((uint64_t)(S - i)) + c2((uint64_t)(S - i - 1));
                     rb = base_i - c2((uint64_t)(S - j)) - (uint64_t)j - 1;
                 }
 #pragma unroll
@@ -864,6 +663,10 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * T3_BUF + 8 * part);
+            // Read again whenever a combination passes what was read before.
+            float thr = MODE == MODE_TOPN ? floor_score() : 0.f;
+            const float hy = BATCH ? jb->hy : a.hy;
+            const float invN = (BATCH ? jb->invN : a.invN) * unscale;
             for (int r = 0; r < nr; ++r, j += 2 * T3_PARTS) {
                 // The cells of two pairs with this lane's genotype of l; those
                 // of the other lane's pair go there.  R[z][2 a + b]: z = 0 this
@@ -907,7 +710,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 const uint32_t T01[9] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x};
                 const uint32_t R12[4] = {(g ? pj.y : pj.x) << 2, (g ? pj.x : pj.y) << 2, (g ? pj.w : pj.z) << 2,
                                          (g ? pj.z : pj.w) << 2};
-                const uint64_t rank = (((uint64_t)r2.z << 32) | r2.y) + (uint64_t)l;
+                const uint64_t rank_of_pair = ((uint64_t)r2.z << 32) | r2.y;   // less l
                 // Cells (x, y, 0) and (x, y, 1); (x, y, 2) is the rest of
                 // T01(x, y).
                 F2 hs[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
@@ -931,7 +734,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                         if ((3 * x + y) % 2 == 1 || 3 * x + y == 8)   // (a cell of no sample adds 0)
                             hs[1] = add_terms(hs[1], odd, 3 * x + y == 8 ? 0u : c[2]);
                         if (MODE == MODE_DUMP && a.dump_tables && lv && j < l) {
-                            uint32_t *o = a.dump_tables + (size_t)rank * 54 + 18 * x + 6 * y;
+                            uint32_t *o = a.dump_tables + (size_t)(rank_of_pair + (uint64_t)l) * 54 + 18 * x + 6 * y;
 #pragma unroll
                             for (int z = 0; z < 3; ++z) {
                                 const int zz = z < 2 ? z ^ g : 2;   // genotype of l
@@ -942,27 +745,28 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     }
                 const float2 h2 = f2_split(f2_add(hs[0], hs[1]));
                 const float score = fmaf(-LN2F * (h2.x + h2.y), invN, hy);
-                const bool valid = lv && j < l && (whole || (rank >= a.rank_begin && rank < a.rank_end));
-                if (MODE == MODE_DUMP && valid && a.dump_scores) a.dump_scores[rank] = score;
+                const bool valid = lv && j < l;
+                if (MODE == MODE_DUMP && valid && a.dump_scores) a.dump_scores[rank_of_pair + (uint64_t)l] = score;
                 if (MODE == MODE_TOPN) {
-                    // A combination has to reach the list's last score, which
-                    // only rises (a racy read is a score it had at some time),
-                    // and the score that enough combinations of all CTAs are
-                    // known to reach.
-                    const float lthr = *(volatile float *)(lscore + L - 1);
-                    const unsigned long long t2 = *(volatile unsigned long long *)&threshold;
-                    const bool low = (int)(t2 >> 32) == job && score < __uint_as_float((uint32_t)t2);
-                    const bool cand = valid && score >= lthr && !low && better(score, rank, thr_s, thr_r);
-                    const unsigned mk = __ballot_sync(FULL, cand);
-                    if (mk) {
-                        if (cand) {
-                            const int p = cnt + __popc(mk & ((1u << lane) - 1u));
-                            ws[p] = score;
-                            wr[p] = rank;
+                    // Few combinations reach the threshold: ranks only after
+                    // the vote.
+                    const bool near = valid && score >= thr;
+                    if (__any_sync(FULL, near)) {
+                        thr = floor_score();
+                        const uint64_t rank = rank_of_pair + (uint64_t)l;
+                        const bool cand = near && score >= thr && (whole || (rank >= a.rank_begin && rank < a.rank_end)) &&
+                                          better(score, rank, thr_s, thr_r);
+                        const unsigned mk = __ballot_sync(FULL, cand);
+                        if (mk) {
+                            if (cand) {
+                                const int p = cnt + __popc(mk & ((1u << lane) - 1u));
+                                ws[p] = score;
+                                wr[p] = rank;
+                            }
+                            cnt += __popc(mk);
+                            __syncwarp();
+                            if (cnt > TC_WBUF - 32) merge();
                         }
-                        cnt += __popc(mk);
-                        __syncwarp();
-                        if (cnt > T3_WBUF - 32) merge();
                     }
                 }
             }
@@ -1112,7 +916,7 @@ size_t triples_smem_bytes(int stages, int M, int L)
 {
     // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
     return 2048 + (size_t)(M + 1) * 4 + (size_t)stages * T3_STAGE + (size_t)T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS * 4 +
-           (size_t)(L + T3_EPI_WARPS * T3_WBUF) * (8 + 4);
+           (size_t)(L + T3_EPI_WARPS * TC_WBUF) * (8 + 4);
 }
 
 int triples_stages(int M, int L, size_t smem_cap)
@@ -1131,7 +935,7 @@ float triples_scale(int64_t M)
 
 void triples_publish(int L, int grid, int *pub_m, int *pub_r)
 {
-    const int half = std::max(1, std::min(grid, 32 * T3_PUB_PER_LANE) / 2);
+    const int half = std::max(1, std::min(grid, 32 * TC_PUB_PER_LANE) / 2);
     *pub_m = std::min(L, (L + half - 1) / half);
     *pub_r = (L + *pub_m - 1) / *pub_m;
 }
