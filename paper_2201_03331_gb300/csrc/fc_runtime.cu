@@ -740,13 +740,13 @@ int Dataset::triples_form(int L) const
     return !(f && strcmp(f, "0") == 0) && cls <= 4095 ? 1 : 0;
 }
 
-bool Dataset::triples_tc_eligible(int L)
+bool Dataset::triples_tc_eligible(int L, int64_t min_snps)
 {
     const char *mode = getenv("FC_TRIPLES_PATH");
     if (mode && strcmp(mode, "popc") == 0) return false;
     if (!allow_tc) return false;
     const bool forced = mode && strcmp(mode, "tc") == 0;
-    if (!forced && S < 384) return false;
+    if (!forced && S < min_snps) return false;
     if (S < 3 || S > 65535 || L > 2048) return false;
     // Both classes need samples (each accumulator is written by its chunks).
     if (W0 == 0 || Wt == W0) return false;

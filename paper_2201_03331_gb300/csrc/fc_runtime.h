@@ -29,6 +29,12 @@ void fault_counters_reset();
 int check_device(int *dev, int *sms);
 int list_capacity(int64_t N);
 float score_error_bound(int k, int64_t M);
+// SNPs from which order 3 takes the tensor cores: at 200 SNPs a search takes
+// 207 to 265 us there for 500 to 8,000 samples (top 10) and 428 to 2,199 in the
+// sweep, loaded and searched 412 to 595 and 578 to 2,412; at 100 SNPs and 500
+// samples the sweep is the better one (155 and 168 us).
+constexpr int64_t TRIPLES_TC_MIN_SNPS = 192;
+constexpr int64_t TRIPLES_TC_MIN_SNPS_BATCH = 384;   // of a batch's jobs
 int pow2_at_least(int v);
 // 2-D TMA descriptor over bytes: rows of inner_bytes (pitch apart), boxes of
 // 128 bytes x box_rows.
@@ -205,7 +211,7 @@ struct Dataset {
     int prepare_xlog2x();
     int pairs_grid(int n) const;   // CTAs for n order-2 tiles
     int pairs_dense(float *scores, uint32_t *tables);
-    bool triples_tc_eligible(int L);
+    bool triples_tc_eligible(int L, int64_t min_snps = TRIPLES_TC_MIN_SNPS);
     int triples_form(int L) const;
     int prepare_triples(int L);
     int build_slab3(int s);

@@ -83,3 +83,18 @@ def test_batch_of_both_forms(fc, monkeypatch):
                 return float(oracle.mi(oracle.tables(ds.genotypes, ph, 3, [c]), 3)[0])
             assert cnt[j] == 7
             assert_topn_equal(idx[j], score[j], o_idx, o_s, score_of)
+
+
+@pytest.mark.parametrize("S,kind", [(191, 3), (192, 6)])
+def test_default_path_by_snps(fc, monkeypatch, S, kind):
+    """From 192 SNPs the tensor cores by default; both sides give the sweep's
+    list."""
+    monkeypatch.delenv("FC_TRIPLES_PATH", raising=False)
+    ds = make_dataset("path", seed=960, S=S, cases=260, controls=301, k=3, top_n=40)
+    h = fc.fc_load(ds.genotypes, ds.phenotype)
+    a = fc.fc_search(h, 3, 40)
+    assert fc.fc_last_search_kind(h) == kind
+    monkeypatch.setenv("FC_TRIPLES_PATH", "popc")
+    b = fc.fc_search(h, 3, 40)
+    assert fc.fc_last_search_kind(h) == 3
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
