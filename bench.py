@@ -567,7 +567,7 @@ def run_batch(args):
         bf16 = peaks.get("bf16_tflops")
         peak = 6.0 * float(bf16) if bf16 else 6.0 * 1900.0
         achieved = flops / sweep_s / 1e12 if sweeps else None
-        roof = {"bound": "tensor", "kernel": "k_triples_tc (order-3 jobs >= 384 SNPs) + k_search_batch (the rest)",
+        roof = {"bound": "tensor", "kernel": "k_triples_tc (order-3 jobs >= 256 SNPs) + k_search_batch (the rest)",
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak if achieved else None,
                 "traffic": None, "kernel_ms_per_step": 1e3 * sweep_s, "tensor_core_jobs": len(tc_jobs),
                 "tensor_core_combinations": sum(math.comb(job_ds[j].S, k) for j in tc_jobs),

@@ -229,9 +229,9 @@ int fc_search_job(fc_handle *h, int job, int k, int64_t top_n, uint32_t *out_idx
  * fc_batch_job_kind - the path the last fc_search_batch on h took for job
  * `job` (values of fc_last_search_kind): the persistent batched sweep
  * (1, 3 or 4); for order-3 jobs large enough for the tensor cores, the
- * batched tensor-core launches (8: the replicates of a data set share its
- * pair-row slab, one persistent launch per group of data sets whose slabs
- * fit the slab buffer together, all in the same CUDA graph as the sweep),
+ * batched tensor-core launches (8: one persistent launch per group of jobs
+ * of one form, each with its own pair-row slab, all in the same CUDA graph
+ * as the sweep),
  * or the per-job tensor-core search (6) for such jobs that the batched form
  * does not take (FC_BATCH_TC3=0: none), run one after another.
  * FC_BATCH_TC=0 keeps every job in the persistent sweep.  0 before the
@@ -284,7 +284,7 @@ int fc_pairs_dense(fc_handle *h, float *scores, uint32_t *tables);
 
 /*
  * fc_triples_dense - every order-3 table or FP32 score computed by the
- * tensor-core triple kernel (the k = 3 path fc_search takes for S >= 384):
+ * tensor-core triple kernel (the k = 3 path fc_search takes for S >= 192):
  * the 8 cells with genotypes in {0,1} from the tensor-core contraction of
  * pair rows with SNP rows, the other 19 by inclusion-exclusion.  A parity
  * hook for the contraction and its epilogue (Section "Computing the
@@ -318,7 +318,7 @@ int fc_tuples_dense(fc_handle *h, int k, float *scores, uint32_t *tables);
 /*
  * fc_triples_form - the form the order-3 tensor-core kernel takes for this
  * data set: 1 = one FP32 accumulator per cell holding n_case + 4096 n_ctrl
- * (control samples enter the contraction with the e4m3 value 64; exact
+ * (control samples enter the contraction with block scale 4096; exact
  * while both classes have at most 4095 samples and the kernel's shared
  * memory fits), 0 = one accumulator per class, -1 = the kernel does not
  * fit (the order-3 search takes the sweep).  Environment FC_TRIPLES_ENC=0

@@ -447,7 +447,7 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
         cudaMemcpyAsync(T->d_desc1, desc1.data(), sizeof(JobDesc) * desc1.size(), cudaMemcpyHostToDevice, st);
     T->desc = desc;
     // Slabs that fit together are built once, here (four data sets of 300 to
-    // 1,200 SNPs x eight replicates in two launches of different forms: 115
+    // 1,200 SNPs x eight replicates in two launches of different forms: 161
     // ms a search instead of 176).
     if (!T->rebuild) {
         for (const Tc3Batch::Slot &ss : T->slots)

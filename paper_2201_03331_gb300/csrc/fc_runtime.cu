@@ -78,7 +78,7 @@ struct PoolEntry {
 std::mutex g_pool_mu;
 std::vector<PoolEntry> g_pool;
 // Two classes: slabs (>= 64 MB, at most 2 kept per device) and the smaller
-// per-search operand buffers (e4m3 rows, tile lists; at most 16 kept per
+// per-search operand buffers (packed rows, tile lists; at most 16 kept per
 // device).  At most 32 GiB are kept in total, per process.  A buffer freed
 // into a full class evicts the oldest of that class (the one least likely to
 // fit the next request when data sets come largest first).

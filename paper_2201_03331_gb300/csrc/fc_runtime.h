@@ -16,7 +16,7 @@ int set_error(int status, const char *fmt, ...);
 int cuda_status(cudaError_t e, const char *what);
 cudaError_t dev_alloc(void **p, size_t bytes);
 // Operand buffers rebuilt per data set or per search (pair-row and
-// tuple-row slabs, e4m3 rows, tile lists): a freed buffer of 4 KB or more is
+// tuple-row slabs, packed rows, tile lists): a freed buffer of 4 KB or more is
 // kept in a small per-process pool and handed to the next request that it
 // fits (at most twice its size), so that searching data sets one after
 // another neither maps and unmaps gigabytes nor pays cudaFree's implicit
@@ -34,7 +34,9 @@ float score_error_bound(int k, int64_t M);
 // sweep, loaded and searched 412 to 595 and 578 to 2,412; at 100 SNPs and 500
 // samples the sweep is the better one (155 and 168 us).
 constexpr int64_t TRIPLES_TC_MIN_SNPS = 192;
-constexpr int64_t TRIPLES_TC_MIN_SNPS_BATCH = 384;   // of a batch's jobs
+// Of a batch's jobs (smaller ones share one launch of the persistent sweep, where
+// eight jobs of 300 SNPs x 7,026 samples took 46 ms).
+constexpr int64_t TRIPLES_TC_MIN_SNPS_BATCH = 256;
 int pow2_at_least(int v);
 // 2-D TMA descriptor over bytes: rows of inner_bytes (pitch apart), boxes of
 // 128 bytes x box_rows.
