@@ -1520,7 +1520,8 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         // with SNP rows, one launch per slab of pair rows.
         // A rank range takes the tiles of its first SNPs, and the kernel
         // drops the combinations outside the range.
-        const bool tc3 = k == 3 && triples_tc_eligible(L) && (!no_alloc || triples_ready);
+        const bool tc3 = k == 3 && triples_tc_eligible(L, whole ? TRIPLES_TC_MIN_SNPS : TRIPLES_TC_MIN_SNPS_RANGE) &&
+                         (!no_alloc || triples_ready);
         // Orders 4-6: tensor-core contraction of tuple rows with tuple rows.
         // A rank range takes the tiles of the left blocks holding a left
         // tuple whose combinations meet the range, and the kernel drops the

@@ -34,6 +34,9 @@ float score_error_bound(int k, int64_t M);
 // sweep, loaded and searched 412 to 595 and 578 to 2,412; at 100 SNPs and 500
 // samples the sweep is the better one (155 and 168 us).
 constexpr int64_t TRIPLES_TC_MIN_SNPS = 192;
+// Of a rank range, which may be a small part of the search: a 64th of 250 SNPs x
+// 2,000 samples, top 1,000, takes 921 us in the sweep and 1,044 there.
+constexpr int64_t TRIPLES_TC_MIN_SNPS_RANGE = 384;
 // Of a batch's jobs (smaller ones share one launch of the persistent sweep, where
 // eight jobs of 300 SNPs x 7,026 samples took 46 ms).
 constexpr int64_t TRIPLES_TC_MIN_SNPS_BATCH = 256;
