@@ -249,6 +249,8 @@ cudaError_t launch_final_sort_batch(const JobDesc *jobs, int n_jobs, double *res
 // ---- order-2 tensor-core path (fc_pairs_tc.cu) -----------------------------
 
 constexpr int TC_MAX_STAGES = 6;
+// Static shared memory of a tensor-core kernel, rounded up (256 to 320 bytes).
+constexpr size_t TC_STATIC_SMEM = 512;
 enum { MODE_DUMP = 2 };
 // Time budget of one mbarrier wait in the tensor-core kernels, in clock64
 // ticks (about 2 s).  The pipeline waits of the order-2 kernel take theirs
@@ -290,7 +292,8 @@ int pairs_rows_i(int enc);
 int pairs_rows_j(int enc);
 int pairs_block_rows();
 // The load stages that fit smem_cap bytes of shared memory beside the table of
-// M samples and lists of L; 0 if not even two do.
+// M samples and lists of L (0: a dump, which keeps no candidates); 0 if not
+// even two do.
 int pairs_stages(int M, int L, size_t smem_cap);
 size_t pairs_smem_bytes(int stages, int M, int L);
 cudaError_t launch_marginals(const uint4 *X, int64_t S, int64_t S_pad, int W0, int Wt, uint16_t *marg,

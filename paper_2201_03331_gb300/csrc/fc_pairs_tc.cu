@@ -680,9 +680,10 @@ int pairs_block_rows() { return T2_N; }
 
 size_t pairs_smem_bytes(int stages, int M, int L)
 {
-    // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
-    return 2048 + (size_t)(M + 1) * 4 + (size_t)stages * T2_STAGE + (size_t)T2_EPI_WARPS * T2_WARP_SNPS * 8 +
-           (size_t)(L + T2_EPI_WARPS * TC_WBUF) * (8 + 4);
+    // 1 KiB for the alignment of the stages; the list and the warps' buffers
+    // where there is a list.
+    return 1024 + TC_STATIC_SMEM + (size_t)(M + 1) * 4 + (size_t)stages * T2_STAGE + (size_t)T2_EPI_WARPS * T2_WARP_SNPS * 8 +
+           (L > 0 ? (size_t)(L + T2_EPI_WARPS * TC_WBUF) * (8 + 4) : 0);
 }
 
 int pairs_stages(int M, int L, size_t smem_cap)
@@ -702,7 +703,9 @@ cudaError_t launch_marginals(const uint4 *X, int64_t S, int64_t S_pad, int W0, i
 cudaError_t launch_pairs_tc(int mode, const CUtensorMap &tmapI, const CUtensorMap &tmapJ, const PairsArgs &a, int grid,
                             cudaStream_t st)
 {
-    const size_t bytes = pairs_smem_bytes(a.stages, a.M, a.L) - 1024;
+    // (The pipeline's arrays and addresses hold for two stages and more.)
+    if (a.stages < 2 || a.stages > TC_MAX_STAGES) return cudaErrorInvalidValue;
+    const size_t bytes = pairs_smem_bytes(a.stages, a.M, a.L) - TC_STATIC_SMEM;
     void *fn = mode == MODE_TOPN ? (a.enc ? reinterpret_cast<void *>(&k_pairs_tc<MODE_TOPN, 1>)
                                           : reinterpret_cast<void *>(&k_pairs_tc<MODE_TOPN, 0>))
                                  : (a.enc ? reinterpret_cast<void *>(&k_pairs_tc<MODE_DUMP, 1>)

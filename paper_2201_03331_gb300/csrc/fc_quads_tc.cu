@@ -728,8 +728,8 @@ cudaError_t launch_quads_small_terms(float *t, cudaStream_t st)
 
 size_t quads_smem_bytes(int enc, int stages, int M, int P2)
 {
-    // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
-    return 2048 + (size_t)stages * (TC_A_BYTES + T4_BLOCK * TC_BK) + (size_t)((M + 1 + 3) & ~3) * 4 +
+    // 1 KiB for the alignment of the stages.
+    return 1024 + TC_STATIC_SMEM + (size_t)stages * (TC_A_BYTES + T4_BLOCK * TC_BK) + (size_t)((M + 1 + 3) & ~3) * 4 +
            (enc ? (size_t)T4_SMALL_FLOATS * 4 : 0) + (size_t)P2 * (8 + 4);
 }
 
@@ -746,7 +746,8 @@ void *quads_kernel(int mode, int enc)
 cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUtensorMap &tmapR, const QuadsArgs &a,
                             int grid, cudaStream_t st)
 {
-    const size_t bytes = quads_smem_bytes(a.enc, a.stages, a.M, a.P2) - 1024;
+    if (a.stages < 2 || a.stages > TC_MAX_STAGES) return cudaErrorInvalidValue;
+    const size_t bytes = quads_smem_bytes(a.enc, a.stages, a.M, a.P2) - TC_STATIC_SMEM;
     void *fn = nullptr;
     if (k == 4) fn = quads_kernel<2, 2>(mode, a.enc);
     if (k == 5) fn = quads_kernel<2, 3>(mode, a.enc);

@@ -2245,13 +2245,6 @@ int fc_timing(fc_handle *h, int enable, double *sweep_ms, int64_t *sweeps, int64
     return FC_OK;
 }
 
-// The samples that the dense outputs take: those whose log table fits beside
-// two 32-KiB load stages in shared memory.
-static bool dense_samples_fit(const Dataset &d)
-{
-    return 1024 + 2 * (size_t)32768 + (size_t)((d.M + 4) & ~3) * 4 <= (size_t)d.max_smem_optin;
-}
-
 int fc_tuples_dense(fc_handle *h, int k, float *scores, uint32_t *tables)
 {
     return guarded([&]() -> int {
@@ -2266,7 +2259,7 @@ int fc_tuples_dense(fc_handle *h, int k, float *scores, uint32_t *tables)
             return set_error(FC_ERANGE, "dense tables need C(S,k) * 3^k <= 2^25");
         if (h->ds.W0 == 0 || h->ds.Wt == h->ds.W0)
             return set_error(FC_EINVAL, "the tensor-core path needs both cases and controls");
-        if (!dense_samples_fit(h->ds))
+        if (quads_smem_bytes(h->ds.tuples_form(), 2, (int)h->ds.M, 0) > (size_t)h->ds.max_smem_optin)
             return set_error(FC_ERANGE, "too many samples for the tensor-core path");
         DeviceGuard g(h->ds.device);
         return h->ds.tuples_dense(k, scores, tables);
@@ -2292,7 +2285,7 @@ int fc_triples_dense(fc_handle *h, float *scores, uint32_t *tables)
         if (tables && h->ds.S > 160) return set_error(FC_ERANGE, "dense order-3 tables need S <= 160");
         if (h->ds.W0 == 0 || h->ds.Wt == h->ds.W0)
             return set_error(FC_EINVAL, "the tensor-core path needs both cases and controls");
-        if (!dense_samples_fit(h->ds))
+        if (h->ds.triples_form(0) < 0)
             return set_error(FC_ERANGE, "too many samples for the tensor-core path");
         DeviceGuard g(h->ds.device);
         return h->ds.triples_dense(scores, tables);
@@ -2309,7 +2302,7 @@ int fc_pairs_dense(fc_handle *h, float *scores, uint32_t *tables)
         if (tables && h->ds.S > 1024) return set_error(FC_ERANGE, "dense tables need S <= 1024");
         if (h->ds.W0 == 0 || h->ds.Wt == h->ds.W0)
             return set_error(FC_EINVAL, "the tensor-core path needs both cases and controls");
-        if (!dense_samples_fit(h->ds))
+        if (pairs_stages((int)h->ds.M, 0, (size_t)h->ds.max_smem_optin) == 0)
             return set_error(FC_ERANGE, "too many samples for the tensor-core path");
         DeviceGuard g(h->ds.device);
         return h->ds.pairs_dense(scores, tables);

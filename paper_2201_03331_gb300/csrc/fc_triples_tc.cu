@@ -914,8 +914,8 @@ int triples_block_rows() { return T3_N; }
 
 size_t triples_smem_bytes(int stages, int M, int L)
 {
-    // 1 KiB for the alignment of the stages, 1 KiB for the static arrays.
-    return 2048 + (size_t)(M + 1) * 4 + (size_t)stages * T3_STAGE + (size_t)T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS * 4 +
+    // 1 KiB for the alignment of the stages.
+    return 1024 + TC_STATIC_SMEM + (size_t)(M + 1) * 4 + (size_t)stages * T3_STAGE + (size_t)T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS * 4 +
            (size_t)(L + T3_EPI_WARPS * TC_WBUF) * (8 + 4);
 }
 
@@ -955,14 +955,14 @@ cudaError_t prepare_triples_tc_batch(int enc, size_t smem_bytes)
 {
     if (enc != 0 && enc != 1) return cudaErrorInvalidValue;
     void *fn = enc == 1 ? kernel_ptr<MODE_TOPN, 1, true>() : kernel_ptr<MODE_TOPN, 0, true>();
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes - 1024);
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem_bytes - TC_STATIC_SMEM));
 }
 
 cudaError_t launch_triples_tc(int mode, const CUtensorMap &tmapA, const CUtensorMap &tmapP, const TriplesArgs &a,
                               int grid, cudaStream_t st, bool set_attr)
 {
-    const size_t bytes = triples_smem_bytes(a.stages, a.M, a.L) - 1024;
-    if (a.enc != 0 && a.enc != 1) return cudaErrorInvalidValue;
+    const size_t bytes = triples_smem_bytes(a.stages, a.M, a.L) - TC_STATIC_SMEM;
+    if ((a.enc != 0 && a.enc != 1) || a.stages < 2 || a.stages > T3_MAX_STAGES) return cudaErrorInvalidValue;
     void *fn = nullptr;
     if (a.jobs) {
         if (mode != MODE_TOPN) return cudaErrorInvalidValue;
