@@ -378,25 +378,41 @@ bool Dataset::ie_eligible(int k) const
     return true;
 }
 
+namespace {
+// Runs `undo` at the end of its scope unless `keep` is set: what a failed
+// preparation has allocated goes back, and the next call starts afresh.
+template <class F>
+struct Undo {
+    F undo;
+    bool keep = false;
+    explicit Undo(F f) : undo(f) {}
+    ~Undo() { if (!keep) undo(); }
+};
+
+// Builds a table of a data set on its first use: the pointer is set only once
+// the kernel that fills the table has been launched.
+template <class T, class F>
+int build_once(Dataset &d, T *&table, size_t bytes, const char *what, F fill)
+{
+    if (table) return FC_OK;
+    T *p = nullptr;
+    cudaError_t e = dev_alloc((void **)&p, bytes);
+    if (e == cudaSuccess && ((e = launch_gate()) != cudaSuccess || (e = fill(p)) != cudaSuccess)) cudaFree(p);
+    if (e != cudaSuccess) return cuda_status(e, what);
+    d.note_launches(1);
+    table = p;
+    return FC_OK;
+}
+}  // namespace
+
 int Dataset::prepare_ie(int k)
 {
-    cudaError_t e;
-    if (!marg) {
-        if ((e = dev_alloc((void **)&marg, sizeof(uint16_t) * 8 * (size_t)S)) != cudaSuccess)
-            return cuda_status(e, "marginal allocation");
-        if ((e = launch_gate()) != cudaSuccess || (e = launch_marginals(X, S, S_pad, W0, Wt, marg, stream)) != cudaSuccess)
-            return cuda_status(e, "marginal kernel");
-        note_launches(1);
-    }
-    if (k == 3 && !PR) {
-        if ((e = dev_alloc((void **)&PR, sizeof(uint4) * (size_t)S_pad * S_pad)) != cudaSuccess)
-            return cuda_status(e, "restricted pair table allocation");
-        if ((e = launch_gate()) != cudaSuccess ||
-            (e = launch_restricted_pairs(X, S, S_pad, W0, Wt, PR, stream)) != cudaSuccess)
-            return cuda_status(e, "restricted pair kernel");
-        note_launches(1);
-    }
-    return FC_OK;
+    int rc = build_once(*this, marg, sizeof(uint16_t) * 8 * (size_t)S, "genotype counts",
+                        [&](uint16_t *p) { return launch_marginals(X, S, S_pad, W0, Wt, p, stream); });
+    if (rc == FC_OK && k == 3)
+        rc = build_once(*this, PR, sizeof(uint4) * (size_t)S_pad * S_pad, "restricted pair table",
+                        [&](uint4 *p) { return launch_restricted_pairs(X, S, S_pad, W0, Wt, p, stream); });
+    return rc;
 }
 
 void Dataset::fill_search_args(SearchArgs &sa) const
@@ -621,33 +637,23 @@ int Dataset::pairs_grid(int n) const
 
 int Dataset::prepare_xlog2x()
 {
-    if (xlog2x) return FC_OK;
-    cudaError_t e;
-    if ((e = dev_alloc((void **)&xlog2x, sizeof(float) * (size_t)(M + 1))) != cudaSuccess)
-        return cuda_status(e, "x log2 x table allocation");
-    if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(xlog2x, M, stream, true, triples_scale(M))) != cudaSuccess)
-        return cuda_status(e, "x log2 x table");
-    note_launches(1);
-    return FC_OK;
+    return build_once(*this, xlog2x, sizeof(float) * (size_t)(M + 1), "x log2 x table",
+                      [&](float *p) { return launch_xlogx(p, M, stream, true, triples_scale(M)); });
 }
 
 int Dataset::prepare_pairs()
 {
     if (pairs_ready) return FC_OK;
+    Undo undo([this] { release_pairs(); });
     enc2 = std::max(M1, M0) <= 4095 ? 1 : 0;
     int rc = prepare_xlog2x();
-    if (rc) return rc;
+    if (rc || (rc = prepare_ie(2)) != FC_OK) return rc;
     const int64_t rows = triples_rows(S);
     const uint64_t kbytes = (uint64_t)Wt * 64, pitch = (uint64_t)triples_pitch(Wt);
     cudaError_t e;
-    if (!E) {
-        e_bytes = (size_t)rows * pitch;
-        if ((e = dev_alloc_pooled((void **)&E, e_bytes, device)) != cudaSuccess)
-            return cuda_status(e, "packed SNP row allocation");
-    }
-    const bool need_marg = marg == nullptr;
-    if (need_marg && (e = dev_alloc((void **)&marg, sizeof(uint16_t) * 8 * (size_t)S)) != cudaSuccess)
-        return cuda_status(e, "marginal allocation");
+    e_bytes = (size_t)rows * pitch;
+    if ((e = dev_alloc_pooled((void **)&E, e_bytes, device)) != cudaSuccess)
+        return cuda_status(e, "packed SNP row allocation");
     const int64_t IB = pairs_rows_i(enc2), JB = pairs_rows_j(enc2);
     const int nI = (int)((S - 1 + IB - 1) / IB), nJ = (int)((S + JB - 1) / JB);
     std::vector<uint32_t> t;
@@ -663,23 +669,32 @@ int Dataset::prepare_pairs()
         }
     ntiles = (int)t.size();
     tiles_host = t;
-    if (!tiles) {
-        tiles_bytes = sizeof(uint32_t) * t.size();
-        if ((e = dev_alloc_pooled((void **)&tiles, tiles_bytes, device)) != cudaSuccess)
-            return cuda_status(e, "tile list allocation");
-    }
+    tiles_bytes = sizeof(uint32_t) * t.size();
+    if ((e = dev_alloc_pooled((void **)&tiles, tiles_bytes, device)) != cudaSuccess)
+        return cuda_status(e, "tile list allocation");
     cudaMemcpyAsync(tiles, t.data(), sizeof(uint32_t) * t.size(), cudaMemcpyHostToDevice, stream);
     if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E, stream)) != cudaSuccess ||
-        (need_marg && (e = launch_marginals(X, S, S_pad, W0, Wt, marg, stream)) != cudaSuccess))
+        (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E, stream)) != cudaSuccess)
         return cuda_status(e, "pair operand preparation");
-    note_launches(need_marg ? 2 : 1);
+    note_launches(1);
     if ((rc = encode_tmap_u8(&tmapI, E, kbytes, pitch, (uint64_t)rows, 128, true)) != FC_OK ||
         (rc = encode_tmap_u8(&tmapJ, E, kbytes, pitch, (uint64_t)rows, (uint32_t)pairs_block_rows(), true)) != FC_OK)
         return rc;
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_status(e, "pair operand preparation");
-    pairs_ready = true;
+    pairs_ready = undo.keep = true;
     return FC_OK;
+}
+
+void Dataset::release_pairs()
+{
+    if (stream) cudaStreamSynchronize(stream);
+    dev_free_pooled(E, e_bytes, device);
+    dev_free_pooled(tiles, tiles_bytes, device);
+    E = nullptr;
+    tiles = nullptr;
+    ntiles = 0;
+    tiles_host.clear();
+    pairs_ready = false;
 }
 
 int Dataset::pairs_dense(float *scores, uint32_t *tables)
@@ -858,6 +873,7 @@ int Dataset::prepare_triples(int L)
     if (form < 0) return set_error(FC_ERANGE, "order-3 tensor-core kernel does not fit in shared memory");
     if (triples_ready && enc3 == form) return FC_OK;
     if (triples_ready) release_triples();
+    Undo undo([this] { release_triples(); });
     enc3 = form;
     int rc = prepare_ie(3);
     if (rc) return rc;
@@ -866,15 +882,13 @@ int Dataset::prepare_triples(int L)
     const int64_t rows = triples_rows(S);
     const uint64_t kbytes = (uint64_t)Wt * 64;
     const uint64_t pitch = (uint64_t)triples_pitch(Wt);
-    if (!E3) {
-        e3_bytes = (size_t)rows * pitch;
-        if ((e = dev_alloc_pooled((void **)&E3, e3_bytes, device)) != cudaSuccess)
-            return cuda_status(e, "packed SNP row allocation");
-        if ((e = launch_gate()) != cudaSuccess ||
-            (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E3, stream)) != cudaSuccess)
-            return cuda_status(e, "packed SNP rows");
-        note_launches(1);
-    }
+    e3_bytes = (size_t)rows * pitch;
+    if ((e = dev_alloc_pooled((void **)&E3, e3_bytes, device)) != cudaSuccess)
+        return cuda_status(e, "packed SNP row allocation");
+    if ((e = launch_gate()) != cudaSuccess ||
+        (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E3, stream)) != cudaSuccess)
+        return cuda_status(e, "packed SNP rows");
+    note_launches(1);
     const int NP = triples_pairs_per_tile(1);
     size_t cap = (size_t)16 << 30;
     if (const char *mb = getenv("FC_TRIPLES_SLAB_MB")) {
@@ -908,7 +922,7 @@ int Dataset::prepare_triples(int L)
     built_slab3 = -1;
     if ((rc = build_slab3(0)) != FC_OK) return rc;
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_status(e, "pair-row slab");
-    triples_ready = true;
+    triples_ready = undo.keep = true;
     return FC_OK;
 }
 
@@ -1220,8 +1234,7 @@ QuadsArgs Dataset::tuples_args(int k, int L, float hy, float invN)
 void Dataset::release_tuples(int k)
 {
     TupleTC &u = tup[k - 4];
-    if (!u.QL && !u.QR && !u.lt && !u.groups) return;
-    if (stream) cudaStreamSynchronize(stream);
+    if (u.QL && stream) cudaStreamSynchronize(stream);   // (QL is the first of them)
     dev_free_pooled(u.QL, u.ql_bytes, device);
     dev_free_pooled(u.QR, u.qr_bytes, device);
     dev_free_pooled(u.QX, u.qx_bytes, device);
@@ -1325,21 +1338,14 @@ int Dataset::prepare_tuples(int k)
     if (u.ready) return FC_OK;
     for (int k2 = 4; k2 <= 6; ++k2)
         if (k2 != k) release_tuples(k2);
+    Undo undo([this, k] { release_tuples(k); });
     cudaError_t e;
-    if (!xlogx) {
-        if ((e = dev_alloc((void **)&xlogx, sizeof(float) * (size_t)(M + 1))) != cudaSuccess)
-            return cuda_status(e, "x ln x table allocation");
-        if ((e = launch_gate()) != cudaSuccess || (e = launch_xlogx(xlogx, M, stream)) != cudaSuccess)
-            return cuda_status(e, "x ln x table");
-        note_launches(1);
-    }
-    if (!small_terms) {
-        if ((e = dev_alloc((void **)&small_terms, sizeof(float) * (size_t)quads_small_floats())) != cudaSuccess)
-            return cuda_status(e, "cell term table allocation");
-        if ((e = launch_gate()) != cudaSuccess || (e = launch_quads_small_terms(small_terms, stream)) != cudaSuccess)
-            return cuda_status(e, "cell term table");
-        note_launches(1);
-    }
+    int rc = build_once(*this, xlogx, sizeof(float) * (size_t)(M + 1), "x ln x table",
+                        [&](float *p) { return launch_xlogx(p, M, stream); });
+    if (rc == FC_OK)
+        rc = build_once(*this, small_terms, sizeof(float) * (size_t)quads_small_floats(), "cell term table",
+                        [&](float *p) { return launch_quads_small_terms(p, stream); });
+    if (rc) return rc;
     const int LT = tc_left_size(k), RT = k - LT;
     // Form 1 takes blocks in pairs on either side: a "block" of the left
     // side is then a pair, and the right slab gets an even count.
@@ -1394,8 +1400,7 @@ int Dataset::prepare_tuples(int k)
     u.amax_host = tuple_amax(u, u.lmin_host);
     const std::vector<int> &amax = u.amax_host;
     u.sub = tuple_strip(u.group, bl, u.rchunk, sms, (double)u.rblk * rowsR * (double)pitch);
-    int rc = tuple_chunk_groups(u, amax, u.sub, bl, nullptr, u.groups_host, u.cg0, u.citems);
-    if (rc) return rc;
+    if ((rc = tuple_chunk_groups(u, amax, u.sub, bl, nullptr, u.groups_host, u.cg0, u.citems)) != FC_OK) return rc;
     u.n_items = 0;
     for (const int64_t n : u.citems) u.n_items += n;
     u.ngroups = (int)u.groups_host.size();
@@ -1434,7 +1439,7 @@ int Dataset::prepare_tuples(int k)
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_status(e, "tuple operands");
     u.lt_host = std::move(lt);
     u.lr_host = std::move(lr);
-    u.ready = true;
+    u.ready = undo.keep = true;
     return FC_OK;
 }
 

@@ -213,6 +213,7 @@ struct Dataset {
     bool pairs_tc_eligible(int L);
     PairsArgs pairs_args(int L, float hy, float invN);
     int prepare_pairs();
+    void release_pairs();
     int prepare_xlog2x();
     int pairs_grid(int n) const;   // CTAs for n order-2 tiles
     int pairs_dense(float *scores, uint32_t *tables);
