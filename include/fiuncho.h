@@ -349,17 +349,20 @@ int fc_last_search_kind(const fc_handle *h);
 int fc_sweep_tables(fc_handle *h, int k, uint64_t rank_begin, int64_t n, uint32_t *out);
 
 /*
- * fc_log2_approx - the base-2 logarithm that the order-3 tensor-core
- * epilogue takes for its n ln n terms (the hardware approximation), of
- * max(n[i], 1) for count integers n[i] < 2^23 (host uint32 in, host float
- * out), computed on the current device.  A parity hook: the epilogue's FP32
- * error bound on the mutual information (Section "Mutual Information test";
- * see fc_search) assumes |result - log2(n)| <= 2^-22 (log2(n) + 1) for
- * 1 <= n <= 2^17, which a test checks for every such n.  The paper has no
- * counterpart.  FC_EINVAL for count < 0 or NULL buffers; FC_ENOMEM /
- * FC_ECUDA as the other calls.
+ * fc_log2_approx - the hardware's base-2 logarithm of max(n[i], 1) for count
+ * integers n[i] < 2^23 (host uint32 in, host float out), computed on the
+ * current device; its error is within 2^-22 (log2(n) + 1).
+ * fc_log2_approx_scaled - the same of n[i] 2^-shift (of 1e-30 where n[i] = 0),
+ * the arguments that the tensor-core epilogues of orders 2 and 3 take it of.
+ * Parity hooks: the epilogues' FP32 error bounds on the mutual information
+ * (Section "Mutual Information test"; see fc_search) assume |result - log2(x)| <=
+ * 2^-22 max(1, |log2(x)|) for every class count and every shift that a sample
+ * count gives (0 to 14), which a test checks for all of them.  The paper has
+ * no counterpart.  FC_EINVAL for count < 0, NULL buffers or a shift outside
+ * [0, 31]; FC_ENOMEM / FC_ECUDA as the other calls.
  */
 int fc_log2_approx(const uint32_t *n, int64_t count, float *out);
+int fc_log2_approx_scaled(const uint32_t *n, int64_t count, int shift, float *out);
 
 /* fc_info - sizes of a loaded data set (any pointer may be NULL). */
 int fc_info(const fc_handle *h, int64_t *S, int64_t *M, int64_t *cases, int64_t *controls);

@@ -45,6 +45,7 @@ _SIGNATURES = {
     "fc_scores": ([P, i32, u64, i64, P], i32),
     "fc_info": ([P, P, P, P, P], i32),
     "fc_log2_approx": ([P, i64, P], i32),
+    "fc_log2_approx_scaled": ([P, i64, i32, P], i32),
     "fc_pairs_dense": ([P, P, P], i32),
     "fc_triples_dense": ([P, P, P], i32),
     "fc_tuples_dense": ([P, i32, P, P], i32),
@@ -185,10 +186,18 @@ def fc_tables(h: Handle, k: int, combos) -> np.ndarray:
 
 
 def fc_log2_approx(n) -> np.ndarray:
-    """The epilogue's hardware base-2 logarithm of ``max(n, 1)`` (float32)."""
+    """The hardware base-2 logarithm of ``max(n, 1)`` (float32)."""
     a = np.ascontiguousarray(np.asarray(n, dtype=np.uint32).ravel())
     out = np.zeros(a.shape[0], dtype=np.float32)
     _check(library().fc_log2_approx(_ptr(a), a.shape[0], _ptr(out)), "fc_log2_approx")
+    return out
+
+
+def fc_log2_approx_scaled(n, shift: int) -> np.ndarray:
+    """The epilogues' hardware base-2 logarithm of ``n 2^-shift`` (float32)."""
+    a = np.ascontiguousarray(np.asarray(n, dtype=np.uint32).ravel())
+    out = np.zeros(a.shape[0], dtype=np.float32)
+    _check(library().fc_log2_approx_scaled(_ptr(a), a.shape[0], shift, _ptr(out)), "fc_log2_approx_scaled")
     return out
 
 

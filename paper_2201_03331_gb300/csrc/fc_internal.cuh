@@ -365,9 +365,10 @@ struct TriplesArgs {
     uint32_t *dump_tables;  // MODE_DUMP: [C(S,3)][27][2]
 };
 
-// The base-2 logarithm the tensor-core epilogues take for n ln n, of
-// max(n & (2^23 - 1), 1), for n[0 .. count).
-cudaError_t launch_log2_approx(const uint32_t *n, int64_t count, float *out, cudaStream_t st);
+// The base-2 logarithm the tensor-core epilogues of orders 2 and 3 take of a class
+// count, for n[0 .. count) (each modulo 2^23): of n times `scale`, a power of two,
+// or 1e-30 where n = 0; scale 0: of max(n, 1).
+cudaError_t launch_log2_approx(const uint32_t *n, int64_t count, float scale, float *out, cudaStream_t st);
 // The load stages that fit smem_cap bytes of shared memory beside the x log2 x
 // table of M samples and lists of L; 0 if not even two do.
 int triples_stages(int M, int L, size_t smem_cap);

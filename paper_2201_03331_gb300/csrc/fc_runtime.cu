@@ -2342,7 +2342,7 @@ int fc_sweep_tables(fc_handle *h, int k, uint64_t rank_begin, int64_t n, uint32_
     });
 }
 
-int fc_log2_approx(const uint32_t *n, int64_t count, float *out)
+static int log2_probe(const uint32_t *n, int64_t count, float scale, float *out)
 {
     return guarded([&]() -> int {
         if (count < 0 || (count > 0 && (!n || !out))) return set_error(FC_EINVAL, "bad buffers");
@@ -2356,12 +2356,20 @@ int fc_log2_approx(const uint32_t *n, int64_t count, float *out)
             return cuda_status(e, "alloc");
         }
         if ((e = cudaMemcpy(dn, n, sizeof(uint32_t) * (size_t)count, cudaMemcpyHostToDevice)) == cudaSuccess &&
-            (e = launch_log2_approx(dn, count, dout, 0)) == cudaSuccess)
+            (e = launch_log2_approx(dn, count, scale, dout, 0)) == cudaSuccess)
             e = cudaMemcpy(out, dout, sizeof(float) * (size_t)count, cudaMemcpyDeviceToHost);
         cudaFree(dn);
         cudaFree(dout);
         return e == cudaSuccess ? FC_OK : cuda_status(e, "log2 probe");
     });
+}
+
+int fc_log2_approx(const uint32_t *n, int64_t count, float *out) { return log2_probe(n, count, 0.f, out); }
+
+int fc_log2_approx_scaled(const uint32_t *n, int64_t count, int shift, float *out)
+{
+    if (shift < 0 || shift > 31) return set_error(FC_EINVAL, "shift %d outside [0, 31]", shift);
+    return log2_probe(n, count, std::ldexp(1.0f, -shift), out);
 }
 
 int fc_info(const fc_handle *h, int64_t *S, int64_t *M, int64_t *cases, int64_t *controls)

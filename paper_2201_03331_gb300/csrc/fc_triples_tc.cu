@@ -58,9 +58,9 @@
 // lg2~(b) = a log2(n/a) + b log2(n/b) (a, b the class counts, n = a + b), and
 // MI = H(Y) - ln 2 sum t / N, where xl is a shared-memory table of x log2 x over
 // the sample counts (entries correctly rounded) and lg2~ the hardware base-2
-// logarithm, with |lg2~(x) - log2 x| <= 2^-22 (|log2 x| + 1) (absolute within
-// [1/2, 2], relative elsewhere; checked on the device for every integer up to
-// 2^17 by a test; fc_log2_approx).  Counts are scored times the power of two
+// logarithm, with |lg2~(x) - log2 x| <= 2^-22 max(1, |log2 x|) (absolute within
+// [1/2, 2], relative elsewhere; a test checks it on the device for every count
+// up to 2^17 under every scale below; fc_log2_approx_scaled).  Counts are scored times the power of two
 // 2^-s, s = floor(log2 M) - 2 (the sum times 2^s is the same): the logarithms of
 // the fullest cells are then near 0, and with them the roundings, while no
 // |log2 x| exceeds log2 M.  Errors of 27-cell scores against FP64 (rms, 4,000
@@ -894,17 +894,20 @@ cudaError_t launch_fill_lists(float *s, uint64_t *r, size_t n, cudaStream_t st)
 }
 
 namespace {
-__global__ void k_log2_approx(const uint32_t *n, int64_t count, float *out)
+__global__ void k_log2_approx(const uint32_t *n, int64_t count, float scale, float *out)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) out[i] = lg2_approx(fmaxf(u2f_small(n[i] & 0x7fffffu), 1.0f));
+    if (i >= count) return;
+    const float x = u2f_small(n[i] & 0x7fffffu);
+    // (add_terms' argument: the scaled count, 1e-30 for a count of 0)
+    out[i] = lg2_approx(scale > 0.f ? fmaf(x, scale, 1e-30f) : fmaxf(x, 1.0f));
 }
 }  // namespace
 
-cudaError_t launch_log2_approx(const uint32_t *n, int64_t count, float *out, cudaStream_t st)
+cudaError_t launch_log2_approx(const uint32_t *n, int64_t count, float scale, float *out, cudaStream_t st)
 {
     if (count <= 0) return cudaSuccess;
-    k_log2_approx<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(n, count, out);
+    k_log2_approx<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(n, count, scale, out);
     return cudaGetLastError();
 }
 
