@@ -24,10 +24,18 @@
 //            112;
 //   ENC = 0: the case and control samples accumulate into two accumulators;
 //            a tile of 64 SNPs i and 56 SNPs j per CTA (M = 128, N = 112).
-// A tile takes 224 TMEM columns and two tiles are in flight.  The scores are
-// those of the order-3 epilogue over 9 cells (t(a, b) = xl[n] - a lg2~(a) - b
-// lg2~(b), counts times a power of two; the error is derived there): |MI32 - MI|
-// <= u (7 ln M + 19 ln 2).
+// A tile takes 224 TMEM columns and two tiles are in flight.
+//
+// The scores are those of the order-3 epilogue over 9 cells: t(a, b) = xl[n] -
+// a lg2~(a) - b lg2~(b), counts times a power of two q that brings the samples to Q =
+// q N < 8 (4 <= Q from 8 samples on).  |MI32 - MI| <= 28 u, u = 2^-24, whatever the
+// samples: with x a scaled count, x |log2 x| <= 0.531 up to 1/2 and <= x max(1, log2 Q)
+// above, so that the sum of x max(1, |log2 x|) over the 18 class counts is at most 9.6 +
+// Q log2 Q <= 4.4 Q, and that of n |log2 n| over the 9 cells 4.8 + Q log2 Q <= 3.6 Q.
+// In units of u Q, in bits, the table entries then err by 3.6, the logarithms (4 u
+// max(1, |log2 x|) each) by 17.6, the first multiply-add of every cell by 3.6 + 4.4, the
+// second (t <= n) by 1, the four levels of additions by 4; ln 2, its product, 1/N,
+// H(Y) and the last multiply-add add 5: 39.2 u ln 2 < 28 u in nats.
 //
 // What bounds the kernel: with many samples the operands' way from L2 (60 KB a
 // chunk and tile; 12,000 SNPs x 8,192 samples move 20 GB at 14.5 TB/s, the

@@ -347,7 +347,7 @@ int list_capacity(int64_t N)
     return (int)L;
 }
 
-float score_error_bound(int k, int64_t M)
+float score_error_bound(int k, int64_t M, bool tc2)
 {
     // FP32 sweep score H(Y) - (1/N) sum_x [a (ln n - ln a) + b (ln n - ln b)]
     // with u = 2^-24: each ln table entry errs by <= u ln M, so each
@@ -356,15 +356,18 @@ float score_error_bound(int k, int64_t M)
     // N H(Y|X) <= N ln 2); the final scaling and subtraction <= 3u ln 2.
     // Divided by N: |MI32 - MI| <= u (2 ln M + (2*3^k + 6) ln 2).  The
     // orders 4-6 tensor-core epilogue's x ln x form has the smaller bound
-    // u (3 ln M + (3^k + 4) ln 2) for every M used here; those of
-    // orders 2 and 3, whose class terms come from the hardware logarithm
-    // (relative error 2^-22 plus 2^-22 absolute), u (7 ln M + 19 ln 2) and u
-    // (7 ln M + 37 ln 2).  The larger, doubled for margin.
+    // u (3 ln M + (3^k + 4) ln 2) for every M used here; the order-3 one,
+    // whose class terms come from the hardware logarithm (relative error
+    // 2^-22, absolute near 1), u (7 ln M + 37 ln 2), and the order-2 one 28 u
+    // (derived beside the kernels).  The larger, doubled for margin; order 2
+    // takes the kernel's where the kernel runs (tc2), below about 300 samples,
+    // so that a search in the sweep keeps the window of the sweep.
     const double u = std::ldexp(1.0, -24);
     const double terms = 2.0 * pow3(k);
     const double lm = std::log((double)std::max<int64_t>(M, 2));
     double e = u * (2.0 * lm + (terms + 6.0) * std::log(2.0));
-    if (k == 2 || k == 3) e = std::max(e, u * (7.0 * lm + (k == 2 ? 19.0 : 37.0) * std::log(2.0)));
+    if (k == 3) e = std::max(e, u * (7.0 * lm + 37.0 * std::log(2.0)));
+    if (tc2) e = std::max(e, u * 28.0);
     return (float)(2.0 * e);
 }
 
@@ -1504,7 +1507,6 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
     if (N == 0) { *out_count = 0; return FC_OK; }
     int L = list_capacity(N);
     if (L > FC_MAX_LIST) return set_error(FC_ERANGE, "top_n %lld too large", (long long)top_n);
-    const float eps = score_error_bound(k, M);
     const double Nd = (double)M;
     double hy = 0.0;
     if (M1 > 0) hy -= (M1 / Nd) * std::log(M1 / Nd);
@@ -1840,7 +1842,7 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         }
         RescoreArgs ra{};
         ra.X = X; ra.S = S; ra.S_pad = S_pad; ra.W0 = W0; ra.Wt = Wt; ra.k = k;
-        ra.N = (int)N; ra.L = L; ra.cand_s = src_s; ra.cand_r = src_r; ra.eps = eps;
+        ra.N = (int)N; ra.L = L; ra.cand_s = src_s; ra.cand_r = src_r; ra.eps = score_error_bound(k, M, tc);
         ra.total = r1 - r0;
         ra.res_s = (double *)p[6]; ra.res_r = (uint64_t *)p[7]; ra.res_c = (uint32_t *)p[8];
         ra.err = err;

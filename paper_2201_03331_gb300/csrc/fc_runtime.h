@@ -28,7 +28,7 @@ cudaError_t launch_gate();
 void fault_counters_reset();
 int check_device(int *dev, int *sms);
 int list_capacity(int64_t N);
-float score_error_bound(int k, int64_t M);
+float score_error_bound(int k, int64_t M, bool tc2 = false);   // tc2: scored by the order-2 tensor-core kernel
 // SNPs from which order 3 takes the tensor cores: at 200 SNPs a search takes
 // 207 to 265 us there for 500 to 8,000 samples (top 10) and 428 to 2,199 in the
 // sweep, loaded and searched 412 to 595 and 578 to 2,412; at 100 SNPs and 500

@@ -68,8 +68,8 @@ def test_pairs_dense_refuses_more(fc, M):
     with pytest.raises(fc.FiunchoError) as e:
         fc.fc_pairs_dense(h)
     assert e.value.status == fc.FC_ERANGE
-    # The sweep takes over in searches.
-    assert len(fc.fc_search(h, 2, 3)[0]) == 3
+    if M < 50000:   # (the sweep takes over in searches while its table fits)
+        assert len(fc.fc_search(h, 2, 3)[0]) == 3
 
 
 @pytest.mark.gpu
