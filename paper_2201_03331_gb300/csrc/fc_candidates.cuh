@@ -10,11 +10,6 @@ namespace fc {
 namespace {
 
 constexpr int TC_WBUF = 64;   // candidates of a warp's buffer
-// Lists from this length on are worth waiting (at most 20 us) for the first
-// threshold over all CTAs: 40,000 SNPs x 2,048 samples with lists of 2048 took
-// 8.6 ms with slow merges and no wait, 7.5 now, and 7.1 with lists of 128.
-constexpr int TC_LONG_LIST = 512;
-constexpr long long TC_FIRST_THRESHOLD_TICKS = 40000;
 
 // 8 consecutive FP32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8])
@@ -217,8 +212,8 @@ __device__ __noinline__ int merge_candidates(float *ls, uint64_t *lr, int L, int
 
 // A score that at least L combinations reach, from what the CTAs of the
 // launch have published (pub[n]: the score of the list's entry m - 1 as an
-// ordered int): the r-th largest, r m >= L, to 20 bits downwards.  All lanes
-// of a warp; n <= 32 TC_PUB_PER_LANE.
+// ordered int): the r-th largest, r m >= L, to 20 bits downwards; -FLT_MAX while
+// fewer than r have.  All lanes of a warp; n <= 32 TC_PUB_PER_LANE.
 constexpr int TC_PUB_PER_LANE = 8;
 __device__ __noinline__ float published_threshold(const int *pub, int n, int r, int lane)
 {
@@ -236,8 +231,9 @@ __device__ __noinline__ float published_threshold(const int *pub, int n, int r, 
         for (int x = 0; x < TC_PUB_PER_LANE; ++x) cnt += __popc(__ballot_sync(FULL, key[x] >= c));
         if (cnt >= r) t = c;
     }
-    const float f = from_ordered((int)(t ^ 0x80000000u));
-    return f >= -FLT_MAX ? f : -FLT_MAX;   // (NaN patterns of nothing published)
+    // Below r lists t is the key of the value set before the launch, 0x80808080,
+    // to 20 bits.
+    return t > 0x00808000u ? from_ordered((int)(t ^ 0x80000000u)) : -FLT_MAX;
 }
 
 }  // namespace

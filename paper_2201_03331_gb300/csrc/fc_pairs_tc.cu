@@ -411,14 +411,12 @@ __global__ void __launch_bounds__(T2_THREADS, 1) k_pairs_tc(const __grid_constan
         int cnt = 0;
         float thr_s = -FLT_MAX;
         uint64_t thr_r = NO_RANK;
-        bool waited = false;
         // The least score of a candidate by now: that of the list's last entry
         // (which only rises; a racy read is a score it had at some time), and
         // the one that enough pairs of all CTAs are known to reach.
         auto floor_score = [&]() -> float {
             return fmaxf(*(volatile float *)(lscore + L - 1), *(volatile float *)&threshold);
         };
-        auto known = [&]() -> bool { return *(volatile float *)&threshold > -FLT_MAX; };
         auto merge = [&]() {
             // Sorted outside the lock, against the list's last score then.
             const float racy = *(volatile float *)(lscore + L - 1);
@@ -459,13 +457,6 @@ __global__ void __launch_bounds__(T2_THREADS, 1) k_pairs_tc(const __grid_constan
                     atomicExch(&list_lock, 0);
                 }
             }
-            __syncwarp();
-            if (waited || L < TC_LONG_LIST) return;
-            // A merge into a long list costs microseconds: after its first
-            // one a warp waits a little for the threshold over all CTAs.
-            waited = true;
-            const long long t0 = clock64();
-            while (clock64() - t0 < TC_FIRST_THRESHOLD_TICKS && !known()) __nanosleep(200);
             __syncwarp();
         };
         // hs + (t(c), t(d)) for two packed cells c, d (a | b << 16, times 2^SH).

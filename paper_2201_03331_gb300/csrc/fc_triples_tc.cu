@@ -468,7 +468,6 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         int cnt = 0;
         float thr_s = -FLT_MAX;
         uint64_t thr_r = NO_RANK;
-        bool waited = false;
         // The least score of a candidate by now: that of the list's last entry
         // (which only rises; a racy read is a score it had at some time), and
         // the one that enough combinations of all CTAs are known to reach.
@@ -477,7 +476,6 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             return (int)(t2 >> 32) == cur_job ? __uint_as_float((uint32_t)t2) : -FLT_MAX;
         };
         auto floor_score = [&]() -> float { return fmaxf(*(volatile float *)(lscore + L - 1), published()); };
-        auto known = [&]() -> bool { return published() > -FLT_MAX; };
         auto merge = [&]() {
             // Sorted outside the lock, against the list's last score then.
             const float racy = *(volatile float *)(lscore + L - 1);
@@ -518,13 +516,6 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     atomicExch(&list_lock, 0);
                 }
             }
-            __syncwarp();
-            if (BATCH || waited || L < TC_LONG_LIST) return;
-            // A merge into a long list costs microseconds: after its first
-            // one a warp waits a little for the threshold over all CTAs.
-            waited = true;
-            const long long t0 = clock64();
-            while (clock64() - t0 < TC_FIRST_THRESHOLD_TICKS && !known()) __nanosleep(200);
             __syncwarp();
         };
         // All epilogue warps meet, unless a wait ran out in some role.
