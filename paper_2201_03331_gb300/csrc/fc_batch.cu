@@ -516,12 +516,14 @@ int plan_batch(fc_handle *h, int k, int64_t top_n)
     B.tc3_slot.assign(n_all, -1);
     const char *btc = getenv("FC_BATCH_TC");
     const bool tc_on = k == 3 && !(btc && strcmp(btc, "0") == 0);
+    int n_short = 0;
+    for (const auto &j : h->jobs) n_short += j->S < 384 && j->Wt < 5;
     for (int j = 0; j < n_all; ++j) {
         Dataset &d = *h->jobs[j];
         if (tc_on) {
             d.allow_tc = true;
             // Smaller jobs share one launch of the persistent sweep.
-            B.tc[j] = d.triples_tc_eligible(L, TRIPLES_TC_MIN_SNPS_BATCH) ? 1 : 0;
+            B.tc[j] = d.triples_tc_eligible(L, triples_tc_min_snps_batch(d.Wt, n_short)) ? 1 : 0;
             d.allow_tc = false;
         }
         if (!B.tc[j]) B.sel.push_back(j);

@@ -37,9 +37,18 @@ constexpr int64_t TRIPLES_TC_MIN_SNPS = 192;
 // Of a rank range, which may be a small part of the search: a 64th of 250 SNPs x
 // 2,000 samples, top 1,000, takes 921 us in the sweep and 1,044 there.
 constexpr int64_t TRIPLES_TC_MIN_SNPS_RANGE = 384;
-// Of a batch's jobs (smaller ones share one launch of the persistent sweep, where
-// eight jobs of 300 SNPs x 7,026 samples took 46 ms).
-constexpr int64_t TRIPLES_TC_MIN_SNPS_BATCH = 256;
+// Of a batch's jobs of Wt 128-sample words; n: its jobs of fewer than 384 SNPs and
+// five words.  The others share one launch of the persistent sweep, which takes
+// 4 to 5 ms however few they are, and with many jobs about 28 + 7 Wt ps a combination;
+// the tensor kernel takes about 5 + 15,000 / S ps a combination of S SNPs.  Sweep and
+// tensor cores, ms: 256 SNPs, two words, 8 jobs 4.7 and 1.7, 48 jobs 8.5 and 8.7,
+// 200 jobs 26 and 35; 383 SNPs, two words, 48 jobs 21 and 20, 200 jobs 76 and 81;
+// 200 jobs of three words, 320 SNPs 54.0 and 54.9, 352 SNPs 70 and 67; of four words,
+// 256 SNPs 34.9 and 35.3, 288 SNPs 47.2 and 44.3; of six, 256 SNPs 44 and 36.
+constexpr int64_t triples_tc_min_snps_batch(int Wt, int n)
+{
+    return n < 48 || Wt >= 5 ? 256 : Wt == 4 ? 288 : Wt == 3 ? 352 : 384;
+}
 int pow2_at_least(int v);
 // 2-D TMA descriptor over bytes: rows of inner_bytes (pitch apart), boxes of
 // 128 bytes x box_rows.
