@@ -110,6 +110,12 @@ struct PackArgs {
     uint32_t *err;          // error word
     int64_t *class_count;   // [2] cases, controls
 };
+// Lets launches of kernel fn take `bytes` of dynamic shared memory.  The limit is
+// one value per kernel and device, for all threads of the process, and a launch
+// above it is refused: it is only ever raised (setting every launch's own size,
+// four threads with lists of 64 to 2048 refused each other's launches).
+cudaError_t allow_dynamic_smem(const void *fn, size_t bytes);
+
 cudaError_t launch_class_index(const PackArgs &a, cudaStream_t st);
 cudaError_t launch_pack(const PackArgs &a, int64_t M1, int64_t M0, cudaStream_t st);
 cudaError_t launch_logtab(float *logtab, int64_t M, cudaStream_t st);

@@ -709,7 +709,7 @@ cudaError_t launch_pairs_tc(int mode, const CUtensorMap &tmapI, const CUtensorMa
                                           : reinterpret_cast<void *>(&k_pairs_tc<MODE_TOPN, 0>))
                                  : (a.enc ? reinterpret_cast<void *>(&k_pairs_tc<MODE_DUMP, 1>)
                                           : reinterpret_cast<void *>(&k_pairs_tc<MODE_DUMP, 0>));
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_dynamic_smem(fn, bytes);
     if (e != cudaSuccess) return e;
     CUtensorMap mI = tmapI, mJ = tmapJ;
     PairsArgs args = a;

@@ -753,7 +753,7 @@ cudaError_t launch_quads_tc(int k, int mode, const CUtensorMap &tmapL, const CUt
     if (k == 5) fn = quads_kernel<2, 3>(mode, a.enc);
     if (k == 6) fn = quads_kernel<3, 3>(mode, a.enc);
     if (!fn) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_dynamic_smem(fn, bytes);
     if (e != cudaSuccess) return e;
     CUtensorMap mL = tmapL, mR = tmapR;
     QuadsArgs args = a;

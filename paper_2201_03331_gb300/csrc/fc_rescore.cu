@@ -360,7 +360,7 @@ cudaError_t launch_rescore(const RescoreArgs &a, int sms, cudaStream_t st)
 cudaError_t launch_final(const RescoreArgs &a, cudaStream_t st)
 {
     const size_t bytes = (size_t)a.L * 20;
-    cudaError_t e = cudaFuncSetAttribute(k_final, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(&k_final), bytes);
     if (e != cudaSuccess) return e;
     k_final<<<1, FINAL_THREADS, bytes, st>>>(a);
     return cudaGetLastError();
@@ -376,7 +376,7 @@ cudaError_t launch_rescore_batch(const RescoreBatchArgs &a, cudaStream_t st)
 
 cudaError_t prepare_final_sort_batch(int L)
 {
-    return cudaFuncSetAttribute(k_final_sort_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, L * 16);
+    return allow_dynamic_smem(reinterpret_cast<const void *>(&k_final_sort_batch), (size_t)L * 16);
 }
 
 cudaError_t launch_final_sort_batch(const JobDesc *jobs, int n_jobs, double *res_s, uint64_t *res_r, int L,

@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -150,6 +151,23 @@ void fault_counters_reset()
 {
     g_alloc_count = 0;
     g_launch_count = 0;
+}
+
+// ---- shared memory of kernels ----------------------------------------------
+
+cudaError_t allow_dynamic_smem(const void *fn, size_t bytes)
+{
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, size_t> limits;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t &limit = limits[{fn, dev}];
+    // (Set again each time: a reset of the device forgets it.)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(limit, bytes));
+    if (e == cudaSuccess) limit = std::max(limit, bytes);
+    return e;
 }
 
 // ---- device selection ------------------------------------------------------

@@ -1040,8 +1040,7 @@ int search_max_blocks_per_sm(int k, const TuneConfig &cfg, int mode, int L, int 
     if (!fn) return 0;
     const size_t bytes = search_smem_bytes(k, var, cfg.NW, cfg.WT, (mode == MODE_TOPN || mode == MODE_BATCH) ? L : 0, M);
     if (smem) *smem = bytes;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-        return 0;
+    if (allow_dynamic_smem(fn, bytes) != cudaSuccess) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, cfg.NW * 32, bytes) != cudaSuccess) return 0;
     return nb;
@@ -1055,7 +1054,7 @@ cudaError_t launch_search(int k, const TuneConfig &cfg, int mode, const SearchAr
     if (!fn) return cudaErrorInvalidValue;
     const size_t bytes = search_smem_bytes(k, var, cfg.NW, cfg.WT, mode == MODE_TOPN ? a.L : 0, a.M);
     if (smem_out) *smem_out = bytes;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_dynamic_smem(fn, bytes);
     if (e != cudaSuccess) return e;
     SearchArgs args = a;
     int NW = cfg.NW, WT = cfg.WT;
@@ -1092,7 +1091,7 @@ cudaError_t launch_merge(const float *in_s, const uint64_t *in_r, int nlists, in
     const int F = std::max(2, std::min(nlists, std::min(SEL_MAX / L, std::max(16, 4096 / L))));
     const int blocks = (nlists + F - 1) / F;
     const size_t bytes = (size_t)F * L * 4 + (size_t)2 * L * 12;
-    cudaError_t e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(&k_select), bytes);
     if (e != cudaSuccess) return e;
     k_select<<<blocks, SEL_THREADS, bytes, st>>>(in_s, in_r, nlists, L, F, out_s, out_r);
     *nout = blocks;
@@ -1101,7 +1100,7 @@ cudaError_t launch_merge(const float *in_s, const uint64_t *in_r, int nlists, in
 
 cudaError_t prepare_merge_jobs(int n2)
 {
-    return cudaFuncSetAttribute(k_merge_jobs, cudaFuncAttributeMaxDynamicSharedMemorySize, n2 * 12);
+    return allow_dynamic_smem(reinterpret_cast<const void *>(&k_merge_jobs), (size_t)n2 * 12);
 }
 
 cudaError_t launch_merge_jobs(const JobDesc *jobs, int n_jobs, const float *item_s, const uint64_t *item_r, int L,

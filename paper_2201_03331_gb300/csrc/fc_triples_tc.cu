@@ -949,7 +949,7 @@ cudaError_t prepare_triples_tc_batch(int enc, size_t smem_bytes)
 {
     if (enc != 0 && enc != 1) return cudaErrorInvalidValue;
     void *fn = enc == 1 ? kernel_ptr<MODE_TOPN, 1, true>() : kernel_ptr<MODE_TOPN, 0, true>();
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem_bytes - TC_STATIC_SMEM));
+    return allow_dynamic_smem(fn, smem_bytes - TC_STATIC_SMEM);
 }
 
 cudaError_t launch_triples_tc(int mode, const CUtensorMap &tmapA, const CUtensorMap &tmapP, const TriplesArgs &a,
@@ -966,7 +966,7 @@ cudaError_t launch_triples_tc(int mode, const CUtensorMap &tmapA, const CUtensor
                                : (a.enc ? kernel_ptr<MODE_DUMP, 1, false>() : kernel_ptr<MODE_DUMP, 0, false>());
     }
     if (set_attr) {
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        const cudaError_t e = allow_dynamic_smem(fn, bytes);
         if (e != cudaSuccess) return e;
     }
     if (grid <= 0) return cudaSuccess;   // attributes only
