@@ -181,17 +181,17 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
         st.job = j;
         st.enc = x.triples_form(L);
         st.M = x.M;
-        st.stages = triples_stages((int)st.M, L, (size_t)lead.max_smem_optin);
-        if (st.enc < 0 || st.stages == 0) continue;
+        if (st.enc < 0) continue;
+        st.shape = triples_shape(st.enc, (int)st.M, L, (size_t)lead.max_smem_optin);
         T->slots.push_back(st);
         maxM = std::max(maxM, st.M);
         minM = std::min(minM, st.M);
     }
     if (T->slots.empty()) return FC_OK;
     T->scale = triples_scale(minM);
-    // A launch takes one form and one stage count (its x log2 x table spans
-    // its most samples): one-accumulator jobs first, then by stages.
-    auto key = [](const Tc3Batch::Slot &x) { return std::make_pair(-x.enc, -x.stages); };
+    // A launch takes one form and one shape of shared memory (its x log2 x table
+    // spans its most samples): one-accumulator jobs first, then by shape.
+    auto key = [](const Tc3Batch::Slot &x) { return std::make_tuple(-x.enc, -x.shape.stages, -x.shape.wbuf); };
     std::stable_sort(T->slots.begin(), T->slots.end(),
                      [&](const Tc3Batch::Slot &a, const Tc3Batch::Slot &b) { return key(a) < key(b); });
 
@@ -364,7 +364,7 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
                                items + ss.ntiles > ((int64_t)1 << 30)))
                 close(x);
             cur.enc = ss.enc;
-            cur.stages = ss.stages;
+            cur.shape = ss.shape;
             cur.M = std::max(cur.M, (int)ss.M);
             ss.slab_off = used;
             used += slab_bytes[(size_t)x];
@@ -483,7 +483,8 @@ TriplesArgs tc3_args(const Tc3Batch &T, const Tc3Batch::Launch &ln, int g)
     a.scale = T.scale;
     a.M = ln.M;
     a.L = T.L;
-    a.stages = ln.stages;
+    a.stages = ln.shape.stages;
+    a.wbuf = ln.shape.wbuf;
     a.wait_ticks = TC_WAIT_TICKS;
     a.list_score = T.list_s;
     a.list_rank = T.list_r;
@@ -707,7 +708,7 @@ int plan_batch(fc_handle *h, int k, int64_t top_n)
         // Each form's kernel takes the shared memory of its largest launch.
         size_t bytes[2] = {0, 0};
         for (const Tc3Batch::Launch &ln : T->launches)
-            bytes[ln.enc] = std::max(bytes[ln.enc], triples_smem_bytes(ln.stages, ln.M, T->L));
+            bytes[ln.enc] = std::max(bytes[ln.enc], triples_smem_bytes(ln.enc, ln.shape.stages, ln.shape.wbuf, ln.M, T->L));
         for (int enc = 0; enc <= 1; ++enc)
             if (bytes[enc] && (e = prepare_triples_tc_batch(enc, bytes[enc])) != cudaSuccess)
                 return cuda_status(e, "batched order-3 attributes");

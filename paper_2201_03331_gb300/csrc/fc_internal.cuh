@@ -349,7 +349,7 @@ struct TriplesArgs {
     int W0, Wt;             // 128-sample words: cases [0, W0), controls [W0, Wt)
     const uint4 *marg4;     // per-SNP genotype counts (one uint4 per SNP)
     const uint4 *PR;        // restricted pair table [S_pad][S_pad]
-    int stages;             // load stages (triples_stages)
+    int stages, wbuf;       // load stages, candidates of a warp's buffer (triples_shape)
     const float *xlogx;     // y log2 y, y = scale x, for x = 0..M (FP64 rounded once to FP32)
     float scale;            // the power of two the kernel scores counts in (triples_scale)
     int M;                  // extent of the kernel's table: the samples
@@ -375,10 +375,14 @@ struct TriplesArgs {
 // count, for n[0 .. count) (each modulo 2^23): of n times `scale`, a power of two,
 // or 1e-30 where n = 0; scale 0: of max(n, 1).
 cudaError_t launch_log2_approx(const uint32_t *n, int64_t count, float scale, float *out, cudaStream_t st);
-// The load stages that fit smem_cap bytes of shared memory beside the x log2 x
-// table of M samples and lists of L; 0 if not even two do.
-int triples_stages(int M, int L, size_t smem_cap);
-size_t triples_smem_bytes(int stages, int M, int L);
+// The load stages and the entries of a warp's candidate buffer that fit smem_cap
+// bytes of shared memory beside the x log2 x table of M samples and lists of L;
+// no stages if not even two do.
+struct TriplesShape {
+    int stages, wbuf;
+};
+TriplesShape triples_shape(int enc, int M, int L, size_t smem_cap);
+size_t triples_smem_bytes(int enc, int stages, int wbuf, int M, int L);
 // The power of two the kernel scores the counts of M samples in.
 float triples_scale(int64_t M);
 // pub_m and pub_r for lists of L and `grid` CTAs: pub_m pub_r >= L, pub_r at most

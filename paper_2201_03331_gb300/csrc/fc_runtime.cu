@@ -771,9 +771,9 @@ int Dataset::pairs_dense(float *scores, uint32_t *tables)
 int Dataset::triples_form(int L) const
 {
     const int64_t cls = std::max(M1, M0);
-    if (cls > 16383 || triples_stages((int)M, std::max(L, 1), (size_t)max_smem_optin) == 0) return -1;
     const char *f = getenv("FC_TRIPLES_ENC");
-    return !(f && strcmp(f, "0") == 0) && cls <= 4095 ? 1 : 0;
+    const int form = !(f && strcmp(f, "0") == 0) && cls <= 4095 ? 1 : 0;
+    return cls > 16383 || triples_shape(form, (int)M, std::max(L, 1), (size_t)max_smem_optin).stages == 0 ? -1 : form;
 }
 
 bool Dataset::triples_tc_eligible(int L, int64_t min_snps)
@@ -812,7 +812,9 @@ TriplesArgs Dataset::triples_args(int L, float hy, float invN)
     ta.rank_begin = 0;
     ta.rank_end = ~0ull;
     ta.L = std::max(L, 1);
-    ta.stages = triples_stages(ta.M, ta.L, (size_t)max_smem_optin);
+    const TriplesShape shape = triples_shape(enc3, ta.M, ta.L, (size_t)max_smem_optin);
+    ta.stages = shape.stages;
+    ta.wbuf = shape.wbuf;
     ta.wait_ticks = TC_WAIT_TICKS;
     return ta;
 }

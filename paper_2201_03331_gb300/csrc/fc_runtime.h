@@ -286,13 +286,13 @@ struct Tc3Batch {
         int j0 = 0, j1 = 0;          // slots [j0, j1)
         int enc = 1, n_items = 0;
         int M = 0;                   // largest sample count (x log2 x table size)
-        int stages = 2;
+        TriplesShape shape{};
     };
     struct Slot {
         int job = 0;
         int enc = 1;
         int64_t M = 0;               // its samples
-        int stages = 2;
+        TriplesShape shape{};
         int64_t slab_rows = 0;
         size_t slab_off = 0;         // within the slab buffer
         size_t e_off = 0;            // its SNP rows within E

@@ -121,10 +121,15 @@ static_assert(T3_STAGE % 1024 == 0, "swizzled stages");
 constexpr int T3_BUF = 2 * T3_N;                   // TMEM columns of a tile
 constexpr uint32_t T3_SCALE_COL = 2 * T3_BUF;      // TMEM column of scale 1, then of 4096, then of 4
 static_assert(T3_SCALE_COL + 3 * FP4_SCALE_COLS <= TC_TMEM_COLS, "scales behind the accumulators");
-constexpr int T3_WARP_PAIRS = 2 * ((2 * T3_NP / 2 + T3_PARTS - 1) / T3_PARTS);   // pairs of a tile per warp (ENC 1)
+__host__ __device__ constexpr int t3_warp_pairs(int enc)   // pairs of a tile per warp, at most
+{
+    return 2 * (((enc ? 2 : 1) * T3_NP / 2 + T3_PARTS - 1) / T3_PARTS);
+}
+constexpr int T3_WBUF_SHORT = 40;                  // a warp's buffer where one of TC_WBUF does not fit
+static_assert(T3_WBUF_SHORT > 32, "a round's 32 candidates fit after a merge");
 constexpr int T3_REC_WORDS = 12;                   // per pair: T01[9], rank base (2 words)
-static_assert(T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS % 4 == 0 && T3_REC_WORDS % 4 == 0, "records of uint4");
-static_assert(T3_WARP_PAIRS <= 32, "a lane per pair record");
+static_assert(T3_REC_WORDS % 4 == 0, "records of uint4");
+static_assert(t3_warp_pairs(1) <= 32, "a lane per pair record");
 
 __device__ __forceinline__ uint64_t c3(uint64_t n) { return n * (n - 1) * (n - 2) / 6; }   // 0 for n < 3
 __device__ __forceinline__ uint64_t c2(uint64_t n) { return n * (n - 1) / 2; }             // 0 for n < 2
@@ -137,6 +142,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     static_assert(!BATCH || MODE == MODE_TOPN, "the batched launch searches");
     constexpr bool PAIR = ENC == 1;                 // a tile per CTA pair
     constexpr int NPT = PAIR ? 2 * T3_NP : T3_NP;   // pairs per tile
+    constexpr int WPAIRS = t3_warp_pairs(ENC);
+    const int wbuf = PAIR ? TC_WBUF : a.wbuf;       // candidates of a warp's buffer
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[T3_MAX_STAGES], bar_empty[T3_MAX_STAGES];
     __shared__ uint64_t bar_tfull[2], bar_tempty[2], bar_done, bar_epi;
@@ -165,9 +172,9 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     float *xltab = reinterpret_cast<float *>(smem_raw);
     uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)(xltab + a.M + 1) + 1023) & ~(uintptr_t)1023);
     uint32_t *recs = reinterpret_cast<uint32_t *>(smem + (size_t)stages * T3_STAGE);
-    uint64_t *lrank = reinterpret_cast<uint64_t *>(recs + T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS);
+    uint64_t *lrank = reinterpret_cast<uint64_t *>(recs + T3_EPI_WARPS * WPAIRS * T3_REC_WORDS);
     uint64_t *wrank = lrank + a.L;
-    float *lscore = reinterpret_cast<float *>(wrank + T3_EPI_WARPS * TC_WBUF);
+    float *lscore = reinterpret_cast<float *>(wrank + T3_EPI_WARPS * wbuf);
     float *wscore = lscore + a.L;
 
     if (threadIdx.x == 0) {
@@ -455,9 +462,9 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         const int g = lane & 1;                            // genotype of this lane's row
         const uint32_t tempty0 = PAIR ? cluster_addr(&bar_tempty[0], 0) : 0;
         const int L = a.L;
-        float *ws = wscore + ew * TC_WBUF;
-        uint64_t *wr = wrank + ew * TC_WBUF;
-        uint32_t *rec = recs + ew * (T3_WARP_PAIRS * T3_REC_WORDS);
+        float *ws = wscore + ew * wbuf;
+        uint64_t *wr = wrank + ew * wbuf;
+        uint32_t *rec = recs + ew * (WPAIRS * T3_REC_WORDS);
         // The job of the tile (a batched launch reads the job's data again with
         // each tile: kept, they cost the scoring loop its registers).
         int cur_job = BATCH ? -1 : 0;
@@ -756,7 +763,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             }
                             cnt += __popc(mk);
                             __syncwarp();
-                            if (cnt > TC_WBUF - 32) merge();
+                            if (cnt > wbuf - 32) merge();
                         }
                     }
                 }
@@ -906,18 +913,22 @@ int triples_pairs_per_tile(int enc) { return enc ? 2 * T3_NP : T3_NP; }
 int triples_snps_per_tile(int enc) { return enc ? 2 * T3_LB : T3_LB; }
 int triples_block_rows() { return T3_N; }
 
-size_t triples_smem_bytes(int stages, int M, int L)
+size_t triples_smem_bytes(int enc, int stages, int wbuf, int M, int L)
 {
     // 1 KiB for the alignment of the stages.
-    return 1024 + TC_STATIC_SMEM + (size_t)(M + 1) * 4 + (size_t)stages * T3_STAGE + (size_t)T3_EPI_WARPS * T3_WARP_PAIRS * T3_REC_WORDS * 4 +
-           (size_t)(L + T3_EPI_WARPS * TC_WBUF) * (8 + 4);
+    return 1024 + TC_STATIC_SMEM + (size_t)(M + 1) * 4 + (size_t)stages * T3_STAGE +
+           (size_t)T3_EPI_WARPS * t3_warp_pairs(enc) * T3_REC_WORDS * 4 + (size_t)(L + T3_EPI_WARPS * wbuf) * (8 + 4);
 }
 
-int triples_stages(int M, int L, size_t smem_cap)
+TriplesShape triples_shape(int enc, int M, int L, size_t smem_cap)
 {
     for (int st = T3_MAX_STAGES; st >= 2; --st)
-        if (triples_smem_bytes(st, M, L) <= smem_cap) return st;
-    return 0;
+        if (triples_smem_bytes(enc, st, TC_WBUF, M, L) <= smem_cap) return {st, TC_WBUF};
+    // The longest lists beside the tables of the most samples (form 0 takes
+    // 2 x 16,383): shorter buffers.  400 SNPs x 32,766 samples, top 1,000, take 4.2
+    // ms (in the sweep 188).
+    if (!enc && triples_smem_bytes(0, 2, T3_WBUF_SHORT, M, L) <= smem_cap) return {2, T3_WBUF_SHORT};
+    return {0, 0};
 }
 
 float triples_scale(int64_t M)
@@ -955,8 +966,10 @@ cudaError_t prepare_triples_tc_batch(int enc, size_t smem_bytes)
 cudaError_t launch_triples_tc(int mode, const CUtensorMap &tmapA, const CUtensorMap &tmapP, const TriplesArgs &a,
                               int grid, cudaStream_t st, bool set_attr)
 {
-    const size_t bytes = triples_smem_bytes(a.stages, a.M, a.L) - TC_STATIC_SMEM;
-    if ((a.enc != 0 && a.enc != 1) || a.stages < 2 || a.stages > T3_MAX_STAGES) return cudaErrorInvalidValue;
+    const size_t bytes = triples_smem_bytes(a.enc, a.stages, a.wbuf, a.M, a.L) - TC_STATIC_SMEM;
+    if ((a.enc != 0 && a.enc != 1) || a.stages < 2 || a.stages > T3_MAX_STAGES || a.wbuf < T3_WBUF_SHORT ||
+        a.wbuf > TC_WBUF || (a.enc && a.wbuf != TC_WBUF))
+        return cudaErrorInvalidValue;
     void *fn = nullptr;
     if (a.jobs) {
         if (mode != MODE_TOPN) return cudaErrorInvalidValue;
