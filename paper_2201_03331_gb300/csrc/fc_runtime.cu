@@ -1548,7 +1548,8 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
         // A rank range takes the tiles of its first SNPs, and the kernel
         // drops the combinations outside the range.
         const bool tc3 = k == 3 && triples_tc_eligible(L, whole ? TRIPLES_TC_MIN_SNPS : TRIPLES_TC_MIN_SNPS_RANGE) &&
-                         (!no_alloc || triples_ready);
+                         (!no_alloc ||
+                          (triples_ready && triples_shape(enc3, (int)M, L, (size_t)max_smem_optin).stages > 0));
         // Orders 4-6: tensor-core contraction of tuple rows with tuple rows.
         // A rank range takes the tiles of the left blocks holding a left
         // tuple whose combinations meet the range, and the kernel drops the
@@ -1589,7 +1590,8 @@ int Dataset::search(int k, int64_t top_n, uint32_t *out_idx, double *out_score, 
             }
             grid = pairs_grid(pa.ntiles);
         } else if (tc3) {
-            int rc = prepare_triples(L);
+            // (Without allocating: the operands as built, in either form.)
+            int rc = no_alloc ? FC_OK : prepare_triples(L);
             if (rc) return rc;
             ta = triples_args(L, (float)hy, (float)(1.0 / Nd));
             ta.rank_begin = r0;

@@ -84,3 +84,20 @@ def test_around_2500_samples(fc, monkeypatch, k, S, kind, M, n):
         o_idx, o_s, _ = oracle.search(ds.genotypes, ds.phenotype, k, n)
         assert_topn_equal(a[0], a[1], o_idx, o_s, lambda c: float(
             oracle.mi(oracle.tables(ds.genotypes, ds.phenotype, k, [c]), k)[0]))
+
+
+def test_static_search_keeps_the_form_of_its_operands(fc, monkeypatch):
+    """fc_search_static takes the order-3 operands as they were built, in
+    whichever form, and allocates nothing."""
+    ds = make_dataset("form", seed=1560, S=200, cases=300, controls=330, k=3, top_n=20)
+    h = fc.fc_load(ds.genotypes, ds.phenotype)
+    want = fc.fc_search(h, 3, 20)
+    for form in ("0", "1"):
+        monkeypatch.setenv("FC_TRIPLES_ENC", form)
+        monkeypatch.setenv("FC_FAULT_ALLOC_ALL", "1")
+        got = fc.fc_search_static(h, 3, 20)
+        assert fc.fc_last_search_kind(h) == 6
+        assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+        monkeypatch.delenv("FC_FAULT_ALLOC_ALL")
+        got = fc.fc_search(h, 3, 20)   # builds the operands of that form
+        assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
