@@ -349,7 +349,6 @@ Dataset::~Dataset()
     dev_free_pooled(tiles3, tiles3_bytes, device);
     dev_free_pooled(rowbase3, rowbase3_bytes, device);
     dev_free_pooled(P3, p3_bytes, device);
-    dev_free_pooled(E3, e3_bytes, device);
     if (ev_sweep0) cudaEventDestroy(ev_sweep0);
     if (ev_sweep1) cudaEventDestroy(ev_sweep1);
     if (own_stream && own_stream_handle) cudaStreamDestroy(own_stream_handle);
@@ -662,6 +661,32 @@ int Dataset::prepare_xlog2x()
                       [&](float *p) { return launch_xlogx(p, M, stream, true, triples_scale(M)); });
 }
 
+// The packed SNP rows, one copy for orders 2 and 3.
+int Dataset::prepare_rows()
+{
+    if (E) return FC_OK;
+    uint8_t *p = nullptr;
+    e_bytes = (size_t)triples_rows(S) * (size_t)triples_pitch(Wt);
+    cudaError_t e = dev_alloc_pooled((void **)&p, e_bytes, device);
+    if (e != cudaSuccess) return cuda_status(e, "packed SNP row allocation");
+    if ((e = launch_gate()) != cudaSuccess ||
+        (e = launch_expand_fp4(X, S, S_pad, Wt, triples_pitch(Wt), p, stream)) != cudaSuccess) {
+        dev_free_pooled(p, e_bytes, device);
+        return cuda_status(e, "packed SNP rows");
+    }
+    note_launches(1);
+    E = p;
+    return FC_OK;
+}
+
+// Gives the rows back once neither order's operands point at them.
+void Dataset::release_rows()
+{
+    if (pairs_ready || triples_ready) return;
+    dev_free_pooled(E, e_bytes, device);
+    E = nullptr;
+}
+
 int Dataset::prepare_pairs()
 {
     if (pairs_ready) return FC_OK;
@@ -669,12 +694,10 @@ int Dataset::prepare_pairs()
     enc2 = std::max(M1, M0) <= 4095 ? 1 : 0;
     int rc = prepare_xlog2x();
     if (rc || (rc = prepare_ie(2)) != FC_OK) return rc;
+    if ((rc = prepare_rows()) != FC_OK) return rc;
     const int64_t rows = triples_rows(S);
     const uint64_t kbytes = (uint64_t)Wt * 64, pitch = (uint64_t)triples_pitch(Wt);
     cudaError_t e;
-    e_bytes = (size_t)rows * pitch;
-    if ((e = dev_alloc_pooled((void **)&E, e_bytes, device)) != cudaSuccess)
-        return cuda_status(e, "packed SNP row allocation");
     const int64_t IB = pairs_rows_i(enc2), JB = pairs_rows_j(enc2);
     const int nI = (int)((S - 1 + IB - 1) / IB), nJ = (int)((S + JB - 1) / JB);
     std::vector<uint32_t> t;
@@ -694,10 +717,6 @@ int Dataset::prepare_pairs()
     if ((e = dev_alloc_pooled((void **)&tiles, tiles_bytes, device)) != cudaSuccess)
         return cuda_status(e, "tile list allocation");
     cudaMemcpyAsync(tiles, t.data(), sizeof(uint32_t) * t.size(), cudaMemcpyHostToDevice, stream);
-    if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E, stream)) != cudaSuccess)
-        return cuda_status(e, "pair operand preparation");
-    note_launches(1);
     if ((rc = encode_tmap_u8(&tmapI, E, kbytes, pitch, (uint64_t)rows, 128, true)) != FC_OK ||
         (rc = encode_tmap_u8(&tmapJ, E, kbytes, pitch, (uint64_t)rows, (uint32_t)pairs_block_rows(), true)) != FC_OK)
         return rc;
@@ -709,13 +728,12 @@ int Dataset::prepare_pairs()
 void Dataset::release_pairs()
 {
     if (stream) cudaStreamSynchronize(stream);
-    dev_free_pooled(E, e_bytes, device);
     dev_free_pooled(tiles, tiles_bytes, device);
-    E = nullptr;
     tiles = nullptr;
     ntiles = 0;
     tiles_host.clear();
     pairs_ready = false;
+    release_rows();
 }
 
 int Dataset::pairs_dense(float *scores, uint32_t *tables)
@@ -901,17 +919,10 @@ int Dataset::prepare_triples(int L)
     int rc = prepare_ie(3);
     if (rc) return rc;
     cudaError_t e;
-    if ((rc = prepare_xlog2x()) != FC_OK) return rc;
+    if ((rc = prepare_xlog2x()) != FC_OK || (rc = prepare_rows()) != FC_OK) return rc;
     const int64_t rows = triples_rows(S);
     const uint64_t kbytes = (uint64_t)Wt * 64;
     const uint64_t pitch = (uint64_t)triples_pitch(Wt);
-    e3_bytes = (size_t)rows * pitch;
-    if ((e = dev_alloc_pooled((void **)&E3, e3_bytes, device)) != cudaSuccess)
-        return cuda_status(e, "packed SNP row allocation");
-    if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_expand_fp4(X, S, S_pad, Wt, (int64_t)pitch, E3, stream)) != cudaSuccess)
-        return cuda_status(e, "packed SNP rows");
-    note_launches(1);
     const int NP = triples_pairs_per_tile(1);
     size_t cap = (size_t)16 << 30;
     if (const char *mb = getenv("FC_TRIPLES_SLAB_MB")) {
@@ -939,7 +950,7 @@ int Dataset::prepare_triples(int L)
         return cuda_status(e, "slab row table allocation");
     cudaMemcpyAsync(tiles3, tiles.data(), sizeof(uint4) * tiles.size(), cudaMemcpyHostToDevice, stream);
     cudaMemcpyAsync(rowbase3, plan->rowbase.data(), sizeof(int64_t) * (size_t)S, cudaMemcpyHostToDevice, stream);
-    if ((rc = encode_tmap_u8(&tmap3A, E3, kbytes, pitch, (uint64_t)rows, 128, true)) != FC_OK) return rc;
+    if ((rc = encode_tmap_u8(&tmap3A, E, kbytes, pitch, (uint64_t)rows, 128, true)) != FC_OK) return rc;
     if ((rc = encode_tmap_u8(&tmap3P, P3, kbytes, pitch, (uint64_t)plan->max_rows, (uint32_t)triples_block_rows(), true)) != FC_OK)
         return rc;
     built_slab3 = -1;
@@ -955,7 +966,7 @@ int Dataset::build_slab3(int s)
     const TripleSlab &sl = slabs3[(size_t)s];
     cudaError_t e;
     if ((e = launch_gate()) != cudaSuccess ||
-        (e = launch_pair_rows(E3, triples_pitch(Wt), Wt, S, sl.i0, sl.i1, rowbase3 + sl.i0, P3, stream)) != cudaSuccess)
+        (e = launch_pair_rows(E, triples_pitch(Wt), Wt, S, sl.i0, sl.i1, rowbase3 + sl.i0, P3, stream)) != cudaSuccess)
         return cuda_status(e, "pair-row kernel");
     note_launches(1);
     built_slab3 = s;
@@ -968,16 +979,15 @@ void Dataset::release_triples()
     dev_free_pooled(P3, p3_bytes, device);
     dev_free_pooled(tiles3, tiles3_bytes, device);
     dev_free_pooled(rowbase3, rowbase3_bytes, device);
-    dev_free_pooled(E3, e3_bytes, device);
     P3 = nullptr;
     tiles3 = nullptr;
     rowbase3 = nullptr;
-    E3 = nullptr;
     ntiles3 = 0;
     slabs3.clear();
     first_tile3.clear();
     built_slab3 = -1;
     triples_ready = false;
+    release_rows();
 }
 
 int Dataset::triples_dense(float *scores, uint32_t *tables)

@@ -90,12 +90,14 @@ struct Dataset {
     bool last_path_tc = false;
     int max_smem_optin = 0;
 
-    // Order-2 tensor-core operands, built on first use: E = packed SNP rows
-    // (row 2s+g for genotypes g = 0, 1; triples_rows), per-SNP genotype counts,
-    // the block-pair tile list, E's TMA descriptors (boxes of the SNPs i and j)
-    // and the form (PairsArgs::enc).
+    // Packed SNP rows of orders 2 and 3 on the tensor cores (row 2s+g for genotypes
+    // g = 0, 1; triples_rows), built by the first that asks and kept while
+    // either's operands point at them.
     uint8_t *E = nullptr;
     size_t e_bytes = 0;
+    // Order-2 tensor-core operands, built on first use: per-SNP genotype counts,
+    // the block-pair tile list, E's TMA descriptors (boxes of the SNPs i and j)
+    // and the form (PairsArgs::enc).
     uint16_t *marg = nullptr;
     uint32_t *tiles = nullptr;
     size_t tiles_bytes = 0;
@@ -105,12 +107,11 @@ struct Dataset {
     int enc2 = 0;
     bool pairs_ready = false;
 
-    // Order-3 tensor-core operands, built on first use: the packed SNP rows
-    // E3, slabs of pair rows (E3[i, a] AND E3[j, b], four rows per pair (i, j),
-    // from the pair (i, i + 1)) for consecutive ranges of
-    // first SNPs i, the tiles of every slab, each i's first row within its
-    // slab, the x log2 x table, and the kernel's two TMA descriptors (SNP
-    // rows, slab).  One slab is built once and kept; with several, each
+    // Order-3 tensor-core operands, built on first use: slabs of pair rows (E[i,
+    // a] AND E[j, b], four rows per pair (i, j), from the pair (i, i + 1)) for
+    // consecutive ranges of first SNPs i, the tiles of every slab, each i's
+    // first row within its slab, the x log2 x table, and the kernel's two TMA
+    // descriptors (SNP rows, slab).  One slab is built once and kept; with several, each
     // search rebuilds them in turn in the same buffer.
     struct TripleSlab {
         int64_t i0 = 0, i1 = 0;   // first SNPs [i0, i1)
@@ -121,7 +122,7 @@ struct Dataset {
     std::vector<int64_t> first_tile3;   // [S + 1] first tile of each first SNP
     float *xlogx = nullptr;   // x ln x, x = 0..M (the orders 4-6 epilogue's MI table)
     float *small_terms = nullptr;   // cell terms of small class counts (orders 4-6)
-    float *xlog2x = nullptr;  // of x = 0..M times triples_scale(M) (the order-3 epilogue's)
+    float *xlog2x = nullptr;  // of x = 0..M times triples_scale(M) (the epilogues of orders 2 and 3)
     uint8_t *P3 = nullptr;
     size_t p3_bytes = 0;
     uint4 *tiles3 = nullptr;
@@ -131,8 +132,6 @@ struct Dataset {
     size_t rowbase3_bytes = 0;
     int built_slab3 = -1;
     int enc3 = 0;             // form of the order-3 kernel (triples_form)
-    uint8_t *E3 = nullptr;    // packed SNP rows (triples_rows)
-    size_t e3_bytes = 0;
     CUtensorMap tmap3A{}, tmap3P{};
     bool triples_ready = false;
     bool last_path_tc3 = false;
@@ -223,6 +222,8 @@ struct Dataset {
     PairsArgs pairs_args(int L, float hy, float invN);
     int prepare_pairs();
     void release_pairs();
+    int prepare_rows();
+    void release_rows();
     int prepare_xlog2x();
     int pairs_grid(int n) const;   // CTAs for n order-2 tiles
     int pairs_dense(float *scores, uint32_t *tables);
