@@ -1108,6 +1108,12 @@ int64_t tuple_count(int64_t S, int T, int other)
 }
 }  // namespace
 
+// The candidate list of the orders 4-6 kernel: L entries and a buffer of at
+// least 512 (a tile adds up to 288), the rest of shared memory to the load
+// stages (three stages were 15 % slower than four, more than four made no
+// difference).
+static int tuples_list(int L) { return L > 0 ? pow2_at_least(L + 512) : 0; }
+
 bool Dataset::tuples_tc_eligible(int k, int L)
 {
     if (k < 4 || k > 6) return false;
@@ -1138,9 +1144,7 @@ bool Dataset::tuples_tc_eligible(int k, int L)
         if ((double)(bl / group + 1) * (double)rchunk * (double)((group + sub - 1) / sub) >= 2147483647.0)
             return false;
     }
-    const int Bcap = std::max(L, 1024);
-    const int P2 = pow2_at_least(L + Bcap);
-    return quads_smem_bytes(enc, 2, (int)M, P2) <= (size_t)max_smem_optin;
+    return quads_smem_bytes(enc, 2, (int)M, tuples_list(L)) <= (size_t)max_smem_optin;
 }
 
 // Right items per chunk of the orders 4-6 right slab (items: right blocks,
@@ -1253,10 +1257,7 @@ QuadsArgs Dataset::tuples_args(int k, int L, float hy, float invN)
     qa.rank_begin = 0;
     qa.rank_end = ~0ull;
     qa.L = L;
-    // A buffer of at least 512 candidates (a tile adds up to 288), the rest
-    // of shared memory to the load stages (three stages were 15 % slower than
-    // four, more than four made no difference).
-    qa.P2 = L > 0 ? pow2_at_least(L + 512) : 0;
+    qa.P2 = tuples_list(L);
     qa.Bcap = qa.P2 - L;
     qa.stages = 2;
     for (int st = TC_MAX_STAGES; st >= 2; --st)

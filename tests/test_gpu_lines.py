@@ -86,6 +86,19 @@ def test_around_2500_samples(fc, monkeypatch, k, S, kind, M, n):
             oracle.mi(oracle.tables(ds.genotypes, ds.phenotype, k, [c]), k)[0]))
 
 
+@pytest.mark.parametrize("M,tc", [(36223, True), (36224, True), (39295, True), (39296, False)])
+def test_order_4_at_its_sample_limit(fc, monkeypatch, M, tc):
+    """What fits is asked of the table and the list as they are launched."""
+    ds = make_dataset("most", seed=1550, S=64, cases=M // 2, controls=M - M // 2, k=4, top_n=10)
+    h = fc.fc_load(ds.genotypes, ds.phenotype)
+    a = fc.fc_search(h, 4, 10)
+    assert (fc.fc_last_search_kind(h) == 7) == tc
+    monkeypatch.setenv("FC_QUADS_PATH", "popc")
+    b = fc.fc_search(h, 4, 10)
+    assert fc.fc_last_search_kind(h) != 7
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
 def test_static_search_keeps_the_form_of_its_operands(fc, monkeypatch):
     """fc_search_static takes the order-3 operands as they were built, in
     whichever form, and allocates nothing."""
