@@ -210,6 +210,11 @@ int fc_load_batch(int n_data, const uint8_t *const *genotypes, const int64_t *S,
  * device queue, per-job lists are merged, rescored in FP64 and ordered on
  * the device.  The launch sequence is captured once per (k, top_n) as a CUDA
  * graph and replayed.  Results per job are those fc_search returns for it.
+ * At order 3 every job on the tensor cores has a slab of pair rows of its own
+ * (1,000 SNPs x 4,000 samples: 4.2 GB).  Where all fit in three quarters of the
+ * free memory less 8 GiB the handle keeps them until it is freed or searched
+ * with another (k, top_n); otherwise it keeps a buffer of that size and every
+ * search rebuilds them.  Environment FC_BATCH_SLAB_MB caps the buffer.
  *
  * out_idx   : host uint32 [jobs][top_n][k]
  * out_score : host double [jobs][top_n]

@@ -172,7 +172,6 @@ int plan_tc3(fc_handle *h, int L, int64_t top_n, std::unique_ptr<Tc3Batch> &out)
     std::unique_ptr<Tc3Batch> T(new Tc3Batch());
     T->L = L;
     T->grid = grid;
-    T->smem_cap = lead.max_smem_optin;
     int64_t maxM = 0, minM = INT64_MAX;
     for (int j = 0; j < (int)h->jobs.size(); ++j) {
         if (!B.tc[j]) continue;
@@ -851,9 +850,8 @@ int fc_load_batch(int n_data, const uint8_t *const *genotypes, const int64_t *S,
                 job->max_smem_optin = h->ds.max_smem_optin;
                 job->stream = st;
                 job->own_stream = false;
-                // Jobs are searched by the batched sweep; the per-job path
-                // runs the same sweep, and no job keeps a pair-row slab
-                // (many resident jobs could not each hold one).
+                // Tensor cores where the batch's plan allows them; a job of its
+                // own keeps no pair-row slab.
                 job->allow_tc = false;
                 rc = job->load(dG, dph + (size_t)r * M[d], S[d], M[d]);
                 if (rc) {
@@ -963,7 +961,7 @@ int fc_search_batch(fc_handle *h, int k, int64_t top_n, uint32_t *out_idx, doubl
                     rc = d.search(k, top_n, oi, os, &out_count[j]);
                     d.allow_tc = false;
                     d.release_triples();
-                                if (rc) return rc;
+                    if (rc) return rc;
                     B.job_kind[j] = d.last_path_tc3 ? 6 : (d.last_sweep_var == VAR_IE ? 3 : d.last_sweep_var == VAR_JR ? 4 : 1);
                     continue;
                 }
@@ -995,7 +993,7 @@ int fc_search_batch(fc_handle *h, int k, int64_t top_n, uint32_t *out_idx, doubl
             rc = d.search(k, top_n, out_idx + (size_t)j * top_n * k, out_score + (size_t)j * top_n, &out_count[j]);
             d.allow_tc = false;
             d.release_triples();
-                if (rc) return rc;
+            if (rc) return rc;
             B.job_kind[j] = d.last_path_tc3 ? 6 : (d.last_sweep_var == VAR_IE ? 3 : d.last_sweep_var == VAR_JR ? 4 : 1);
             if (lead.timing) {
                 lead.sweep_ms += d.sweep_ms;

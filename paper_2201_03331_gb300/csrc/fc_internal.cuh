@@ -34,10 +34,10 @@ __host__ __device__ inline uint64_t binom(int64_t n, int r)
     // variable takes some 70 instructions, and a rank is turned into its
     // combination by up to 30 of these.
     uint64_t c = 1;
+    static_assert(KMAX_TABLES <= 6, "r is at most the order");
 #pragma unroll
     for (int i = 1; i <= 6; ++i)
         if (i <= r) c = c * (uint64_t)(n - r + i) / (uint64_t)i;
-    for (int i = 7; i <= r; ++i) c = c * (uint64_t)(n - r + i) / (uint64_t)i;
     return c;
 }
 
@@ -122,9 +122,9 @@ cudaError_t launch_logtab(float *logtab, int64_t M, cudaStream_t st);
 // y ln y (base2: y log2 y), y = scale x, for x = 0..M, each the FP64 product
 // rounded once.
 cudaError_t launch_xlogx(float *t, int64_t M, cudaStream_t st, bool base2 = false, double scale = 1.0);
-// t(a, b) = a log(n/a) + b log(n/b), n = a + b (base2: in bits), for a, b < n_max
-// at b stride + a, each rounded once; 0 in the rest of `floats` entries.
-cudaError_t launch_small_terms(float *t, int n_max, int stride, int floats, bool base2, cudaStream_t st);
+// t(a, b) = a ln(n/a) + b ln(n/b), n = a + b, for a, b < n_max at b stride + a, each
+// rounded once; 0 in the rest of `floats` entries.
+cudaError_t launch_small_terms(float *t, int n_max, int stride, int floats, cudaStream_t st);
 
 struct SearchArgs {
     const uint4 *X;

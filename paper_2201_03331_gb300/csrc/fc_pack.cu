@@ -110,9 +110,9 @@ __global__ void k_xlogx(float *t, int64_t M, bool base2, double scale)
     if (n <= M) t[n] = n == 0 ? 0.0f : (float)(y * (base2 ? log2(y) : log(y)));
 }
 
-// t(a, b) = a log(n/a) + b log(n/b), n = a + b, for a, b < n_max at b stride + a
-// (base2: in bits), in FP64 rounded once; 0 elsewhere.
-__global__ void k_small_terms(float *t, int n_max, int stride, int floats, bool base2)
+// t(a, b) = a ln(n/a) + b ln(n/b), n = a + b, for a, b < n_max at b stride + a, in
+// FP64 rounded once; 0 elsewhere.
+__global__ void k_small_terms(float *t, int n_max, int stride, int floats)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= floats) return;
@@ -120,16 +120,16 @@ __global__ void k_small_terms(float *t, int n_max, int stride, int floats, bool 
     double v = 0.0;
     if (a < n_max && b < n_max && a > 0 && b > 0) {
         const double n = a + b;
-        v = base2 ? (double)a * log2(n / a) + (double)b * log2(n / b) : (double)a * log(n / a) + (double)b * log(n / b);
+        v = (double)a * log(n / a) + (double)b * log(n / b);
     }
     t[i] = (float)v;
 }
 
 }  // namespace
 
-cudaError_t launch_small_terms(float *t, int n_max, int stride, int floats, bool base2, cudaStream_t st)
+cudaError_t launch_small_terms(float *t, int n_max, int stride, int floats, cudaStream_t st)
 {
-    k_small_terms<<<(floats + 255) / 256, 256, 0, st>>>(t, n_max, stride, floats, base2);
+    k_small_terms<<<(floats + 255) / 256, 256, 0, st>>>(t, n_max, stride, floats);
     return cudaGetLastError();
 }
 

@@ -723,7 +723,7 @@ int quads_small_floats() { return T4_SMALL_FLOATS; }
 
 cudaError_t launch_quads_small_terms(float *t, cudaStream_t st)
 {
-    return launch_small_terms(t, T4_SMALL, T4_SMALL_STRIDE, T4_SMALL_FLOATS, false, st);
+    return launch_small_terms(t, T4_SMALL, T4_SMALL_STRIDE, T4_SMALL_FLOATS, st);
 }
 
 size_t quads_smem_bytes(int enc, int stages, int M, int P2)

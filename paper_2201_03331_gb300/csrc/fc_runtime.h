@@ -16,8 +16,8 @@ int set_error(int status, const char *fmt, ...);
 int cuda_status(cudaError_t e, const char *what);
 cudaError_t dev_alloc(void **p, size_t bytes);
 // Operand buffers rebuilt per data set or per search (pair-row and
-// tuple-row slabs, packed rows, tile lists): a freed buffer of 4 KB or more is
-// kept in a small per-process pool and handed to the next request that it
+// tuple-row slabs, packed rows, tile lists): a freed buffer is kept in a small
+// per-process pool and handed to the next request that it
 // fits (at most twice its size), so that searching data sets one after
 // another neither maps and unmaps gigabytes nor pays cudaFree's implicit
 // device synchronization each time.  The caller has synchronized every
@@ -302,7 +302,7 @@ struct Tc3Batch {
     std::vector<Slot> slots;
     std::vector<Launch> launches;
     std::vector<int> slot_job;       // job index of every slot
-    int n = 0, L = 0, grid = 0, smem_cap = 0;
+    int n = 0, L = 0, grid = 0;
     int level1 = 0, F = 0;           // two-level merge: groups of F lists per job
     bool rebuild = false;            // slabs rebuilt before every launch (several groups)
     std::vector<void *> allocs;      // device allocations of the plan
