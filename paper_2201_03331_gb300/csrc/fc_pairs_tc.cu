@@ -37,14 +37,15 @@
 // second (t <= n) by 1, the four levels of additions by 4; ln 2, its product, 1/N,
 // H(Y) and the last multiply-add add 5: 39.2 u ln 2 < 28 u in nats.
 //
-// What bounds the kernel: with many samples the operands' way from L2 (60 KB a
-// chunk and tile; 12,000 SNPs x 8,192 samples move 20 GB at 14.5 TB/s, the
-// tensor pipe 33 % active), with few the scoring.  40,000 SNPs x 8,192 samples,
-// lists of 2048: 13.1 ms, x 2,048 samples: 7.5 ms.  (The kernel before, byte rows
-// in 128 x 128 tiles of one CTA and four epilogue warps that met at barriers
-// and sorted a shared buffer of candidates, took 37 ms for the first, and 15 of
-// the 16 ms of a search of 12,001 SNPs x 2,987 samples met once, now 1.5: it
-// sorted after nearly every 16 SNPs while its list filled.)
+// What bounds the kernel: with many samples the operands' way from L2 (30 KB a
+// chunk and CTA; 12,000 SNPs x 8,192 samples, form 0, move 20 GB at 15 TB/s, the
+// tensor pipe 37 % active, 1.6 instructions a cycle), with few the scoring.
+// 40,000 SNPs x 8,192 samples, lists of 2048: 12.9 ms, x 2,048 samples: 7.1 ms; a
+// search with its tail 13.1 and 7.3.  (The kernel before, byte rows in 128 x 128
+// tiles of one CTA and four epilogue warps that met at barriers and sorted a
+// shared buffer of candidates, took 37 ms for the first, and 15 of the 16 ms of
+// a search of 12,001 SNPs x 2,987 samples met once, now 1.6: it sorted after
+// nearly every 16 SNPs while its list filled.)
 //
 // TMEM lane 2 i + g holds genotype g of SNP i, columns 2 j + h genotype h of SNP
 // j.  The two lanes of a SNP i take two SNPs j at a time, one each: they

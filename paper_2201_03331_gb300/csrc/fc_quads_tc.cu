@@ -30,7 +30,11 @@
 // holds a larger count; the others take three reads of a table of x ln x.
 // (A 64 x 64 table leaves room for two more load stages, but at 2,048
 // samples more cells are above it: order 4, a 64th of 1,001 SNPs, 57.7 ms
-// against 46.9; order 5 at 152 SNPs 120 against 112.)
+// against 46.9; order 5 at 152 SNPs 120 against 112.)  What bounds the kernel is
+// the tensor pipe (74 % active at order 4, 120 SNPs x 6,000 samples, operands at
+// 14.5 TB/s from L2) and with few samples the epilogue: 300 SNPs x 6,000 samples
+// take 53.7 ms, that 64th of 1,001 SNPs 46.0, orders 5 and 6 at 152 and 76 SNPs
+// x 2,048 samples 111 and 113.
 // The accumulator n_case + 4096 n_ctrl plus 2^21 holds four times the packed
 // counts in its mantissa, so the table offset 4 a + 532 b takes a shift and a
 // multiply-add.  Each thread sums the terms of its row's cells, the 3^LT lanes

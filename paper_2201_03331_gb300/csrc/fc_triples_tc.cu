@@ -26,14 +26,16 @@
 //            a tile of 64 SNPs and 28 pairs per CTA (M = 128, N = 112).
 // Either way a CTA's stage is 128 + 112 rows, a tile takes 224 TMEM columns,
 // and two tiles are in flight.  What bounds the kernel is the scoring, about
-// 400 instructions per 32 combinations: 1,000 SNPs x 4,000 samples take 5.3 ms
-// (5.9 with byte rows and both genotypes of a SNP from different tiles), of
-// which the tiles alone are 1.9 ms, the logarithms 0.95, the table reads 0.86
-// and the exchange of the cells 0.45.  (One CTA per 128 x 24 tile with both
-// genotypes of a SNP in one lane needed no exchange of cells, but 1,000 bytes
-// of shared memory per combination against about 530 here: 5.2 ms there, but
-// 3.9 ms instead of 2.9 at 701 SNPs x 9,001 samples, 6.5 before.  12 epilogue
-// warps with more registers: 5.5 and 3.2 ms.)
+// 400 instructions per 32 combinations: 1,000 SNPs x 4,000 samples take 4.56 ms,
+// 701 x 9,001 2.49, a search with its tail 4.7 and 2.6 (5.9 and 6.5 with byte rows
+// and both genotypes of a SNP from different tiles); at 500 SNPs 1.8 instructions
+// are issued a cycle and the tensor pipe is 31 % active.  Parts left out, when the
+// first search took 5.3 ms (its selection and merges were slower): the tiles alone
+// were 1.9 ms, the logarithms 0.95, the table reads 0.86 and the exchange of the
+// cells 0.45.  (One CTA per 128 x 24 tile with both genotypes of a SNP in one lane
+// needed no exchange of cells, but 1,000 bytes of shared memory per combination
+// against about 530 here: 5.2 ms then, but 3.9 ms instead of 2.9 for the second.
+// 12 epilogue warps with more registers: 5.5 and 3.2 ms.)
 //
 // The pair rows live in a slab in device memory, the paper's `combine` of
 // two genotype tables done once per data set (k_pair_rows): for each first
