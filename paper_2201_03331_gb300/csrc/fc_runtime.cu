@@ -1155,7 +1155,7 @@ bool Dataset::tuples_tc_eligible(int k, int L)
 // what the rows take), so that a setting gives the chunks it always gave.
 // The search then builds each chunk's right rows in turn and runs the
 // chunk's tiles (the paper's order-5 and order-6 runs on one node, 561 and
-// 223 variants, need 2 TB and 122 GB of right rows at 2048 samples).
+// 223 variants, need 0.93 TB and 56 GB of right rows at 2048 samples).
 int64_t Dataset::tuple_right_chunk(int k) const
 {
     const int LT = tc_left_size(k), RT = k - LT;
