@@ -38,6 +38,7 @@ int set_error(int status, const char *fmt, ...)
 int cuda_status(cudaError_t e, const char *what)
 {
     if (e == cudaSuccess) return FC_OK;
+    cudaGetLastError();   // reported here: the thread's next launch has no part in it
     if (e == cudaErrorMemoryAllocation)
         return set_error(FC_ENOMEM, "%s: %s", what, cudaGetErrorString(e));
     return set_error(FC_ECUDA, "%s: %s", what, cudaGetErrorString(e));
@@ -167,6 +168,7 @@ cudaError_t allow_dynamic_smem(const void *fn, size_t bytes)
     // (Set again each time: a reset of the device forgets it.)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(limit, bytes));
     if (e == cudaSuccess) limit = std::max(limit, bytes);
+    else cudaGetLastError();   // (a size that does not fit is not the next launch's error)
     return e;
 }
 
